@@ -369,8 +369,12 @@ static pf_status upload_tables(pf_handle* h) {
         int prev = -2;
         for (int lt = 0; lt < tx * ty; ++lt) {
           const int sx = lt % tx, cy = lt / tx;
-          const bool edge = (sx == 0 && dd.bc[0]) || (sx == tx - 1 && dd.bc[1]) ||
-                            (cy == 0 && dd.bc[2]) || (cy == ty - 1 && dd.bc[3]);
+          // a tile pulls the ring of sites around it, and those pulls reach one
+          // site further: plain tiles stay two sites away from such a side
+          // (a last strip or tile row of one site leaves its neighbour an edge)
+          const int x0 = sx * YM_W, ya = cy * h->chunk;
+          const bool edge = (x0 < 2 && dd.bc[0]) || (x0 + YM_W > dd.nx - 2 && dd.bc[1]) ||
+                            (ya < 2 && dd.bc[2]) || (ya + h->chunk > dd.ny - 2 && dd.bc[3]);
           if (edge != (pass == 1)) continue;
           if (lt != prev + 1) {
             DomDesc r = dd;
