@@ -60,7 +60,8 @@ struct pf_handle {
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
   int variant = STEP_YMARCH;  // step kernel traversal
   int tx = 32, ty = 8;      // tile of the 2-D variant
-  int chunk = 32;           // rows per tile of the y-march variants (tuned at 4096^2)
+  int chunk = 32;           // rows per tile of the y-march variants
+  int own_chunk = 0;        // 1: set by the caller or the autotuner, else chosen by size
   int ntiles = 0;
   int grid = 0;
   int launch_mode = 0;      // 0: one launch over all domains; 1: one launch per domain
@@ -339,6 +340,57 @@ static void release(pf_handle* h) {
   h->fields = h->grain = nullptr;
 }
 
+// Rows per tile of the y-march traversals for the handle's domains.  A tile
+// streams its rows one after the other, `warm` more than it updates, so a step
+// takes about (waves of tiles over the resident CTAs) x (chunk + warm) row
+// times: long tiles waste little on a large lattice, short ones are what fills
+// the chip on a small one.  Whole waves up to four; beyond that the CTAs run
+// out of step and only half a wave is lost at the end.  Measured (FP32, us per
+// step at 32 rows and at the rows chosen): 128^2 43.1 -> 6.2 (1 row), 256^2
+// 45.1 -> 8.2 (1), 512^2 51.1 -> 18.5 (4), 1024^2 88.5 -> 66.2 (16), 4096^2
+// 868 (32; 24 rows 878, 16 rows 884).  FP64 is bound by the FP64 units, so
+// there the SM with the most tiles sets the time and a row costs its update
+// (5.6 pulls' worth with its own pull) plus two warm-up pulls per tile: 128^2
+// 763 -> 34.9 (1 row), 256^2 765 -> 105 (4).
+static int chunk_by_size(const pf_handle* h, int sms, int ctas_per_sm) {
+  const bool staged = h->variant == STEP_STAGED;
+  const int top = staged ? 48 : 32;
+  const double warm = staged ? 3.0 : 2.0;
+  double best = 0.0;
+  int pick = top;
+  for (int c = top; c >= 1; --c) {
+    long long tiles = 0;
+    for (const DomDesc& d : h->ddesc)
+      tiles += (long long)((d.nx + YM_W - 1) / YM_W) * ((d.ny + c - 1) / c);
+    double cost;
+    if (h->prec == PF_FP64) {
+      cost = (double)((tiles + sms - 1) / sms) * (5.6 * c + 2.0);
+    } else {
+      const double w = (double)tiles / ((double)sms * ctas_per_sm);
+      cost = (w > 4.0 ? w + 0.5 : std::ceil(w)) * (c + warm);
+    }
+    // shorter tiles only where they are clearly ahead: they pull more rows twice
+    if (c == top || cost < 0.97 * best) {
+      best = cost;
+      pick = c;
+    }
+  }
+  return pick;
+}
+
+static pf_status choose_chunk(pf_handle* h) {
+  if (h->own_chunk || h->variant == STEP_TILE) return PF_OK;
+  int sms = 0;
+  PF_CUDA(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
+  return dispatch(h, [&](auto s_t, auto r_t) {
+    PF_TYPES(s_t, r_t);
+    const int k = step_blocks_per_sm<S, R>(h->variant, h->tx, h->ty, h->plane_stride,
+                                           h->thermal != 0, h->any_bc != 0);
+    h->chunk = chunk_by_size(h, std::max(1, sms), std::max(1, k));
+    return PF_OK;
+  });
+}
+
 static pf_status upload_tables(pf_handle* h) {
   // tiles of every domain, in domain order
   std::vector<int> tile_dom;
@@ -503,11 +555,9 @@ extern "C" pf_status pf_create(const pf_params* p, const pf_domain* doms, int n_
     return bail(PF_ERR_CUDA, "grain table upload failed");
   // default traversal: the staged y-march for the 16-bit storage forms
   // (measured faster at 4096^2), the plain y-march otherwise
-  if ((prec == PF_FP16_OFFSET || prec == PF_BF16_OFFSET) && staged_ok(h)) {
+  if ((prec == PF_FP16_OFFSET || prec == PF_BF16_OFFSET) && staged_ok(h))
     h->variant = STEP_STAGED;
-    h->chunk = 48;
-  }
-  if (upload_tables(h) != PF_OK) return bail(PF_ERR_CUDA, h->err.c_str());
+  if (choose_chunk(h) != PF_OK || upload_tables(h) != PF_OK) return bail(PF_ERR_CUDA, h->err.c_str());
   *out = h;
   return PF_OK;
 }
@@ -992,6 +1042,7 @@ extern "C" pf_status pf_set_step_config(pf_handle* h, int variant, int a, int b)
   } else {
     return fail(h, PF_ERR_BAD_ARG, "unknown step variant");
   }
+  h->own_chunk = 1;
   PF_CUDA(h, cudaStreamSynchronize(h->stream));
   h->variant = variant;
   // captured graphs hold the old tile table's size and chunk: drop them
@@ -1094,6 +1145,7 @@ static pf_status autotune_t(pf_handle* h, int trial_steps, int out[4]) {
   h->variant = bc.variant;
   if (bc.variant != STEP_TILE) h->chunk = bc.a; else { h->tx = bc.a; h->ty = bc.b; }
   h->persistent = bc.persistent;
+  h->own_chunk = 1;
   for (auto& g : h->gexec)   // graphs captured before hold the old tiles
     if (g) { cudaGraphExecDestroy(g); g = nullptr; }
   h->coop_graph_failed = 0;
@@ -1336,7 +1388,10 @@ extern "C" pf_status pf_run(pf_handle* h, const double* fields6, size_t n, int n
     return fail(h, PF_ERR_BAD_ARG, "output buffer too small");
   const bool strip = h->variant == STEP_YMARCH || h->variant == STEP_STAGED;
   const int th = strip ? h->chunk : h->ty;
-  const int B = std::min(PF_RUN_BANDS, ((dd.ny + th - 1) / th) / 4);
+  int B = std::min(PF_RUN_BANDS, ((dd.ny + th - 1) / th) / 4);
+  // tiles chosen by size are short on a small lattice, whose bands would step
+  // faster than the host can launch them one by one: 2^18 sites a band (13 us)
+  if (!h->own_chunk) B = (int)std::min<size_t>(B, nn >> 18);
   if (n_steps == 0 || h->thermal || h->any_bc || B < 3) {
     // one after the other
     pf_status st = pf_set_fields(h, 0, fields6, nullptr, n);
@@ -1462,8 +1517,10 @@ extern "C" pf_status pf_set_boundaries(pf_handle* h, int dom, const int bc[4]) {
     }
   if (h->any_bc && h->variant != STEP_YMARCH) {
     h->variant = STEP_YMARCH;
-    h->chunk = 32;
+    h->own_chunk = 0;
   }
+  pf_status cs = choose_chunk(h);
+  if (cs != PF_OK) return cs;
   for (auto& g : h->gexec)
     if (g) { cudaGraphExecDestroy(g); g = nullptr; }
   return upload_tables(h);

@@ -1,4 +1,6 @@
-"""Tiles of the y-march at the sizes where they can go wrong."""
+"""Tiles of the y-march, their rows chosen by size, at the sizes where they can
+go wrong."""
+import numpy as np
 import pytest
 
 from paper_2407_01651_gb300 import pf
@@ -10,6 +12,25 @@ pytestmark = pytest.mark.gpu
 
 def small(nx, ny):
     return wl.Layout(nx, ny, seeds=[(nx / 2, ny / 2, 0.4)], bubbles=[(nx / 4, ny / 4, min(nx, ny) / 8)])
+
+
+@pytest.mark.parametrize("shape", [(4, 4), (64, 64), (129, 5), (300, 301), (512, 96)])
+@pytest.mark.parametrize("precision,thermal", [("fp32", 0), ("fp32", 1), ("fp64", 0), ("fp16", 0)])
+def test_rows_per_tile_do_not_change_the_bits(shape, precision, thermal):
+    """The rows per tile follow the lattice's size; every choice gives the bits
+    of 32-row tiles of the same traversal."""
+    lay = small(*shape)
+    par = dict(lay.params, thermal=thermal)
+    res = []
+    for fixed in (False, True):
+        sim = pf.Simulation([shape], par, precision)
+        if fixed:
+            sim.set_step_config(sim.step_config()[0], 32)
+        sim.init_fields(0, lay.seeds, lay.R_s, lay.bubbles)
+        sim.step(5)
+        res.append(sim.get_state())
+        assert sim.step_config()[1] == 32 if fixed else 1 <= sim.step_config()[1] <= 48
+    assert np.array_equal(res[0], res[1])
 
 
 @pytest.mark.parametrize("shape,bc,rows", [
