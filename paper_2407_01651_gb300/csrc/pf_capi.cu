@@ -84,7 +84,9 @@ struct pf_handle {
   int* d_tile_dom = nullptr;
   double* partial = nullptr;
   double* d_diag = nullptr;
-  unsigned int* d_err = nullptr;  // device error bits written by the step kernels
+  // device error bits written by the step kernels, then the block counter of
+  // the reductions (0 between them)
+  unsigned int* d_err = nullptr;
   int* d_tile_ctr = nullptr;      // two tile counters of the one-launch mode
   int drop_copies = 0;            // testing only (pf_test_drop_staged_copies)
   double* staging = nullptr;    // FP64 device staging (largest domain x 39 planes)
@@ -539,14 +541,14 @@ extern "C" pf_status pf_create(const pf_params* p, const pf_domain* doms, int n_
   h->grain_cs = (double2*)dev_alloc(h, (size_t)n_doms * MAX_GRAINS * sizeof(double2));
   h->d_doms = (DomDesc*)dev_alloc(h, (size_t)n_doms * sizeof(DomDesc));
   h->partial = (double*)dev_alloc(h, (size_t)REDUCE_BLOCKS * NDIAG * sizeof(double));
-  h->d_diag = (double*)dev_alloc(h, NDIAG * sizeof(double));
-  h->d_err = (unsigned int*)dev_alloc(h, sizeof(unsigned int));
+  h->d_diag = (double*)dev_alloc(h, (NDIAG + 1) * sizeof(double));
+  h->d_err = (unsigned int*)dev_alloc(h, 2 * sizeof(unsigned int));
   (void)max_n;
   if (!h->fields || !h->grain || !h->grain_cs || !h->d_doms || !h->partial || !h->d_diag ||
       !h->d_err)
     return bail(PF_ERR_OOM, "device allocation failed");
   if (cudaMemsetAsync(h->fields, 0, ps * N_FIELDS * h->celem, h->stream) != cudaSuccess ||
-      cudaMemsetAsync(h->d_err, 0, sizeof(unsigned int), h->stream) != cudaSuccess ||
+      cudaMemsetAsync(h->d_err, 0, 2 * sizeof(unsigned int), h->stream) != cudaSuccess ||
       cudaMemsetAsync(h->grain, 0, ps, h->stream) != cudaSuccess)
     return bail(PF_ERR_CUDA, "memset failed");
   std::vector<double2> cs((size_t)n_doms * MAX_GRAINS, make_double2(1.0, 0.0));
@@ -578,15 +580,22 @@ extern "C" const char* pf_last_error(const pf_handle* h) {
 extern "C" long long pf_steps_taken(const pf_handle* h) { return h ? h->steps : -1; }
 extern "C" long long pf_launch_count(const pf_handle* h) { return h ? h->launches : -1; }
 
-// Device error bits set by the step kernels (read after a synchronisation).
-static pf_status check_device_error(pf_handle* h) {
-  unsigned int bits = 0;
-  PF_CUDA(h, cudaMemcpy(&bits, h->d_err, sizeof(bits), cudaMemcpyDeviceToHost));
+// Device error bits set by the step kernels.
+static pf_status report_device_error(pf_handle* h, unsigned int bits) {
   if (bits & ERR_STAGED_TIMEOUT)
     return fail(h, PF_ERR_TIMEOUT,
                 "staged step: a bulk copy of an input row did not complete within 1 s; the "
                 "state is invalid");
   return PF_OK;
+}
+
+// Waits for the stream and reports the error bits: the copy of the bits is in
+// the stream, so one wait covers it and everything before it.
+static pf_status check_device_error(pf_handle* h) {
+  unsigned int bits = 0;
+  PF_CUDA(h, cudaMemcpyAsync(&bits, h->d_err, sizeof(bits), cudaMemcpyDeviceToHost, h->stream));
+  PF_CUDA(h, cudaStreamSynchronize(h->stream));
+  return report_device_error(h, bits);
 }
 
 // A re-initialised state is valid again: clear the device error bits.
@@ -607,9 +616,9 @@ extern "C" pf_status pf_test_drop_staged_copies(pf_handle* h, int on) {
 
 extern "C" pf_status pf_sync(pf_handle* h) {
   if (!h) return PF_ERR_BAD_ARG;
-  PF_CUDA(h, cudaStreamSynchronize(h->stream));
+  pf_status st = check_device_error(h);
   PF_CUDA(h, cudaGetLastError());
-  return check_device_error(h);
+  return st;
 }
 
 // ---------------------------------------------------------------------------
@@ -1214,7 +1223,6 @@ extern "C" pf_status pf_get_fields(pf_handle* h, int dom, uint32_t mask, double*
   if (!direct)
     PF_CUDA(h, cudaMemcpyAsync(host_out, h->staging, need * sizeof(double), cudaMemcpyDeviceToHost,
                                h->stream));
-  PF_CUDA(h, cudaStreamSynchronize(h->stream));
   return check_device_error(h);
 }
 
@@ -1243,12 +1251,11 @@ static pf_status run_banded(pf_handle* h, const double* in6, int n_steps, uint32
   std::vector<int> tr(B + 1);
   for (int b = 0; b <= B; ++b) tr[b] = (int)((long long)tiles_y * b / B);
   auto row = [&](int b) { return std::min(tr[b] * th, dd.ny); };
-  pf_status st = ensure_staging(h, (size_t)(6 + ns) * nn + REDUCE_BLOCKS + 1);
+  pf_status st = ensure_staging(h, (size_t)(6 + ns) * nn + REDUCE_BLOCKS);
   if (st != PF_OK) return st;
   double* d_in = h->staging;
   double* d_out = d_in + 6 * nn;
   double* d_part = d_out + (size_t)ns * nn;
-  double* d_sum = d_part + REDUCE_BLOCKS;
   // Streams by distance from the periodic seam (between bands B-1 and 0):
   // the bands far from it can run steps ahead of it, so they get the higher
   // priorities, finish first and start their copies back while the bands at
@@ -1284,13 +1291,12 @@ static pf_status run_banded(pf_handle* h, const double* in6, int n_steps, uint32
   // phi first; the bands' copies follow it
   PF_CUDA(h, cudaMemcpyAsync(d_in, in6, nn * sizeof(double), cudaMemcpyHostToDevice, S0));
   PF_CUDA(h, cudaEventRecord(h->run_phi, S0));
-  PF_CUDA(h, launch_sum_as<R>(d_in, nn, d_part, d_sum, S0));
   // rho_bar written into the device descriptor by a kernel: a copy from the
   // host would queue on the copy engine behind the bands' copies
-  PF_CUDA(h, launch_set_rho_bar(h->d_doms, 0, d_sum, (double)nn, h->p.rho_g,
-                                h->p.rho_l - h->p.rho_g, S0));
+  PF_CUDA(h, launch_rho_bar<R>(d_in, nn, d_part, h->d_err + 1, h->d_doms, 0, h->p.rho_g,
+                               h->p.rho_l - h->p.rho_g, S0));
   PF_CUDA(h, cudaEventRecord(h->run_ctl, S0));
-  h->launches += 3;
+  h->launches++;
   const int cur = h->cur;
   // the bands' copies one after the other, from the middle band outwards to
   // the seam, so that the middle bands' data arrive (and their steps start)
@@ -1428,7 +1434,6 @@ extern "C" pf_status pf_get_state(pf_handle* h, int dom, double* host_out, size_
   h->launches++;
   PF_CUDA(h, cudaMemcpyAsync(host_out, h->staging, nn * np * sizeof(double),
                              cudaMemcpyDeviceToHost, h->stream));
-  PF_CUDA(h, cudaStreamSynchronize(h->stream));
   return check_device_error(h);
 }
 
@@ -1469,8 +1474,8 @@ static pf_status reduce_t(pf_handle* h, int dom, const pf_probe* probe) {
   a.dom = h->ddesc[dom];
   a.probe = probe != nullptr;
   if (probe) { a.xc = probe->xc; a.yc = probe->yc; a.Rp = probe->R; a.W = probe->W; }
-  PF_CUDA(h, launch_reduce<R>(a, h->partial, h->d_diag, h->stream));
-  h->launches += 2;
+  PF_CUDA(h, launch_reduce<R>(a, h->partial, h->d_diag, h->d_err + 1, h->d_err, h->stream));
+  h->launches++;
   return PF_OK;
 }
 
@@ -1480,12 +1485,12 @@ extern "C" pf_status pf_reduce(pf_handle* h, int dom, const pf_probe* probe, pf_
     return fail(h, PF_ERR_BAD_ARG, "bad domain or output");
   pf_status st = h->prec == PF_FP64 ? reduce_t<double>(h, dom, probe) : reduce_t<float>(h, dom, probe);
   if (st != PF_OK) return st;
-  double buf[NDIAG];
+  double buf[NDIAG + 1];   // the diagnostics and the error bits in one copy
   PF_CUDA(h, cudaMemcpyAsync(buf, h->d_diag, sizeof(buf), cudaMemcpyDeviceToHost, h->stream));
   PF_CUDA(h, cudaStreamSynchronize(h->stream));
   static_assert(sizeof(pf_diag) == NDIAG * sizeof(double), "pf_diag layout");
-  std::memcpy(out, buf, sizeof(buf));
-  return check_device_error(h);
+  std::memcpy(out, buf, sizeof(pf_diag));
+  return report_device_error(h, (unsigned int)buf[NDIAG]);
 }
 
 // ---------------------------------------------------------------------------
@@ -1578,15 +1583,16 @@ extern "C" pf_status pf_reduce_thermal(pf_handle* h, int dom, double out[3]) {
     PF_TYPES(s_t, r_t);
     PF_CUDA(h, launch_reduce_thermal<S, R>((const S*)h->pop[h->cur], fields_ptr<R>(h),
                                            h->plane_stride, dd, h->partial, h->d_diag,
-                                           h->stream));
+                                           h->d_err + 1, h->d_err, h->stream));
     return PF_OK;
   });
   if (st != PF_OK) return st;
-  h->launches += 2;
-  PF_CUDA(h, cudaMemcpyAsync(out, h->d_diag, 3 * sizeof(double), cudaMemcpyDeviceToHost,
-                             h->stream));
+  h->launches++;
+  double buf[4];
+  PF_CUDA(h, cudaMemcpyAsync(buf, h->d_diag, sizeof(buf), cudaMemcpyDeviceToHost, h->stream));
   PF_CUDA(h, cudaStreamSynchronize(h->stream));
-  return check_device_error(h);
+  std::memcpy(out, buf, 3 * sizeof(double));
+  return report_device_error(h, (unsigned int)buf[3]);
 }
 
 // ---------------------------------------------------------------------------

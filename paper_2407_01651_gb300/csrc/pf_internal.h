@@ -140,7 +140,8 @@ cudaError_t launch_set_temperature(S* out, R* aout, R* fields, long long ps, con
                                    const double* theta, const KParams<R>& kp, cudaStream_t st);
 template <typename S, typename R>
 cudaError_t launch_reduce_thermal(const S* pop, const R* fields, long long ps, const DomDesc& d,
-                                  double* partial, double* out, cudaStream_t st);
+                                  double* partial, double* out, unsigned int* ctr,
+                                  const unsigned int* err, cudaStream_t st);
 template <typename R>
 cudaError_t launch_fields_to_f64(const R* fields, long long ps, long long off, long long n,
                                  uint32_t mask, double* out, cudaStream_t st);
@@ -149,18 +150,18 @@ template <typename R>
 cudaError_t launch_fields_to_f64_range(const R* fields, long long ps, long long off, long long n,
                                        long long j0, long long j1, uint32_t mask, double* out,
                                        cudaStream_t st);
-// *out = the FP64 sum over the n values phi[i] rounded to R, in the order of
-// the diagnostics reduction (launch_reduce): equal to its sum of phi over the
-// fields that pf_set_fields writes from the same values.  partial: REDUCE_BLOCKS doubles.
+// doms[dom].rho_bar = fma(sum / n, drho, rho_g) on the device, sum the FP64 sum
+// over the n values phi[i] rounded to R in the order of the diagnostics
+// reduction: bit for bit the rho_bar that pf_set_fields forms from the same
+// values.  partial: REDUCE_BLOCKS doubles; ctr: a device counter at 0.
 template <typename R>
-cudaError_t launch_sum_as(const double* phi, long long n, double* partial, double* out,
-                          cudaStream_t st);
-// doms[dom].rho_bar = fma(*sum / n, drho, rho_g), on the device.
-cudaError_t launch_set_rho_bar(DomDesc* doms, int dom, const double* sum, double n, double rho_g,
-                               double drho, cudaStream_t st);
+cudaError_t launch_rho_bar(const double* phi, long long n, double* partial, unsigned int* ctr,
+                           DomDesc* doms, int dom, double rho_g, double drho, cudaStream_t st);
+// FP64 diagnostics: out holds NDIAG of them (thermal totals: 3), then the
+// device error bits read from err; partial holds REDUCE_BLOCKS records.
 template <typename R>
-cudaError_t launch_reduce(const ReduceArgs<R>& a, double* partial, double* out,
-                          cudaStream_t st);
+cudaError_t launch_reduce(const ReduceArgs<R>& a, double* partial, double* out, unsigned int* ctr,
+                          const unsigned int* err, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
 // Discrete adjoint

@@ -3,13 +3,15 @@
 // itself is in pf_step.cu:
 //   k_init_spec initial fields from seeds and bubbles, equilibrium populations
 //   k_set_fields equilibrium populations from given macroscopic fields
-//   k_reduce*   FP64 diagnostics (conservation, centroid, Laplace probe)
+//   k_reduce, k_reduce_thermal, k_rho_bar  FP64 sums (conservation, centroid,
+//               Laplace probe, mean density)
 //   k_*_state   raw state to / from FP64
 //
 // Layout: structure of arrays, one plane per population / scalar, x fastest,
 // periodic domains concatenated in every plane.
 #include "pf_internal.h"
 #include "pf_device.cuh"
+#include "pf_reduce.cuh"
 
 #include <cuda_fp16.h>
 #include <cuda_bf16.h>
@@ -283,15 +285,24 @@ __global__ void k_fields_to_f64(const R* __restrict__ fields, long long ps, long
 }
 
 // ---------------------------------------------------------------------------
-// FP64 reductions: each block writes NDIAG partials, one block sums them in a
-// fixed order (deterministic).
+// FP64 reductions: each block writes one record of partial sums, the block
+// that finishes last adds them in a fixed order (pf_reduce.cuh), so that a
+// reduction is one launch.
 // ---------------------------------------------------------------------------
+// out: NDIAG diagnostics, then the device error bits.  Diagnostics cost FP64
+// instructions, of which this GPU retires few: the site's row and column come
+// from one 32-bit division, and the speed's square root is taken once, of the
+// largest square (the square root is monotone and correctly rounded).
 template <typename R>
-__global__ void k_reduce_partial(ReduceArgs<R> a, double* __restrict__ partial) {
+__global__ void __launch_bounds__(RED_THREADS) k_reduce(ReduceArgs<R> a, double* __restrict__ partial,
+                                                        double* __restrict__ out,
+                                                        unsigned int* __restrict__ ctr,
+                                                        const unsigned int* __restrict__ err) {
   double acc[NDIAG];
+#pragma unroll
   for (int q = 0; q < NDIAG; ++q) acc[q] = 0.0;
   const DomDesc d = a.dom;
-  const long long n = (long long)d.nx * d.ny;
+  const long long n = (long long)d.nx * d.ny;   // at most 2^32
   const long long ps = a.plane_stride;
   const double Rin = a.Rp - 2.0 * a.W, Rout = a.Rp + 4.0 * a.W;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -303,47 +314,41 @@ __global__ void k_reduce_partial(ReduceArgs<R> a, double* __restrict__ partial) 
     const double p = (double)a.fields[FLD_P * ps + site];
     const double vx = (double)a.fields[FLD_VX * ps + site];
     const double vy = (double)a.fields[FLD_VY * ps + site];
-    const double x = (double)(i % d.nx), y = (double)(i / d.nx);
+    const unsigned row = (unsigned)i / (unsigned)d.nx, col = (unsigned)i - row * (unsigned)d.nx;
+    const double x = (double)col, y = (double)row, gas = 1.0 - phi;
     acc[0] += phi;
     acc[1] += C;
     acc[2] += 0.5 * (1.0 + psi);
-    acc[3] += 1.0 - phi;
-    acc[4] += x * (1.0 - phi);
-    acc[5] += y * (1.0 - phi);
+    acc[3] += gas;
+    acc[4] += x * gas;
+    acc[5] += y * gas;
     if (a.probe) {
       const double dx = min_image(x - a.xc, (double)d.nx), dy = min_image(y - a.yc, (double)d.ny);
       const double r = sqrt(dx * dx + dy * dy);
       if (r < Rin) { acc[6] += p; acc[7] += 1.0; }
       if (r > Rout) { acc[8] += p; acc[9] += 1.0; }
     }
-    const double vm = sqrt(vx * vx + vy * vy);
+    const double vm = vx * vx + vy * vy;
     if (vm > acc[10]) acc[10] = vm;
     if (!isfinite(phi) || !isfinite(psi) || !isfinite(C) || !isfinite(p) || !isfinite(vx) ||
         !isfinite(vy))
       acc[11] += 1.0;
   }
-  __shared__ double sh[NDIAG][256];
-  for (int q = 0; q < NDIAG; ++q) sh[q][threadIdx.x] = acc[q];
-  __syncthreads();
-  for (int stride = blockDim.x / 2; stride > 0; stride >>= 1) {
-    if ((int)threadIdx.x < stride)
-      for (int q = 0; q < NDIAG; ++q) {
-        if (q == 10)
-          sh[q][threadIdx.x] = fmax(sh[q][threadIdx.x], sh[q][threadIdx.x + stride]);
-        else
-          sh[q][threadIdx.x] += sh[q][threadIdx.x + stride];
-      }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0)
-    for (int q = 0; q < NDIAG; ++q) partial[blockIdx.x * NDIAG + q] = sh[q][0];
+  const double r = block_sum256<NDIAG, 10>(acc);
+  if (threadIdx.x < NDIAG) partial[blockIdx.x * NDIAG + threadIdx.x] = r;
+  if (!last_block(ctr)) return;
+  const double t = sum_records256<NDIAG, 10>(partial, gridDim.x);
+  if (threadIdx.x < NDIAG) out[threadIdx.x] = threadIdx.x == 10 ? sqrt(t) : t;
+  if (threadIdx.x == 0) out[NDIAG] = (double)*err;
 }
 
 // Thermal totals (FP64): sum over sites of the five temperature populations
-// (the total of rho H), sum theta, sum psi; fixed-order partials as above.
+// (the total of rho H), sum theta, sum psi; then the device error bits.
 template <typename S, typename R>
-__global__ void k_reduce_thermal_partial(const S* __restrict__ pop, const R* __restrict__ fields,
-                                         long long ps, DomDesc d, double* __restrict__ partial) {
+__global__ void __launch_bounds__(RED_THREADS) k_reduce_thermal(
+    const S* __restrict__ pop, const R* __restrict__ fields, long long ps, DomDesc d,
+    double* __restrict__ partial, double* __restrict__ out, unsigned int* __restrict__ ctr,
+    const unsigned int* __restrict__ err) {
   double acc[3] = {0.0, 0.0, 0.0};
   const long long n = (long long)d.nx * d.ny;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
@@ -355,37 +360,12 @@ __global__ void k_reduce_thermal_partial(const S* __restrict__ pop, const R* __r
     acc[1] += (double)fields[FLD_THETA * ps + site];
     acc[2] += (double)fields[FLD_PSI * ps + site];
   }
-  __shared__ double sh[3][256];
-  for (int q = 0; q < 3; ++q) sh[q][threadIdx.x] = acc[q];
-  __syncthreads();
-  for (int stride = blockDim.x / 2; stride > 0; stride >>= 1) {
-    if ((int)threadIdx.x < stride)
-      for (int q = 0; q < 3; ++q) sh[q][threadIdx.x] += sh[q][threadIdx.x + stride];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0)
-    for (int q = 0; q < 3; ++q) partial[blockIdx.x * 3 + q] = sh[q][0];
-}
-
-__global__ void k_reduce_thermal_final(const double* __restrict__ partial, int nblocks,
-                                       double* __restrict__ out) {
-  const int q = threadIdx.x;
-  if (q >= 3) return;
-  double acc = 0.0;
-  for (int b = 0; b < nblocks; ++b) acc += partial[b * 3 + q];
-  out[q] = acc;
-}
-
-__global__ void k_reduce_final(const double* __restrict__ partial, int nblocks,
-                               double* __restrict__ out) {
-  const int q = threadIdx.x;
-  if (q >= NDIAG) return;
-  double acc = 0.0;
-  for (int b = 0; b < nblocks; ++b) {
-    const double v = partial[b * NDIAG + q];
-    acc = (q == 10) ? fmax(acc, v) : acc + v;
-  }
-  out[q] = acc;
+  const double r = block_sum256<3>(acc);
+  if (threadIdx.x < 3) partial[blockIdx.x * 3 + threadIdx.x] = r;
+  if (!last_block(ctr)) return;
+  const double t = sum_records256<3>(partial, gridDim.x);
+  if (threadIdx.x < 3) out[threadIdx.x] = t;
+  if (threadIdx.x == 0) out[3] = (double)*err;
 }
 
 // Fields [j0, j1) of a domain to FP64 (the band form of k_fields_to_f64).
@@ -405,36 +385,24 @@ __global__ void k_fields_to_f64_range(const R* __restrict__ fields, long long ps
   }
 }
 
-// FP64 sum of n values rounded to R, with the thread order and block tree of
-// the phi sum in k_reduce_partial / k_reduce_final (REDUCE_BLOCKS x 256).
+// Buoyancy reference of a domain from its n values of phi rounded to R: the
+// sum with the thread order and block tree of the phi sum in k_reduce, then
+// doms[dom].rho_bar = fma(sum / n, drho, rho_g) in the device descriptor.
 template <typename R>
-__global__ void k_sum_as_partial(const double* __restrict__ v, long long n,
-                                 double* __restrict__ partial) {
-  double acc = 0.0;
+__global__ void __launch_bounds__(RED_THREADS) k_rho_bar(const double* __restrict__ v, long long n,
+                                                         double* __restrict__ partial,
+                                                         unsigned int* __restrict__ ctr,
+                                                         DomDesc* doms, int dom, double rho_g,
+                                                         double drho) {
+  double acc[1] = {0.0};
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
-    acc += (double)static_cast<R>(v[i]);
-  __shared__ double sh[256];
-  sh[threadIdx.x] = acc;
-  __syncthreads();
-  for (int stride = blockDim.x / 2; stride > 0; stride >>= 1) {
-    if ((int)threadIdx.x < stride) sh[threadIdx.x] += sh[threadIdx.x + stride];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) partial[blockIdx.x] = sh[0];
-}
-
-__global__ void k_sum_final(const double* __restrict__ partial, int nblocks,
-                            double* __restrict__ out) {
-  if (threadIdx.x != 0) return;
-  double acc = 0.0;
-  for (int b = 0; b < nblocks; ++b) acc = acc + partial[b];
-  *out = acc;
-}
-
-__global__ void k_set_rho_bar(DomDesc* doms, int dom, const double* __restrict__ sum, double n,
-                              double rho_g, double drho) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) doms[dom].rho_bar = fma(*sum / n, drho, rho_g);
+    acc[0] += (double)static_cast<R>(v[i]);
+  const double r = block_sum256<1>(acc);
+  if (threadIdx.x == 0) partial[blockIdx.x] = r;
+  if (!last_block(ctr)) return;
+  const double t = sum_records256<1>(partial, gridDim.x);
+  if (threadIdx.x == 0) doms[dom].rho_bar = fma(t / (double)n, drho, rho_g);
 }
 
 // ---------------------------------------------------------------------------
@@ -500,11 +468,18 @@ cudaError_t launch_set_temperature(S* out, R* aout, R* fields, long long ps, con
   return cudaGetLastError();
 }
 
+// Blocks of a reduction over n sites (a record each; the phi sums of k_reduce
+// and k_rho_bar agree bit for bit because both take this grid).
+static int reduce_grid(long long n) {
+  return (int)std::min<long long>((n + RED_THREADS - 1) / RED_THREADS, REDUCE_BLOCKS);
+}
+
 template <typename S, typename R>
 cudaError_t launch_reduce_thermal(const S* pop, const R* fields, long long ps, const DomDesc& d,
-                                  double* partial, double* out, cudaStream_t st) {
-  k_reduce_thermal_partial<S, R><<<REDUCE_BLOCKS, 256, 0, st>>>(pop, fields, ps, d, partial);
-  k_reduce_thermal_final<<<1, 32, 0, st>>>(partial, REDUCE_BLOCKS, out);
+                                  double* partial, double* out, unsigned int* ctr,
+                                  const unsigned int* err, cudaStream_t st) {
+  k_reduce_thermal<S, R><<<reduce_grid((long long)d.nx * d.ny), RED_THREADS, 0, st>>>(
+      pop, fields, ps, d, partial, out, ctr, err);
   return cudaGetLastError();
 }
 
@@ -525,24 +500,18 @@ cudaError_t launch_fields_to_f64_range(const R* fields, long long ps, long long 
 }
 
 template <typename R>
-cudaError_t launch_sum_as(const double* phi, long long n, double* partial, double* out,
-                          cudaStream_t st) {
-  k_sum_as_partial<R><<<REDUCE_BLOCKS, 256, 0, st>>>(phi, n, partial);
-  k_sum_final<<<1, 32, 0, st>>>(partial, REDUCE_BLOCKS, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_set_rho_bar(DomDesc* doms, int dom, const double* sum, double n, double rho_g,
-                               double drho, cudaStream_t st) {
-  k_set_rho_bar<<<1, 32, 0, st>>>(doms, dom, sum, n, rho_g, drho);
+cudaError_t launch_rho_bar(const double* phi, long long n, double* partial, unsigned int* ctr,
+                           DomDesc* doms, int dom, double rho_g, double drho, cudaStream_t st) {
+  k_rho_bar<R><<<reduce_grid(n), RED_THREADS, 0, st>>>(phi, n, partial, ctr, doms, dom, rho_g,
+                                                       drho);
   return cudaGetLastError();
 }
 
 template <typename R>
-cudaError_t launch_reduce(const ReduceArgs<R>& a, double* partial, double* out,
-                          cudaStream_t st) {
-  k_reduce_partial<R><<<REDUCE_BLOCKS, 256, 0, st>>>(a, partial);
-  k_reduce_final<<<1, 32, 0, st>>>(partial, REDUCE_BLOCKS, out);
+cudaError_t launch_reduce(const ReduceArgs<R>& a, double* partial, double* out, unsigned int* ctr,
+                          const unsigned int* err, cudaStream_t st) {
+  k_reduce<R><<<reduce_grid((long long)a.dom.nx * a.dom.ny), RED_THREADS, 0, st>>>(a, partial, out,
+                                                                                   ctr, err);
   return cudaGetLastError();
 }
 
@@ -558,6 +527,7 @@ cudaError_t launch_reduce(const ReduceArgs<R>& a, double* partial, double* out,
                                                     cudaStream_t);                           \
   template cudaError_t launch_reduce_thermal<S, R>(const S*, const R*, long long,            \
                                                    const DomDesc&, double*, double*,         \
+                                                   unsigned int*, const unsigned int*,       \
                                                    cudaStream_t);
 
 PF_INST(double, double)
@@ -575,13 +545,13 @@ template cudaError_t launch_fields_to_f64_range<double>(const double*, long long
 template cudaError_t launch_fields_to_f64_range<float>(const float*, long long, long long,
                                                        long long, long long, long long, uint32_t,
                                                        double*, cudaStream_t);
-template cudaError_t launch_sum_as<double>(const double*, long long, double*, double*,
-                                           cudaStream_t);
-template cudaError_t launch_sum_as<float>(const double*, long long, double*, double*,
-                                          cudaStream_t);
+template cudaError_t launch_rho_bar<double>(const double*, long long, double*, unsigned int*,
+                                            DomDesc*, int, double, double, cudaStream_t);
+template cudaError_t launch_rho_bar<float>(const double*, long long, double*, unsigned int*,
+                                           DomDesc*, int, double, double, cudaStream_t);
 template cudaError_t launch_reduce<double>(const ReduceArgs<double>&, double*, double*,
-                                           cudaStream_t);
+                                           unsigned int*, const unsigned int*, cudaStream_t);
 template cudaError_t launch_reduce<float>(const ReduceArgs<float>&, double*, double*,
-                                          cudaStream_t);
+                                          unsigned int*, const unsigned int*, cudaStream_t);
 
 }  // namespace pf

@@ -18,6 +18,7 @@
 
 #include "../../include/pf.h"
 #include "pf_internal.h"
+#include "pf_reduce.cuh"
 
 namespace {
 
@@ -95,17 +96,11 @@ __global__ void __launch_bounds__(kThreads) k_noalloc_partial(
   if (threadIdx.x < pf::NDIAG) scratch[blockIdx.x * pf::NDIAG + threadIdx.x] = red[threadIdx.x][0];
 }
 
-// One warp: record q of the final result sums (or maxes) the block records
-// in block order, so the result does not depend on scheduling.
-__global__ void k_noalloc_final(double* __restrict__ scratch, int nblocks) {
-  const int q = threadIdx.x;
-  if (q >= pf::NDIAG) return;
-  double acc = 0.0;
-  for (int b = 0; b < nblocks; ++b) {
-    const double v = scratch[b * pf::NDIAG + q];
-    acc = q == 10 ? fmax(acc, v) : acc + v;
-  }
-  scratch[kMaxBlocks * pf::NDIAG + q] = acc;
+// One block: the final result, in an order fixed by the record numbers.
+__global__ void __launch_bounds__(pf::RED_THREADS) k_noalloc_final(double* __restrict__ scratch,
+                                                                   int nblocks) {
+  const double r = pf::sum_records256<pf::NDIAG, 10>(scratch, nblocks);
+  if (threadIdx.x < pf::NDIAG) scratch[kMaxBlocks * pf::NDIAG + threadIdx.x] = r;
 }
 
 // Device address of the scratch array in the current context.  The host-side
@@ -162,7 +157,7 @@ extern "C" pf_status pf_reduce_noalloc(const void* fields, int fields_fp64, long
   else
     k_noalloc_partial<float><<<nblocks, kThreads, 0, stream>>>(
         static_cast<const float*>(fields), plane_stride, offset, nx, ny, pr, xc, yc, R, W, scratch);
-  k_noalloc_final<<<1, 32, 0, stream>>>(scratch, nblocks);
+  k_noalloc_final<<<1, pf::RED_THREADS, 0, stream>>>(scratch, nblocks);
   double res[pf::NDIAG];
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess)

@@ -20,6 +20,7 @@
 
 #include "../../include/pf.h"
 #include "pf_d3.cuh"
+#include "pf_reduce.cuh"
 
 namespace pf {
 namespace d3 {
@@ -554,12 +555,6 @@ __global__ void k_reduce3(const R* f, unsigned long long ps, unsigned long long 
   }
   if (threadIdx.x == 0) { part[2 * blockIdx.x] = sh[0][0]; part[2 * blockIdx.x + 1] = sh[1][0]; }
 }
-__global__ void k_reduce3_final(const double* part, int nb, int k, double* out) {
-  if ((int)threadIdx.x >= k) return;
-  double acc = 0.0;
-  for (int b = 0; b < nb; ++b) acc += part[k * b + threadIdx.x];
-  out[threadIdx.x] = acc;
-}
 
 // Thermal totals: sum of the seven temperature populations (rho H), sum theta,
 // sum psi; fixed-order partials.
@@ -1036,7 +1031,7 @@ extern "C" pf_status pf3_reduce(pf3_handle* h, double out[2]) {
   if (st != PF_OK) return st;
   if (h->prec == PF_FP64) k_reduce3<double><<<nb, 256, 0, h->stream>>>((const double*)h->fields, h->n, h->n, h->scratch);
   else k_reduce3<float><<<nb, 256, 0, h->stream>>>((const float*)h->fields, h->n, h->n, h->scratch);
-  k_reduce3_final<<<1, 32, 0, h->stream>>>(h->scratch, nb, 2, h->scratch + 2 * nb);
+  k_sum_records<2><<<1, RED_THREADS, 0, h->stream>>>(h->scratch, nb, h->scratch + 2 * nb);
   PF3_CUDA(h, cudaGetLastError());
   h->launches += 2;
   PF3_CUDA(h, cudaMemcpyAsync(out, h->scratch + 2 * nb, 2 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
@@ -1056,7 +1051,7 @@ extern "C" pf_status pf3_reduce_thermal(pf3_handle* h, double out[3]) {
     using R = decltype(r_t);
     k_reduce3_th<S, R><<<nb, 256, 0, h->stream>>>((const S*)h->pop[h->cur], (const R*)h->fields,
                                                    h->n, h->n, h->scratch);
-    k_reduce3_final<<<1, 32, 0, h->stream>>>(h->scratch, nb, 3, h->scratch + 3 * nb);
+    k_sum_records<3><<<1, RED_THREADS, 0, h->stream>>>(h->scratch, nb, h->scratch + 3 * nb);
     PF3_CUDA(h, cudaGetLastError());
     return PF_OK;
   });

@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "pf_step3f.cuh"
+#include "pf_reduce.cuh"
 
 namespace pf {
 namespace d3f {
@@ -220,12 +221,6 @@ __global__ void k_reducef(const R* f, unsigned long long ps, unsigned long long 
   if (threadIdx.x == 0)
     for (int q = 0; q < 3; ++q) part[3 * blockIdx.x + q] = sh[q][0];
 }
-__global__ void k_reducef_final(const double* part, int nb, double* out) {
-  if (threadIdx.x >= 3) return;
-  double acc = 0.0;
-  for (int b = 0; b < nb; ++b) acc += part[3 * b + threadIdx.x];
-  out[threadIdx.x] = acc;
-}
 
 }  // namespace d3f
 }  // namespace pf
@@ -367,7 +362,7 @@ static pf_status reduce_fields(pf3f_handle* h, double out[3]) {
   if (st != PF_OK) return st;
   if (h->prec == PF_FP64) k_reducef<double><<<nb, 256, 0, h->stream>>>((const double*)h->fields, h->n, h->n, h->scratch);
   else k_reducef<float><<<nb, 256, 0, h->stream>>>((const float*)h->fields, h->n, h->n, h->scratch);
-  k_reducef_final<<<1, 32, 0, h->stream>>>(h->scratch, nb, h->scratch + 3 * nb);
+  k_sum_records<3><<<1, RED_THREADS, 0, h->stream>>>(h->scratch, nb, h->scratch + 3 * nb);
   PF3F_CUDA(h, cudaGetLastError());
   h->launches += 2;
   PF3F_CUDA(h, cudaMemcpyAsync(out, h->scratch + 3 * nb, 3 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
@@ -766,7 +761,7 @@ extern "C" pf_status pf3f_reduce_thermal(pf3f_handle* h, double out[3]) {
     using R = decltype(r_t);
     k_reducef_th<S, R><<<nb, 256, 0, h->stream>>>((const S*)h->pop[h->cur], (const R*)h->fields,
                                                    h->n, h->n, h->scratch);
-    k_reducef_final<<<1, 32, 0, h->stream>>>(h->scratch, nb, h->scratch + 3 * nb);
+    k_sum_records<3><<<1, RED_THREADS, 0, h->stream>>>(h->scratch, nb, h->scratch + 3 * nb);
     PF3F_CUDA(h, cudaGetLastError());
     return PF_OK;
   });

@@ -1,5 +1,5 @@
-"""Tiles of the y-march, their rows chosen by size, at the sizes where they can
-go wrong."""
+"""Tiles chosen by size, tiles next to non-periodic sides, and the one-launch
+FP64 reductions, at the sizes where they can go wrong."""
 import numpy as np
 import pytest
 
@@ -54,3 +54,24 @@ def test_tiles_next_to_a_side(shape, bc, rows):
         o.step(1)
         sim.step(1)
         compare(o, sim, 1e-11, early=True)
+
+
+@pytest.mark.parametrize("shape", [(4, 4), (16, 16), (33, 31), (700, 600)])
+def test_reductions_equal_the_sums_of_the_fields(shape):
+    """pf_reduce against numpy FP64 sums of the fields it reads; a sum of n
+    terms in another order differs by at most n eps of the sum of magnitudes."""
+    lay = small(*shape)
+    sim = pf.Simulation([shape], lay.params, "fp64")
+    sim.init_fields(0, lay.seeds, lay.R_s, lay.bubbles)
+    sim.step(2)
+    for _ in range(2):     # the block counter is back at zero after a call
+        d, f = sim.reduce(0), sim.fields()
+        x, y = np.arange(shape[0])[None, :], np.arange(shape[1])[:, None]
+        gas = 1.0 - f["phi"]
+        want = dict(sum_phi=f["phi"], sum_C=f["C"], sum_hpsi=0.5 * (1 + f["psi"]), gas=gas,
+                    gas_x=x * gas, gas_y=y * gas)
+        for k, v in want.items():
+            assert abs(d[k] - v.sum()) <= v.size * 2.3e-16 * np.abs(v).sum() + 1e-300, k
+        assert d["max_v"] == np.sqrt(f["vx"] ** 2 + f["vy"] ** 2).max() or np.isclose(
+            d["max_v"], np.sqrt(f["vx"] ** 2 + f["vy"] ** 2).max(), rtol=1e-15)
+        assert d["nonfinite"] == 0
