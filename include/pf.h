@@ -171,8 +171,10 @@ pf_status pf_params_derived(const pf_params *p, double out[3]);
 /* Create a handle for n_doms periodic domains (n_doms >= 1, each nx, ny in
  * [4, 65536]; fewer than 2^32 sites in all, each domain padded to a multiple
  * of 64).  cuda_stream: a cudaStream_t (NULL = legacy default stream).
- * alloc may be NULL (cudaMalloc).  Allocates two copies of the 39-plane state
- * (about 2 x 160 B per site in FP32), the field planes and reduction scratch.
+ * alloc may be NULL (cudaMalloc).  Allocates two copies of the state (23
+ * population planes, of each opposite pair of a lattice whose even moments
+ * are slaved to its density only one, and 7 lagged planes: about 2 x 120 B
+ * per site in FP32), the field planes and reduction scratch.
  * Errors: BAD_ARG, OOM, CUDA. */
 pf_status pf_create(const pf_params *p, const pf_domain *doms, int n_doms,
                     pf_precision prec, void *cuda_stream, const pf_allocator *alloc,
@@ -279,7 +281,9 @@ pf_status pf_run(pf_handle *h, const double *fields6, size_t n, int n_steps, uin
 
 /* Raw state of domain dom (pf_state_planes(h) planes, FP64) to / from the
  * host: checkpoint and restart.  Synchronise the stream.  pf_set_state marks
- * the domain initialised.  Errors: BAD_ARG (domain, NULL, a buffer of the
+ * the domain initialised.  Its populations may be any: where they are not what
+ * a step leaves behind (to a few ulp), the planes stay on the device in FP64
+ * until the domain's next step, which starts from them.  Errors: BAD_ARG (domain, NULL, a buffer of the
  * wrong size: at least / exactly planes x nx x ny values), OOM (staging),
  * CUDA; pf_get_state also TIMEOUT (a staged step's wait ran out before the
  * call: the state is invalid), which pf_set_state clears. */

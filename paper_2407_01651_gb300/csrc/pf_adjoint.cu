@@ -17,7 +17,7 @@
 // Adjoint planes are in the compute precision.  The FP32 and FP64 storage
 // forms are supported.
 #include "pf_local.cuh"
-#include "pf_pull.cuh"
+#include "pf_raw.cuh"
 
 namespace pf {
 
@@ -46,7 +46,9 @@ __device__ __forceinline__ local::Coef<R> make_coef(const KParams<R>& kp, const 
 }  // namespace
 
 // ---------------------------------------------------------------------------
-template <typename S, typename R, bool BIG>
+// RAW: x_t is a raw state (its pulls from a.raw; the first state after a
+// pf_set_state of populations that no collision made).
+template <typename S, typename R, bool BIG, bool RAW>
 __global__ void __launch_bounds__(256, 2) k_adj_local(AdjArgs<S, R> a) {
   __shared__ R sphi[ADJ_TY + 2][ADJ_TX + 2], spsi[ADJ_TY + 2][ADJ_TX + 2];
   __shared__ R svx[ADJ_TY + 2][ADJ_TX + 2], svy[ADJ_TY + 2][ADJ_TX + 2];
@@ -57,6 +59,21 @@ __global__ void __launch_bounds__(256, 2) k_adj_local(AdjArgs<S, R> a) {
   const int tid = threadIdx.y * ADJ_TX + threadIdx.x;
   const int tiles_x = (d.nx + ADJ_TX - 1) / ADJ_TX;
   const int ntiles = tiles_x * ((d.ny + ADJ_TY - 1) / ADJ_TY);
+  const RawState<S, R> rs{a.raw, (long long)d.nx * d.ny};
+  const GeneralPull<S, R, false> raw{rs, st, d};
+  // streamed dendrite populations, phi, psi and the lagged velocity of a site
+  auto pull = [&](const Src9& src, int x, int y, R (&g)[5], R& phi, R& psi, R& psio, R& vx, R& vy) {
+    V2<R> J;
+    if constexpr (RAW) {
+      raw.hg(x, y, J, g, phi, psi, psio);
+      vx = rs.x(X_VX, raw.local(src.s[0]));
+      vy = rs.x(X_VY, raw.local(src.s[0]));
+    } else {
+      pull_hg<S, R, BIG>(st, src, J, g, phi, psi, psio);
+      vx = ld<R>(st.ain + A_VXO * ps, src.s[0]);
+      vy = ld<R>(st.ain + A_VYO * ps, src.s[0]);
+    }
+  };
   R pe = R(0), po = R(0), psg = R(0);
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     const int x0 = (tile % tiles_x) * ADJ_TX, y0 = (tile / tiles_x) * ADJ_TY;
@@ -71,11 +88,13 @@ __global__ void __launch_bounds__(256, 2) k_adj_local(AdjArgs<S, R> a) {
     {
       R phi, psi;
       src = sources(d, x % d.nx, y % d.ny);
-      pull_hg<S, R, BIG>(st, src, in.h, in.g, phi, psi, in.psio);
-      sphi[threadIdx.y + 1][threadIdx.x + 1] = phi;
-      spsi[threadIdx.y + 1][threadIdx.x + 1] = psi;
-      svx[threadIdx.y + 1][threadIdx.x + 1] = ld<R>(st.ain + A_VXO * ps, src.s[0]);
-      svy[threadIdx.y + 1][threadIdx.x + 1] = ld<R>(st.ain + A_VYO * ps, src.s[0]);
+      const int ty = threadIdx.y + 1, tx = threadIdx.x + 1;
+      pull(src, x % d.nx, y % d.ny, in.g, phi, psi, in.psio, svx[ty][tx], svy[ty][tx]);
+      sphi[ty][tx] = phi;
+      spsi[ty][tx] = psi;
+      // the reverse reads the streamed h only through their sum
+      in.h[0] = phi;
+      for (int i = 1; i < 9; ++i) in.h[i] = R(0);
     }
     if (tid < 2 * (ADJ_TX + 2) + 2 * ADJ_TY) {
       int lx, ly;
@@ -86,18 +105,16 @@ __global__ void __launch_bounds__(256, 2) k_adj_local(AdjArgs<S, R> a) {
       int gx = x0 + lx - 1, gy = y0 + ly - 1;
       gx = ((gx % d.nx) + d.nx) % d.nx;
       gy = ((gy % d.ny) + d.ny) % d.ny;
-      R h[9], g[5], phi, psi, pso;
-      const Src9 hs = sources(d, gx, gy);
-      pull_hg<S, R, BIG>(st, hs, h, g, phi, psi, pso);
+      R g[5], phi, psi, pso;
+      pull(sources(d, gx, gy), gx, gy, g, phi, psi, pso, svx[ly][lx], svy[ly][lx]);
       sphi[ly][lx] = phi;
       spsi[ly][lx] = psi;
-      svx[ly][lx] = ld<R>(st.ain + A_VXO * ps, hs.s[0]);
-      svy[ly][lx] = ld<R>(st.ain + A_VYO * ps, hs.s[0]);
     }
     __syncthreads();
     if (inside) {
       SiteIn<R> si;
-      load_site<S, R, BIG>(st, src, si);
+      if constexpr (RAW) raw.site(x, y, si);
+      else load_site<S, R, BIG>(st, src, si);
       for (int i = 0; i < 9; ++i) in.f[i] = si.f[i];
       for (int i = 0; i < 5; ++i) in.s[i] = si.s[i];
       in.phio = si.phio;
@@ -274,6 +291,8 @@ __global__ void __launch_bounds__(ADJ_TX * ADJ_TY) k_adj_transpose(AdjArgs<S, R>
     }
     rr_own = __ldg(plane(X, A_RR, ps) + site);
     apsio = __ldg(plane(A, AI_PSIO, ps) + site);
+    const R gm = ld<R>(plane(P, P_GPOST, ps), site), gbase = q5_base(gm);
+    const S gpair[2] = {__ldg(plane(P, P_GPOST + 1, ps) + site), __ldg(plane(P, P_GPOST + 2, ps) + site)};
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
       const unsigned t = src.s[OPP[q]];   // destination of q
@@ -282,7 +301,10 @@ __global__ void __launch_bounds__(ADJ_TX * ADJ_TY) k_adj_transpose(AdjArgs<S, R>
       gown[q] = __ldg(plane(A, AI_G + q, ps) + site);
       gdst[q] = __ldg(plane(A, AI_G + q, ps) + t);
       rsrc[q] = __ldg(plane(X, A_RR, ps) + sq);
-      gdiff[q] = ld<R>(plane(P, P_GPOST + q, ps), site) - ld<R>(plane(P, P_GPRE + q, ps), t);
+      const R gp = q == 0 ? q5_rest(gm, gbase)
+                          : (minus9(q) ? pair_m<S, R>(gpair[(q - 1) & 1], gbase)
+                                       : pair_p<S, R>(gpair[(q - 1) & 1], gbase));
+      gdiff[q] = gp - ld<R>(plane(P, P_GPRE + q, ps), t);
     }
     plane(L, 34, ps)[site] = __ldg(plane(A, AI_PHIO, ps) + site);
     plane(L, 35, ps)[site] = __ldg(plane(A, AI_CO, ps) + site);
@@ -357,10 +379,12 @@ __global__ void k_adj_omega_init(const R* __restrict__ L, const S* __restrict__ 
 // ---------------------------------------------------------------------------
 template <typename S, typename R>
 cudaError_t launch_adjoint_step(const AdjArgs<S, R>& a, int grid, cudaStream_t st) {
-  if ((unsigned long long)a.step.plane_stride * N_POP >= (1ull << 32))
-    k_adj_local<S, R, true><<<grid, dim3(ADJ_TX, ADJ_TY), 0, st>>>(a);
+  if (a.raw)
+    k_adj_local<S, R, true, true><<<grid, dim3(ADJ_TX, ADJ_TY), 0, st>>>(a);
+  else if ((unsigned long long)a.step.plane_stride * N_POP >= (1ull << 32))
+    k_adj_local<S, R, true, false><<<grid, dim3(ADJ_TX, ADJ_TY), 0, st>>>(a);
   else
-    k_adj_local<S, R, false><<<grid, dim3(ADJ_TX, ADJ_TY), 0, st>>>(a);
+    k_adj_local<S, R, false, false><<<grid, dim3(ADJ_TX, ADJ_TY), 0, st>>>(a);
   const int tiles = ((a.dom.nx + ADJ_TX - 1) / ADJ_TX) * ((a.dom.ny + ADJ_TY - 1) / ADJ_TY);
   k_adj_transpose<S, R><<<tiles, dim3(ADJ_TX, ADJ_TY), 0, st>>>(a);
   return cudaGetLastError();

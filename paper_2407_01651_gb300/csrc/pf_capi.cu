@@ -1,8 +1,8 @@
 // pf_capi.cu -- implementation of the C ABI declared in include/pf.h.
 //
 // A handle owns, for all of its domains together:
-//   - two copies of the 39-plane state (45 in thermal mode; ping-pong of the
-//     pull scheme),
+//   - two copies of the 29-plane state (33 in thermal mode; ping-pong of the
+//     pull scheme; pf_model.cuh),
 //   - 9 field planes in compute precision (written by the last step of each
 //     pf_step call and by the initialisation),
 //   - a uint8 grain id per site and a (cos, sin) table per domain,
@@ -42,7 +42,6 @@ struct pf_handle {
   size_t celem = 4;         // bytes per compute value
   int thermal = 0;          // temperature lattice and finite-Le F(U)
   int n_pop = N_POP;        // population planes per state copy
-  int n_aux = N_AUX;        // lagged-scalar planes per state copy
   int n_phys = N_PHYS;      // planes of the raw FP64 state
   int any_bc = 0;           // some domain has a non-periodic side
   int any_io = 0;           // ... among them an inlet or an outlet
@@ -91,6 +90,10 @@ struct pf_handle {
   int drop_copies = 0;            // testing only (pf_test_drop_staged_copies)
   double* staging = nullptr;    // FP64 device staging (largest domain x 39 planes)
   size_t staging_elems = 0;
+  // raw FP64 planes of a domain whose state pf_set_state gave populations that
+  // no collision made (pf_step_general.cu), until its next step; else nullptr
+  std::vector<double*> raw;
+  std::vector<double*> spent;   // raw planes a step has consumed, freed at the next wait
   long long steps = 0;
   long long launches = 0;
   std::string err;
@@ -264,9 +267,29 @@ static pf_status check_params(const pf_params* p) {
 template <typename R>
 static R* fields_ptr(pf_handle* h) { return reinterpret_cast<R*>(h->fields); }
 
+// The raw planes of a domain are not its state any more; work that reads them
+// may still be in the stream, so they are freed where the stream was waited for.
+static void drop_raw(pf_handle* h, int dom) {
+  if (h->raw[dom]) h->spent.push_back(h->raw[dom]);
+  h->raw[dom] = nullptr;
+}
+static void free_spent(pf_handle* h) {
+  for (double* r : h->spent) dev_free(h, r);
+  h->spent.clear();
+}
+static bool any_raw(const pf_handle* h) {
+  for (const double* r : h->raw)
+    if (r) return true;
+  return false;
+}
+
 // FP64 device staging for host transfers, grown on demand (never on the
 // stepping path).
 static pf_status ensure_staging(pf_handle* h, size_t elems) {
+  if (!h->spent.empty()) {
+    cudaStreamSynchronize(h->stream);
+    free_spent(h);
+  }
   if (elems <= h->staging_elems) return PF_OK;
   cudaStreamSynchronize(h->stream);
   dev_free(h, h->staging);
@@ -322,6 +345,9 @@ static void release(pf_handle* h) {
   dev_free(h, h->d_tile_ctr);
   h->d_tile_ctr = nullptr;
   dev_free(h, h->staging);
+  for (double*& r : h->raw) { dev_free(h, r); r = nullptr; }
+  for (double* r : h->spent) dev_free(h, r);
+  h->spent.clear();
   dev_free(h, h->adj_ws);
   h->adj_ws = nullptr;
   for (auto& g : h->gexec)
@@ -496,10 +522,10 @@ extern "C" pf_status pf_create(const pf_params* p, const pf_domain* doms, int n_
   h->celem = prec == PF_FP64 ? 8 : 4;
   h->thermal = p->thermal;
   h->n_pop = p->thermal ? N_POP_TH : N_POP;
-  h->n_aux = p->thermal ? N_AUX_TH : N_AUX;
   h->n_phys = p->thermal ? N_PHYS_TH : N_PHYS;
   h->doms.assign(doms, doms + n_doms);
   h->inited.assign(n_doms, 0);
+  h->raw.assign(n_doms, nullptr);
   long long off = 0;
   size_t max_n = 0;
   for (int d = 0; d < n_doms; ++d) {
@@ -533,7 +559,7 @@ extern "C" pf_status pf_create(const pf_params* p, const pf_domain* doms, int n_
   };
   for (int c = 0; c < 2; ++c) {
     h->pop[c] = dev_alloc(h, ps * h->n_pop * h->elem);
-    h->aux[c] = dev_alloc(h, ps * h->n_aux * h->celem);
+    h->aux[c] = dev_alloc(h, ps * N_AUX * h->celem);
     if (!h->pop[c] || !h->aux[c]) return bail(PF_ERR_OOM, "state allocation failed");
   }
   h->fields = dev_alloc(h, ps * N_FIELDS * h->celem);
@@ -696,6 +722,7 @@ extern "C" pf_status pf_init_fields(pf_handle* h, int dom, const pf_init_spec* s
     if (!std::isfinite(spec->bubbles[i])) return fail(h, PF_ERR_BAD_ARG, "non-finite bubble");
   std::vector<double> angles;
   for (int s = 0; s < spec->n_seeds; ++s) angles.push_back(spec->seeds[3 * s + 2]);
+  drop_raw(h, dom);
   pf_status st = clear_device_error(h);
   if (st != PF_OK) return st;
   st = upload_grain_table(h, dom, angles);
@@ -764,6 +791,7 @@ extern "C" pf_status pf_set_fields(pf_handle* h, int dom, const double* fields6,
       ids[i] = (uint8_t)it->second;
     }
   }
+  drop_raw(h, dom);
   pf_status st = clear_device_error(h);
   if (st != PF_OK) return st;
   st = upload_grain_table(h, dom, angles);
@@ -935,6 +963,42 @@ static pf_status step_t(pf_handle* h, bool write_fields, cudaStream_t stream = n
   return PF_OK;
 }
 
+// The step after a pf_set_state of populations that no collision made: those
+// domains from their raw planes, the others as ever, one launch per domain.
+template <typename S, typename R>
+static pf_status step_general_t(pf_handle* h, bool write_fields) {
+  const StepArgs<S, R> a0 = make_step_args<S, R>(h, h->pop[h->cur], h->aux[h->cur],
+                                                 h->pop[h->cur ^ 1], h->aux[h->cur ^ 1],
+                                                 write_fields);
+  auto go = [&](int t0, int t1, int bc) -> pf_status {
+    if (t1 <= t0) return PF_OK;
+    StepArgs<S, R> a = a0;
+    a.tile_base = t0;
+    a.ntiles = t1;
+    a.bc = bc;
+    PF_CUDA(h, launch_step<S, R>(a, h->variant, h->tx, h->ty, t1 - t0, h->stream));
+    h->launches++;
+    return PF_OK;
+  };
+  for (size_t d = 0; d < h->ddesc.size(); ++d) {
+    pf_status st;
+    if (h->raw[d]) {
+      PF_CUDA(h, launch_step_general<S, R>(a0, h->ddesc[d], h->raw[d], h->stream));
+      h->launches++;
+    } else if (h->any_bc) {
+      if ((st = go(h->plain0[d], h->plain1[d], 0)) != PF_OK) return st;
+      if ((st = go(h->edge0[d], h->edge1[d], h->any_io ? 2 : 1)) != PF_OK) return st;
+    } else {
+      const int t1 = d + 1 < h->ddesc.size() ? h->ddesc[d + 1].tile0 : h->ntiles;
+      if ((st = go(h->ddesc[d].tile0, t1, 0)) != PF_OK) return st;
+    }
+  }
+  for (size_t d = 0; d < h->raw.size(); ++d) drop_raw(h, (int)d);
+  h->cur ^= 1;
+  h->steps++;
+  return PF_OK;
+}
+
 // Executable graph of graph_steps steps (no field output) starting from the
 // current buffer parity; captured on an internal stream, replayed on the
 // handle's stream.  graph_steps is even, so the parity is unchanged.
@@ -975,6 +1039,11 @@ static pf_status ensure_graph(pf_handle* h) {
 template <typename S, typename R>
 static pf_status step_n(pf_handle* h, int n_steps) {
   int done = 0;
+  if (n_steps > 0 && any_raw(h)) {
+    pf_status st = step_general_t<S, R>(h, n_steps == 1);
+    if (st != PF_OK) return st;
+    done = 1;
+  }
   if (steps_in_one_launch(h)) {
     // graph_steps > 0: whole graph_steps-step launches replayed from graphs,
     // then the rest (with the field output) in one more launch
@@ -1093,7 +1162,7 @@ extern "C" pf_status pf_set_launch(pf_handle* h, int per_domain, int persistent,
 template <typename S, typename R>
 static pf_status autotune_t(pf_handle* h, int trial_steps, int out[4]) {
   const size_t ps = (size_t)h->plane_stride;
-  const size_t pop_b = ps * h->n_pop * sizeof(S), aux_b = ps * h->n_aux * sizeof(R);
+  const size_t pop_b = ps * h->n_pop * sizeof(S), aux_b = ps * N_AUX * sizeof(R);
   void* snap_p = dev_alloc(h, pop_b);
   void* snap_a = dev_alloc(h, aux_b);
   if (!snap_p || !snap_a) {
@@ -1284,6 +1353,7 @@ static pf_status run_banded(pf_handle* h, const double* in6, int n_steps, uint32
   if (!h->run_phi) PF_CUDA(h, cudaEventCreateWithFlags(&h->run_phi, cudaEventDisableTiming));
   if (!h->run_ctl) PF_CUDA(h, cudaEventCreateWithFlags(&h->run_ctl, cudaEventDisableTiming));
   cudaStream_t S0 = h->stream;
+  drop_raw(h, 0);
   st = clear_device_error(h);
   if (st != PF_OK) return st;
   st = upload_grain_table(h, 0, {});
@@ -1425,9 +1495,14 @@ extern "C" pf_status pf_get_state(pf_handle* h, int dom, double* host_out, size_
   if (st != PF_OK) return st;
   st = dispatch(h, [&](auto s_t, auto r_t) {
     PF_TYPES(s_t, r_t);
-    PF_CUDA(h, launch_state_to_f64<S, R>((const S*)h->pop[h->cur], (const R*)h->aux[h->cur],
-                                         h->plane_stride, dd.off, (long long)nn, h->staging,
-                                         h->thermal, h->stream));
+    if (h->raw[dom])
+      PF_CUDA(h, launch_raw_rounded<S, R>(h->raw[dom], (long long)nn, (int)np, h->staging,
+                                          h->stream));
+    else
+      PF_CUDA(h, launch_state_to_f64<S, R>((const S*)h->pop[h->cur], (const R*)h->aux[h->cur],
+                                           h->plane_stride, dd.off, (long long)nn, h->staging,
+                                           h->thermal, h->p.rho_g, h->p.rho_l - h->p.rho_g,
+                                           h->stream));
     return PF_OK;
   });
   if (st != PF_OK) return st;
@@ -1446,6 +1521,7 @@ extern "C" pf_status pf_set_state(pf_handle* h, int dom, const double* host_in, 
   const size_t np = (size_t)h->n_phys;
   if (n != nn * np)
     return fail(h, PF_ERR_BAD_ARG, "input must hold pf_state_planes(h) planes of nx*ny");
+  drop_raw(h, dom);
   pf_status st = clear_device_error(h);
   if (st != PF_OK) return st;
   st = ensure_staging(h, nn * np);
@@ -1456,12 +1532,22 @@ extern "C" pf_status pf_set_state(pf_handle* h, int dom, const double* host_in, 
     PF_TYPES(s_t, r_t);
     PF_CUDA(h, launch_state_from_f64<S, R>((S*)h->pop[h->cur], (R*)h->aux[h->cur],
                                            h->plane_stride, dd.off, (long long)nn, h->staging,
-                                           h->thermal, h->stream));
+                                           h->thermal, h->p.rho_g, h->p.rho_l - h->p.rho_g,
+                                           h->d_err, h->stream));
     return PF_OK;
   });
   if (st != PF_OK) return st;
   h->launches++;
+  unsigned int bits = 0;
+  PF_CUDA(h, cudaMemcpyAsync(&bits, h->d_err, sizeof(bits), cudaMemcpyDeviceToHost, h->stream));
   PF_CUDA(h, cudaStreamSynchronize(h->stream));
+  if (bits & ERR_GENERAL_STATE) {
+    // the staged planes are the domain's state until its next step
+    h->raw[dom] = h->staging;
+    h->staging = nullptr;
+    h->staging_elems = 0;
+    if ((st = clear_device_error(h)) != PF_OK) return st;
+  }
   h->inited[dom] = 1;
   return PF_OK;
 }
@@ -1565,6 +1651,12 @@ extern "C" pf_status pf_set_temperature(pf_handle* h, int dom, const double* the
     PF_CUDA(h, launch_set_temperature<S, R>((S*)h->pop[h->cur], (R*)h->aux[h->cur],
                                             fields_ptr<R>(h), h->plane_stride, dd, h->staging,
                                             make_kparams<R>(h->p), h->stream));
+    if (h->raw[dom]) {
+      PF_CUDA(h, launch_raw_temperature<S, R>((const S*)h->pop[h->cur], (const R*)h->aux[h->cur],
+                                              h->plane_stride, dd.off, (long long)nn, h->raw[dom],
+                                              h->p.rho_g, h->p.rho_l - h->p.rho_g, h->stream));
+      h->launches++;
+    }
     return PF_OK;
   });
   if (st != PF_OK) return st;
@@ -1582,7 +1674,7 @@ extern "C" pf_status pf_reduce_thermal(pf_handle* h, int dom, double out[3]) {
   pf_status st = dispatch(h, [&](auto s_t, auto r_t) {
     PF_TYPES(s_t, r_t);
     PF_CUDA(h, launch_reduce_thermal<S, R>((const S*)h->pop[h->cur], fields_ptr<R>(h),
-                                           h->plane_stride, dd, h->partial, h->d_diag,
+                                           h->plane_stride, dd, h->raw[dom], h->partial, h->d_diag,
                                            h->d_err + 1, h->d_err, h->stream));
     return PF_OK;
   });
@@ -1655,6 +1747,14 @@ static pf_status adjoint_t(pf_handle* h, int n, const pf_objective* obj, double*
   auto buf_of = [&](int seg) -> std::vector<char*>& { return sg[nbuf == 2 ? (seg & 1) : 0]; };
   const bool fresh = h->steps == 0;
   cudaStream_t A = h->stream;
+  // x_0 may be a raw state: its step and its reverse take their own kernels
+  const double* raw0 = h->raw[0];
+  auto forward = [&](const StepArgs<S, R>& a, int t, cudaStream_t sx) -> pf_status {
+    if (t > 0 || !raw0) return launch_all<S, R>(h, a, sx);
+    PF_CUDA(h, launch_step_general<S, R>(a, dd, raw0, sx));
+    h->launches++;
+    return PF_OK;
+  };
 
   // forward sweep: a checkpoint every K steps; the last segment's input
   // states stay in its segment buffer, and its last step writes the handle's
@@ -1667,8 +1767,11 @@ static pf_status adjoint_t(pf_handle* h, int n, const pf_objective* obj, double*
       PF_CUDA(h, cudaMemcpyAsync(aux_of(ck[t / K]), h->aux[h->cur], aux_b,
                                  cudaMemcpyDeviceToDevice, A));
     }
-    pf_status st = step_t<S, R>(h, false);
+    pf_status st = forward(make_step_args<S, R>(h, h->pop[h->cur], h->aux[h->cur],
+                                                h->pop[h->cur ^ 1], h->aux[h->cur ^ 1], false), t, A);
     if (st != PF_OK) return st;
+    h->cur ^= 1;
+    h->steps++;
   }
   {
     std::vector<char*>& bl = buf_of(nseg - 1);
@@ -1680,7 +1783,7 @@ static pf_status adjoint_t(pf_handle* h, int n, const pf_objective* obj, double*
       const StepArgs<S, R> a = make_step_args<S, R>(
           h, pop_of(bl[j]), aux_of(bl[j]), last ? h->pop[h->cur ^ 1] : pop_of(bl[j + 1]),
           last ? h->aux[h->cur ^ 1] : aux_of(bl[j + 1]), last);
-      pf_status sl = launch_all<S, R>(h, a, A);
+      pf_status sl = forward(a, t_last + j, A);
       if (sl != PF_OK) return sl;
     }
     h->cur ^= 1;
@@ -1708,7 +1811,7 @@ static pf_status adjoint_t(pf_handle* h, int n, const pf_objective* obj, double*
     for (int j = 0; j + 1 < K; ++j) {
       const StepArgs<S, R> a = make_step_args<S, R>(h, pop_of(b[j]), aux_of(b[j]),
                                                     pop_of(b[j + 1]), aux_of(b[j + 1]), false);
-      pf_status sl = launch_all<S, R>(h, a, sx);
+      pf_status sl = forward(a, s * K + j, sx);
       if (sl != PF_OK) return sl;
     }
     return PF_OK;
@@ -1728,6 +1831,7 @@ static pf_status adjoint_t(pf_handle* h, int n, const pf_objective* obj, double*
       aa.ai = ai;
       aa.partial = partial;
       aa.dfs_dsigma = dfs;
+      aa.raw = t0 + j == 0 ? raw0 : nullptr;
       PF_CUDA(h, launch_adjoint_step<S, R>(aa, grid, A));
       h->launches += ADJ_LAUNCHES_PER_STEP;
       cl ^= 1;
@@ -1792,6 +1896,8 @@ static pf_status adjoint_t(pf_handle* h, int n, const pf_objective* obj, double*
   PF_CUDA(h, cudaMemcpyAsync(hp.data(), partial, hp.size() * sizeof(double),
                              cudaMemcpyDeviceToHost, A));
   PF_CUDA(h, cudaStreamSynchronize(A));
+  drop_raw(h, 0);
+  free_spent(h);
   double g[3] = {0.0, 0.0, 0.0};
   for (int b = 0; b < grid; ++b)
     for (int q = 0; q < 3; ++q) g[q] += hp[(size_t)b * 3 + q];

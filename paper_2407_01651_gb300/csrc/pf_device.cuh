@@ -135,6 +135,61 @@ __device__ __forceinline__ void st_off_w(S* __restrict__ p, I i, R v, R w, R M) 
   }
 }
 
+// Products and differences that are never contracted: the bases below are
+// formed at every site that reads a population, and all of them have to get
+// the same bits.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
+
+// Bases of the pair-stored lattices: two opposite populations of a site add up
+// to twice the base, the rest population is what the pairs leave of the
+// density.  All differences here are exact (Sterbenz), so the populations of a
+// site sum to its density up to the unbiased rounding of the odd parts: a
+// uniform bulk, where every site rounds the same value the same way, would
+// otherwise lose a fixed fraction of a conserved total at every step.
+// CAC (D2Q9): axis phi/9; diagonal phi/36 as t - axis with t = fl(axis +
+// phi/36), so that 4 axis + 4 diagonal = 4 t and the rest is phi - 4 t.
+template <typename R>
+struct CacBase {
+  R axis, t;
+  __device__ __forceinline__ explicit CacBase(R phi)
+      : axis(mul_rn(phi, R(1.0 / 9.0))), t(fma(phi, R(1.0 / 36.0), axis)) {}
+  __device__ __forceinline__ R diag() const { return sub_rn(t, axis); }
+  __device__ __forceinline__ R rest(R phi) const { return fma(R(-4), t, phi); }
+};
+// D2Q5: axis m/6, rest m - 4 (m/6).
+template <typename R>
+__device__ __forceinline__ R q5_base(R m) {
+  return mul_rn(m, R(1.0 / 6.0));
+}
+template <typename R>
+__device__ __forceinline__ R q5_rest(R m, R base) {
+  return fma(R(-4), base, m);
+}
+// Population of the stored direction of a pair, and of the opposite one.  The
+// 16-bit forms hold the offset from the base (pos: an offset the direction's
+// populations share), the others the population.
+template <typename S, typename R>
+__device__ __forceinline__ R pair_p(S v, R base) {
+  if constexpr (Codec<S>::kOffset) return dec_off<S, R>(v, base);
+  else return Codec<S>::template dec<R>(v);
+}
+template <typename S, typename R>
+__device__ __forceinline__ R pair_m(S v, R base) {
+  const R raw = Codec<S>::template dec<R>(v);
+  if constexpr (!Codec<S>::kOffset) return fma(R(2), base, -raw);
+  else return fma(raw, R(-1.0f / Codec<S>::kOffScale), base);
+}
+// Store of the pair: base + odd, or the scaled odd part in the 16-bit forms.
+template <typename S, typename R>
+__device__ __forceinline__ S enc_pair(R base, R odd) {
+  if constexpr (!Codec<S>::kOffset) return Codec<S>::template enc<R>(base + odd);
+  else if constexpr (Codec<S>::kOffScale == 1.0f) return Codec<S>::template enc<R>(odd);
+  else return Codec<S>::template enc<R>(odd * R(Codec<S>::kOffScale));
+}
+
 // Compensated (Neumaier) accumulation: the zeroth moments phi, psi, C are sums
 // of 5 or 9 populations of similar size; in FP32 plain summation loses up to
 // ~8 ulp(phi), which the W_phi^2-weighted Laplacian in mu_phi then amplifies.

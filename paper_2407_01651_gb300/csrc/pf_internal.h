@@ -79,6 +79,7 @@ struct SetFieldsArgs {
 // Device error bits (pf_handle::d_err).
 constexpr unsigned int ERR_STAGED_TIMEOUT = 1u;   // a staged bulk copy did not complete
 constexpr unsigned int ERR_NONFINITE_INPUT = 2u;  // pf_set_fields met a non-finite value
+constexpr unsigned int ERR_GENERAL_STATE = 4u;    // pf_set_state: not a collision's output
 
 template <typename R>
 struct ReduceArgs {
@@ -129,10 +130,25 @@ cudaError_t launch_flag_nonfinite(const double* p, long long n, unsigned int* fl
                                   cudaStream_t st);
 template <typename S, typename R>
 cudaError_t launch_state_to_f64(const S* pin, const R* ain, long long ps, long long off,
-                                long long n, double* out, int thermal, cudaStream_t st);
+                                long long n, double* out, int thermal, double rho_g, double drho,
+                                cudaStream_t st);
 template <typename S, typename R>
 cudaError_t launch_state_from_f64(S* pout, R* aout, long long ps, long long off, long long n,
-                                  const double* in, int thermal, cudaStream_t st);
+                                  const double* in, int thermal, double rho_g, double drho,
+                                  unsigned int* err, cudaStream_t st);
+// One step of a domain from raw FP64 planes, whatever their populations.
+template <typename S, typename R>
+cudaError_t launch_step_general(const StepArgs<S, R>& a, const DomDesc& d, const double* raw,
+                                cudaStream_t st);
+// Raw planes: their temperature planes from the stored state; rounded to the
+// storage form.
+template <typename S, typename R>
+cudaError_t launch_raw_temperature(const S* pin, const R* ain, long long ps, long long off,
+                                   long long n, double* raw, double rho_g, double drho,
+                                   cudaStream_t st);
+template <typename S, typename R>
+cudaError_t launch_raw_rounded(const double* raw, long long n, int planes, double* out,
+                               cudaStream_t st);
 // Thermal mode: temperature lattice at equilibrium for a theta field (device,
 // n of the domain), and the FP64 totals (sum e, sum theta, sum psi).
 template <typename S, typename R>
@@ -140,7 +156,7 @@ cudaError_t launch_set_temperature(S* out, R* aout, R* fields, long long ps, con
                                    const double* theta, const KParams<R>& kp, cudaStream_t st);
 template <typename S, typename R>
 cudaError_t launch_reduce_thermal(const S* pop, const R* fields, long long ps, const DomDesc& d,
-                                  double* partial, double* out, unsigned int* ctr,
+                                  const double* raw, double* partial, double* out, unsigned int* ctr,
                                   const unsigned int* err, cudaStream_t st);
 template <typename R>
 cudaError_t launch_fields_to_f64(const R* fields, long long ps, long long off, long long n,
@@ -183,6 +199,7 @@ struct AdjArgs {
   R* lam_out;              // lambda_t, 39 planes
   R* ai;                   // input adjoints, N_AI planes
   double* partial;         // per-block parameter adjoints (eps, Omega, sigma), accumulated
+  const double* raw;       // x_t as raw FP64 planes (pf_step_general.cu), or nullptr
   double dfs_dsigma;       // d(surface-tension coefficient)/d sigma
 };
 

@@ -10,7 +10,7 @@
 // Layout: structure of arrays, one plane per population / scalar, x fastest,
 // periodic domains concatenated in every plane.
 #include "pf_internal.h"
-#include "pf_device.cuh"
+#include "pf_site.cuh"
 #include "pf_reduce.cuh"
 
 #include <cuda_fp16.h>
@@ -34,20 +34,19 @@ __device__ __forceinline__ double min_image(double d, double L) {
 
 // Temperature lattice of one site at equilibrium (thermal mode): H =
 // c_p [theta - (c_p^s/c_p) h(psi)], e = g^eq(rho H, theta, rho H v) of
-// Appendix B (with the axis base rounded as in collide_th), lagged H = H and
-// the lagged dendrite source at its pointwise part Q_psi(theta) / F(U).
+// Appendix B (axis base rounded as in the collision), and the lagged dendrite
+// source at its pointwise part Q_psi(theta) / F(U).
 template <typename S, typename R>
 __device__ void write_thermal(S* out, R* aout, R* fields, long long ps, long long site, R phi,
                               R psi, R U, R vx, R vy, R theta, const KParams<R>& kp) {
   const R rho = kp.rho_g + phi * kp.drho;
   const R H = kp.th_cp * (theta - kp.th_lh * (R(1) + psi));
   const R m0 = rho * H;
-  const R b = round_to_multiple(theta * R(1.0 / 6.0), quantum_quarter_ulp(m0));
-  const R jx = m0 * vx, jy = m0 * vy;
-  const R e[5] = {m0 - R(4) * b, b + R(0.5) * jx, b + R(0.5) * jy, b - R(0.5) * jx,
-                  b - R(0.5) * jy};
-  for (int i = 0; i < 5; ++i) st<S, R>(out + (P_E + i) * ps, site, e[i]);
-  aout[A_HO * ps + site] = H;
+  const R b = th_base(m0, theta);
+  st<S, R>(out + (P_E + 0) * ps, site, m0);
+  st<S, R>(out + (P_E + 1) * ps, site, b);
+  st<S, R>(out + (P_E + 2) * ps, site, b + R(0.5) * (m0 * vx));
+  st<S, R>(out + (P_E + 3) * ps, site, b + R(0.5) * (m0 * vy));
   const R omp2 = R(1) - psi * psi, ophi = R(1) - phi;
   const R Q = kp.four_bpsi * psi * omp2 - kp.two_bint * ophi * ophi * (R(1) + psi) -
               kp.lam * omp2 * omp2 * (theta + kp.Mcinf * U);
@@ -69,35 +68,33 @@ __device__ void write_equilibrium(S* out, R* aout, R* fields, long long ps, long
                                   double theta_d) {
   const R phi = static_cast<R>(phi_d), psi = static_cast<R>(psi_d), C = static_cast<R>(C_d);
   const R vx = static_cast<R>(vx_d), vy = static_cast<R>(vy_d), p = static_cast<R>(p_d);
-  const R rho = kp.rho_g + phi * kp.drho;
-  R f[9];
-  feq_ns(p, rho, vx, vy, f);
-  // CAC h_eq = w_i phi (1 + 3 c.v); dendrite w_i psi; solute w_i C (1 + 3 c.v)
-  const R cu[9] = {R(0), vx, vy, -vx, -vy, vx + vy, -vx + vy, -vx - vy, vx - vy};
-  for (int i = 0; i < 9; ++i) {
-    st_ns<S, R>(out + (P_F + i) * ps, site, f[i]);
-    st_off<S, R>(out + (P_H + i) * ps, site, w9<R>(i) * phi * (R(1) + R(3) * cu[i]),
-                 w9<R>(i) * phi);
-  }
-  for (int i = 0; i < 5; ++i) {
-    st_off<S, R>(out + (P_GPRE + i) * ps, site, w5<R>(i) * psi, w5<R>(i) * psi);
-    st_off<S, R>(out + (P_GPOST + i) * ps, site, w5<R>(i) * psi, w5<R>(i) * psi);
-    st_off<S, R>(out + (P_S + i) * ps, site, w5<R>(i) * C * (R(1) + R(3) * cu[i]),
-                 w5<R>(i) * C);
-  }
   const R omk = R(1) - kp.k;
   const R U = (R(2) * C / (R(1) + kp.k - omk * psi) - R(1)) / omk;
   const R omp2 = R(1) - psi * psi;
   const R ophi = R(1) - phi;
-  const R Q = kp.four_bpsi * psi * omp2 - kp.two_bint * ophi * ophi * (R(1) + psi) -
-              kp.lam * omp2 * omp2 * (kp.theta + kp.Mcinf * U);
-  aout[A_RR * ps + site] = R(1);
-  aout[A_PHIO * ps + site] = phi;
-  aout[A_CO * ps + site] = C;
-  aout[A_VXO * ps + site] = vx;
-  aout[A_VYO * ps + site] = vy;
-  aout[A_QO * ps + site] = Q;
-  aout[A_PSIO * ps + site] = psi;
+  SiteOut<R> o;
+  feq_ns(p, kp.rho_g + phi * kp.drho, vx, vy, o.f);
+  // CAC h_eq = w_i phi (1 + 3 c.v); dendrite w_i psi; solute w_i C (1 + 3 c.v)
+  o.hA = (w9<R>(1) * phi * R(3)) * vec2(vx, vy);
+  o.hD = (w9<R>(5) * phi * R(3)) * vec2(vx + vy, vy - vx);
+  o.g = vec2(R(0), R(0));
+  o.F = R(0);
+  o.s = (w5<R>(1) * C * R(3)) * vec2(vx, vy);
+  R g[5];
+  for (int i = 0; i < 5; ++i) g[i] = w5<R>(i) * psi;
+  o.ias2 = R(1);
+  o.phi = phi;
+  o.psi = psi;
+  o.C = C;
+  o.vx = vx;
+  o.vy = vy;
+  o.Q = kp.four_bpsi * psi * omp2 - kp.two_bint * ophi * ophi * (R(1) + psi) -
+        kp.lam * omp2 * omp2 * (kp.theta + kp.Mcinf * U);
+  StepArgs<S, R> to{};
+  to.out = out;
+  to.aout = aout;
+  to.plane_stride = ps;
+  store_state<S, R>(to, (unsigned)site, o, g);
   if (fields) {
     fields[FLD_PHI * ps + site] = phi;
     fields[FLD_PSI * ps + site] = psi;
@@ -200,71 +197,229 @@ __global__ void k_set_temperature(S* out, R* aout, R* fields, long long ps, DomD
 // Raw state / fields conversion to and from FP64.
 // ---------------------------------------------------------------------------
 // Raw state of one site <-> the 39 physical planes (f, h, g_pre, g_post, r,
-// s, phi, C, vx, vy, Q_psi), decoding / encoding the storage form.  In the
-// offset forms a population stored at site x is relative to the lagged
-// moment of x itself.
-// Thermal mode adds planes 39..43 (e_0..e_4) and 44 (H of the last step).
+// s, phi, C, vx, vy, Q_psi), every population of a pair, in FP64.  In the
+// offset forms a population stored at site x is relative to the lagged moment
+// of x itself.  Thermal mode adds planes 39..43 (e_0..e_4) and 44 (H of the last
+// step).  A state taken out and put back gives the same stored values: the
+// stored populations and the densities pass through unchanged, and the density
+// of a lattice without a plane of its own (g_post, e) is the FP64 sum of its
+// populations in sum5's order, of which the rest one is written as density
+// minus the others (exact).
+__device__ __forceinline__ double sum_pairs5(const double (&v)[5]) {
+  return (v[1] + v[3]) + (v[2] + v[4]);
+}
+__device__ __forceinline__ double sum5(const double (&v)[5]) { return sum_pairs5(v) + v[0]; }
+
 template <typename S, typename R>
 __global__ void k_state_to_f64(const S* __restrict__ pin, const R* __restrict__ ain, long long ps,
                                long long off, long long n, double* __restrict__ out,
-                               int thermal) {
+                               int thermal, double rho_g, double drho) {
   constexpr bool offs = Codec<S>::kOffset;
   for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n;
        j += (long long)gridDim.x * blockDim.x) {
     const long long s = off + j;
+    auto pop = [&](int k) { return pin[k * ps + s]; };
+    // stored and opposite population of a pair with this base
+    auto plus = [&](S v, R base) {
+      return offs ? (double)base + (double)dec_off<S, R>(v, R(0)) : (double)pair_p<S, R>(v, base);
+    };
+    auto minus = [&](S v, R base) {
+      return offs ? (double)base - (double)dec_off<S, R>(v, R(0)) : (double)pair_m<S, R>(v, base);
+    };
     const R phio = ain[A_PHIO * ps + s], Co = ain[A_CO * ps + s];
     const R psio = offs ? ain[A_PSIO * ps + s] : R(0);
-    for (int i = 0; i < 9; ++i) {
-      out[(0 + i) * n + j] = (double)pop_ns<S, R>(pin + (P_F + i) * ps, s);
-      out[(9 + i) * n + j] = (double)pop_off<S, R>(pin + (P_H + i) * ps, s, w9<R>(i) * phio);
+    for (int i = 0; i < 9; ++i) out[(X_F + i) * n + j] = (double)pop_ns<S, R>(pin + (P_F + i) * ps, s);
+    const CacBase<R> b(phio);
+    out[X_H * n + j] = (double)b.rest(phio);
+    for (int i = 1; i < 9; ++i) {
+      const R base = i < 5 ? b.axis : b.diag();
+      const S v = pop(P_H + pair9(i));
+      out[(X_H + i) * n + j] = minus9(i) ? minus(v, base) : plus(v, base);
     }
-    for (int i = 0; i < 5; ++i) {
-      out[(18 + i) * n + j] = (double)pop_off<S, R>(pin + (P_GPRE + i) * ps, s, w5<R>(i) * psio);
-      out[(23 + i) * n + j] = (double)pop_off<S, R>(pin + (P_GPOST + i) * ps, s, w5<R>(i) * psio);
-      out[(29 + i) * n + j] = (double)pop_off<S, R>(pin + (P_S + i) * ps, s, w5<R>(i) * Co);
+    for (int i = 0; i < 5; ++i)
+      out[(X_GPRE + i) * n + j] = (double)pop_off<S, R>(pin + (P_GPRE + i) * ps, s, w5<R>(i) * psio);
+    {
+      // density m; in the offset forms psi_o + F with F/6 in the first plane
+      const double f6 = offs ? (double)dec_off<S, R>(pop(P_GPOST), R(0)) : 0.0;
+      const R m = offs ? psio : (R)Codec<S>::template dec<R>(pop(P_GPOST));
+      const R base = q5_base(m);
+      double g[5];
+      for (int i = 1; i < 3; ++i) {
+        const S v = pop(P_GPOST + i);
+        g[i] = plus(v, base);
+        g[i + 2] = minus(v, base) + 2.0 * f6;
+      }
+      g[0] = ((double)m + 6.0 * f6) - sum_pairs5(g);
+      for (int i = 0; i < 5; ++i) out[(X_GPOST + i) * n + j] = g[i];
     }
-    out[28 * n + j] = (double)ain[A_RR * ps + s];
-    out[34 * n + j] = (double)phio;
-    out[35 * n + j] = (double)Co;
-    out[36 * n + j] = (double)ain[A_VXO * ps + s];
-    out[37 * n + j] = (double)ain[A_VYO * ps + s];
-    out[38 * n + j] = (double)ain[A_QO * ps + s];
+    {
+      const R base = q5_base(Co);
+      out[X_S * n + j] = (double)q5_rest(Co, base);
+      for (int i = 1; i < 3; ++i) {
+        const S v = pop(P_S + i - 1);
+        out[(X_S + i) * n + j] = plus(v, base);
+        out[(X_S + i + 2) * n + j] = minus(v, base);
+      }
+    }
+    out[X_RR * n + j] = (double)ain[A_RR * ps + s];
+    out[X_PHI * n + j] = (double)phio;
+    out[X_C * n + j] = (double)Co;
+    out[X_VX * n + j] = (double)ain[A_VXO * ps + s];
+    out[X_VY * n + j] = (double)ain[A_VYO * ps + s];
+    out[X_Q * n + j] = (double)ain[A_QO * ps + s];
     if (thermal) {
-      for (int i = 0; i < 5; ++i) out[(39 + i) * n + j] = (double)ld<R>(pin + (P_E + i) * ps, s);
-      out[44 * n + j] = (double)ain[A_HO * ps + s];
+      const R m = Codec<S>::template dec<R>(pop(P_E)), base = Codec<S>::template dec<R>(pop(P_E + 1));
+      double e[5];
+      for (int i = 1; i < 3; ++i) {
+        e[i] = plus(pop(P_E + 1 + i), base);
+        e[i + 2] = minus(pop(P_E + 1 + i), base);
+      }
+      e[0] = (double)m - sum_pairs5(e);
+      for (int i = 0; i < 5; ++i) out[(X_E + i) * n + j] = e[i];
+      out[X_HO * n + j] = (double)m / (rho_g + (double)phio * drho);
     }
   }
 }
 
+// Sets ERR_GENERAL_STATE where the populations are not a collision's output to
+// rounding (4 ulp of the pair's size in FP32 arithmetic, 16 in FP64): the step
+// that follows then starts from the raw planes (pf_step_general.cu).
 template <typename S, typename R>
 __global__ void k_state_from_f64(S* __restrict__ pout, R* __restrict__ aout, long long ps,
                                  long long off, long long n, const double* __restrict__ in,
-                                 int thermal) {
+                                 int thermal, double rho_g, double drho, unsigned int* err) {
+  constexpr double tol = sizeof(R) == 8 ? 16.0 * 2.220446049250313e-16 : 4.0 * 1.1920928955078125e-7;
+  constexpr bool offs = Codec<S>::kOffset;
+  bool general = false;
+  // a and b are equal to rounding on the scale of their parts
+  auto same = [&](double a, double b, double size) {
+    if (!(fabs(a - b) <= tol * size)) general = true;
+  };
   for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n;
        j += (long long)gridDim.x * blockDim.x) {
     const long long s = off + j;
-    const R phio = (R)in[34 * n + j], Co = (R)in[35 * n + j];
+    auto x = [&](int k) { return in[k * n + j]; };
+    auto put = [&](int k, double v, R base) {
+      if constexpr (offs) pout[k * ps + s] = enc_off<S, R>((R)(v - (double)base), R(0));
+      else pout[k * ps + s] = Codec<S>::template enc<R>((R)v);
+    };
+    const R phio = (R)x(X_PHI), Co = (R)x(X_C);
     R psio = R(0);  // psi of the last step = sum of g_pre
-    for (int i = 0; i < 5; ++i) psio += (R)in[(18 + i) * n + j];
-    for (int i = 0; i < 9; ++i) {
-      st_ns<S, R>(pout + (P_F + i) * ps, s, (R)in[(0 + i) * n + j]);
-      st_off<S, R>(pout + (P_H + i) * ps, s, (R)in[(9 + i) * n + j], w9<R>(i) * phio);
+    for (int i = 0; i < 5; ++i) psio += (R)x(X_GPRE + i);
+    for (int i = 0; i < 9; ++i) st_ns<S, R>(pout + (P_F + i) * ps, s, (R)x(X_F + i));
+    {
+      const CacBase<R> b(phio);
+      double size = fabs(x(X_PHI));
+      for (int i = 0; i < 9; ++i) size = fmax(size, fabs(x(X_H + i)));
+      same(x(X_H), (double)b.rest(phio), size);
+      for (int i : {1, 2, 5, 6}) {
+        const R base = i < 5 ? b.axis : b.diag();
+        same(x(X_H + i) + x(X_H + i + 2), 2.0 * (double)base, size);
+        put(P_H + pair9(i), x(X_H + i), base);
+      }
     }
-    for (int i = 0; i < 5; ++i) {
-      st_off<S, R>(pout + (P_GPRE + i) * ps, s, (R)in[(18 + i) * n + j], w5<R>(i) * psio);
-      st_off<S, R>(pout + (P_GPOST + i) * ps, s, (R)in[(23 + i) * n + j], w5<R>(i) * psio);
-      st_off<S, R>(pout + (P_S + i) * ps, s, (R)in[(29 + i) * n + j], w5<R>(i) * Co);
+    for (int i = 0; i < 5; ++i)
+      st_off<S, R>(pout + (P_GPRE + i) * ps, s, (R)x(X_GPRE + i), w5<R>(i) * psio);
+    {
+      double g[5], size = 0.0;
+      for (int i = 0; i < 5; ++i) {
+        g[i] = x(X_GPOST + i);
+        size = fmax(size, fabs(g[i]));
+      }
+      const double m = sum5(g);
+      same(g[1] + g[3], m / 3.0, 2.0 * size);
+      same(g[2] + g[4], m / 3.0, 2.0 * size);
+      if constexpr (offs) {
+        const R base = q5_base(psio);
+        pout[P_GPOST * ps + s] = enc_off<S, R>((R)((m - (double)psio) / 6.0), R(0));
+        put(P_GPOST + 1, g[1], base);
+        put(P_GPOST + 2, g[2], base);
+      } else {
+        put(P_GPOST, m, R(0));
+        put(P_GPOST + 1, g[1], R(0));
+        put(P_GPOST + 2, g[2], R(0));
+      }
     }
-    aout[A_RR * ps + s] = (R)in[28 * n + j];
+    {
+      const R base = q5_base(Co);
+      double size = fabs(x(X_C));
+      for (int i = 0; i < 5; ++i) size = fmax(size, fabs(x(X_S + i)));
+      same(x(X_S), (double)q5_rest(Co, base), size);
+      for (int i = 1; i < 3; ++i) {
+        same(x(X_S + i) + x(X_S + i + 2), 2.0 * (double)base, size);
+        put(P_S + i - 1, x(X_S + i), base);
+      }
+    }
+    aout[A_RR * ps + s] = (R)x(X_RR);
     aout[A_PHIO * ps + s] = phio;
     aout[A_CO * ps + s] = Co;
-    aout[A_VXO * ps + s] = (R)in[36 * n + j];
-    aout[A_VYO * ps + s] = (R)in[37 * n + j];
-    aout[A_QO * ps + s] = (R)in[38 * n + j];
-    aout[A_PSIO * ps + s] = psio;
+    aout[A_VXO * ps + s] = (R)x(X_VX);
+    aout[A_VYO * ps + s] = (R)x(X_VY);
+    aout[A_QO * ps + s] = (R)x(X_Q);
+    if constexpr (offs) aout[A_PSIO * ps + s] = psio;
     if (thermal) {
-      for (int i = 0; i < 5; ++i) st<S, R>(pout + (P_E + i) * ps, s, (R)in[(39 + i) * n + j]);
-      aout[A_HO * ps + s] = (R)in[44 * n + j];
+      double e[5], size = 0.0;
+      for (int i = 0; i < 5; ++i) {
+        e[i] = x(X_E + i);
+        size = fmax(size, fabs(e[i]));
+      }
+      const double md = sum5(e), rhoH = (rho_g + x(X_PHI) * drho) * x(X_HO);
+      const R m = (R)md, b = round_to_multiple((R)(0.5 * (e[1] + e[3])), quantum_quarter_ulp(m));
+      same(e[1] + e[3], 2.0 * (double)b, 2.0 * size);
+      same(e[2] + e[4], 2.0 * (double)b, 2.0 * size);
+      same(md, rhoH, 2.0 * size);
+      st<S, R>(pout + (P_E + 0) * ps, s, m);
+      st<S, R>(pout + (P_E + 1) * ps, s, b);
+      st<S, R>(pout + (P_E + 2) * ps, s, (R)e[1]);
+      st<S, R>(pout + (P_E + 3) * ps, s, (R)e[2]);
+    }
+  }
+  if (general) atomicOr(err, ERR_GENERAL_STATE);
+}
+
+// The temperature planes of a raw state from the stored ones (after
+// pf_set_temperature rewrote those).
+template <typename S, typename R>
+__global__ void k_raw_temperature(const S* __restrict__ pin, const R* __restrict__ ain,
+                                  long long ps, long long off, long long n,
+                                  double* __restrict__ raw, double rho_g, double drho) {
+  for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n;
+       j += (long long)gridDim.x * blockDim.x) {
+    const long long s = off + j;
+    const R m = ld<R>(pin + P_E * ps, s), b = ld<R>(pin + (P_E + 1) * ps, s);
+    const R e1 = ld<R>(pin + (P_E + 2) * ps, s), e2 = ld<R>(pin + (P_E + 3) * ps, s);
+    raw[X_E * n + j] = (double)q5_rest(m, b);
+    raw[(X_E + 1) * n + j] = (double)e1;
+    raw[(X_E + 2) * n + j] = (double)e2;
+    raw[(X_E + 3) * n + j] = (double)fma(R(2), b, -e1);
+    raw[(X_E + 4) * n + j] = (double)fma(R(2), b, -e2);
+    raw[X_HO * n + j] = (double)m / (rho_g + raw[X_PHI * n + j] * drho);
+    raw[X_Q * n + j] = (double)ain[A_QO * ps + s];
+  }
+}
+
+// A raw state rounded to the storage form (as pf_get_state returns it).
+template <typename S, typename R>
+__global__ void k_raw_rounded(const double* __restrict__ raw, long long n, int planes,
+                              double* __restrict__ out) {
+  for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n;
+       j += (long long)gridDim.x * blockDim.x) {
+    auto x = [&](int k) { return (R)raw[k * n + j]; };
+    R psio = R(0);
+    for (int i = 0; i < 5; ++i) psio += x(X_GPRE + i);
+    for (int k = 0; k < planes; ++k) {
+      R v = x(k);
+      if (k < X_H) {
+        if constexpr (Codec<S>::kOffset)
+          v = Codec<S>::template dec<R>(Codec<S>::template enc<R>(v * R(kNSScale))) * R(kNSInvScale);
+      } else if (k < X_PHI && k != X_RR) {
+        const R wm = k < X_GPRE ? w9<R>(k - X_H) * x(X_PHI)
+                                : (k < X_GPOST ? w5<R>(k - X_GPRE) * psio
+                                               : (k < X_RR ? w5<R>(k - X_GPOST) * psio
+                                                           : w5<R>(k - X_S) * x(X_C)));
+        v = dec_off<S, R>(enc_off<S, R>(v, wm), wm);
+      }
+      out[k * n + j] = (double)v;
     }
   }
 }
@@ -343,20 +498,25 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce(ReduceArgs<R> a, double*
 }
 
 // Thermal totals (FP64): sum over sites of the five temperature populations
-// (the total of rho H), sum theta, sum psi; then the device error bits.
+// (the total of rho H: their density plane, or the raw state's populations),
+// sum theta, sum psi; then the device error bits.
 template <typename S, typename R>
 __global__ void __launch_bounds__(RED_THREADS) k_reduce_thermal(
     const S* __restrict__ pop, const R* __restrict__ fields, long long ps, DomDesc d,
-    double* __restrict__ partial, double* __restrict__ out, unsigned int* __restrict__ ctr,
+    const double* __restrict__ raw, double* __restrict__ partial, double* __restrict__ out, unsigned int* __restrict__ ctr,
     const unsigned int* __restrict__ err) {
   double acc[3] = {0.0, 0.0, 0.0};
   const long long n = (long long)d.nx * d.ny;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
     const long long site = d.off + i;
-    double se = 0.0;
-    for (int q = 0; q < 5; ++q) se += (double)ld<R>(pop + (P_E + q) * ps, site);
-    acc[0] += se;
+    if (raw) {
+      double se = 0.0;
+      for (int q = 0; q < 5; ++q) se += (double)(R)raw[(X_E + q) * n + i];
+      acc[0] += se;
+    } else {
+      acc[0] += (double)ld<R>(pop + P_E * ps, site);
+    }
     acc[1] += (double)fields[FLD_THETA * ps + site];
     acc[2] += (double)fields[FLD_PSI * ps + site];
   }
@@ -447,15 +607,33 @@ cudaError_t launch_set_fields(const SetFieldsArgs<S, R>& a, cudaStream_t st) {
 
 template <typename S, typename R>
 cudaError_t launch_state_to_f64(const S* pin, const R* ain, long long ps, long long off,
-                                long long n, double* out, int thermal, cudaStream_t st) {
-  k_state_to_f64<S, R><<<1024, 256, 0, st>>>(pin, ain, ps, off, n, out, thermal);
+                                long long n, double* out, int thermal, double rho_g, double drho,
+                                cudaStream_t st) {
+  k_state_to_f64<S, R><<<1024, 256, 0, st>>>(pin, ain, ps, off, n, out, thermal, rho_g, drho);
   return cudaGetLastError();
 }
 
 template <typename S, typename R>
 cudaError_t launch_state_from_f64(S* pout, R* aout, long long ps, long long off, long long n,
-                                  const double* in, int thermal, cudaStream_t st) {
-  k_state_from_f64<S, R><<<1024, 256, 0, st>>>(pout, aout, ps, off, n, in, thermal);
+                                  const double* in, int thermal, double rho_g, double drho,
+                                  unsigned int* err, cudaStream_t st) {
+  k_state_from_f64<S, R><<<1024, 256, 0, st>>>(pout, aout, ps, off, n, in, thermal, rho_g, drho,
+                                               err);
+  return cudaGetLastError();
+}
+
+template <typename S, typename R>
+cudaError_t launch_raw_temperature(const S* pin, const R* ain, long long ps, long long off,
+                                   long long n, double* raw, double rho_g, double drho,
+                                   cudaStream_t st) {
+  k_raw_temperature<S, R><<<1024, 256, 0, st>>>(pin, ain, ps, off, n, raw, rho_g, drho);
+  return cudaGetLastError();
+}
+
+template <typename S, typename R>
+cudaError_t launch_raw_rounded(const double* raw, long long n, int planes, double* out,
+                               cudaStream_t st) {
+  k_raw_rounded<S, R><<<1024, 256, 0, st>>>(raw, n, planes, out);
   return cudaGetLastError();
 }
 
@@ -476,10 +654,10 @@ static int reduce_grid(long long n) {
 
 template <typename S, typename R>
 cudaError_t launch_reduce_thermal(const S* pop, const R* fields, long long ps, const DomDesc& d,
-                                  double* partial, double* out, unsigned int* ctr,
+                                  const double* raw, double* partial, double* out, unsigned int* ctr,
                                   const unsigned int* err, cudaStream_t st) {
   k_reduce_thermal<S, R><<<reduce_grid((long long)d.nx * d.ny), RED_THREADS, 0, st>>>(
-      pop, fields, ps, d, partial, out, ctr, err);
+      pop, fields, ps, d, raw, partial, out, ctr, err);
   return cudaGetLastError();
 }
 
@@ -519,15 +697,23 @@ cudaError_t launch_reduce(const ReduceArgs<R>& a, double* partial, double* out, 
   template cudaError_t launch_init_spec<S, R>(const InitArgs<S, R>&, cudaStream_t);          \
   template cudaError_t launch_set_fields<S, R>(const SetFieldsArgs<S, R>&, cudaStream_t);    \
   template cudaError_t launch_state_to_f64<S, R>(const S*, const R*, long long, long long,   \
-                                                 long long, double*, int, cudaStream_t);     \
+                                                 long long, double*, int, double, double,    \
+                                                 cudaStream_t);                              \
   template cudaError_t launch_state_from_f64<S, R>(S*, R*, long long, long long, long long,  \
-                                                   const double*, int, cudaStream_t);        \
+                                                   const double*, int, double, double,       \
+                                                   unsigned int*, cudaStream_t);             \
+  template cudaError_t launch_raw_temperature<S, R>(const S*, const R*, long long, long long, \
+                                                    long long, double*, double, double,      \
+                                                    cudaStream_t);                           \
+  template cudaError_t launch_raw_rounded<S, R>(const double*, long long, int, double*,      \
+                                                cudaStream_t);                               \
   template cudaError_t launch_set_temperature<S, R>(S*, R*, R*, long long, const DomDesc&,   \
                                                     const double*, const KParams<R>&,        \
                                                     cudaStream_t);                           \
   template cudaError_t launch_reduce_thermal<S, R>(const S*, const R*, long long,            \
-                                                   const DomDesc&, double*, double*,         \
-                                                   unsigned int*, const unsigned int*,       \
+                                                   const DomDesc&, const double*, double*,   \
+                                                   double*, unsigned int*,                   \
+                                                   const unsigned int*,                      \
                                                    cudaStream_t);
 
 PF_INST(double, double)

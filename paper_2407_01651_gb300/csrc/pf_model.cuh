@@ -22,15 +22,23 @@ namespace pf {
 // live in one buffer of the storage type, the lagged scalars in another of
 // the compute type.
 // ---------------------------------------------------------------------------
+//
+// CAC, post-collision dendrite, solute and temperature populations come out of
+// a collision whose even moments are functions of the conserved one, so that
+// two opposite populations add up to a known function of that density: their
+// base (pf_device.cuh) times two.  One population of each pair is stored, the
+// density plane gives the others back: 29 values per site instead of 39
+// (thermal 33 instead of 45).
 enum PopPlane : int {
   P_F = 0,        // NS populations f_0..f_8 (post-collision)
-  P_H = 9,        // CAC populations h_0..h_8 (post-collision)
-  P_GPRE = 18,    // dendrite populations before collision g_0..g_4
-  P_GPOST = 23,   // dendrite populations after collision
-  P_S = 28,       // solute populations s_0..s_4 (post-collision)
-  N_POP = 33,
-  P_E = 33,       // temperature populations e_0..e_4 (post-collision; thermal mode)
-  N_POP_TH = 38
+  P_H = 9,        // CAC: h_1, h_2, h_5, h_6; density phi of the last step (A_PHIO)
+  P_GPRE = 13,    // dendrite populations before collision g_0..g_4
+  P_GPOST = 18,   // dendrite after collision: density (16-bit forms: its share F/6
+                  // of the offsets), g_1, g_2
+  P_S = 21,       // solute: s_1, s_2; density C of the last step (A_CO)
+  N_POP = 23,
+  P_E = 23,       // temperature (thermal mode): density rho H, axis base, e_1, e_2
+  N_POP_TH = 27
 };
 
 enum AuxPlane : int {
@@ -41,13 +49,14 @@ enum AuxPlane : int {
   A_VYO = 4,      // vy of the last step
   A_QO = 5,       // Q_psi of the last step
   A_PSIO = 6,     // psi of the last step (offset storage forms only)
-  N_AUX = 7,
-  A_HO = 7,       // H = c_p theta - c_p^s h(psi) of the last step (thermal mode)
-  N_AUX_TH = 8
+  N_AUX = 7
 };
 
 // Raw state exchanged with the host (pf_get_state / pf_set_state): 39 planes
-// f[9], h[9], g_pre[5], g_post[5], r, s[5], phi, C, vx, vy, Q_psi.
+// f[9], h[9], g_pre[5], g_post[5], r, s[5], phi, C, vx, vy, Q_psi (every
+// population of a pair; first plane of each group below).
+constexpr int X_F = 0, X_H = 9, X_GPRE = 18, X_GPOST = 23, X_RR = 28, X_S = 29, X_PHI = 34,
+              X_C = 35, X_VX = 36, X_VY = 37, X_Q = 38, X_E = 39, X_HO = 44;
 constexpr int N_PHYS = 39;
 // Thermal mode: + e[5], H_o.
 constexpr int N_PHYS_TH = 45;
@@ -149,22 +158,6 @@ __device__ __forceinline__ void f_from_moments(T axis, T diag, V2<T> DF, V2<T> E
   f[5] = f56.x; f[6] = f56.y; f[7] = f78.x; f[8] = f78.y;
 }
 
-// D2Q5 post-collision populations from (m0, jx, jy) with the energy moment at
-// -(2/3) m0 and the anisotropic moment at 0 (their equilibria, rate 1):
-// s_0 = m0/3, s_{1,3} = m0/6 +- jx/2, s_{2,4} = m0/6 +- jy/2.
-// s_0 is formed as m0 - 4 (m0/6): by Sterbenz's lemma that difference is
-// exact, so sum_i s_i = m0 up to the unbiased rounding of the +-j/2 terms.
-// (Rounding m0 * fl(1/3) and m0 * fl(1/6) separately would bias every site's
-// sum the same way, a drift of ~0.5 ulp per step in a conserved total.)
-template <typename T>
-__device__ __forceinline__ void q5_from_m(T m0, V2<T> J, T s[5]) {
-  const T a0 = m0 * T(1.0 / 6.0);
-  const V2<T> a = splat(a0);
-  const V2<T> s12 = fma(T(0.5), J, a), s34 = fma(T(-0.5), J, a);
-  s[0] = m0 - T(4) * a0;
-  s[1] = s12.x; s[2] = s12.y; s[3] = s34.x; s[4] = s34.y;
-}
-
 // NS collision, D2Q9 MRT with forcing through (I - S/2):
 //   m* = m - S (m - m_eq) + (I - S/2) M G,
 // m_eq = (0, 6p + 3 rho v^2, -9p - 3 rho v^2, rho vx, -rho vx, rho vy, -rho vy,
@@ -209,48 +202,38 @@ __device__ __forceinline__ void collide_ns(T f[9], T p, T rho, V2<T> v, V2<T> F,
 }
 
 // CAC collision, D2Q9: h_eq = w_i phi (1 + 3 c.v), G_i = 3 w_i c.G1.  Flux
-// moments relax with s_phi, all others with 1:
-// m* = (phi, -2 phi, phi, j*x, -phi vx - G1x/2, j*y, -phi vy - G1y/2, 0, 0),
-// whose back-transform has axis = phi/9, diag = phi/36, h_0 = 4 phi/9.  The
-// rest population is formed as h_0 = phi - 4 t with t = fl(axis + diag), an
-// exact difference (Sterbenz), and the diagonal base is shifted by the exact
-// rounding error of t (Fast2Sum), so that h_0 + 4 axis + 4 diag = phi holds
-// exactly.  Otherwise a uniform bulk, where every site rounds the same value
-// the same way, would lose a fixed fraction of phi at every step.
+// moments (J before the collision) relax with s_phi, all others with 1:
+// m* = (phi, -2 phi, phi, j*x, -phi vx - G1x/2, j*y, -phi vy - G1y/2, 0, 0).
+// Its back-transform is h_i = base +- odd, base = phi/9 on the axes and phi/36
+// on the diagonals; the odd parts of directions 1, 2 (A) and 5, 6 (D) are
+// returned, the opposite directions have them with the other sign.
 template <typename T, typename R>
-__device__ __forceinline__ void collide_cac(T h[9], T phi, V2<T> v, V2<T> G1,
+__device__ __forceinline__ void collide_cac(V2<T> J, T phi, V2<T> v, V2<T> G1, V2<T>& A, V2<T>& D,
                                             const KParams<R>& kp) {
-  const V2<T> Dl = vec2(h[1], h[2]) - vec2(h[3], h[4]);
-  const V2<T> U = vec2(h[5], h[6]) - vec2(h[7], h[8]);
-  const V2<T> J = Dl + vec2(U.x - U.y, U.x + U.y);
   const R hs = R(1) - R(0.5) * kp.s_phi;
   const V2<T> pv = phi * v;
   const V2<T> JS = fma(splat(T(hs)), G1, fma(splat(T(-kp.s_phi)), J - pv, J));
   const V2<T> q46 = fma(T(-0.5), G1, splat(T(0)) - pv);   // (-phi vx - G1x/2, ...)
-  const T axis = phi * T(1.0 / 9.0), diag = phi * T(1.0 / 36.0);
-  const T t = axis + diag;
-  const T e = diag - (t - axis);   // axis + diag - t, exact (|axis| >= |diag|)
-  h[0] = phi - T(4) * t;
-  f_from_moments(axis, diag - e, T(1.0 / 6.0) * JS, T(1.0 / 12.0) * q46, T(0), T(0), h);
+  const V2<T> DF = T(1.0 / 6.0) * JS, EG = T(1.0 / 12.0) * q46;
+  A = fma(T(-2), EG, DF);
+  const V2<T> S = DF + EG;
+  D = vec2(S.y + S.x, S.y - S.x);
 }
 
-// D2Q5 collision with conserved zeroth moment m0 (after the direct source),
-// flux moments j relaxing with rate s towards jeq plus (1 - s/2) Gj, and the
-// other moments at their equilibria.
+// D2Q5 collision: flux moments J relax with rate s towards jeq plus (1 - s/2)
+// Gj, the other moments are at their equilibria, so the populations are the
+// rest one and base +- J*/2.  Returns J*/2, the odd parts of directions 1, 2.
 template <typename T>
-__device__ __forceinline__ void collide_q5(T q[5], T m0, T s, V2<T> Jeq, V2<T> G) {
-  const V2<T> J = vec2(q[1], q[2]) - vec2(q[3], q[4]);
+__device__ __forceinline__ V2<T> collide_q5(V2<T> J, T s, V2<T> Jeq, V2<T> G) {
   const T hs = T(1) - T(0.5) * s;
-  const V2<T> JS = fma(splat(hs), G, fma(splat(-s), J - Jeq, J));
-  q5_from_m(m0, JS, q);
+  return T(0.5) * fma(splat(hs), G, fma(splat(-s), J - Jeq, J));
 }
 
 // Temperature collision, D2Q5 (Appendix B): g_0^eq = rho H + (w_0 - 1) theta,
 // g_i^eq = w_i theta + w_i c_i.(rho H v)/c_s^2, G_i = w_i c_i.dJ/c_s^2 with
-// dJ = d_t(rho H v); flux moments relax with s, the others with 1.  In moment
-// space the energy moment is at -4 m0 + (10/3) theta and the anisotropic one
-// at 0, whose back-transform is e_0 = m0 - (2/3) theta, e_{1,3} = theta/6 +- j*x/2,
-// e_{2,4} = theta/6 +- j*y/2.  m0 = rho H is conserved as it came in.  The
+// dJ = d_t(rho H v); flux moments relax with s, the others with 1: e_0 = m0 -
+// 4 b, axis populations b +- J*/2 (collide_q5) with b = theta/6 (th_base).
+// m0 = rho H is conserved as it came in.  The
 // base theta/6 of the axis populations is rounded to a multiple of ulp(m0)/4,
 // which makes m0 - 4 (theta/6) exact in the common case: a uniform region
 // would otherwise round every site's e_0 the same way and drift the conserved
@@ -275,15 +258,8 @@ __device__ __forceinline__ T round_to_multiple(T v, T q) {
   else return rint(v * __drcp_rn(q)) * q;
 }
 template <typename T>
-__device__ __forceinline__ void collide_th(T e[5], T m0, T theta, T s, V2<T> Jeq, V2<T> G) {
-  const V2<T> J = vec2(e[1], e[2]) - vec2(e[3], e[4]);
-  const T hs = T(1) - T(0.5) * s;
-  const V2<T> JS = fma(splat(hs), G, fma(splat(-s), J - Jeq, J));
-  const T b = round_to_multiple(theta * T(1.0 / 6.0), quantum_quarter_ulp(m0));
-  const V2<T> a = splat(b);
-  const V2<T> e12 = fma(T(0.5), JS, a), e34 = fma(T(-0.5), JS, a);
-  e[0] = m0 - T(4) * b;
-  e[1] = e12.x; e[2] = e12.y; e[3] = e34.x; e[4] = e34.y;
+__device__ __forceinline__ T th_base(T m0, T theta) {
+  return round_to_multiple(theta * T(1.0 / 6.0), quantum_quarter_ulp(m0));
 }
 
 }  // namespace pf

@@ -43,33 +43,83 @@ __device__ __forceinline__ unsigned pidx(int k, unsigned ps, unsigned s) {
   else return (unsigned)k * ps + s;
 }
 
-// Streamed CAC populations h and dendrite populations g (with the a_s^2 time
-// stretch g = g_pre + r_src (g_post,src - g_pre)) at (x, y); returns phi, psi
-// (compensated sums) and psi_o, the psi of the previous step (sum of g_pre, or
-// the stored lagged psi in the offset forms).  In the offset forms a
-// population held by site s decodes as w_i M_o(s) + stored value.
+// The nine loaded CAC values of a pull, before they are combined: rest density
+// phi_o of the site, the stored population of each direction's pair at its
+// source, and the sources' phi_o (16-bit forms: of every direction; else of the
+// directions that are not stored: 3, 4, 7, 8).
+__device__ __forceinline__ constexpr int pair9(int i) { return ((i - 1) & 1) + (i >= 5 ? 2 : 0); }
+__device__ __forceinline__ constexpr bool minus9(int i) { return ((i - 1) & 2) != 0; }
+
+// phi and the flux J = sum c h of the streamed CAC populations.
+template <typename S, typename R>
+__device__ __forceinline__ void cac_moments(const S (&v)[9], const R (&ph)[9], R& phi, V2<R>& J) {
+  R h[9];
+  h[0] = CacBase<R>(ph[0]).rest(ph[0]);
+#pragma unroll
+  for (int i = 1; i < 9; ++i) {
+    R base = R(0);
+    if (Codec<S>::kOffset || minus9(i)) {
+      const CacBase<R> b(ph[i]);
+      base = i < 5 ? b.axis : b.diag();
+    }
+    h[i] = minus9(i) ? pair_m<S, R>(v[i], base) : pair_p<S, R>(v[i], base);
+  }
+  CSum<R> sh;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) sh.add(h[i]);
+  phi = sh.value();
+  const V2<R> U = vec2(h[5], h[6]) - vec2(h[7], h[8]);
+  J = (vec2(h[1], h[2]) - vec2(h[3], h[4])) + vec2(U.x - U.y, U.x + U.y);
+}
+
+// Streamed CAC moments (phi and the flux J) and dendrite populations g (with
+// the a_s^2 time stretch g = g_pre + r_src (g_post,src - g_pre)) at (x, y);
+// phi and psi are compensated sums, psi_o is the psi of the previous step (sum
+// of g_pre, or the stored lagged psi in the offset forms).
 template <typename S, typename R, bool BIG = false>
-__device__ __forceinline__ void pull_hg(const StepArgs<S, R>& a, const Src9& src, R h[9],
+__device__ __forceinline__ void pull_hg(const StepArgs<S, R>& a, const Src9& src, V2<R>& J,
                                         R g[5], R& phi, R& psi, R& psio) {
   const unsigned ps = (unsigned)a.plane_stride;
   constexpr bool off = Codec<S>::kOffset;
-  CSum<R> sh;
+  auto pop = [&](int k, unsigned s) { return __ldg(pbase<BIG>(a.in, k, ps) + pidx<BIG>(k, ps, s)); };
+  auto aux = [&](int k, unsigned s) { return __ldg(pbase<BIG>(a.ain, k, ps) + pidx<BIG>(k, ps, s)); };
+  {
+    S v[9];
+    R ph[9];
+    ph[0] = aux(A_PHIO, src.s[0]);
 #pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    const R wm = off ? w9<R>(i) * ld<R>(pbase<BIG>(a.ain, A_PHIO, ps), pidx<BIG>(A_PHIO, ps, src.s[i])) : R(0);
-    h[i] = pop_off<S, R>(pbase<BIG>(a.in, P_H + i, ps), pidx<BIG>(P_H + i, ps, src.s[i]), wm);
-    sh.add(h[i]);
+    for (int i = 1; i < 9; ++i) {
+      v[i] = pop(P_H + pair9(i), src.s[i]);
+      ph[i] = off || minus9(i) ? aux(A_PHIO, src.s[i]) : R(0);
+    }
+    cac_moments<S, R>(v, ph, phi, J);
   }
-  phi = sh.value();
   CSum<R> sg;
   R po = R(0);
-  const R psio_own = off ? ld<R>(pbase<BIG>(a.ain, A_PSIO, ps), pidx<BIG>(A_PSIO, ps, src.s[0])) : R(0);
+  const R psio_own = off ? aux(A_PSIO, src.s[0]) : R(0);
 #pragma unroll
   for (int i = 0; i < 5; ++i) {
-    const R gold = pop_off<S, R>(pbase<BIG>(a.in, P_GPRE + i, ps), pidx<BIG>(P_GPRE + i, ps, src.s[0]), w5<R>(i) * psio_own);
-    const R wm = off ? w5<R>(i) * ld<R>(pbase<BIG>(a.ain, A_PSIO, ps), pidx<BIG>(A_PSIO, ps, src.s[i])) : R(0);
-    const R gpo = pop_off<S, R>(pbase<BIG>(a.in, P_GPOST + i, ps), pidx<BIG>(P_GPOST + i, ps, src.s[i]), wm);
-    const R rr = ld<R>(pbase<BIG>(a.ain, A_RR, ps), pidx<BIG>(A_RR, ps, src.s[i]));
+    const R gold = dec_off<S, R>(pop(P_GPRE + i, src.s[0]), w5<R>(i) * psio_own);
+    R gpo;
+    if constexpr (off) {
+      // density psi_o + F of the source; its planes: F/6 and the offsets of g_1, g_2
+      const R m = i == 0 ? psio_own : aux(A_PSIO, src.s[i]);
+      const R base = q5_base(m);
+      if (i == 0) gpo = fma(R(2), dec_off<S, R>(pop(P_GPOST, src.s[0]), R(0)), q5_rest(m, base));
+      else if (!minus9(i)) gpo = pair_p<S, R>(pop(P_GPOST + i, src.s[i]), base);
+      else gpo = pair_m<S, R>(pop(P_GPOST + i - 2, src.s[i]),
+                              fma(R(2), dec_off<S, R>(pop(P_GPOST, src.s[i]), R(0)), base));
+    } else {
+      if (i == 0) {
+        const R m = (R)pop(P_GPOST, src.s[0]);
+        gpo = q5_rest(m, q5_base(m));
+      } else if (!minus9(i)) {
+        gpo = (R)pop(P_GPOST + i, src.s[i]);
+      } else {
+        gpo = pair_m<S, R>(pop(P_GPOST + i - 2, src.s[i]), q5_base((R)pop(P_GPOST, src.s[i])));
+      }
+    }
+    const R rr = aux(A_RR, src.s[i]);
     g[i] = gold + (gpo - gold) * rr;
     sg.add(g[i]);
     po += gold;
@@ -93,47 +143,67 @@ struct SiteIn {
   R f[9], s[5];
   R phio, Co, Qo;
   uint8_t gid;
-  R e[5], Ho;     // thermal mode: streamed temperature populations, lagged H
+  R e[5], mo;     // thermal mode: streamed temperature populations, lagged rho H
 };
+
+// Streamed solute populations; Co is C of the last step at the site itself.
+template <typename S, typename R, bool BIG = false>
+__device__ __forceinline__ void pull_s(const StepArgs<S, R>& a, const Src9& src, R Co, R (&s)[5]) {
+  const unsigned ps = (unsigned)a.plane_stride;
+  constexpr bool off = Codec<S>::kOffset;
+  s[0] = q5_rest(Co, q5_base(Co));
+#pragma unroll
+  for (int i = 1; i < 5; ++i) {
+    const int k = P_S + pair9(i);
+    const S v = __ldg(pbase<BIG>(a.in, k, ps) + pidx<BIG>(k, ps, src.s[i]));
+    R base = R(0);
+    if (off || minus9(i))
+      base = q5_base(__ldg(pbase<BIG>(a.ain, A_CO, ps) + pidx<BIG>(A_CO, ps, src.s[i])));
+    s[i] = minus9(i) ? pair_m<S, R>(v, base) : pair_p<S, R>(v, base);
+  }
+}
 
 template <typename S, typename R, bool BIG = false, bool TH = false>
 __device__ __forceinline__ void load_site(const StepArgs<S, R>& a, const Src9& src,
                                           SiteIn<R>& in) {
   const unsigned ps = (unsigned)a.plane_stride;
-  constexpr bool off = Codec<S>::kOffset;
 #pragma unroll
   for (int i = 0; i < 9; ++i) in.f[i] = pop_ns<S, R>(pbase<BIG>(a.in, P_F + i, ps), pidx<BIG>(P_F + i, ps, src.s[i]));
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    const R wm = off ? w5<R>(i) * ld<R>(pbase<BIG>(a.ain, A_CO, ps), pidx<BIG>(A_CO, ps, src.s[i])) : R(0);
-    in.s[i] = pop_off<S, R>(pbase<BIG>(a.in, P_S + i, ps), pidx<BIG>(P_S + i, ps, src.s[i]), wm);
-  }
   in.phio = ld<R>(pbase<BIG>(a.ain, A_PHIO, ps), pidx<BIG>(A_PHIO, ps, src.s[0]));
   in.Co = ld<R>(pbase<BIG>(a.ain, A_CO, ps), pidx<BIG>(A_CO, ps, src.s[0]));
+  pull_s<S, R, BIG>(a, src, in.Co, in.s);
   in.Qo = ld<R>(pbase<BIG>(a.ain, A_QO, ps), pidx<BIG>(A_QO, ps, src.s[0]));
   in.gid = a.grain[src.s[0]];
   if constexpr (TH) {
-#pragma unroll
-    for (int i = 0; i < 5; ++i)
-      in.e[i] = ld<R>(pbase<BIG>(a.in, P_E + i, ps), pidx<BIG>(P_E + i, ps, src.s[i]));
-    in.Ho = ld<R>(pbase<BIG>(a.ain, A_HO, ps), pidx<BIG>(A_HO, ps, src.s[0]));
+    auto pop = [&](int k, unsigned s) { return ld<R>(pbase<BIG>(a.in, k, ps), pidx<BIG>(k, ps, s)); };
+    in.mo = pop(P_E, src.s[0]);
+    in.e[0] = q5_rest(in.mo, pop(P_E + 1, src.s[0]));
+    in.e[1] = pop(P_E + 2, src.s[1]);
+    in.e[2] = pop(P_E + 3, src.s[2]);
+    in.e[3] = fma(R(2), pop(P_E + 1, src.s[3]), -pop(P_E + 2, src.s[3]));
+    in.e[4] = fma(R(2), pop(P_E + 1, src.s[4]), -pop(P_E + 3, src.s[4]));
   }
 }
 
 // Supersaturation U of a site from its streamed solute populations (thermal
 // mode: U on the stencil neighbourhood feeds grad F), with the arithmetic of
 // the site update's own C and U.
+template <typename R>
+__device__ __forceinline__ R supersat(const KParams<R>& kp, const R (&s)[5], R psi) {
+  CSum<R> cs;
+#pragma unroll
+  for (int i = 0; i < 5; ++i) cs.add(s[i]);
+  const R C = cs.value();
+  const R omk = R(1) - kp.k;
+  const R A = (R(1) + kp.k) - omk * psi;
+  return (R(2) * C * frcp(A) - R(1)) * kp.inv_omk;
+}
 template <typename S, typename R, bool BIG = false>
 __device__ __forceinline__ R pull_U(const StepArgs<S, R>& a, const Src9& src, R psi) {
   const unsigned ps = (unsigned)a.plane_stride;
-  CSum<R> cs;
-#pragma unroll
-  for (int i = 0; i < 5; ++i)
-    cs.add(ld<R>(pbase<BIG>(a.in, P_S + i, ps), pidx<BIG>(P_S + i, ps, src.s[i])));
-  const R C = cs.value();
-  const R omk = R(1) - a.kp.k;
-  const R A = (R(1) + a.kp.k) - omk * psi;
-  return (R(2) * C * frcp(A) - R(1)) * a.kp.inv_omk;
+  R s[5];
+  pull_s<S, R, BIG>(a, src, __ldg(pbase<BIG>(a.ain, A_CO, ps) + pidx<BIG>(A_CO, ps, src.s[0])), s);
+  return supersat(a.kp, s, psi);
 }
 
 }  // namespace pf

@@ -22,10 +22,13 @@ struct Nb9 {
   T v[3][3];
 };
 
-// New state and diagnostic fields of a site.
+// New state and diagnostic fields of a site: of the pair-stored lattices the
+// odd parts (CAC: directions 1, 2 and 5, 6; D2Q5: directions 1, 2) and, for
+// the dendrite, the source F that its density psi + F gained.
 template <typename T>
 struct SiteOut {
-  T f[9], h[9], s[5], gpost[5];
+  T f[9], F;
+  V2<T> hA, hD, s, g;
   T ias2, phi, psi, C, U, p, vx, vy, Q, mu;
 };
 
@@ -33,17 +36,19 @@ struct SiteOut {
 template <typename T>
 struct ThermIn {
   T e[5];     // streamed temperature populations
-  T Ho;       // H of the previous step
+  T mo;       // rho H of the previous step
   Nb9<T> U;   // supersaturation on the 3 x 3 neighbourhood (for grad F)
 };
 template <typename T>
 struct ThermOut {
-  T e[5];     // post-collision temperature populations
-  T H, theta;
+  T m0, b;    // density rho H and axis base of the temperature lattice
+  V2<T> e;    // odd parts of directions 1, 2
+  T theta;
 };
 
 // Everything after streaming at one site:
-//   f, h, g, s   streamed populations (g after the a_s^2 time stretch)
+//   f, g, s      streamed populations (g after the a_s^2 time stretch)
+//   hJ           flux of the streamed CAC populations
 //   psio         psi of the previous step
 //   phio, Co, Qo lagged phi, C, Q_psi of the site
 //   P, S, VX, VY phi, psi and the lagged velocity on the 3 x 3 neighbourhood
@@ -56,22 +61,15 @@ struct ThermOut {
 // stored as the lagged source (o.Q) in place of Q.
 template <typename T, typename R, bool TH = false>
 __device__ __forceinline__ void site_math(const KParams<R>& kp, T rho_bar, T eps, T ct, T sn,
-                                          const T (&f_in)[9], const T (&h_in)[9],
-                                          const T (&g)[5], const T (&s_in)[5], T psio, T phio,
+                                          const T (&f_in)[9], V2<T> hJ,
+                                          const T (&g)[5], const T (&s)[5], T psio, T phio,
                                           T Co, T Qo, const Nb9<T>& P, const Nb9<T>& S,
                                           const Nb9<T>& VX, const Nb9<T>& VY, SiteOut<T>& o,
                                           const ThermIn<T>* ti = nullptr,
                                           ThermOut<T>* to = nullptr) {
   T* f = o.f;
-  T* h = o.h;
-  T* s = o.s;
 #pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    f[i] = f_in[i];
-    h[i] = h_in[i];
-  }
-#pragma unroll
-  for (int i = 0; i < 5; ++i) s[i] = s_in[i];
+  for (int i = 0; i < 9; ++i) f[i] = f_in[i];
 
   const T phi = P.v[1][1], psi = S.v[1][1];
   const V2<T> vo = vec2(VX.v[1][1], VY.v[1][1]);
@@ -196,7 +194,7 @@ __device__ __forceinline__ void site_math(const KParams<R>& kp, T rho_bar, T eps
 
   // ---- collisions ----
   collide_ns(f, p, rho, v, F, gr, kp);
-  collide_cac(h, phi, v, fma(T(1.0 / 3.0) * aphi, nf, fma(phi, v, (-phio) * vo)), kp);
+  collide_cac(hJ, phi, v, fma(T(1.0 / 3.0) * aphi, nf, fma(phi, v, (-phio) * vo)), o.hA, o.hD, kp);
   T Qs = Q;        // source stored as the lagged value
   {
     T s1;
@@ -221,27 +219,24 @@ __device__ __forceinline__ void site_math(const KParams<R>& kp, T rho_bar, T eps
     } else {
       s1 = frcp(T(kp.c_s1) * as2 + T(0.5));
     }
-    const T Fs = (Qs + T(0.5) * (Qs - Qo)) * T(kp.inv_tau0);
-#pragma unroll
-    for (int i = 0; i < 5; ++i) o.gpost[i] = g[i];
-    collide_q5(o.gpost, psi + Fs, s1, vec2(T(0), T(0)), (T(-1.0 / 3.0) * ias2) * vec2(Nx, Ny));
+    o.F = (Qs + T(0.5) * (Qs - Qo)) * T(kp.inv_tau0);
+    o.g = collide_q5(vec2(g[1], g[2]) - vec2(g[3], g[4]), s1, vec2(T(0), T(0)),
+                     (T(-1.0 / 3.0) * ias2) * vec2(Nx, Ny));
   }
   {
     const T E = T(2) * omk * T(kp.D) * qf * C * iA * iA;
     const V2<T> jeq = fma(C, v, fma(-E, gs, omk * fma(at, gs, jv * nf)));
     const T DC = T(2 * kp.D) * qf * iA;
     const T sc = frcp(T(3) * DC + T(0.5));
-    collide_q5(s, C, sc, jeq, fma(C, v, (-Co) * vo));
+    o.s = collide_q5(vec2(s[1], s[2]) - vec2(s[3], s[4]), sc, jeq, fma(C, v, (-Co) * vo));
   }
   if constexpr (TH) {
-    // d_t(rho H v) with rho_o H_o v_o of the previous step (backward difference)
-    const T rho_o = T(kp.rho_g) + phio * T(kp.drho);
+    // d_t(rho H v): backward difference with the previous step's rho H and v
     const V2<T> jH = rhoH * v;
-    const V2<T> dJ = fma(-(rho_o * ti->Ho), vo, jH);
-#pragma unroll
-    for (int i = 0; i < 5; ++i) to->e[i] = ti->e[i];
-    collide_th(to->e, rhoH, theta, T(kp.th_s), jH, dJ);
-    to->H = rhoH * irho;
+    to->m0 = rhoH;
+    to->b = th_base(rhoH, theta);
+    to->e = collide_q5(vec2(ti->e[1], ti->e[2]) - vec2(ti->e[3], ti->e[4]), T(kp.th_s), jH,
+                       fma(-ti->mo, vo, jH));
     to->theta = theta;
   }
   o.ias2 = ias2;
@@ -256,13 +251,55 @@ __device__ __forceinline__ void site_math(const KParams<R>& kp, T rho_bar, T eps
   o.mu = mu;
 }
 
+// Store the new state of a site (g: its streamed dendrite populations).
+template <typename S, typename R>
+__device__ __forceinline__ void store_state(const StepArgs<S, R>& a, unsigned site,
+                                            const SiteOut<R>& o, const R (&g)[5]) {
+  const unsigned ps = (unsigned)a.plane_stride;
+  auto put = [&](int k, S v) { plane(a.out, k, ps)[site] = v; };
+#pragma unroll
+  for (int i = 0; i < 9; ++i) st_ns<S, R>(plane(a.out, P_F + i, ps), site, o.f[i]);
+  {
+    const CacBase<R> b(o.phi);
+    put(P_H + 0, enc_pair<S, R>(b.axis, o.hA.x));
+    put(P_H + 1, enc_pair<S, R>(b.axis, o.hA.y));
+    put(P_H + 2, enc_pair<S, R>(b.diag(), o.hD.x));
+    put(P_H + 3, enc_pair<S, R>(b.diag(), o.hD.y));
+  }
+#pragma unroll
+  for (int i = 0; i < 5; ++i) st_off_w<S, R>(plane(a.out, P_GPRE + i, ps), site, g[i], w5<R>(i), o.psi);
+  if constexpr (Codec<S>::kOffset) {
+    const R f6 = q5_base(o.F);
+    put(P_GPOST + 0, enc_pair<S, R>(R(0), f6));
+    put(P_GPOST + 1, enc_pair<S, R>(R(0), f6 + o.g.x));
+    put(P_GPOST + 2, enc_pair<S, R>(R(0), f6 + o.g.y));
+  } else {
+    const R m = o.psi + o.F, base = q5_base(m);
+    put(P_GPOST + 0, Codec<S>::template enc<R>(m));
+    put(P_GPOST + 1, enc_pair<S, R>(base, o.g.x));
+    put(P_GPOST + 2, enc_pair<S, R>(base, o.g.y));
+  }
+  {
+    const R base = q5_base(o.C);
+    put(P_S + 0, enc_pair<S, R>(base, o.s.x));
+    put(P_S + 1, enc_pair<S, R>(base, o.s.y));
+  }
+  plane(a.aout, A_RR, ps)[site] = o.ias2;
+  plane(a.aout, A_PHIO, ps)[site] = o.phi;
+  plane(a.aout, A_CO, ps)[site] = o.C;
+  plane(a.aout, A_VXO, ps)[site] = o.vx;
+  plane(a.aout, A_VYO, ps)[site] = o.vy;
+  plane(a.aout, A_QO, ps)[site] = o.Q;
+  if constexpr (Codec<S>::kOffset) plane(a.aout, A_PSIO, ps)[site] = o.psi;
+}
+
 // One site: gather the stencil values from the traversal's shared-memory rows,
 // run site_math and store the new state and (if requested) the fields.
-// TH: thermal mode, with SU the supersaturation rows and in.e / in.Ho loaded.
+// TH: thermal mode, with SU the supersaturation rows and in.e / in.mo loaded.
 template <typename S, typename R, bool TH = false>
 __device__ __forceinline__ void site_update(const StepArgs<S, R>& a, const DomDesc& d,
                                             const Src9& src, const SiteIn<R>& in,
-                                            const R (&h_in)[9], const R (&g_in)[5], R psio,
+                                            V2<R> hJ, const R (&g_in)[5], R psio,
                                             Rows3<R> SP, Rows3<R> SS, Rows3<R> SVX,
                                             Rows3<R> SVY, int c, Rows3<R> SU = Rows3<R>{}) {
   const unsigned ps = (unsigned)a.plane_stride;
@@ -284,38 +321,21 @@ __device__ __forceinline__ void site_update(const StepArgs<S, R>& a, const DomDe
   if constexpr (TH) {
 #pragma unroll
     for (int i = 0; i < 5; ++i) ti.e[i] = in.e[i];
-    ti.Ho = in.Ho;
+    ti.mo = in.mo;
     ti.U = nb(SU);
   }
   site_math<R, R, TH>(a.kp, static_cast<R>(d.rho_bar), static_cast<R>(d.eps_s),
-                      static_cast<R>(cs.x), static_cast<R>(cs.y), in.f, h_in, g_in, in.s, psio,
+                      static_cast<R>(cs.x), static_cast<R>(cs.y), in.f, hJ, g_in, in.s, psio,
                       in.phio, in.Co, in.Qo, nb(SP), nb(SS), nb(SVX), nb(SVY), o, &ti, &to);
 
-  // ---- store ----
-  const R phi = o.phi, psi = o.psi, C = o.C;
-#pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    st_ns<S, R>(plane(a.out, P_F + i, ps), site, o.f[i]);
-    st_off_w<S, R>(plane(a.out, P_H + i, ps), site, o.h[i], w9<R>(i), phi);
-  }
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    st_off_w<S, R>(plane(a.out, P_GPRE + i, ps), site, g_in[i], w5<R>(i), psi);
-    st_off_w<S, R>(plane(a.out, P_GPOST + i, ps), site, o.gpost[i], w5<R>(i), psi);
-    st_off_w<S, R>(plane(a.out, P_S + i, ps), site, o.s[i], w5<R>(i), C);
-  }
-  plane(a.aout, A_RR, ps)[site] = o.ias2;
-  plane(a.aout, A_PHIO, ps)[site] = phi;
-  plane(a.aout, A_CO, ps)[site] = C;
-  plane(a.aout, A_VXO, ps)[site] = o.vx;
-  plane(a.aout, A_VYO, ps)[site] = o.vy;
-  plane(a.aout, A_QO, ps)[site] = o.Q;
-  if constexpr (Codec<S>::kOffset) plane(a.aout, A_PSIO, ps)[site] = psi;
+  store_state<S, R>(a, site, o, g_in);
   if constexpr (TH) {
-#pragma unroll
-    for (int i = 0; i < 5; ++i) st<S, R>(plane(a.out, P_E + i, ps), site, to.e[i]);
-    plane(a.aout, A_HO, ps)[site] = to.H;
+    st<S, R>(plane(a.out, P_E, ps), site, to.m0);
+    st<S, R>(plane(a.out, P_E + 1, ps), site, to.b);
+    st<S, R>(plane(a.out, P_E + 2, ps), site, to.b + to.e.x);
+    st<S, R>(plane(a.out, P_E + 3, ps), site, to.b + to.e.y);
   }
+  const R phi = o.phi, psi = o.psi, C = o.C;
   if (a.fields) {
     R* fl = a.fields;
     plane(fl, FLD_PHI, ps)[site] = phi;

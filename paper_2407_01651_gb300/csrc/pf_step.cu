@@ -41,8 +41,9 @@ __global__ void __launch_bounds__(256) k_step_tile(StepArgs<S, R> a) {
 
     for (int i = tid; i < SW * SH; i += nthr) {
       const int gx = wrapi(x0 + (i % SW) - 1, nx), gy = wrapi(y0 + (i / SW) - 1, ny);
-      R h[9], g[5], phi, psi, po;
-      pull_hg<S, R, BIG>(a, sources(d, gx, gy), h, g, phi, psi, po);
+      V2<R> J;
+      R g[5], phi, psi, po;
+      pull_hg<S, R, BIG>(a, sources(d, gx, gy), J, g, phi, psi, po);
       sphi[i] = phi;
       spsi[i] = psi;
       const unsigned site = (unsigned)d.off + (unsigned)gy * (unsigned)nx + (unsigned)gx;
@@ -54,13 +55,14 @@ __global__ void __launch_bounds__(256) k_step_tile(StepArgs<S, R> a) {
     const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
     if (x < nx && y < ny) {
       const Src9 src = sources(d, x, y);
-      R h[9], g[5], phi, psi, po;
-      pull_hg<S, R, BIG>(a, src, h, g, phi, psi, po);
+      V2<R> J;
+      R g[5], phi, psi, po;
+      pull_hg<S, R, BIG>(a, src, J, g, phi, psi, po);
       const int r = threadIdx.y + 1;
       auto rows = [&](const R* X) { return Rows3<R>{X + (r - 1) * SW, X + r * SW, X + (r + 1) * SW}; };
       SiteIn<R> in;
       load_site<S, R, BIG>(a, src, in);
-      site_update(a, d, src, in, h, g, po, rows(sphi), rows(spsi), rows(svx), rows(svy),
+      site_update(a, d, src, in, J, g, po, rows(sphi), rows(spsi), rows(svx), rows(svy),
                   threadIdx.x + 1);
     }
     __syncthreads();
@@ -122,23 +124,24 @@ __device__ __forceinline__ void ymarch_tiles(const StepArgs<S, R>& a,
       sc = w + 1;
     }
 
-    R hC[9], gC[5], poC = R(0);
+    V2<R> JC = vec2(R(0), R(0));
+    R gC[5], poC = R(0);
     // rows ya-1 and ya into the ring (warm-up)
     for (int k = 0; k < 2; ++k) {
       const int yy = wrapi(ya - 1 + k, ny);
       const int slot = (ya - 1 + k) & 3;
       if (active) {
         const Src9 src = sources(d, col, yy);
-        R h[9], g[5], phi, psi, po;
-        pull_hg<S, R, BIG>(a, src, h, g, phi, psi, po);
+        V2<R> J;
+        R g[5], phi, psi, po;
+        pull_hg<S, R, BIG>(a, src, J, g, phi, psi, po);
         ring[0][slot][sc] = phi;
         ring[1][slot][sc] = psi;
         ring[2][slot][sc] = ld<R>(pbase<BIG>(a.ain, A_VXO, ps), pidx<BIG>(A_VXO, ps, src.s[0]));
         ring[3][slot][sc] = ld<R>(pbase<BIG>(a.ain, A_VYO, ps), pidx<BIG>(A_VYO, ps, src.s[0]));
         if constexpr (TH) ring[NF - 1][slot][sc] = pull_U<S, R, BIG>(a, src, psi);
         if (k == 1) {
-#pragma unroll
-          for (int i = 0; i < 9; ++i) hC[i] = h[i];
+          JC = J;
 #pragma unroll
           for (int i = 0; i < 5; ++i) gC[i] = g[i];
           poC = po;
@@ -152,12 +155,13 @@ __device__ __forceinline__ void ymarch_tiles(const StepArgs<S, R>& a,
       SiteIn<R> in;
       const Src9 srcj = sources(d, col, j);
       if (interior) load_site<S, R, BIG, TH>(a, srcj, in);
-      R hL[9], gL[5], poL = R(0);
+      V2<R> JL = vec2(R(0), R(0));
+      R gL[5], poL = R(0);
       if (active) {
         const int yn = j + 1 >= ny ? j + 1 - ny : j + 1;
         const Src9 src = sources(d, col, yn);
         R phi, psi;
-        pull_hg<S, R, BIG>(a, src, hL, gL, phi, psi, poL);
+        pull_hg<S, R, BIG>(a, src, JL, gL, phi, psi, poL);
         const int slot = (j + 1) & 3;
         ring[0][slot][sc] = phi;
         ring[1][slot][sc] = psi;
@@ -169,11 +173,10 @@ __device__ __forceinline__ void ymarch_tiles(const StepArgs<S, R>& a,
       if (interior) {
         const int m = (j - 1) & 3, c0 = j & 3, pp = (j + 1) & 3;
         auto rows = [&](int f) { return Rows3<R>{ring[f][m], ring[f][c0], ring[f][pp]}; };
-        site_update<S, R, TH>(a, d, srcj, in, hC, gC, poC, rows(0), rows(1), rows(2), rows(3),
+        site_update<S, R, TH>(a, d, srcj, in, JC, gC, poC, rows(0), rows(1), rows(2), rows(3),
                               sc, rows(NF - 1));
       }
-#pragma unroll
-      for (int i = 0; i < 9; ++i) hC[i] = hL[i];
+      JC = JL;
 #pragma unroll
       for (int i = 0; i < 5; ++i) gC[i] = gL[i];
       poC = poL;
@@ -218,7 +221,7 @@ __global__ void __launch_bounds__(YM_THREADS, sizeof(R) == 4 ? (TH ? 3 : 4) : 2)
   }
 }
 
-// Buffers of more than 2^32 elements (plane stride x 33 population planes)
+// Buffers of more than 2^32 elements (plane stride x population planes)
 // take the 64-bit plane-base addressing of the pull helpers.
 inline bool big_handle(long long plane_stride, bool thermal) {
   return (unsigned long long)plane_stride * (thermal ? N_POP_TH : N_POP) >= (1ull << 32);

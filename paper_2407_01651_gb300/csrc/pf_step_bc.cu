@@ -27,143 +27,102 @@
 // FP32 and FP64 storage only.
 #include <type_traits>
 
-#include "pf_site.cuh"
+#include "pf_sides.cuh"
 
 namespace pf {
 
 namespace {
 
-__device__ __forceinline__ constexpr int cx9(int i) {
-  return (i == 1 || i == 5 || i == 8) ? 1 : ((i == 3 || i == 6 || i == 7) ? -1 : 0);
-}
-__device__ __forceinline__ constexpr int cy9(int i) {
-  return (i == 2 || i == 5 || i == 6) ? 1 : ((i == 4 || i == 7 || i == 8) ? -1 : 0);
-}
-__device__ __forceinline__ constexpr int opp9(int i) {
-  return i == 0 ? 0 : (i <= 4 ? (i + 1) % 4 + 1 : (i + 1) % 4 + 5);
-}
-// reflections that flip c_x / c_y
-__device__ __forceinline__ int mirx9(int i) {
-  switch (i) {
-    case 1: return 3; case 3: return 1; case 5: return 6; case 6: return 5;
-    case 7: return 8; case 8: return 7; default: return i;
-  }
-}
-__device__ __forceinline__ int miry9(int i) {
-  switch (i) {
-    case 2: return 4; case 4: return 2; case 5: return 8; case 8: return 5;
-    case 6: return 7; case 7: return 6; default: return i;
-  }
-}
+// Populations of the pair-stored lattices with the direction known at run time
+// only: plane of the pair and whether the opposite one is stored.
+__device__ __forceinline__ int pair_rt(int q) { return ((q - 1) & 1) + (q >= 5 ? 2 : 0); }
+__device__ __forceinline__ bool minus_rt(int q) { return ((q - 1) & 2) != 0; }
 
-__device__ __forceinline__ unsigned site_at(const DomDesc& d, int x, int y) {
-  return (unsigned)d.off + (unsigned)y * (unsigned)d.nx + (unsigned)x;
-}
-
-// Source of the population of direction i pulled by (x, y): site, direction
-// to read and mode (0 plain or reflected, 1 wall bounce, 2 far-field bounce,
-// 3 inlet bounce, 4 outlet: source clamped to the last site, 5 extrapolation
-// inlet: the source is the ghost node beyond the side, whose NS population is
-// built from the fluid site next to it, the one returned).
-struct PullSrc {
-  unsigned site;
-  int q, mode;
-};
-// IO: some side of the launch is an inlet or an outlet; without them the
-// compiler drops those branches from the boundary pulls
-template <bool IO>
-__device__ __forceinline__ int bounce_rank(int t) {
-  return t == BC_WALL ? 1 : (t == BC_FARFIELD ? 2 : (IO && t == BC_INLET ? 3 : 0));
-}
-template <bool IO>
-__device__ __forceinline__ PullSrc pull_src(const DomDesc& d, int x, int y, int i) {
-  const int nx = d.nx, ny = d.ny;
-  int sx = x - cx9(i), sy = y - cy9(i), q = i, bounce = 0, outlet = 0, nee = 0;
-  if (sx < 0 || sx >= nx) {
-    const int t = d.bc[sx < 0 ? 0 : 1];
-    if (t == BC_PERIODIC) sx += sx < 0 ? nx : -nx;
-    else if (t == BC_SYMMETRIC) { sx = sx < 0 ? -1 - sx : 2 * nx - 1 - sx; q = mirx9(q); }
-    else if (IO && t == BC_OUTLET) { sx = sx < 0 ? 0 : nx - 1; outlet = 1; }
-    else if (IO && t == BC_INLET_NEE) { sx = sx < 0 ? 0 : nx - 1; nee = 1; }
-    else bounce = bounce_rank<IO>(t);
-  }
-  if (sy < 0 || sy >= ny) {
-    const int t = d.bc[sy < 0 ? 2 : 3];
-    if (t == BC_PERIODIC) sy += sy < 0 ? ny : -ny;
-    else if (t == BC_SYMMETRIC) { sy = sy < 0 ? -1 - sy : 2 * ny - 1 - sy; q = miry9(q); }
-    else if (IO && t == BC_OUTLET) { sy = sy < 0 ? 0 : ny - 1; outlet = 1; }
-    else if (IO && t == BC_INLET_NEE) { sy = sy < 0 ? 0 : ny - 1; nee = 1; }
-    else bounce = max(bounce, bounce_rank<IO>(t));
-  }
-  if (bounce) return {site_at(d, x, y), opp9(i), bounce};
-  return {site_at(d, sx, sy), q, nee ? 5 : (outlet ? 4 : 0)};
-}
-
-// The lattices other than NS see an extrapolation inlet as an inlet:
-// anti-bounce-back at the site itself.
-template <bool IO>
-__device__ __forceinline__ PullSrc scalar_src(const DomDesc& d, int x, int y, int i) {
-  PullSrc p = pull_src<IO>(d, x, y, i);
-  if (IO && p.mode == 5) p = {site_at(d, x, y), opp9(i), 3};
-  return p;
-}
-
-// A pull source of (x, y) lies beyond a non-periodic side.
-__device__ __forceinline__ bool near_side(const DomDesc& d, int x, int y) {
-  return (x == 0 && d.bc[0]) || (x == d.nx - 1 && d.bc[1]) || (y == 0 && d.bc[2]) ||
-         (y == d.ny - 1 && d.bc[3]);
-}
-
-// Ring fields: 0 phi, 1 psi, 2 vx_o, 3 vy_o, 4 U.  Ghost value across one side
-// of type t on axis (0: x, 1: y) from the mirror site's value v.
-template <typename R, bool IO>
-__device__ __forceinline__ R ghost_map(const KParams<R>& kp, int t, int axis, int field, R v) {
-  if (IO && t == BC_OUTLET) return v;
-  if (field == 2 || field == 3) {
-    const bool normal = (field == 2) == (axis == 0);
-    if (t == BC_SYMMETRIC) return normal ? -v : v;
-    if (IO && t == BC_INLET) return R(2) * (field == 2 ? kp.vin_x : kp.vin_y) - v;
-    if (IO && t == BC_INLET_NEE) return field == 2 ? kp.vin_x : kp.vin_y;   // the ghost is the node
-    return -v;
-  }
-  if (t == BC_FARFIELD || (IO && (t == BC_INLET || t == BC_INLET_NEE))) {
-    if (field == 1) return R(-2) - v;   // 2 psi_far - psi, psi_far = -1
-    if (field == 4) return -v;          // 2 U_far - U, U_far = 0
-    if (IO && field == 0 && t != BC_FARFIELD) return R(2) - v;   // liquid inflow, phi = 1
-  }
-  return v;
-}
-
+// The pulls at a side first issue every load and then combine the values: with
+// the source of each direction decided and used one after the other, each
+// load's latency was waited for in turn (4.6 us a row of tiles, 1.5 us in the
+// periodic kernel).
 template <typename S, typename R, bool BIG, bool IO>
 __device__ __forceinline__ void pull_hg_b(const StepArgs<S, R>& a, const DomDesc& d, int x,
-                                          int y, R h[9], R g[5], R& phi, R& psi, R& psio) {
+                                          int y, V2<R>& J, R g[5], R& phi, R& psi, R& psio) {
   const unsigned ps = (unsigned)a.plane_stride;
   const unsigned own = site_at(d, x, y);
+  auto pop = [&](int k, unsigned s) { return ld<R>(pbase<BIG>(a.in, k, ps), pidx<BIG>(k, ps, s)); };
+  auto aux = [&](int k, unsigned s) { return ld<R>(pbase<BIG>(a.ain, k, ps), pidx<BIG>(k, ps, s)); };
+  R v[9], ph[9], gv[5], m[5], rr[5], gold[5];
+  int how[9];       // 4 q + class of the mode (0 as is, 2 far field, 3 inlet)
+  ph[0] = aux(A_PHIO, own);
+  m[0] = pop(P_GPOST, own);
+  rr[0] = aux(A_RR, own);
+#pragma unroll
+  for (int i = 0; i < 5; ++i) gold[i] = pop(P_GPRE + i, own);
+#pragma unroll
+  for (int i = 1; i < 9; ++i) {
+    const PullSrc p = scalar_src<IO>(d, x, y, i);
+    how[i] = 4 * p.q + (p.mode == 2 || p.mode == 3 ? p.mode : 0);
+    v[i] = pop(P_H + pair_rt(p.q), p.site);
+    ph[i] = aux(A_PHIO, p.site);
+    if (i < 5) {
+      gv[i] = pop(P_GPOST + 1 + pair_rt(p.q), p.site);
+      m[i] = pop(P_GPOST, p.site);
+      rr[i] = aux(A_RR, p.site);
+    }
+  }
+  R h[9];
+  h[0] = CacBase<R>(ph[0]).rest(ph[0]);
+#pragma unroll
+  for (int i = 1; i < 9; ++i) {
+    const CacBase<R> b(ph[i]);
+    const R base = i < 5 ? b.axis : b.diag();   // a reflection keeps axes and diagonals apart
+    h[i] = minus_rt(how[i] >> 2) ? fma(R(2), base, -v[i]) : v[i];
+    if (IO && (how[i] & 3) == 3) h[i] = -h[i] + R(2) * w9<R>(i) * R(1);   // inlet: phi = 1
+  }
   CSum<R> sh;
 #pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    const PullSrc p = scalar_src<IO>(d, x, y, i);
-    R v = ld<R>(pbase<BIG>(a.in, P_H + p.q, ps), pidx<BIG>(P_H + p.q, ps, p.site));
-    if (IO && p.mode == 3) v = -v + R(2) * w9<R>(i) * R(1);   // inlet: phi = 1
-    h[i] = v;
-    sh.add(h[i]);
-  }
+  for (int i = 0; i < 9; ++i) sh.add(h[i]);
   phi = sh.value();
+  const V2<R> U = vec2(h[5], h[6]) - vec2(h[7], h[8]);
+  J = (vec2(h[1], h[2]) - vec2(h[3], h[4])) + vec2(U.x - U.y, U.x + U.y);
   CSum<R> sg;
   R po = R(0);
 #pragma unroll
   for (int i = 0; i < 5; ++i) {
-    const PullSrc p = scalar_src<IO>(d, x, y, i);
-    const R gold = ld<R>(pbase<BIG>(a.in, P_GPRE + i, ps), pidx<BIG>(P_GPRE + i, ps, own));
-    R gpo = ld<R>(pbase<BIG>(a.in, P_GPOST + p.q, ps), pidx<BIG>(P_GPOST + p.q, ps, p.site));
-    if (p.mode == 2 || p.mode == 3) gpo = -gpo + R(2) * w5<R>(i) * R(-1);
-    const R rr = ld<R>(pbase<BIG>(a.ain, A_RR, ps), pidx<BIG>(A_RR, ps, p.site));
-    g[i] = gold + (gpo - gold) * rr;
+    const R base = q5_base(m[i]);
+    R gpo;
+    if (i == 0) gpo = q5_rest(m[0], base);
+    else {
+      gpo = minus_rt(how[i] >> 2) ? fma(R(2), base, -gv[i]) : gv[i];
+      if (how[i] & 3) gpo = -gpo + R(2) * w5<R>(i) * R(-1);
+    }
+    g[i] = gold[i] + (gpo - gold[i]) * rr[i];
     sg.add(g[i]);
-    po += gold;
+    po += gold[i];
   }
   psi = sg.value();
   psio = po;
+}
+
+// Streamed solute populations next to a side (C_far = 1).
+template <typename S, typename R, bool BIG, bool IO>
+__device__ __forceinline__ void pull_s_b(const StepArgs<S, R>& a, const DomDesc& d, int x, int y,
+                                         R Co, R (&s)[5]) {
+  const unsigned ps = (unsigned)a.plane_stride;
+  R v[5], c[5];
+  int how[5];
+#pragma unroll
+  for (int i = 1; i < 5; ++i) {
+    const PullSrc p = scalar_src<IO>(d, x, y, i);
+    how[i] = 2 * p.q + (p.mode == 2 || p.mode == 3);
+    const int k = P_S + pair_rt(p.q);
+    v[i] = ld<R>(pbase<BIG>(a.in, k, ps), pidx<BIG>(k, ps, p.site));
+    c[i] = ld<R>(pbase<BIG>(a.ain, A_CO, ps), pidx<BIG>(A_CO, ps, p.site));
+  }
+  s[0] = q5_rest(Co, q5_base(Co));
+#pragma unroll
+  for (int i = 1; i < 5; ++i) {
+    s[i] = minus_rt(how[i] >> 1) ? fma(R(2), q5_base(c[i]), -v[i]) : v[i];
+    if (how[i] & 1) s[i] = -s[i] + R(2) * w5<R>(i) * R(1);
+  }
 }
 
 template <typename S, typename R, bool BIG, bool TH, bool IO>
@@ -171,79 +130,65 @@ __device__ __forceinline__ void load_site_b(const StepArgs<S, R>& a, const DomDe
                                             int y, SiteIn<R>& in) {
   const unsigned ps = (unsigned)a.plane_stride;
   const unsigned own = site_at(d, x, y);
-  in.phio = ld<R>(pbase<BIG>(a.ain, A_PHIO, ps), pidx<BIG>(A_PHIO, ps, own));
+  auto pop = [&](int k, unsigned s) { return ld<R>(pbase<BIG>(a.in, k, ps), pidx<BIG>(k, ps, s)); };
+  auto aux = [&](int k, unsigned s) { return ld<R>(pbase<BIG>(a.ain, k, ps), pidx<BIG>(k, ps, s)); };
+  in.phio = aux(A_PHIO, own);
+  in.Co = aux(A_CO, own);
+  in.Qo = aux(A_QO, own);
+  in.gid = a.grain[own];
   R vxo = R(0), vyo = R(0);
   if constexpr (IO) {
-    vxo = ld<R>(pbase<BIG>(a.ain, A_VXO, ps), pidx<BIG>(A_VXO, ps, own));
-    vyo = ld<R>(pbase<BIG>(a.ain, A_VYO, ps), pidx<BIG>(A_VYO, ps, own));
+    vxo = aux(A_VXO, own);
+    vyo = aux(A_VYO, own);
   }
-  const R rho_o = a.kp.rho_g + in.phio * a.kp.drho;
+  PullSrc p[9];
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
-    const PullSrc p = pull_src<IO>(d, x, y, i);
-    if (IO && p.mode == 4) {
-      // pressure outlet p = 0: -f*_opp(own) + 2 rho_o w_i [(c.v_o)^2 / (2 cs^4) - v_o^2 / (2 cs^2)]
-      const R fo = ld<R>(pbase<BIG>(a.in, P_F + opp9(i), ps), pidx<BIG>(P_F + opp9(i), ps, own));
-      const R cu = R(cx9(i)) * vxo + R(cy9(i)) * vyo;
-      in.f[i] = -fo + R(2) * rho_o * w9<R>(i) * (R(4.5) * cu * cu - R(1.5) * (vxo * vxo + vyo * vyo));
-    } else {
-      R v = ld<R>(pbase<BIG>(a.in, P_F + p.q, ps), pidx<BIG>(P_F + p.q, ps, p.site));
-      if (IO && p.mode == 3)   // inlet: moving-wall bounce-back
-        v += R(2) * (a.kp.rho_g + a.kp.drho) * w9<R>(i) * R(3) *
-             (R(cx9(i)) * a.kp.vin_x + R(cy9(i)) * a.kp.vin_y);
-      if (IO && p.mode == 5) {
-        // extrapolation inlet: the ghost node's post-collision population is
-        // f_q^eq(p_b, rho_l, u_in) + f*_q(x_f) - f_q^eq(p_f, rho_f, v_f) with
-        // p_b = p_f, i.e. f*_q(x_f) + rho_l s_q(u_in) - rho_f s_q(v_f), with
-        // s_q(v) = w_q [3 c.v + 4.5 (c.v)^2 - 1.5 v^2] and the fluid site's
-        // last-step rho and v
-        const R fx = ld<R>(pbase<BIG>(a.ain, A_VXO, ps), pidx<BIG>(A_VXO, ps, p.site));
-        const R fy = ld<R>(pbase<BIG>(a.ain, A_VYO, ps), pidx<BIG>(A_VYO, ps, p.site));
-        const R fphi = ld<R>(pbase<BIG>(a.ain, A_PHIO, ps), pidx<BIG>(A_PHIO, ps, p.site));
-        const R cb = R(cx9(p.q)) * a.kp.vin_x + R(cy9(p.q)) * a.kp.vin_y;
-        const R cf = R(cx9(p.q)) * fx + R(cy9(p.q)) * fy;
-        const R sb = R(3) * cb + R(4.5) * cb * cb -
-                     R(1.5) * (a.kp.vin_x * a.kp.vin_x + a.kp.vin_y * a.kp.vin_y);
-        const R sf = R(3) * cf + R(4.5) * cf * cf - R(1.5) * (fx * fx + fy * fy);
-        v += w9<R>(p.q) * ((a.kp.rho_g + a.kp.drho) * sb - (a.kp.rho_g + fphi * a.kp.drho) * sf);
-      }
-      in.f[i] = v;
-    }
+    p[i] = pull_src<IO>(d, x, y, i);
+    // a pressure outlet takes the site's own opposite population
+    const bool outlet = IO && p[i].mode == 4;
+    in.f[i] = pop(P_F + (outlet ? opp9(i) : p[i].q), outlet ? own : p[i].site);
   }
+  pull_s_b<S, R, BIG, IO>(a, d, x, y, in.Co, in.s);
+  if constexpr (TH) {
+    R v[5], b[5];
+    int how[5];
+    in.mo = pop(P_E, own);
+    b[0] = pop(P_E + 1, own);
 #pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    const PullSrc p = scalar_src<IO>(d, x, y, i);
-    R v = ld<R>(pbase<BIG>(a.in, P_S + p.q, ps), pidx<BIG>(P_S + p.q, ps, p.site));
-    if (p.mode == 2 || p.mode == 3) v = -v + R(2) * w5<R>(i) * R(1);   // C_far = 1
-    in.s[i] = v;
-    if constexpr (TH) {
-      R e = ld<R>(pbase<BIG>(a.in, P_E + p.q, ps), pidx<BIG>(P_E + p.q, ps, p.site));
-      if (p.mode == 2 || p.mode == 3) e = -e + R(2) * w5<R>(i) * a.kp.th_far;
-      in.e[i] = e;
+    for (int i = 1; i < 5; ++i) {
+      const PullSrc q = scalar_src<IO>(d, x, y, i);
+      how[i] = 2 * q.q + (q.mode == 2 || q.mode == 3);
+      v[i] = pop(P_E + 2 + pair_rt(q.q), q.site);
+      b[i] = pop(P_E + 1, q.site);
+    }
+    in.e[0] = q5_rest(in.mo, b[0]);
+#pragma unroll
+    for (int i = 1; i < 5; ++i) {
+      in.e[i] = minus_rt(how[i] >> 1) ? fma(R(2), b[i], -v[i]) : v[i];
+      if (how[i] & 1) in.e[i] = -in.e[i] + R(2) * w5<R>(i) * a.kp.th_far;
     }
   }
-  in.Co = ld<R>(pbase<BIG>(a.ain, A_CO, ps), pidx<BIG>(A_CO, ps, own));
-  in.Qo = ld<R>(pbase<BIG>(a.ain, A_QO, ps), pidx<BIG>(A_QO, ps, own));
-  in.gid = a.grain[own];
-  if constexpr (TH) in.Ho = ld<R>(pbase<BIG>(a.ain, A_HO, ps), pidx<BIG>(A_HO, ps, own));
+  if constexpr (IO) {
+    const R rho_o = a.kp.rho_g + in.phio * a.kp.drho;
+#pragma unroll
+    for (int i = 0; i < 9; ++i)
+      in.f[i] = side_ns<R>(a.kp, p[i], i, in.f[i], rho_o, vxo, vyo, [&](R& fx, R& fy, R& fphi) {
+        fx = aux(A_VXO, p[i].site);
+        fy = aux(A_VYO, p[i].site);
+        fphi = aux(A_PHIO, p[i].site);
+      });
+  }
 }
 
 template <typename S, typename R, bool BIG, bool IO>
 __device__ __forceinline__ R pull_U_b(const StepArgs<S, R>& a, const DomDesc& d, int x, int y,
                                       R psi) {
   const unsigned ps = (unsigned)a.plane_stride;
-  CSum<R> cs;
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    const PullSrc p = scalar_src<IO>(d, x, y, i);
-    R v = ld<R>(pbase<BIG>(a.in, P_S + p.q, ps), pidx<BIG>(P_S + p.q, ps, p.site));
-    if (p.mode == 2 || p.mode == 3) v = -v + R(2) * w5<R>(i) * R(1);
-    cs.add(v);
-  }
-  const R C = cs.value();
-  const R omk = R(1) - a.kp.k;
-  const R A = (R(1) + a.kp.k) - omk * psi;
-  return (R(2) * C * frcp(A) - R(1)) * a.kp.inv_omk;
+  R s[5];
+  pull_s_b<S, R, BIG, IO>(a, d, x, y, ld<R>(pbase<BIG>(a.ain, A_CO, ps),
+                                            pidx<BIG>(A_CO, ps, site_at(d, x, y))), s);
+  return supersat(a.kp, s, psi);
 }
 
 }  // namespace
@@ -285,7 +230,7 @@ __global__ void __launch_bounds__(YM_THREADS, sizeof(R) == 4 ? 3 : 2)
 
     // ring values of row yr (ya-1 .. yb, possibly a ghost row) and the
     // streamed h, g of the site (col, row) they were computed at
-    auto fill = [&](int yr, R (&h)[9], R (&g)[5], R& po) {
+    auto fill = [&](int yr, V2<R>& J, R (&g)[5], R& po) {
       int ey = yr, ty = -1;
       if (yr < 0) {
         if (d.bc[2]) { ey = 0; ty = d.bc[2]; } else ey = yr + ny;
@@ -293,9 +238,10 @@ __global__ void __launch_bounds__(YM_THREADS, sizeof(R) == 4 ? 3 : 2)
         if (d.bc[3]) { ey = ny - 1; ty = d.bc[3]; } else ey = yr - ny;
       }
       R v[NF];
-      const bool near = near_side(d, col, ey);
-      if (near) pull_hg_b<S, R, BIG, IO>(a, d, col, ey, h, g, v[0], v[1], po);
-      else pull_hg<S, R, BIG>(a, sources(d, col, ey), h, g, v[0], v[1], po);
+      // one path per warp: lanes away from the side pull the same values there
+      const bool near = __any_sync(__activemask(), near_side(d, col, ey));
+      if (near) pull_hg_b<S, R, BIG, IO>(a, d, col, ey, J, g, v[0], v[1], po);
+      else pull_hg<S, R, BIG>(a, sources(d, col, ey), J, g, v[0], v[1], po);
       const unsigned s0 = site_at(d, col, ey);
       v[2] = ld<R>(pbase<BIG>(a.ain, A_VXO, ps), pidx<BIG>(A_VXO, ps, s0));
       v[3] = ld<R>(pbase<BIG>(a.ain, A_VYO, ps), pidx<BIG>(A_VYO, ps, s0));
@@ -311,14 +257,15 @@ __global__ void __launch_bounds__(YM_THREADS, sizeof(R) == 4 ? 3 : 2)
       }
     };
 
-    R hC[9], gC[5], poC = R(0);
+    V2<R> JC = vec2(R(0), R(0));
+    R gC[5], poC = R(0);
     for (int k = 0; k < 2; ++k) {
       if (active) {
-        R h[9], g[5], po;
-        fill(ya - 1 + k, h, g, po);
+        V2<R> J;
+        R g[5], po;
+        fill(ya - 1 + k, J, g, po);
         if (k == 1) {
-#pragma unroll
-          for (int i = 0; i < 9; ++i) hC[i] = h[i];
+          JC = J;
 #pragma unroll
           for (int i = 0; i < 5; ++i) gC[i] = g[i];
           poC = po;
@@ -330,7 +277,7 @@ __global__ void __launch_bounds__(YM_THREADS, sizeof(R) == 4 ? 3 : 2)
       SiteIn<R> in;
       Src9 srcj;
       if (interior) {
-        if (near_side(d, col, j)) {
+        if (__any_sync(__activemask(), near_side(d, col, j))) {
           load_site_b<S, R, BIG, TH, IO>(a, d, col, j, in);
           srcj.s[0] = site_at(d, col, j);
         } else {
@@ -338,17 +285,17 @@ __global__ void __launch_bounds__(YM_THREADS, sizeof(R) == 4 ? 3 : 2)
           load_site<S, R, BIG, TH>(a, srcj, in);
         }
       }
-      R hL[9], gL[5], poL = R(0);
-      if (active) fill(j + 1, hL, gL, poL);
+      V2<R> JL = vec2(R(0), R(0));
+      R gL[5], poL = R(0);
+      if (active) fill(j + 1, JL, gL, poL);
       __syncthreads();
       if (interior) {
         const int m = (j - 1) & 3, c0 = j & 3, pp = (j + 1) & 3;
         auto rows = [&](int f) { return Rows3<R>{ring[f][m], ring[f][c0], ring[f][pp]}; };
-        site_update<S, R, TH>(a, d, srcj, in, hC, gC, poC, rows(0), rows(1), rows(2), rows(3),
+        site_update<S, R, TH>(a, d, srcj, in, JC, gC, poC, rows(0), rows(1), rows(2), rows(3),
                               sc, rows(NF - 1));
       }
-#pragma unroll
-      for (int i = 0; i < 9; ++i) hC[i] = hL[i];
+      JC = JL;
 #pragma unroll
       for (int i = 0; i < 5; ++i) gC[i] = gL[i];
       poC = poL;

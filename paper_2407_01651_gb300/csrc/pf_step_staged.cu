@@ -4,12 +4,12 @@
 //
 // The arithmetic per site is the one of every other traversal (pf_site.cuh);
 // what differs is how the inputs reach it.  Every plane that a site reads at
-// its neighbours (f, h, g_post, s and r = 1/a_s^2; in the 16-bit forms also
-// the lagged phi, C, psi that decode the neighbours' offsets) is copied row by
-// row with cp.async.bulk into a ring of NSLOT row slots, each completing on
-// its own mbarrier.  Planes that only the site itself reads (g_pre, the lagged
-// velocity, Q_psi, the grain id; phi_o and C_o in FP32/FP64) are loaded into
-// registers one row ahead of their use.  So no warp waits on HBM inside the
+// its neighbours (f, h, g_post, s, r = 1/a_s^2 and the lagged phi and C that
+// give the opposite populations of the stored pairs; in the 16-bit forms also
+// the lagged psi) is copied row by row with cp.async.bulk into a ring of NSLOT
+// row slots, each completing on its own mbarrier.  Planes that only the site
+// itself reads (g_pre, the lagged velocity, Q_psi, the grain id) are loaded
+// into registers one row ahead of their use.  So no warp waits on HBM inside the
 // arithmetic of a row: the copies of row j+4 are in flight while row j is
 // computed.
 //
@@ -32,16 +32,16 @@ struct Stage {
   static constexpr int HR = 16 / (int)sizeof(R);   // halo columns of a compute plane
   static constexpr int PWS = YM_W + 2 * HS;        // staged width, storage planes
   static constexpr int PWR = YM_W + 2 * HR;        // staged width, compute planes
-  static constexpr int NPS = 28;                   // f[9], h[9], g_post[5], s[5]
+  static constexpr int NPS = 18;                   // f[9], h[4], g_post[3], s[2]
   static constexpr bool OFF = Codec<S>::kOffset;
-  static constexpr int NAS = OFF ? 4 : 1;          // r (+ phi_o, C_o, psi_o)
+  static constexpr int NAS = OFF ? 4 : 3;          // r, phi_o, C_o (+ psi_o)
   static constexpr int POP_BYTES = NPS * PWS * (int)sizeof(S);
   static constexpr int SLOT_BYTES = POP_BYTES + NAS * PWR * (int)sizeof(R);
   static constexpr int NSLOT = 6;
   static constexpr int RW = YM_W + 2;
   static constexpr int RING_BYTES = 4 * 4 * RW * (int)sizeof(R);
   static constexpr int SMEM = NSLOT * SLOT_BYTES + RING_BYTES + NSLOT * 8;
-  static constexpr int MIN_BLOCKS = sizeof(S) == 8 ? 1 : (sizeof(S) == 4 ? 2 : 3);
+  static constexpr int MIN_BLOCKS = sizeof(S) == 8 ? 1 : (sizeof(S) == 4 ? 2 : 4);
   static_assert(POP_BYTES % 16 == 0 && SLOT_BYTES % 16 == 0, "16-byte staged planes");
   static_assert(HS >= 2 && HR >= 2, "the halo streaming reaches two columns out");
 };
@@ -52,7 +52,7 @@ __device__ __forceinline__ int aux_plane(int u) {
   return u == U_RR ? A_RR : (u == U_PHIO ? A_PHIO : (u == U_CO ? A_CO : A_PSIO));
 }
 // staged storage plane q -> population plane (f, h, then g_post, s)
-__device__ __forceinline__ int pop_plane(int q) { return q < 18 ? q : q + 5; }
+__device__ __forceinline__ int pop_plane(int q) { return q < P_GPRE ? q : q + 5; }
 
 // ---- mbarrier and bulk copy (PTX) ----
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
@@ -200,9 +200,9 @@ struct OwnHG {
   R vxo, vyo;
 };
 // Own-site inputs of the update of one row (loaded a row ahead).
-template <typename S, typename R>
+template <typename R>
 struct OwnSite {
-  R phio, Co, Qo;
+  R Qo;
   uint8_t gid;
 };
 
@@ -216,32 +216,33 @@ __device__ __forceinline__ void load_own_hg(const StepArgs<S, R>& a, unsigned si
 }
 template <typename S, typename R>
 __device__ __forceinline__ void load_own_site(const StepArgs<S, R>& a, unsigned site,
-                                              OwnSite<S, R>& o) {
+                                              OwnSite<R>& o) {
   const unsigned ps = (unsigned)a.plane_stride;
-  if constexpr (!Codec<S>::kOffset) {
-    o.phio = __ldg(plane(a.ain, A_PHIO, ps) + site);
-    o.Co = __ldg(plane(a.ain, A_CO, ps) + site);
-  }
   o.Qo = __ldg(plane(a.ain, A_QO, ps) + site);
   o.gid = __ldg(a.grain + site);
 }
 
-// Streamed h and g of the site at column offset dx of the middle row of
-// (rm, rc, rp), from the staged rows; same arithmetic as pull_hg.
+// Streamed CAC moments and g of the site at column offset dx of the middle row
+// of (rm, rc, rp), from the staged rows; same arithmetic as pull_hg.
 template <typename S, typename R>
 __device__ __forceinline__ void stream_hg(const SlotView<S, R> (&rows)[3], int dx,
-                                          const OwnHG<S, R>& own, R h[9], R g[5], R& phi,
+                                          const OwnHG<S, R>& own, V2<R>& J, R g[5], R& phi,
                                           R& psi, R& psio) {
   constexpr bool off = Codec<S>::kOffset;
-  CSum<R> sh;
+  {
+    S v[9];
+    R ph[9];
+    ph[0] = rows[1].x(U_PHIO, dx);
 #pragma unroll
-  for (int i = 0; i < 9; ++i) {
-    const SlotView<S, R>& r = rows[src_row(i)];
-    const int sx = dx + src_dx(i);
-    h[i] = dec_off<S, R>(r.p(9 + i, sx), off ? w9<R>(i) * r.x(U_PHIO, sx) : R(0));
-    sh.add(h[i]);
+    for (int i = 1; i < 9; ++i) {
+      const SlotView<S, R>& r = rows[src_row(i)];
+      const int sx = dx + src_dx(i);
+      v[i] = r.p(P_H + pair9(i), sx);
+      ph[i] = off || minus9(i) ? r.x(U_PHIO, sx) : R(0);
+    }
+    cac_moments<S, R>(v, ph, phi, J);
   }
-  phi = sh.value();
+  constexpr int G = 13;   // staged index of the g_post planes
   CSum<R> sg;
   R po = R(0);
   const R psio_own = off ? rows[1].x(U_PSIO, dx) : R(0);
@@ -250,7 +251,23 @@ __device__ __forceinline__ void stream_hg(const SlotView<S, R> (&rows)[3], int d
     const SlotView<S, R>& r = rows[src_row(i)];
     const int sx = dx + src_dx(i);
     const R gold = dec_off<S, R>(own.gpre[i], w5<R>(i) * psio_own);
-    const R gpo = dec_off<S, R>(r.p(18 + i, sx), off ? w5<R>(i) * r.x(U_PSIO, sx) : R(0));
+    R gpo;
+    if constexpr (off) {
+      const R m = i == 0 ? psio_own : r.x(U_PSIO, sx);
+      const R base = q5_base(m);
+      if (i == 0) gpo = fma(R(2), dec_off<S, R>(r.p(G, sx), R(0)), q5_rest(m, base));
+      else if (!minus9(i)) gpo = pair_p<S, R>(r.p(G + i, sx), base);
+      else gpo = pair_m<S, R>(r.p(G + i - 2, sx), fma(R(2), dec_off<S, R>(r.p(G, sx), R(0)), base));
+    } else {
+      if (i == 0) {
+        const R m = (R)r.p(G, sx);
+        gpo = q5_rest(m, q5_base(m));
+      } else if (!minus9(i)) {
+        gpo = (R)r.p(G + i, sx);
+      } else {
+        gpo = pair_m<S, R>(r.p(G + i - 2, sx), q5_base((R)r.p(G, sx)));
+      }
+    }
     const R rr = r.x(U_RR, sx);
     g[i] = gold + (gpo - gold) * rr;
     sg.add(g[i]);
@@ -263,22 +280,21 @@ __device__ __forceinline__ void stream_hg(const SlotView<S, R> (&rows)[3], int d
 // Streamed f and s and the lagged scalars of the site at column offset dx.
 template <typename S, typename R>
 __device__ __forceinline__ void site_inputs(const SlotView<S, R> (&rows)[3], int dx,
-                                            const OwnSite<S, R>& own, SiteIn<R>& in) {
+                                            const OwnSite<R>& own, SiteIn<R>& in) {
   constexpr bool off = Codec<S>::kOffset;
+  constexpr int Q = 16;   // staged index of the s planes
 #pragma unroll
   for (int i = 0; i < 9; ++i) in.f[i] = dec_ns<S, R>(rows[src_row(i)].p(i, dx + src_dx(i)));
+  in.phio = rows[1].x(U_PHIO, dx);
+  in.Co = rows[1].x(U_CO, dx);
+  in.s[0] = q5_rest(in.Co, q5_base(in.Co));
 #pragma unroll
-  for (int i = 0; i < 5; ++i) {
+  for (int i = 1; i < 5; ++i) {
     const SlotView<S, R>& r = rows[src_row(i)];
     const int sx = dx + src_dx(i);
-    in.s[i] = dec_off<S, R>(r.p(23 + i, sx), off ? w5<R>(i) * r.x(U_CO, sx) : R(0));
-  }
-  if constexpr (off) {
-    in.phio = rows[1].x(U_PHIO, dx);
-    in.Co = rows[1].x(U_CO, dx);
-  } else {
-    in.phio = own.phio;
-    in.Co = own.Co;
+    const S v = r.p(Q + pair9(i), sx);
+    const R base = off || minus9(i) ? q5_base(r.x(U_CO, sx)) : R(0);
+    in.s[i] = minus9(i) ? pair_m<S, R>(v, base) : pair_p<S, R>(v, base);
   }
   in.Qo = own.Qo;
   in.gid = own.gid;
@@ -348,7 +364,8 @@ __global__ void __launch_bounds__(YM_THREADS, Stage<S, R>::MIN_BLOCKS)
 
     // ring rows ya-1 and ya (streaming reads staged rows ya-2 .. ya+1)
     OwnHG<S, R> ohg;
-    R hC[9], gC[5], poC = R(0);
+    V2<R> JC = vec2(R(0), R(0));
+    R gC[5], poC = R(0);
     for (int r = k0; r <= ya + 1; ++r) wait_row(r);
     waited = ya + 1;
     for (int k = 0; k < 2; ++k) {
@@ -358,15 +375,15 @@ __global__ void __launch_bounds__(YM_THREADS, Stage<S, R>::MIN_BLOCKS)
         const SlotView<S, R> rows[3] = {slot_view<S, R>(slots, slot_of(y - 1)),
                                         slot_view<S, R>(slots, slot_of(y)),
                                         slot_view<S, R>(slots, slot_of(y + 1))};
-        R h[9], g[5], phi, psi, po;
-        stream_hg(rows, dx, ohg, h, g, phi, psi, po);
+        V2<R> J;
+        R g[5], phi, psi, po;
+        stream_hg(rows, dx, ohg, J, g, phi, psi, po);
         ring[0][y & 3][sc] = phi;
         ring[1][y & 3][sc] = psi;
         ring[2][y & 3][sc] = ohg.vxo;
         ring[3][y & 3][sc] = ohg.vyo;
         if (k == 1) {
-#pragma unroll
-          for (int i = 0; i < 9; ++i) hC[i] = h[i];
+          JC = J;
 #pragma unroll
           for (int i = 0; i < 5; ++i) gC[i] = g[i];
           poC = po;
@@ -374,7 +391,7 @@ __global__ void __launch_bounds__(YM_THREADS, Stage<S, R>::MIN_BLOCKS)
       }
     }
     // own inputs one row ahead
-    OwnSite<S, R> osC{};
+    OwnSite<R> osC{};
     if (active) load_own_hg(a, site_of(ya + 1), ohg);
     if (interior) load_own_site(a, site_of(ya), osC);
 
@@ -382,21 +399,22 @@ __global__ void __launch_bounds__(YM_THREADS, Stage<S, R>::MIN_BLOCKS)
       wait_row(j + 2);
       waited = j + 2;
       // streaming of row j+1 into the ring
-      R hL[9], gL[5], poL = R(0);
+      V2<R> JL = vec2(R(0), R(0));
+      R gL[5], poL = R(0);
       if (active) {
         const int y = j + 1;
         const SlotView<S, R> rows[3] = {slot_view<S, R>(slots, slot_of(y - 1)),
                                         slot_view<S, R>(slots, slot_of(y)),
                                         slot_view<S, R>(slots, slot_of(y + 1))};
         R phi, psi;
-        stream_hg(rows, dx, ohg, hL, gL, phi, psi, poL);
+        stream_hg(rows, dx, ohg, JL, gL, phi, psi, poL);
         ring[0][y & 3][sc] = phi;
         ring[1][y & 3][sc] = psi;
         ring[2][y & 3][sc] = ohg.vxo;
         ring[3][y & 3][sc] = ohg.vyo;
         if (j + 2 < yb + 1) load_own_hg(a, site_of(j + 2), ohg);
       }
-      OwnSite<S, R> osN{};
+      OwnSite<R> osN{};
       if (interior && j + 1 < yb) load_own_site(a, site_of(j + 1), osN);
       if (__syncthreads_or(bad)) {
         // drain the copies still in flight (bounded), report, stop
@@ -425,10 +443,9 @@ __global__ void __launch_bounds__(YM_THREADS, Stage<S, R>::MIN_BLOCKS)
         src.s[0] = site_of(j);
         const int m = (j - 1) & 3, c0 = j & 3, pp = (j + 1) & 3;
         auto rws = [&](int f) { return Rows3<R>{ring[f][m], ring[f][c0], ring[f][pp]}; };
-        site_update(a, d, src, in, hC, gC, poC, rws(0), rws(1), rws(2), rws(3), sc);
+        site_update(a, d, src, in, JC, gC, poC, rws(0), rws(1), rws(2), rws(3), sc);
       }
-#pragma unroll
-      for (int i = 0; i < 9; ++i) hC[i] = hL[i];
+      JC = JL;
 #pragma unroll
       for (int i = 0; i < 5; ++i) gC[i] = gL[i];
       poC = poL;
