@@ -209,7 +209,8 @@ pf_status pf_step(pf_handle *h, int n_steps);
  * tiles of a rows (b ignored; the default for FP32/FP64, a chosen from the
  * domains' sizes, at most 32); variant 2 = the same strips with their input
  * rows staged in shared memory by bulk copies (b ignored; the default for
- * FP16/BF16 storage, a chosen by size, at most 48; needs every
+ * FP16/BF16 storage and, from 786,432 sites on, for FP32, a chosen by size, at
+ * most 48; needs every
  * domain's nx to be a multiple of 16 bytes of storage: 4 FP32, 8 FP16/BF16,
  * 2 FP64 sites).  Synchronises the stream and rebuilds the tile table.
  * Errors: BAD_ARG. */

@@ -28,7 +28,7 @@ __device__ constexpr int CY9[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
 
 template <typename R>
 __device__ __forceinline__ local::Coef<R> make_coef(const KParams<R>& kp, const DomDesc& d,
-                                                    double2 cs) {
+                                                    GrainCS<R> cs) {
   local::Coef<R> c;
   c.rho_g = kp.rho_g; c.drho = kp.drho; c.ge2 = kp.ge2; c.gat2 = kp.gat2; c.kappa = kp.kappa;
   c.fs_coef = kp.fs_coef; c.Wphi2 = kp.Wphi2; c.M_phi = kp.M_phi; c.two_bphi = kp.two_bphi;
@@ -37,8 +37,8 @@ __device__ __forceinline__ local::Coef<R> make_coef(const KParams<R>& kp, const 
   c.k = kp.k; c.D = kp.D; c.g = kp.g; c.s_e = kp.s_e; c.s_eps = kp.s_eps; c.s_q = kp.s_q;
   c.s_nu = kp.s_nu; c.s_phi = kp.s_phi;
   c.eps = static_cast<R>(d.eps_s);
-  c.ct = static_cast<R>(cs.x);
-  c.sn = static_cast<R>(cs.y);
+  c.ct = cs.x;
+  c.sn = cs.y;
   c.rho_bar = static_cast<R>(d.rho_bar);
   return c;
 }

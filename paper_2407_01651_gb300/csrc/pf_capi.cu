@@ -61,6 +61,7 @@ struct pf_handle {
   int tx = 32, ty = 8;      // tile of the 2-D variant
   int chunk = 32;           // rows per tile of the y-march variants
   int own_chunk = 0;        // 1: set by the caller or the autotuner, else chosen by size
+  bool staged_rows = false; // the y-march chosen by size stages its rows (step_variant)
   int ntiles = 0;
   int grid = 0;
   int launch_mode = 0;      // 0: one launch over all domains; 1: one launch per domain
@@ -78,7 +79,7 @@ struct pf_handle {
   int cur = 0;
   void* fields = nullptr;
   uint8_t* grain = nullptr;
-  double2* grain_cs = nullptr;
+  void* grain_cs = nullptr;     // (cos, sin) of each grain angle, compute type
   DomDesc* d_doms = nullptr;
   int* d_tile_dom = nullptr;
   double* partial = nullptr;
@@ -373,16 +374,26 @@ static void release(pf_handle* h) {
 // takes about (waves of tiles over the resident CTAs) x (chunk + warm) row
 // times: long tiles waste little on a large lattice, short ones are what fills
 // the chip on a small one.  Whole waves up to four; beyond that the CTAs run
-// out of step and only half a wave is lost at the end.  Measured (FP32, us per
-// step at 32 rows and at the rows chosen): 128^2 43.1 -> 6.2 (1 row), 256^2
-// 45.1 -> 8.2 (1), 512^2 51.1 -> 18.5 (4), 1024^2 88.5 -> 66.2 (16), 4096^2
-// 868 (32; 24 rows 878, 16 rows 884).  FP64 is bound by the FP64 units, so
-// there the SM with the most tiles sets the time and a row costs its update
-// (5.6 pulls' worth with its own pull) plus two warm-up pulls per tile: 128^2
-// 763 -> 34.9 (1 row), 256^2 765 -> 105 (4).
+// out of step and only half a wave is lost at the end.  Measured (us per step at
+// 32 rows and at the rows chosen): FP32 128^2 43.1 -> 6.2 (1 row), 256^2 45.1 ->
+// 8.2 (1), 512^2 45.1 -> 18.5 (4); staged 1024^2 88.0 -> 55.3 (14), 2048^2 206 ->
+// 183 (27), 4096^2 679 -> 676 (36).
+// FP64 is bound by the FP64 units, so there the SM with the most tiles sets the
+// time, a row costs its update (5.6 pulls' worth with its own pull) plus two
+// warm-up pulls per tile, and one tile alone leaves an SM's units idle for an
+// eighth of the time: 128^2 763 -> 38.9 (1 row), 512^2 804 -> 337 (7).
+// Tiles at a non-periodic side are several times slower per row and too few to
+// fill the chip: their height is held to a share of the lattice's side, so that
+// they end with the others (thermal, sides: 1024^2 at 18 rows 128, at 6 rows 107;
+// 2048^2 at 36 rows 371, at 12 rows 333).
 static int chunk_by_size(const pf_handle* h, int sms, int ctas_per_sm) {
-  const bool staged = h->variant == STEP_STAGED;
-  const int top = staged ? 48 : 32;
+  const bool staged = h->variant == STEP_STAGED || h->staged_rows;
+  int top = h->variant == STEP_STAGED ? 48 : (staged ? 36 : 32);
+  if (h->any_bc) {
+    double n = 0.0;
+    for (const DomDesc& d : h->ddesc) n = std::max(n, (double)d.nx * d.ny);
+    top = std::max(2, std::min(top, (int)(std::sqrt(n) / 160.0)));
+  }
   const double warm = staged ? 3.0 : 2.0;
   double best = 0.0;
   int pick = top;
@@ -392,7 +403,7 @@ static int chunk_by_size(const pf_handle* h, int sms, int ctas_per_sm) {
       tiles += (long long)((d.nx + YM_W - 1) / YM_W) * ((d.ny + c - 1) / c);
     double cost;
     if (h->prec == PF_FP64) {
-      cost = (double)((tiles + sms - 1) / sms) * (5.6 * c + 2.0);
+      cost = (double)((tiles + sms - 1) / sms) * (5.6 * c + 2.0) * (tiles <= sms ? 1.13 : 1.0);
     } else {
       const double w = (double)tiles / ((double)sms * ctas_per_sm);
       cost = (w > 4.0 ? w + 0.5 : std::ceil(w)) * (c + warm);
@@ -406,14 +417,28 @@ static int chunk_by_size(const pf_handle* h, int sms, int ctas_per_sm) {
   return pick;
 }
 
+// The traversal that a step takes.  Where neither the caller nor the autotuner
+// set one, an FP32 y-march stages its rows by bulk copies (the same strips and
+// tiles, the same bits) if the widths allow it and there are sites enough: its
+// prologue fills the stages, so short tiles do not pay.  Measured, us per step
+// y-march / staged: 512^2 18.5 / 22.6, 1024^2 63.6 / 59.5, 2048^2 213 / 183,
+// 4096^2 820 / 677.  FP64 is bound by its arithmetic: 1024^2 1234 / 1261.
+constexpr long long STAGE_SITES = 3ll << 18;
+static StepVariant step_variant(const pf_handle* h) {
+  if (h->variant == STEP_YMARCH && h->staged_rows && !h->own_chunk && h->persistent != 2)
+    return STEP_STAGED;
+  return (StepVariant)h->variant;
+}
+
 static pf_status choose_chunk(pf_handle* h) {
   if (h->own_chunk || h->variant == STEP_TILE) return PF_OK;
+  h->staged_rows = h->prec == PF_FP32 && h->plane_stride >= STAGE_SITES && staged_ok(h);
   int sms = 0;
   PF_CUDA(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
   return dispatch(h, [&](auto s_t, auto r_t) {
     PF_TYPES(s_t, r_t);
-    const int k = step_blocks_per_sm<S, R>(h->variant, h->tx, h->ty, h->plane_stride,
-                                           h->thermal != 0, h->any_bc != 0);
+    const int k = step_blocks_per_sm<S, R>(h->staged_rows ? STEP_STAGED : h->variant, h->tx, h->ty,
+                                           h->plane_stride, h->thermal != 0, h->any_bc != 0);
     h->chunk = chunk_by_size(h, std::max(1, sms), std::max(1, k));
     return PF_OK;
   });
@@ -490,6 +515,21 @@ static pf_status upload_tables(pf_handle* h) {
   return PF_OK;
 }
 
+// Grain table of a domain: the given angles, then the lattice's own frame.
+static pf_status upload_grain_table(pf_handle* h, int dom, const std::vector<double>& angles) {
+  return dispatch(h, [&](auto s_t, auto r_t) {
+    PF_TYPES(s_t, r_t);
+    std::vector<GrainCS<R>> cs(MAX_GRAINS, GrainCS<R>{R(1), R(0)});
+    for (size_t i = 0; i < angles.size(); ++i)
+      cs[i] = GrainCS<R>{(R)std::cos(angles[i]), (R)std::sin(angles[i])};
+    PF_CUDA(h, cudaMemcpyAsync(reinterpret_cast<GrainCS<R>*>(h->grain_cs) + (size_t)dom * MAX_GRAINS,
+                               cs.data(), cs.size() * sizeof(GrainCS<R>), cudaMemcpyHostToDevice,
+                               h->stream));
+    PF_CUDA(h, cudaStreamSynchronize(h->stream));
+    return PF_OK;
+  });
+}
+
 extern "C" pf_status pf_create(const pf_params* p, const pf_domain* doms, int n_doms,
                                pf_precision prec, void* cuda_stream, const pf_allocator* alloc,
                                pf_handle** out) {
@@ -564,7 +604,7 @@ extern "C" pf_status pf_create(const pf_params* p, const pf_domain* doms, int n_
   }
   h->fields = dev_alloc(h, ps * N_FIELDS * h->celem);
   h->grain = (uint8_t*)dev_alloc(h, ps);
-  h->grain_cs = (double2*)dev_alloc(h, (size_t)n_doms * MAX_GRAINS * sizeof(double2));
+  h->grain_cs = dev_alloc(h, (size_t)n_doms * MAX_GRAINS * 2 * h->celem);
   h->d_doms = (DomDesc*)dev_alloc(h, (size_t)n_doms * sizeof(DomDesc));
   h->partial = (double*)dev_alloc(h, (size_t)REDUCE_BLOCKS * NDIAG * sizeof(double));
   h->d_diag = (double*)dev_alloc(h, (NDIAG + 1) * sizeof(double));
@@ -577,10 +617,9 @@ extern "C" pf_status pf_create(const pf_params* p, const pf_domain* doms, int n_
       cudaMemsetAsync(h->d_err, 0, 2 * sizeof(unsigned int), h->stream) != cudaSuccess ||
       cudaMemsetAsync(h->grain, 0, ps, h->stream) != cudaSuccess)
     return bail(PF_ERR_CUDA, "memset failed");
-  std::vector<double2> cs((size_t)n_doms * MAX_GRAINS, make_double2(1.0, 0.0));
-  if (cudaMemcpyAsync(h->grain_cs, cs.data(), cs.size() * sizeof(double2), cudaMemcpyHostToDevice,
-                      h->stream) != cudaSuccess)
-    return bail(PF_ERR_CUDA, "grain table upload failed");
+  for (int d = 0; d < n_doms; ++d)
+    if (upload_grain_table(h, d, {}) != PF_OK)
+      return bail(PF_ERR_CUDA, "grain table upload failed");
   // default traversal: the staged y-march for the 16-bit storage forms
   // (measured faster at 4096^2), the plain y-march otherwise
   if ((prec == PF_FP16_OFFSET || prec == PF_BF16_OFFSET) && staged_ok(h))
@@ -696,15 +735,6 @@ static pf_status init_spec_t(pf_handle* h, int dom, const pf_init_spec* spec, co
   a.theta0 = h->p.theta0;
   PF_CUDA(h, launch_init_spec<S, R>(a, h->stream));
   h->launches++;
-  return PF_OK;
-}
-
-static pf_status upload_grain_table(pf_handle* h, int dom, const std::vector<double>& angles) {
-  std::vector<double2> cs(MAX_GRAINS, make_double2(1.0, 0.0));
-  for (size_t i = 0; i < angles.size(); ++i) cs[i] = make_double2(std::cos(angles[i]), std::sin(angles[i]));
-  PF_CUDA(h, cudaMemcpyAsync(h->grain_cs + (size_t)dom * MAX_GRAINS, cs.data(),
-                             MAX_GRAINS * sizeof(double2), cudaMemcpyHostToDevice, h->stream));
-  PF_CUDA(h, cudaStreamSynchronize(h->stream));
   return PF_OK;
 }
 
@@ -841,7 +871,7 @@ static StepArgs<S, R> make_step_args(const pf_handle* h, const void* pin, const 
   a.aout = reinterpret_cast<R*>(aout);
   a.plane_stride = h->plane_stride;
   a.grain = h->grain;
-  a.grain_cs = h->grain_cs;
+  a.grain_cs = reinterpret_cast<const GrainCS<R>*>(h->grain_cs);
   a.doms = h->any_bc ? h->d_runs : h->d_doms;
   a.tile_dom = h->d_tile_dom;
   a.ntiles = h->ntiles;
@@ -860,9 +890,13 @@ static StepArgs<S, R> make_step_args(const pf_handle* h, const void* pin, const 
 // of the device looping over the tiles (persistent).
 template <typename S, typename R>
 static pf_status launch_all(pf_handle* h, StepArgs<S, R> a, cudaStream_t stream) {
+  // a state outside the handle's buffers (the adjoint's) has to be aligned too
+  const bool aligned = !((reinterpret_cast<uintptr_t>(a.in) | reinterpret_cast<uintptr_t>(a.ain)) & 15u);
+  const StepVariant variant =
+      step_variant(h) == STEP_STAGED && !aligned ? STEP_YMARCH : step_variant(h);
   auto cap_of = [&](bool bc) {
     return h->persistent ? std::max(1, h->sms) *
-                               step_blocks_per_sm<S, R>(h->variant, h->tx, h->ty,
+                               step_blocks_per_sm<S, R>(bc ? STEP_YMARCH : variant, h->tx, h->ty,
                                                         h->plane_stride, h->thermal != 0, bc)
                          : 1 << 30;
   };
@@ -872,8 +906,8 @@ static pf_status launch_all(pf_handle* h, StepArgs<S, R> a, cudaStream_t stream)
     a.tile_base = t0;
     a.ntiles = t1;
     a.bc = bc;
-    PF_CUDA(h, launch_step<S, R>(a, h->variant, h->tx, h->ty, std::min(t1 - t0, cap_of(bc != 0)),
-                                 sx));
+    PF_CUDA(h, launch_step<S, R>(a, bc ? STEP_YMARCH : variant, h->tx, h->ty,
+                                 std::min(t1 - t0, cap_of(bc != 0)), sx));
     h->launches++;
     return PF_OK;
   };
@@ -976,7 +1010,8 @@ static pf_status step_general_t(pf_handle* h, bool write_fields) {
     a.tile_base = t0;
     a.ntiles = t1;
     a.bc = bc;
-    PF_CUDA(h, launch_step<S, R>(a, h->variant, h->tx, h->ty, t1 - t0, h->stream));
+    PF_CUDA(h, launch_step<S, R>(a, bc ? STEP_YMARCH : step_variant(h), h->tx, h->ty, t1 - t0,
+                                 h->stream));
     h->launches++;
     return PF_OK;
   };
@@ -1174,8 +1209,12 @@ static pf_status autotune_t(pf_handle* h, int trial_steps, int out[4]) {
   const long long steps0 = h->steps, launches0 = h->launches;
   PF_CUDA(h, cudaMemcpyAsync(snap_p, h->pop[cur0], pop_b, cudaMemcpyDeviceToDevice, h->stream));
   PF_CUDA(h, cudaMemcpyAsync(snap_a, h->aux[cur0], aux_b, cudaMemcpyDeviceToDevice, h->stream));
-  struct Cand { int variant, a, b, persistent; };
+  // own: as pf_set_step_config would take it; else the tiles chosen by size
+  struct Cand { int variant, a, b, persistent, own = 1; };
   std::vector<Cand> cands;
+  const int own0 = h->own_chunk;
+  if (!own0 && h->staged_rows)
+    for (int pers : {0, 1}) cands.push_back({h->variant, h->chunk, 0, pers, 0});
   for (int ch : {4, 8, 16, 24, 32, 48, 64, 96})
     for (int pers : {0, 1}) cands.push_back({STEP_YMARCH, ch, 0, pers});
   if (!h->thermal && !h->any_bc) {
@@ -1195,6 +1234,7 @@ static pf_status autotune_t(pf_handle* h, int trial_steps, int out[4]) {
     h->variant = c.variant;
     if (c.variant != STEP_TILE) h->chunk = c.a; else { h->tx = c.a; h->ty = c.b; }
     h->persistent = c.persistent;
+    h->own_chunk = c.own;
     st = upload_tables(h);
     if (st != PF_OK) break;
     for (int t = 0; t < 2 && st == PF_OK; ++t) st = step_t<S, R>(h, false);
@@ -1219,17 +1259,21 @@ static pf_status autotune_t(pf_handle* h, int trial_steps, int out[4]) {
   h->cur = cur0;
   h->steps = steps0;
   h->launches = launches0;
+  h->own_chunk = own0;
   if (st != PF_OK) return st;
   h->variant = bc.variant;
   if (bc.variant != STEP_TILE) h->chunk = bc.a; else { h->tx = bc.a; h->ty = bc.b; }
   h->persistent = bc.persistent;
-  h->own_chunk = 1;
+  h->own_chunk = bc.own;
   for (auto& g : h->gexec)   // graphs captured before hold the old tiles
     if (g) { cudaGraphExecDestroy(g); g = nullptr; }
   h->coop_graph_failed = 0;
   st = upload_tables(h);
   if (st != PF_OK) return st;
-  if (out) { out[0] = bc.variant; out[1] = bc.a; out[2] = bc.b; out[3] = bc.persistent; }
+  if (out) {
+    pf_get_step_config(h, out);
+    out[3] = bc.persistent;
+  }
   return PF_OK;
 }
 
@@ -1248,7 +1292,8 @@ extern "C" pf_status pf_autotune(pf_handle* h, int trial_steps, int out[4]) {
 
 extern "C" pf_status pf_get_step_config(const pf_handle* h, int out[3]) {
   if (!h || !out) return PF_ERR_BAD_ARG;
-  out[0] = h->variant;
+  // what pf_set_step_config would take to run the same kernels
+  out[0] = !h->thermal && !h->any_bc ? (int)step_variant(h) : h->variant;
   out[1] = h->variant != STEP_TILE ? h->chunk : h->tx;
   out[2] = h->variant == STEP_TILE ? h->ty : 0;
   return PF_OK;
@@ -1417,7 +1462,7 @@ static pf_status run_banded(pf_handle* h, const double* in6, int n_steps, uint32
       }
       a.tile_base = dd.tile0 + tr[b] * dd.tiles_x;
       a.ntiles = dd.tile0 + tr[b + 1] * dd.tiles_x;
-      PF_CUDA(h, launch_step<S, R>(a, h->variant, h->tx, h->ty, a.ntiles - a.tile_base, sb));
+      PF_CUDA(h, launch_step<S, R>(a, step_variant(h), h->tx, h->ty, a.ntiles - a.tile_base, sb));
       h->launches++;
       PF_CUDA(h, cudaEventRecord(h->run_ev[s & 1][b], sb));
     }

@@ -20,6 +20,12 @@ enum StepVariant : int { STEP_TILE = 0, STEP_YMARCH = 1, STEP_STAGED = 2 };
 constexpr int YM_W = 128;            // interior columns of a y-march strip
 constexpr int YM_THREADS = YM_W + 32;  // + one warp whose lanes 0, 1 own the halo columns
 
+// (cos, sin) of a grain angle in the type of the arithmetic.
+template <typename R>
+struct alignas(2 * sizeof(R)) GrainCS {
+  R x, y;
+};
+
 template <typename S, typename R>
 struct StepArgs {
   const S* __restrict__ in;     // population planes read this step
@@ -28,7 +34,7 @@ struct StepArgs {
   R* __restrict__ aout;         // lagged-scalar planes written this step
   long long plane_stride;       // sites per plane (all domains, padded)
   const uint8_t* __restrict__ grain;    // grain id per site
-  const double2* __restrict__ grain_cs; // (cos, sin) of each grain angle
+  const GrainCS<R>* __restrict__ grain_cs; // (cos, sin) of each grain angle
   const DomDesc* __restrict__ doms;
   const int* __restrict__ tile_dom;     // domain of each tile
   int tile_base;                // first tile of this launch
@@ -104,11 +110,9 @@ cudaError_t launch_ymarch_bc(const StepArgs<S, R>& a, bool big, int grid, cudaSt
 template <typename S, typename R>
 int ymarch_bc_blocks_per_sm(bool big, bool thermal);
 template <typename S, typename R>
-int staged_smem_bytes();
-template <typename S, typename R>
 int staged_halo_columns();
 template <typename S, typename R>
-int staged_blocks_per_sm();
+int staged_blocks_per_sm(bool thermal);
 // Every step of a call in one cooperative launch (y-march, periodic domains),
 // and the resident CTAs per SM of that kernel.
 // ctr: two device ints (tile counters), owned by the caller.

@@ -43,14 +43,14 @@ __device__ __forceinline__ unsigned pidx(int k, unsigned ps, unsigned s) {
   else return (unsigned)k * ps + s;
 }
 
-// The nine loaded CAC values of a pull, before they are combined: rest density
-// phi_o of the site, the stored population of each direction's pair at its
-// source, and the sources' phi_o (16-bit forms: of every direction; else of the
-// directions that are not stored: 3, 4, 7, 8).
+// Plane of the pair of a D2Q9 (or D2Q5) direction within its lattice's pairs,
+// and whether the pair stores the opposite direction.
 __device__ __forceinline__ constexpr int pair9(int i) { return ((i - 1) & 1) + (i >= 5 ? 2 : 0); }
 __device__ __forceinline__ constexpr bool minus9(int i) { return ((i - 1) & 2) != 0; }
 
-// phi and the flux J = sum c h of the streamed CAC populations.
+// phi and the flux J = sum c h of the streamed CAC populations: v the stored
+// population of each direction's pair at its source, ph the sources' phi_o (own
+// in ph[0]; 16-bit forms: of every direction, else of 3, 4, 7, 8).
 template <typename S, typename R>
 __device__ __forceinline__ void cac_moments(const S (&v)[9], const R (&ph)[9], R& phi, V2<R>& J) {
   R h[9];
@@ -75,57 +75,75 @@ __device__ __forceinline__ void cac_moments(const S (&v)[9], const R (&ph)[9], R
 // Streamed CAC moments (phi and the flux J) and dendrite populations g (with
 // the a_s^2 time stretch g = g_pre + r_src (g_post,src - g_pre)) at (x, y);
 // phi and psi are compensated sums, psi_o is the psi of the previous step (sum
-// of g_pre, or the stored lagged psi in the offset forms).
+// of g_pre, or the stored lagged psi in the offset forms).  In two parts, so
+// that a traversal may issue the loads of a row well before it combines them.
+template <typename S, typename R>
+struct HgLoads {
+  S h[9], gpre[5], gp[5], gm[5];   // h and g_post of each direction's pair at its source, the
+                                   // sources' g_post density (or F/6)
+  R ph[9], po[5], rr[5];           // phi_o, psi_o (offset forms) and r of the sources
+};
+
 template <typename S, typename R, bool BIG = false>
-__device__ __forceinline__ void pull_hg(const StepArgs<S, R>& a, const Src9& src, V2<R>& J,
-                                        R g[5], R& phi, R& psi, R& psio) {
+__device__ __forceinline__ void load_hg(const StepArgs<S, R>& a, const Src9& src,
+                                        HgLoads<S, R>& l) {
   const unsigned ps = (unsigned)a.plane_stride;
   constexpr bool off = Codec<S>::kOffset;
   auto pop = [&](int k, unsigned s) { return __ldg(pbase<BIG>(a.in, k, ps) + pidx<BIG>(k, ps, s)); };
   auto aux = [&](int k, unsigned s) { return __ldg(pbase<BIG>(a.ain, k, ps) + pidx<BIG>(k, ps, s)); };
-  {
-    S v[9];
-    R ph[9];
-    ph[0] = aux(A_PHIO, src.s[0]);
+  l.ph[0] = aux(A_PHIO, src.s[0]);
 #pragma unroll
-    for (int i = 1; i < 9; ++i) {
-      v[i] = pop(P_H + pair9(i), src.s[i]);
-      ph[i] = off || minus9(i) ? aux(A_PHIO, src.s[i]) : R(0);
-    }
-    cac_moments<S, R>(v, ph, phi, J);
+  for (int i = 1; i < 9; ++i) {
+    l.h[i] = pop(P_H + pair9(i), src.s[i]);
+    if (off || minus9(i)) l.ph[i] = aux(A_PHIO, src.s[i]);
   }
-  CSum<R> sg;
-  R po = R(0);
-  const R psio_own = off ? aux(A_PSIO, src.s[0]) : R(0);
 #pragma unroll
   for (int i = 0; i < 5; ++i) {
-    const R gold = dec_off<S, R>(pop(P_GPRE + i, src.s[0]), w5<R>(i) * psio_own);
+    l.gpre[i] = pop(P_GPRE + i, src.s[0]);
+    if (i > 0) l.gp[i] = pop(P_GPOST + 1 + pair9(i), src.s[i]);
+    if (i == 0 || minus9(i)) l.gm[i] = pop(P_GPOST, src.s[i]);
+    if (off) l.po[i] = aux(A_PSIO, src.s[i]);
+    l.rr[i] = aux(A_RR, src.s[i]);
+  }
+}
+
+template <typename S, typename R>
+__device__ __forceinline__ void finish_hg(const HgLoads<S, R>& l, V2<R>& J, R g[5], R& phi, R& psi,
+                                          R& psio) {
+  constexpr bool off = Codec<S>::kOffset;
+  cac_moments<S, R>(l.h, l.ph, phi, J);
+  CSum<R> sg;
+  R po = R(0);
+  const R psio_own = off ? l.po[0] : R(0);
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    const R gold = dec_off<S, R>(l.gpre[i], w5<R>(i) * psio_own);
     R gpo;
     if constexpr (off) {
       // density psi_o + F of the source; its planes: F/6 and the offsets of g_1, g_2
-      const R m = i == 0 ? psio_own : aux(A_PSIO, src.s[i]);
-      const R base = q5_base(m);
-      if (i == 0) gpo = fma(R(2), dec_off<S, R>(pop(P_GPOST, src.s[0]), R(0)), q5_rest(m, base));
-      else if (!minus9(i)) gpo = pair_p<S, R>(pop(P_GPOST + i, src.s[i]), base);
-      else gpo = pair_m<S, R>(pop(P_GPOST + i - 2, src.s[i]),
-                              fma(R(2), dec_off<S, R>(pop(P_GPOST, src.s[i]), R(0)), base));
+      const R base = q5_base(l.po[i]);
+      if (i == 0) gpo = fma(R(2), dec_off<S, R>(l.gm[0], R(0)), q5_rest(l.po[0], base));
+      else if (!minus9(i)) gpo = pair_p<S, R>(l.gp[i], base);
+      else gpo = pair_m<S, R>(l.gp[i], fma(R(2), dec_off<S, R>(l.gm[i], R(0)), base));
     } else {
-      if (i == 0) {
-        const R m = (R)pop(P_GPOST, src.s[0]);
-        gpo = q5_rest(m, q5_base(m));
-      } else if (!minus9(i)) {
-        gpo = (R)pop(P_GPOST + i, src.s[i]);
-      } else {
-        gpo = pair_m<S, R>(pop(P_GPOST + i - 2, src.s[i]), q5_base((R)pop(P_GPOST, src.s[i])));
-      }
+      if (i == 0) gpo = q5_rest((R)l.gm[0], q5_base((R)l.gm[0]));
+      else if (!minus9(i)) gpo = (R)l.gp[i];
+      else gpo = pair_m<S, R>(l.gp[i], q5_base((R)l.gm[i]));
     }
-    const R rr = aux(A_RR, src.s[i]);
-    g[i] = gold + (gpo - gold) * rr;
+    g[i] = gold + (gpo - gold) * l.rr[i];
     sg.add(g[i]);
     po += gold;
   }
   psi = sg.value();
   psio = off ? psio_own : po;
+}
+
+template <typename S, typename R, bool BIG = false>
+__device__ __forceinline__ void pull_hg(const StepArgs<S, R>& a, const Src9& src, V2<R>& J,
+                                        R g[5], R& phi, R& psi, R& psio) {
+  HgLoads<S, R> l;
+  load_hg<S, R, BIG>(a, src, l);
+  finish_hg<S, R>(l, J, g, phi, psi, psio);
 }
 
 // Three rows of a shared-memory field around a site: row y-1, y, y+1.
@@ -143,8 +161,29 @@ struct SiteIn {
   R f[9], s[5];
   R phio, Co, Qo;
   uint8_t gid;
+  GrainCS<R> cs;  // of that grain: load_grain, once gid has arrived
   R e[5], mo;     // thermal mode: streamed temperature populations, lagged rho H
 };
+
+// What a tile's sites take from their domain, in the type of the arithmetic:
+// converted once per tile, since FP64 conversions run on units that this GPU
+// has few of.
+template <typename R>
+struct SiteDom {
+  R rho_bar, eps;
+  int grain_off;
+  __device__ __forceinline__ explicit SiteDom(const DomDesc& d)
+      : rho_bar(static_cast<R>(d.rho_bar)), eps(static_cast<R>(d.eps_s)), grain_off(d.grain_off) {}
+};
+
+// The grain rotation of a site.  Issued before the barrier that ends a row's
+// streaming: it depends on the grain id, and in the middle of the update every
+// warp waited for it.
+template <typename S, typename R>
+__device__ __forceinline__ void load_grain(const StepArgs<S, R>& a, const SiteDom<R>& sd,
+                                           SiteIn<R>& in) {
+  in.cs = a.grain_cs[sd.grain_off + in.gid];
+}
 
 // Streamed solute populations; Co is C of the last step at the site itself.
 template <typename S, typename R, bool BIG = false>

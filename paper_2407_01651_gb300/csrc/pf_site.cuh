@@ -295,9 +295,9 @@ __device__ __forceinline__ void store_state(const StepArgs<S, R>& a, unsigned si
 
 // One site: gather the stencil values from the traversal's shared-memory rows,
 // run site_math and store the new state and (if requested) the fields.
-// TH: thermal mode, with SU the supersaturation rows and in.e / in.mo loaded.
+// TH: thermal mode, with SU the supersaturation rows and in.e / in.mo loaded; in.cs is the grain's.
 template <typename S, typename R, bool TH = false>
-__device__ __forceinline__ void site_update(const StepArgs<S, R>& a, const DomDesc& d,
+__device__ __forceinline__ void site_update(const StepArgs<S, R>& a, const SiteDom<R>& sd,
                                             const Src9& src, const SiteIn<R>& in,
                                             V2<R> hJ, const R (&g_in)[5], R psio,
                                             Rows3<R> SP, Rows3<R> SS, Rows3<R> SVX,
@@ -314,7 +314,6 @@ __device__ __forceinline__ void site_update(const StepArgs<S, R>& a, const DomDe
     }
     return n;
   };
-  const double2 cs = a.grain_cs[d.grain_off + in.gid];
   SiteOut<R> o;
   ThermIn<R> ti;
   ThermOut<R> to;
@@ -324,8 +323,7 @@ __device__ __forceinline__ void site_update(const StepArgs<S, R>& a, const DomDe
     ti.mo = in.mo;
     ti.U = nb(SU);
   }
-  site_math<R, R, TH>(a.kp, static_cast<R>(d.rho_bar), static_cast<R>(d.eps_s),
-                      static_cast<R>(cs.x), static_cast<R>(cs.y), in.f, hJ, g_in, in.s, psio,
+  site_math<R, R, TH>(a.kp, sd.rho_bar, sd.eps, in.cs.x, in.cs.y, in.f, hJ, g_in, in.s, psio,
                       in.phio, in.Co, in.Qo, nb(SP), nb(SS), nb(SVX), nb(SVY), o, &ti, &to);
 
   store_state<S, R>(a, site, o, g_in);

@@ -62,7 +62,9 @@ __global__ void __launch_bounds__(256) k_step_tile(StepArgs<S, R> a) {
       auto rows = [&](const R* X) { return Rows3<R>{X + (r - 1) * SW, X + r * SW, X + (r + 1) * SW}; };
       SiteIn<R> in;
       load_site<S, R, BIG>(a, src, in);
-      site_update(a, d, src, in, J, g, po, rows(sphi), rows(spsi), rows(svx), rows(svy),
+      const SiteDom<R> sd(d);
+      load_grain(a, sd, in);
+      site_update(a, sd, src, in, J, g, po, rows(sphi), rows(spsi), rows(svx), rows(svy),
                   threadIdx.x + 1);
     }
     __syncthreads();
@@ -124,6 +126,7 @@ __device__ __forceinline__ void ymarch_tiles(const StepArgs<S, R>& a,
       sc = w + 1;
     }
 
+    const SiteDom<R> sd(d);
     V2<R> JC = vec2(R(0), R(0));
     R gC[5], poC = R(0);
     // rows ya-1 and ya into the ring (warm-up)
@@ -169,11 +172,12 @@ __device__ __forceinline__ void ymarch_tiles(const StepArgs<S, R>& a,
         ring[3][slot][sc] = ld<R>(pbase<BIG>(a.ain, A_VYO, ps), pidx<BIG>(A_VYO, ps, src.s[0]));
         if constexpr (TH) ring[NF - 1][slot][sc] = pull_U<S, R, BIG>(a, src, psi);
       }
+      if (interior) load_grain(a, sd, in);
       __syncthreads();
       if (interior) {
         const int m = (j - 1) & 3, c0 = j & 3, pp = (j + 1) & 3;
         auto rows = [&](int f) { return Rows3<R>{ring[f][m], ring[f][c0], ring[f][pp]}; };
-        site_update<S, R, TH>(a, d, srcj, in, JC, gC, poC, rows(0), rows(1), rows(2), rows(3),
+        site_update<S, R, TH>(a, sd, srcj, in, JC, gC, poC, rows(0), rows(1), rows(2), rows(3),
                               sc, rows(NF - 1));
       }
       JC = JL;
@@ -321,7 +325,7 @@ static int traversal_blocks_per_sm(int variant, int tx, int ty, bool thermal) {
 template <typename S, typename R>
 int step_blocks_per_sm(int variant, int tx, int ty, long long plane_stride, bool thermal,
                        bool bc) {
-  if (variant == STEP_STAGED) return staged_blocks_per_sm<S, R>();
+  if (variant == STEP_STAGED) return staged_blocks_per_sm<S, R>(thermal);
   if (variant == STEP_YMARCH && bc)
     return ymarch_bc_blocks_per_sm<S, R>(big_handle(plane_stride, thermal), thermal);
   return big_handle(plane_stride, thermal)

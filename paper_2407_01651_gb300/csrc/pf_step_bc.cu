@@ -257,6 +257,7 @@ __global__ void __launch_bounds__(YM_THREADS, sizeof(R) == 4 ? 3 : 2)
       }
     };
 
+    const SiteDom<R> sd(d);
     V2<R> JC = vec2(R(0), R(0));
     R gC[5], poC = R(0);
     for (int k = 0; k < 2; ++k) {
@@ -288,11 +289,12 @@ __global__ void __launch_bounds__(YM_THREADS, sizeof(R) == 4 ? 3 : 2)
       V2<R> JL = vec2(R(0), R(0));
       R gL[5], poL = R(0);
       if (active) fill(j + 1, JL, gL, poL);
+      if (interior) load_grain(a, sd, in);
       __syncthreads();
       if (interior) {
         const int m = (j - 1) & 3, c0 = j & 3, pp = (j + 1) & 3;
         auto rows = [&](int f) { return Rows3<R>{ring[f][m], ring[f][c0], ring[f][pp]}; };
-        site_update<S, R, TH>(a, d, srcj, in, JC, gC, poC, rows(0), rows(1), rows(2), rows(3),
+        site_update<S, R, TH>(a, sd, srcj, in, JC, gC, poC, rows(0), rows(1), rows(2), rows(3),
                               sc, rows(NF - 1));
       }
       JC = JL;

@@ -67,11 +67,13 @@ __global__ void __launch_bounds__(GX * GY) k_step_general(StepArgs<S, R> a, DomD
   pull.hg(x, y, J, g, phi, psi, po);
   SiteIn<R> in;
   pull.site(x, y, in);
+  const SiteDom<R> sd(d);
+  load_grain(a, sd, in);
   Src9 src;
   src.s[0] = site_at(d, x, y);
   const int r = threadIdx.y;
   auto rows = [&](int f) { return Rows3<R>{ring[f][r], ring[f][r + 1], ring[f][r + 2]}; };
-  site_update<S, R, TH>(a, d, src, in, J, g, po, rows(0), rows(1), rows(2), rows(3),
+  site_update<S, R, TH>(a, sd, src, in, J, g, po, rows(0), rows(1), rows(2), rows(3),
                         threadIdx.x + 1, rows(NF - 1));
 }
 

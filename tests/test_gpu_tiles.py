@@ -33,6 +33,27 @@ def test_rows_per_tile_do_not_change_the_bits(shape, precision, thermal):
     assert np.array_equal(res[0], res[1])
 
 
+@pytest.mark.parametrize("shape", [(1024, 768), (1028, 800), (900, 900), (132, 6000)])
+@pytest.mark.parametrize("thermal,bc", [(0, None), (1, None), (1, (S, S, W, F)), (0, (P, P, W, W))])
+def test_staged_rows_give_the_bits_of_the_plain_march(shape, thermal, bc):
+    """Large FP32 lattices stage their rows by bulk copies where the width allows
+    it: the bits of the y-march set by hand, with the temperature lattice and
+    beside tiles at a side."""
+    lay = small(*shape)
+    par = dict(lay.params, thermal=thermal, g=1e-5)
+    res = []
+    for plain in (False, True):
+        sim = pf.Simulation([shape], par, "fp32")
+        if bc:
+            sim.set_boundaries(0, *bc)
+        if plain:
+            sim.set_step_config(1, sim.step_config()[1])
+        sim.init_fields(0, lay.seeds, lay.R_s, lay.bubbles)
+        sim.step(6)
+        res.append(sim.get_state())
+    assert np.array_equal(res[0], res[1])
+
+
 @pytest.mark.parametrize("shape,bc,rows", [
     ((129, 40), (W, S, P, P), 0),     # a last strip of one column
     ((130, 40), (F, W, P, P), 0),
