@@ -58,11 +58,13 @@ __device__ __forceinline__ void st(S* __restrict__ p, I i, R v) {
   p[i] = Codec<S>::template enc<R>(v);
 }
 
-// Reciprocal and reciprocal square root: IEEE in FP64; in FP32 the hardware
-// approximations (relative error a few 1e-7), far inside the FP32 tolerance.
+// Reciprocal and reciprocal square root: in FP64 IEEE and to one ulp (as the
+// rounded quotient of the rounded root is, at about half its instructions on
+// units that are the bound there); in FP32 the hardware approximations
+// (relative error a few 1e-7), far inside the FP32 tolerance.
 __device__ __forceinline__ double frcp(double x) { return 1.0 / x; }
 __device__ __forceinline__ float frcp(float x) { return __fdividef(1.0f, x); }
-__device__ __forceinline__ double frsqrt(double x) { return 1.0 / sqrt(x); }
+__device__ __forceinline__ double frsqrt(double x) { return rsqrt(x); }
 __device__ __forceinline__ float frsqrt(float x) { return rsqrtf(x); }
 
 // Plane k of a plane-major buffer: a warp-uniform base pointer, so that one
