@@ -448,8 +448,9 @@ typedef struct pf3_handle pf3_handle;
 #define PF3_STATE_PLANES_THERMAL 30
 
 /* Handle of an nx x ny x nz lattice (each in [4, 4096]), FP32 or FP64
- * storage, on cuda_stream; allocates two state copies (23 planes each, 30 in
- * thermal mode) and 3 field planes (4 in thermal mode).  Errors: BAD_ARG, OOM. */
+ * storage, on cuda_stream; allocates two state copies (17 planes each, 22 in
+ * thermal mode: of each opposite pair whose sum the density fixes, one
+ * population) and 3 field planes (4 in thermal mode).  Errors: BAD_ARG, OOM. */
 pf_status pf3_create(const pf_params *p, int nx, int ny, int nz, pf_precision prec,
                      void *cuda_stream, pf3_handle **out);
 /* Spherical seeds n x (x, y, z) of radius R_s: psi = max tanh(sqrt(2 beta_psi)

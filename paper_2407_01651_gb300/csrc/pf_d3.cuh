@@ -32,6 +32,18 @@ __device__ __forceinline__ const T* pl(const T* p, int k, unsigned ps) { return 
 template <typename T>
 __device__ __forceinline__ T* pl(T* p, int k, unsigned ps) { return p + (unsigned)k * ps; }
 
+// Pair storage on D3Q7.  The even moments of the dendrite, solute and
+// temperature collisions are set by the density, so the populations of an axis
+// add up to 2 x base (density/8, temperature: a plane of its own); one of each
+// pair is stored, direction 1, 3 or 5, and the density.
+// Plane of the pair of direction q (1..6) and whether q is the opposite one.
+__device__ __forceinline__ constexpr int pair7(int q) { return (q - 1) / 2; }
+__device__ __forceinline__ constexpr bool minus7(int q) { return q % 2 == 0; }
+// opposite population of an axis from its density m: m/4 - g (the products
+// with powers of two are exact)
+template <typename R>
+__device__ __forceinline__ R other7(R m, R v) { return fma(R(0.25), m, -v); }
+
 // Index offset from coordinate v (in [0, n)) to v - c, c in {-1, 0, 1}, with one
 // periodic wrap, times the axis stride. Added to a site index in the unsigned
 // type I, a negative offset wraps modulo 2^bits and the sum is the exact

@@ -25,9 +25,10 @@
 namespace pf {
 namespace d3 {
 
-// planes: g_pre 0..6, g_post 7..13, s 14..20, thermal e 21..27 (storage
-// type); r, Q_o (compute type)
-constexpr int G_PRE = 0, G_POST = 7, S_POP = 14, E_POP = 21, NPOP3 = 21, NPOP3_TH = 28;
+// planes (storage type; pairs as in pf_d3.cuh): g_pre 0..6; g_post density, g_1,
+// g_3, g_5; C, s_1, s_3, s_5; thermal rho H, axis base, e_1, e_3, e_5; r, Q_o
+// (compute type): 17 values per site instead of 23 (thermal 22 instead of 30)
+constexpr int G_PRE = 0, G_POST = 7, S_POP = 11, E_POP = 15, NPOP3 = 15, NPOP3_TH = 20;
 constexpr int A3_RR = 0, A3_QO = 1, NAUX3 = 2;
 constexpr int NSTATE3 = 23, NSTATE3_TH = 30;      // raw FP64 state planes
 
@@ -109,7 +110,16 @@ __device__ __forceinline__ void stream_g(const Args3<S, R, I>& a, int x, int y, 
     int q;
     const int mode = pull7<S, R, BC>(a, x, y, z, i, src, q);
     const R gold = ld<R>(pl(a.in, G_PRE + i, a.ps), own);
-    R gpo = ld<R>(pl(a.in, G_POST + q, a.ps), src);
+    R gpo;
+    if (i == 0) {
+      gpo = R(0.25) * ld<R>(pl(a.in, G_POST, a.ps), own);
+    } else {
+      gpo = ld<R>(pl(a.in, G_POST + 1 + pair7(q), a.ps), src);
+      if (BC || minus7(i)) {
+        const R o = other7(ld<R>(pl(a.in, G_POST, a.ps), src), gpo);
+        if (minus7(q)) gpo = o;
+      }
+    }
     if (BC && mode == 2) gpo = -gpo + R(2) * w7<R>(i) * R(-1);    // psi_far = -1
     const R rr = ld<R>(pl(a.ain, A3_RR, a.ps), src);
     g[i] = gold + (gpo - gold) * rr;
@@ -120,17 +130,26 @@ __device__ __forceinline__ void stream_g(const Args3<S, R, I>& a, int x, int y, 
   psio = po;
 }
 
-// Streamed populations of one D3Q7 lattice (plane base P) at (x, y, z); far:
-// the lattice's far-field value (BC).
-template <typename S, typename R, bool BC, typename I>
-__device__ __forceinline__ void stream7(const Args3<S, R, I>& a, int P, int x, int y, int z, R f[7],
+// Streamed solute (E = false) or temperature populations at (x, y, z); far: the
+// lattice's far-field value (BC).
+template <typename S, typename R, bool BC, bool E, typename I>
+__device__ __forceinline__ void stream7(const Args3<S, R, I>& a, int x, int y, int z, R f[7],
                                         R far) {
+  constexpr int P = E ? E_POP : S_POP, PAIR = E ? E_POP + 2 : S_POP + 1;
+  const unsigned long long own = site3(a, x, y, z);
+  const R m = ld<R>(pl(a.in, P, a.ps), own);
+  f[0] = E ? fma(R(-6), ld<R>(pl(a.in, P + 1, a.ps), own), m) : R(0.25) * m;
 #pragma unroll
-  for (int i = 0; i < 7; ++i) {
+  for (int i = 1; i < 7; ++i) {
     unsigned long long src;
     int q;
     const int mode = pull7<S, R, BC>(a, x, y, z, i, src, q);
-    f[i] = ld<R>(pl(a.in, P + q, a.ps), src);
+    f[i] = ld<R>(pl(a.in, PAIR + pair7(q), a.ps), src);
+    if (BC || minus7(i)) {
+      const R b = ld<R>(pl(a.in, E ? P + 1 : P, a.ps), src);
+      const R o = E ? fma(R(2), b, -f[i]) : other7(b, f[i]);
+      if (minus7(q)) f[i] = o;
+    }
     if (BC && mode == 2) f[i] = -f[i] + R(2) * w7<R>(i) * far;
   }
 }
@@ -241,7 +260,7 @@ __global__ void __launch_bounds__(THREADS, (ctas3d<R, TH, ROT, I>())) k_step3d(A
         ring[(za - 1 + k) & 3][hy][hx] = gpsi(psi, fz);
         if constexpr (TH) {
           R sv[7];
-          stream7<S, R, BC>(a, S_POP, x, y, z, sv, R(1));
+          stream7<S, R, BC, false>(a, x, y, z, sv, R(1));
           const R C = sum7(sv);
           uring[(za - 1 + k) & 3][hy][hx] = gU(supersat3(a.c, C, psi), fz);
           if (k == 1) {
@@ -266,9 +285,9 @@ __global__ void __launch_bounds__(THREADS, (ctas3d<R, TH, ROT, I>())) k_step3d(A
         if constexpr (TH) {
 #pragma unroll
           for (int i = 0; i < 7; ++i) sv[i] = sC[i];
-          stream7<S, R, BC>(a, E_POP, x, y, z, ev, a.c.th0);
+          stream7<S, R, BC, true>(a, x, y, z, ev, a.c.th0);
         } else {
-          stream7<S, R, BC>(a, S_POP, x, y, z, sv, R(1));
+          stream7<S, R, BC, false>(a, x, y, z, sv, R(1));
         }
         Qo = ld<R>(pl(a.ain, A3_QO, a.ps), site);
         // warm L2 with this column's populations two planes ahead
@@ -287,7 +306,7 @@ __global__ void __launch_bounds__(THREADS, (ctas3d<R, TH, ROT, I>())) k_step3d(A
         stream_g<S, R, BC>(a, x, y, zn, gL, psi, poL);
         ring[(z + 1) & 3][hy][hx] = gpsi(psi, fz);
         if constexpr (TH) {
-          stream7<S, R, BC>(a, S_POP, x, y, zn, sL, R(1));
+          stream7<S, R, BC, false>(a, x, y, zn, sL, R(1));
           CL = sum7(sL);
           uring[(z + 1) & 3][hy][hx] = gU(supersat3(a.c, CL, psi), fz);
         }
@@ -358,16 +377,11 @@ __global__ void __launch_bounds__(THREADS, (ctas3d<R, TH, ROT, I>())) k_step3d(A
           const R Sx = fma(hs, gq * Nx, Jx - s1 * Jx), Sy = fma(hs, gq * Ny, Jy - s1 * Jy),
                   Sz = fma(hs, gq * Nz, Jz - s1 * Jz);
           const R b = m0 * R(0.125);
-          R go[7];
-          go[0] = fma(R(-6), b, m0);           // m0 - 6 m0/8 = m0/4, exact
-          go[1] = fma(R(0.5), Sx, b); go[2] = fma(R(-0.5), Sx, b);
-          go[3] = fma(R(0.5), Sy, b); go[4] = fma(R(-0.5), Sy, b);
-          go[5] = fma(R(0.5), Sz, b); go[6] = fma(R(-0.5), Sz, b);
+          const R go[4] = {m0, fma(R(0.5), Sx, b), fma(R(0.5), Sy, b), fma(R(0.5), Sz, b)};
 #pragma unroll
-          for (int i = 0; i < 7; ++i) {
-            st<S, R>(pl(a.out, G_PRE + i, a.ps), site, gC[i]);
-            st<S, R>(pl(a.out, G_POST + i, a.ps), site, go[i]);
-          }
+          for (int i = 0; i < 7; ++i) st<S, R>(pl(a.out, G_PRE + i, a.ps), site, gC[i]);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) st<S, R>(pl(a.out, G_POST + i, a.ps), site, go[i]);
           pl(a.aout, A3_RR, a.ps)[site] = ias2;
           pl(a.aout, A3_QO, a.ps)[site] = Qeff;
         }
@@ -383,13 +397,9 @@ __global__ void __launch_bounds__(THREADS, (ctas3d<R, TH, ROT, I>())) k_step3d(A
           const R Jx = sv[1] - sv[2], Jy = sv[3] - sv[4], Jz = sv[5] - sv[6];
           const R Sx = Jx - sc * (Jx - Ex), Sy = Jy - sc * (Jy - Ey), Sz = Jz - sc * (Jz - Ez);
           const R b = C * R(0.125);
-          R so[7];
-          so[0] = fma(R(-6), b, C);            // C - 6 C/8 = C/4, exact
-          so[1] = fma(R(0.5), Sx, b); so[2] = fma(R(-0.5), Sx, b);
-          so[3] = fma(R(0.5), Sy, b); so[4] = fma(R(-0.5), Sy, b);
-          so[5] = fma(R(0.5), Sz, b); so[6] = fma(R(-0.5), Sz, b);
+          const R so[4] = {C, fma(R(0.5), Sx, b), fma(R(0.5), Sy, b), fma(R(0.5), Sz, b)};
 #pragma unroll
-          for (int i = 0; i < 7; ++i) st<S, R>(pl(a.out, S_POP + i, a.ps), site, so[i]);
+          for (int i = 0; i < 4; ++i) st<S, R>(pl(a.out, S_POP + i, a.ps), site, so[i]);
         }
         // temperature (TH): at rest the equilibrium is e_0 = rho H - (3/4) theta,
         // e_i = theta / 8; the flux relaxes to 0 at s_T from k_T = (1/s_T - 1/2)
@@ -400,13 +410,9 @@ __global__ void __launch_bounds__(THREADS, (ctas3d<R, TH, ROT, I>())) k_step3d(A
           const R b = round_to_multiple(theta * R(0.125), R(2) * quantum_quarter_ulp(m0e));
           const R Sx = c.omsth * (ev[1] - ev[2]), Sy = c.omsth * (ev[3] - ev[4]),
                   Sz = c.omsth * (ev[5] - ev[6]);
-          R eo[7];
-          eo[0] = fma(R(-6), b, m0e);
-          eo[1] = fma(R(0.5), Sx, b); eo[2] = fma(R(-0.5), Sx, b);
-          eo[3] = fma(R(0.5), Sy, b); eo[4] = fma(R(-0.5), Sy, b);
-          eo[5] = fma(R(0.5), Sz, b); eo[6] = fma(R(-0.5), Sz, b);
+          const R eo[5] = {m0e, b, fma(R(0.5), Sx, b), fma(R(0.5), Sy, b), fma(R(0.5), Sz, b)};
 #pragma unroll
-          for (int i = 0; i < 7; ++i) st<S, R>(pl(a.out, E_POP + i, a.ps), site, eo[i]);
+          for (int i = 0; i < 5; ++i) st<S, R>(pl(a.out, E_POP + i, a.ps), site, eo[i]);
         }
         if (a.fields) {
           pl(a.fields, 0, a.ps)[site] = psi;
@@ -435,9 +441,9 @@ template <typename S, typename R>
 __device__ void write_th3(const Args3<S, R>& a, unsigned long long site, R psi, R C, R theta) {
   const Coef3<R>& c = a.c;
   const R m0 = c.rcp * (theta - c.halfL * (R(1) + psi));
+  st<S, R>(pl(a.out, E_POP, a.ps), site, m0);
 #pragma unroll
-  for (int i = 1; i < 7; ++i) st<S, R>(pl(a.out, E_POP + i, a.ps), site, R(0.125) * theta);
-  st<S, R>(pl(a.out, E_POP, a.ps), site, m0 - R(0.75) * theta);
+  for (int i = 1; i < 5; ++i) st<S, R>(pl(a.out, E_POP + i, a.ps), site, R(0.125) * theta);
   const R U = supersat3(c, C, psi);
   const R omp2 = R(1) - psi * psi;
   const R Q = c.four_bpsi * psi * omp2 - c.lam * omp2 * omp2 * (theta + c.Mcinf * U);
@@ -451,10 +457,11 @@ template <typename S, typename R, bool TH>
 __device__ void write_eq3(const Args3<S, R>& a, unsigned long long site, R psi, R C, R theta) {
   const Coef3<R>& c = a.c;
 #pragma unroll
-  for (int i = 0; i < 7; ++i) {
-    st<S, R>(pl(a.out, G_PRE + i, a.ps), site, w7<R>(i) * psi);
-    st<S, R>(pl(a.out, G_POST + i, a.ps), site, w7<R>(i) * psi);
-    st<S, R>(pl(a.out, S_POP + i, a.ps), site, w7<R>(i) * C);
+  for (int i = 0; i < 7; ++i) st<S, R>(pl(a.out, G_PRE + i, a.ps), site, w7<R>(i) * psi);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {      // density, then one population per axis
+    st<S, R>(pl(a.out, G_POST + i, a.ps), site, i ? R(0.125) * psi : psi);
+    st<S, R>(pl(a.out, S_POP + i, a.ps), site, i ? R(0.125) * C : C);
   }
   const R omk = R(1) - c.k;
   const R U = (R(2) * C / ((R(1) + c.k) - omk * psi) - R(1)) * c.inv_omk;
@@ -513,15 +520,23 @@ __global__ void k_state3(const S* pin, const R* ain, unsigned long long ps, unsi
                          int thermal, double* out) {
   for (unsigned long long j = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; j < n;
        j += (unsigned long long)gridDim.x * blockDim.x) {
+    auto v = [&](int k) { return ld<R>(pl(pin, k, ps), j); };
+    const R mg = v(G_POST), mc = v(S_POP);
     for (int i = 0; i < 7; ++i) {
-      out[(0 + i) * n + j] = (double)ld<R>(pl(pin, G_PRE + i, ps), j);
-      out[(7 + i) * n + j] = (double)ld<R>(pl(pin, G_POST + i, ps), j);
-      out[(15 + i) * n + j] = (double)ld<R>(pl(pin, S_POP + i, ps), j);
+      const int k = i ? 1 + pair7(i) : 0;
+      out[(0 + i) * n + j] = (double)v(G_PRE + i);
+      out[(7 + i) * n + j] = (double)(i == 0 ? R(0.25) * mg : (minus7(i) ? other7(mg, v(G_POST + k)) : v(G_POST + k)));
+      out[(15 + i) * n + j] = (double)(i == 0 ? R(0.25) * mc : (minus7(i) ? other7(mc, v(S_POP + k)) : v(S_POP + k)));
     }
     out[14 * n + j] = (double)ain[A3_RR * ps + j];
     out[22 * n + j] = (double)ain[A3_QO * ps + j];
-    if (thermal)
-      for (int i = 0; i < 7; ++i) out[(23 + i) * n + j] = (double)ld<R>(pl(pin, E_POP + i, ps), j);
+    if (thermal) {
+      const R m = v(E_POP), b = v(E_POP + 1);
+      for (int i = 0; i < 7; ++i) {
+        const R e = i ? v(E_POP + 2 + pair7(i)) : R(0);
+        out[(23 + i) * n + j] = (double)(i == 0 ? fma(R(-6), b, m) : (minus7(i) ? fma(R(2), b, -e) : e));
+      }
+    }
   }
 }
 
@@ -564,7 +579,7 @@ __global__ void k_reduce3_th(const S* pin, const R* f, unsigned long long ps, un
   double a0 = 0.0, a1 = 0.0, a2 = 0.0;
   for (unsigned long long j = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; j < n;
        j += (unsigned long long)gridDim.x * blockDim.x) {
-    for (int i = 0; i < 7; ++i) a0 += (double)ld<R>(pl(pin, E_POP + i, ps), j);
+    a0 += (double)ld<R>(pl(pin, E_POP, ps), j);   // rho H, the populations' sum
     a1 += (double)f[3 * ps + j];
     a2 += (double)f[j];
   }
