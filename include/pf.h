@@ -486,8 +486,8 @@ pf_status pf3_set_orientation(pf3_handle *h, const double *seeds7, int n_seeds);
  * both not.  Before initialising (seeds then use plain distances along bounded
  * axes).  Errors: BAD_ARG, STATE (already initialised). */
 pf_status pf3_set_boundaries(pf3_handle *h, const int bc[6]);
-/* Planes per tile of the z-march (default 16).  Errors: BAD_ARG (outside
- * [1, 4096]). */
+/* Planes per tile of the z-march (default: chosen by size, at most 16; the
+ * state does not depend on it).  Errors: BAD_ARG (outside [1, 4096]). */
 pf_status pf3_set_chunk(pf3_handle *h, int chunk);
 /* Index width of the periodic step: by default sites and plane offsets are
  * indexed in 32 bits while PF3_STATE_PLANES_THERMAL x n < 2^32 (fewer address
@@ -587,9 +587,9 @@ pf_status pf3f_set_orientation(pf3f_handle *h, const double *seeds7, int n_seeds
  * all of it at a wall or far side; 2 X_far - X for psi and U at a far side).
  * Before initialising.  Errors: BAD_ARG, STATE. */
 pf_status pf3f_set_boundaries(pf3f_handle *h, const int bc[6]);
-/* Planes per tile of the z-march (default 36, the fastest at 256^3 on a
- * 152-SM GPU: the tiles then fill the last wave of one CTA per SM); the state
- * does not depend on it.  Errors: BAD_ARG (outside [1, 2048]). */
+/* Planes per tile of the z-march (default: chosen by size, at most 36, which
+ * is the fastest at 256^3 on a 152-SM GPU: the tiles then fill the last wave of
+ * one CTA per SM); the state does not depend on it.  Errors: BAD_ARG (outside [1, 2048]). */
 pf_status pf3f_set_chunk(pf3f_handle *h, int chunk);
 /* Index width of the periodic step: by default sites and plane offsets are
  * indexed in 32 bits while PF3F_STATE_PLANES_THERMAL x n < 2^32 (fewer address

@@ -3,6 +3,7 @@
 // set, plane addressing, periodic wrapping and the isotropic D3Q19-weighted
 // gradient and Laplacian over a 4-slot shared-memory ring of planes.
 #pragma once
+#include <algorithm>
 #include <cmath>
 
 #include "pf_device.cuh"
@@ -99,6 +100,37 @@ __device__ __forceinline__ R lap18(const R (*Pm)[HX], const R (*P0)[HX], const R
                   ((d(Pp, 1, 0) + d(Pm, -1, 0)) + (d(Pp, -1, 0) + d(Pm, 1, 0))) +
                   ((d(Pp, 0, 1) + d(Pm, 0, -1)) + (d(Pp, 0, -1) + d(Pm, 0, 1)));
   return R(1.0 / 3.0) * faces + R(1.0 / 6.0) * edges;
+}
+
+// Planes per tile of a z-march over columns of TX x ty sites on `slots` resident
+// CTAs: `top` where that gives waves enough, else the length whose tiles, each
+// with 2 warm-up planes and the columns' last ones shorter, end first. `alone`:
+// what a plane takes longer where a tile has an SM to itself; a shorter length
+// has to be `gain` ahead. Chosen once per handle.
+inline int planes_by_size(int nx, int ny, int nz, int ty, int slots, int top, double alone,
+                          double gain) {
+  const long long xy = (long long)((nx + TX - 1) / TX) * ((ny + ty - 1) / ty);
+  if (xy * ((nz + top - 1) / top) > 6ll * slots) return top;
+  auto planes = [&](int c) {
+    const long long tz = (nz + c - 1) / c, full = xy * (tz - 1);
+    const long long A = c + 2, B = nz - c * (tz - 1) + 2;
+    // whole tiles in rounds; then the columns' last ones on the SMs that are free,
+    // and on the others when their tile ends
+    const long long q = full / slots, r = full % slots;
+    long long t = r ? std::max(A, B) : B;
+    while ((slots - r) * (t / B) + r * (t > A ? (t - A) / B : 0) < xy) ++t;
+    return (double)(q * A + t) * (xy * tz <= slots ? alone : 1.0);
+  };
+  int pick = top;
+  double best = planes(top);
+  for (int c = std::min(top, nz) - 1; c >= 1; --c) {
+    const double cost = planes(c);
+    if (cost < gain * best) {
+      best = cost;
+      pick = c;
+    }
+  }
+  return pick;
 }
 
 // Signed minimum-image offset on a periodic axis of length L.

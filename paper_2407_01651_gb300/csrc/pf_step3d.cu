@@ -607,8 +607,11 @@ struct pf3_handle {
   pf_params p{};
   pf_precision prec = PF_FP32;
   cudaStream_t stream = nullptr;
-  int nx = 0, ny = 0, nz = 0, chunk = 16;
+  int nx = 0, ny = 0, nz = 0;
+  int chunk = 0;    // planes per tile (0: by size)
+  int planes = 16;  // by size (choose_planes)
   int index64 = 0;  // periodic step in 64-bit indices at any size
+  int sms = 1;      // of the device
   int thermal = 0, npop = NPOP3, nfields = 3, nstate = NSTATE3;
   int rotated = 0;                // grain orientations set
   int bc[6] = {0, 0, 0, 0, 0, 0}; // side types x-, x+, y-, y+, z-, z+
@@ -671,9 +674,22 @@ static Coef3<R> coef3(const pf_params& p) {
   return c;
 }
 
+// Planes per tile where the caller sets none. Two CTAs an SM, three in one form;
+// the FP64 form is bound by the SM's FP64 units, which one tile keeps busy five
+// sixths of the time. us per step at 16 planes and at those chosen: FP32 64^3
+// 29.0 -> 16.6, 96x80x72 30.9 -> 24.8, 128^3 87.9 -> 81.1, 256^3 519 (16); FP64
+// 64^3 354 -> 193.
+static void choose_planes(pf3_handle* h) {
+  const bool fp64 = h->elem == 8;
+  const int per_sm = fp64 ? 1 : (h->thermal || h->rotated ? 2 : 3);
+  h->planes = planes_by_size(h->nx, h->ny, h->nz, TY, h->sms * per_sm, 16, fp64 ? 1.2 : 1.0,
+                             fp64 ? 0.9 : 0.97);
+}
+
 template <typename S, typename R, typename I = unsigned long long>
 static Args3<S, R, I> args3(const pf3_handle* h, bool fields) {
   Args3<S, R, I> a{};
+  a.chunk = h->chunk ? h->chunk : h->planes;
   a.in = (const S*)h->pop[h->cur];
   a.out = (S*)h->pop[h->cur ^ 1];
   a.ain = (const R*)h->aux[h->cur];
@@ -683,10 +699,10 @@ static Args3<S, R, I> args3(const pf3_handle* h, bool fields) {
   a.rot = (const R*)h->rot;
   for (int k = 0; k < 6; ++k) a.bc[k] = h->bc[k];
   a.ps = (I)h->n;
-  a.nx = h->nx; a.ny = h->ny; a.nz = h->nz; a.chunk = h->chunk;
+  a.nx = h->nx; a.ny = h->ny; a.nz = h->nz;
   a.tiles_x = (h->nx + TX - 1) / TX;
   a.tiles_y = (h->ny + TY - 1) / TY;
-  a.tiles_z = (h->nz + h->chunk - 1) / h->chunk;
+  a.tiles_z = (h->nz + a.chunk - 1) / a.chunk;
   a.c = coef3<R>(h->p);
   return a;
 }
@@ -742,6 +758,13 @@ extern "C" pf_status pf3_create(const pf_params* p, int nx, int ny, int nz, pf_p
   h->nfields = p->thermal ? 4 : 3;
   h->nstate = p->thermal ? NSTATE3_TH : NSTATE3;
   h->elem = h->celem = prec == PF_FP64 ? 8 : 4;
+  {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || h->sms < 1)
+      h->sms = 1;
+    choose_planes(h);
+  }
   bool ok = true;
   for (int c = 0; c < 2; ++c) {
     ok = ok && cudaMalloc(&h->pop[c], n * h->npop * h->elem) == cudaSuccess;
@@ -892,6 +915,7 @@ extern "C" pf_status pf3_set_orientation(pf3_handle* h, const double* seeds7, in
   if (n_seeds < 0 || (n_seeds > 0 && !seeds7)) return fail3(h, PF_ERR_BAD_ARG, "bad seeds");
   if (n_seeds == 0) {                      // back to the lattice-aligned grain
     h->rotated = 0;
+    choose_planes(h);
     return PF_OK;
   }
   std::vector<double> rot(9 * (size_t)n_seeds);
@@ -929,6 +953,7 @@ extern "C" pf_status pf3_set_orientation(pf3_handle* h, const double* seeds7, in
   }
   PF3_CUDA(h, cudaStreamSynchronize(h->stream));
   h->rotated = 1;
+  choose_planes(h);
   return PF_OK;
 }
 
@@ -975,11 +1000,10 @@ extern "C" pf_status pf3_step(pf3_handle* h, int n_steps) {
     const bool a32 = !h->any_bc && !h->index64 && (unsigned long long)NSTATE3_TH * h->n <= 0xFFFFFFFFull;
     for (int t = 0; t < n_steps; ++t) {
       const bool last = t == n_steps - 1;
-      const int tiles = (int)((long long)((h->nx + TX - 1) / TX) * ((h->ny + TY - 1) / TY) *
-                              ((h->nz + h->chunk - 1) / h->chunk));
       auto go = [&](auto bcv, const auto& a) {
         constexpr bool BC = decltype(bcv)::value;
         using I = decltype(a.ps);
+        const int tiles = a.tiles_x * a.tiles_y * a.tiles_z;
         if (h->rotated) {
           if (h->thermal) k_step3d<S, R, true, true, BC, I><<<tiles, THREADS, 0, h->stream>>>(a);
           else k_step3d<S, R, false, true, BC, I><<<tiles, THREADS, 0, h->stream>>>(a);

@@ -232,7 +232,12 @@ struct pf3f_handle {
   pf_params p{};
   pf_precision prec = PF_FP32;
   cudaStream_t stream = nullptr;
-  int nx = 0, ny = 0, nz = 0, chunk = 36;  // z-march tile (tuned at 256^3 on 152 SMs)
+  int nx = 0, ny = 0, nz = 0;
+  int chunk = 0;    // planes per tile (0: by size)
+  // by size: one CTA an SM; us per step at 36 planes and at those chosen: FP32
+  // 64^3 147 -> 37.6, 96x80x72 152 -> 72.6, 128^3 305 -> 255, 256^3 1885 (36: tuned
+  // there); FP64 64^3 3677 -> 745
+  int planes = 36;
   int index64 = 0;  // periodic step in 64-bit indices at any size
   unsigned long long n = 0;
   size_t elem = 4;
@@ -318,6 +323,7 @@ static CoefF<R> coeff(const pf3f_handle* h) {
 template <typename S, typename R, typename I = unsigned long long>
 static ArgsF<S, R, I> argsf(const pf3f_handle* h, bool fields) {
   ArgsF<S, R, I> a{};
+  a.chunk = h->chunk ? h->chunk : h->planes;
   a.in = (const S*)h->pop[h->cur];
   a.out = (S*)h->pop[h->cur ^ 1];
   a.ain = (const R*)h->aux[h->cur];
@@ -327,10 +333,10 @@ static ArgsF<S, R, I> argsf(const pf3f_handle* h, bool fields) {
   a.rot = (const R*)h->rot;
   for (int k = 0; k < 6; ++k) a.bc[k] = h->bc[k];
   a.ps = (I)h->n;
-  a.nx = h->nx; a.ny = h->ny; a.nz = h->nz; a.chunk = h->chunk;
+  a.nx = h->nx; a.ny = h->ny; a.nz = h->nz;
   a.tiles_x = (h->nx + TX - 1) / TX;
   a.tiles_y = (h->ny + TY - 1) / TY;
-  a.tiles_z = (h->nz + h->chunk - 1) / h->chunk;
+  a.tiles_z = (h->nz + a.chunk - 1) / a.chunk;
   a.c = coeff<R>(h);
   return a;
 }
@@ -411,6 +417,12 @@ extern "C" pf_status pf3f_create(const pf_params* p, int nx, int ny, int nz, pf_
   h->p = *p; h->prec = prec; h->stream = (cudaStream_t)cuda_stream;
   h->nx = nx; h->ny = ny; h->nz = nz; h->n = n;
   h->elem = prec == PF_FP64 ? 8 : 4;
+  {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
+      h->planes = d3::planes_by_size(nx, ny, nz, TY, sms, 36, 1.0, 0.97);
+  }
   h->thermal = p->thermal;
   h->npop = p->thermal ? NPOPF_TH : NPOPF;
   h->naux = p->thermal ? NAUXF_TH : NAUXF;
