@@ -986,10 +986,12 @@ static pf_status steps_one_launch(pf_handle* h, int n, bool write_fields, cudaSt
 }
 
 template <typename S, typename R>
-static pf_status step_t(pf_handle* h, bool write_fields, cudaStream_t stream = nullptr) {
-  const StepArgs<S, R> a = make_step_args<S, R>(h, h->pop[h->cur], h->aux[h->cur],
+static pf_status step_t(pf_handle* h, bool write_fields, cudaStream_t stream = nullptr,
+                        bool chained = false) {
+  StepArgs<S, R> a = make_step_args<S, R>(h, h->pop[h->cur], h->aux[h->cur],
                                                 h->pop[h->cur ^ 1], h->aux[h->cur ^ 1],
                                                 write_fields);
+  a.chained = chained;
   pf_status st = launch_all<S, R>(h, a, stream ? stream : h->stream);
   if (st != PF_OK) return st;
   h->cur ^= 1;
@@ -1106,8 +1108,13 @@ static pf_status step_n(pf_handle* h, int n_steps) {
       h->launches += (long long)h->graph_steps * per_step;
     }
   }
-  for (; done < n_steps; ++done) {
-    pf_status st = step_t<S, R>(h, done == n_steps - 1);
+  // steps behind the first, one launch each: chained (see chain_step), except in
+  // a caller's capture, whose graph keeps plain edges
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (n_steps - done > 1) PF_CUDA(h, cudaStreamIsCapturing(h->stream, &cs));
+  const bool chain = cs == cudaStreamCaptureStatusNone && h->launch_mode == 0 && !h->any_bc;
+  for (bool behind = false; done < n_steps; ++done, behind = chain) {
+    pf_status st = step_t<S, R>(h, done == n_steps - 1, nullptr, behind);
     if (st != PF_OK) return st;
   }
   return PF_OK;

@@ -48,9 +48,34 @@ constexpr float kNSScale = 4096.0f;      // NS populations x 2^12 in the 16-bit 
 constexpr float kNSInvScale = 1.0f / 4096.0f;
 
 
+// Load from a state plane: a plain coherent load (a chained step starts while the
+// step that writes the plane still runs, so the read-only path is not for it) that
+// the compiler may move past the stores, which go to the other state.
+__device__ __forceinline__ float ldp(const float* p) {
+  float v;
+  asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double ldp(const double* p) {
+  double v;
+  asm("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ unsigned short ldp(const unsigned short* p) {
+  unsigned short v;
+  asm("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ __half ldp(const __half* p) {
+  return __ushort_as_half(ldp(reinterpret_cast<const unsigned short*>(p)));
+}
+__device__ __forceinline__ __nv_bfloat16 ldp(const __nv_bfloat16* p) {
+  return __ushort_as_bfloat16(ldp(reinterpret_cast<const unsigned short*>(p)));
+}
+
 template <typename R, typename S, typename I>
 __device__ __forceinline__ R ld(const S* __restrict__ p, I i) {
-  return Codec<S>::template dec<R>(__ldg(p + i));
+  return Codec<S>::template dec<R>(ldp(p + i));
 }
 
 template <typename S, typename R, typename I>
@@ -116,7 +141,7 @@ __device__ __forceinline__ S enc_off(R v, R wm) {
 }
 template <typename S, typename R, typename I>
 __device__ __forceinline__ R pop_off(const S* __restrict__ p, I i, R wm) {
-  return dec_off<S, R>(__ldg(p + i), wm);
+  return dec_off<S, R>(ldp(p + i), wm);
 }
 template <typename S, typename R, typename I>
 __device__ __forceinline__ void st_off(S* __restrict__ p, I i, R v, R wm) {

@@ -43,6 +43,7 @@ struct StepArgs {
   R* fields;                    // 8 field planes, or nullptr
   unsigned int* err;            // device error bits (1: a staged copy timed out), or nullptr
   int drop_copies;              // testing only: the staged kernel skips its bulk copies
+  int chained;                  // launched behind the handle's previous step (chain_step)
   int thermal;                  // 1: temperature lattice and finite-Le F(U) (FP32 / FP64)
   int bc;                       // 1: some domain has a non-periodic side (y-march only)
   KParams<R> kp;
@@ -99,6 +100,21 @@ struct ReduceArgs {
 template <typename S, typename R>
 cudaError_t launch_step(const StepArgs<S, R>& a, int variant, int tx, int ty, int grid,
                         cudaStream_t st);
+// Launch of a step kernel, behind the previous step where a.chained (chain_step).
+template <typename K, typename A>
+cudaError_t launch_chained(K kernel, const A& a, int grid, size_t smem, cudaStream_t st) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(YM_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = a.chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, a);
+}
 // Staged variant (bulk copies of the input rows into shared memory): launch,
 // dynamic shared memory, the x granularity it needs (nx a multiple of it), and
 // resident CTAs per SM.

