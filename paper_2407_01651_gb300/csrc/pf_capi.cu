@@ -88,6 +88,7 @@ struct pf_handle {
   // the reductions (0 between them)
   unsigned int* d_err = nullptr;
   int* d_tile_ctr = nullptr;      // two tile counters of the one-launch mode
+  bool one_bc = false;            // few tiles with sides: one launch (upload_tables)
   int drop_copies = 0;            // testing only (pf_test_drop_staged_copies)
   double* staging = nullptr;    // FP64 device staging (largest domain x 39 planes)
   size_t staging_elems = 0;
@@ -512,6 +513,23 @@ static pf_status upload_tables(pf_handle* h) {
     if (g) { cudaGraphExecDestroy(g); g = nullptr; }
   cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device);
   h->grid = h->ntiles;  // one CTA per tile; the kernel also accepts fewer (grid-stride)
+  // Handles with sides take two launches a step, plain and edge tiles, on two
+  // streams.  Where the tiles are resident at once, one launch of the edge kernel
+  // (the plain one's values away from a side), chained like the periodic step, is
+  // ahead: us per step, two launches and one, FP32 walls 128^2 10.3 and 7.4,
+  // thermal, walls in y 200x400 14.4 and 13.5.  Edge tiles alone are one launch
+  // anyhow; chained they gain while there is one a SM (128^2), and beyond lose the
+  // even spread over the SMs (thermal 256^2 16.7 and 17.5).
+  h->one_bc = false;
+  if (h->any_bc)
+    return dispatch(h, [&](auto s_t, auto r_t) {
+      PF_TYPES(s_t, r_t);
+      const int sms = std::max(1, h->sms);
+      const int k = step_blocks_per_sm<S, R>(STEP_YMARCH, h->tx, h->ty, h->plane_stride,
+                                             h->thermal != 0, true);
+      h->one_bc = h->ntiles <= (h->n_plain > 0 ? sms * k : sms);
+      return PF_OK;
+    });
   return PF_OK;
 }
 
@@ -915,6 +933,8 @@ static pf_status launch_all(pf_handle* h, StepArgs<S, R> a, cudaStream_t stream)
   const int edge_kind = h->any_io ? 2 : 1;   // boundary kernel with or without inlet/outlet code
   pf_status st = PF_OK;
   if (h->any_bc) {
+    // few tiles: one launch of the boundary-aware kernel over all of them
+    if (h->one_bc && h->launch_mode == 0) return go1(0, h->ntiles, edge_kind);
     // plain tiles: the periodic kernel; edge tiles: the boundary-aware one, on
     // the side stream (both read the same state and write disjoint sites)
     if (h->launch_mode == 0) {
@@ -954,7 +974,7 @@ static pf_status launch_all(pf_handle* h, StepArgs<S, R> a, cudaStream_t stream)
 static int launches_per_step(const pf_handle* h) {
   if (!h->any_bc) return h->launch_mode == 0 ? 1 : (int)h->ddesc.size();
   int n = 0;
-  if (h->launch_mode == 0) return (h->n_plain > 0) + (h->ntiles > h->n_plain);
+  if (h->launch_mode == 0) return h->one_bc ? 1 : (h->n_plain > 0) + (h->ntiles > h->n_plain);
   for (size_t d = 0; d < h->ddesc.size(); ++d)
     n += (h->plain1[d] > h->plain0[d]) + (h->edge1[d] > h->edge0[d]);
   return n;
@@ -1112,7 +1132,8 @@ static pf_status step_n(pf_handle* h, int n_steps) {
   // a caller's capture, whose graph keeps plain edges
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   if (n_steps - done > 1) PF_CUDA(h, cudaStreamIsCapturing(h->stream, &cs));
-  const bool chain = cs == cudaStreamCaptureStatusNone && h->launch_mode == 0 && !h->any_bc;
+  const bool chain = cs == cudaStreamCaptureStatusNone && h->launch_mode == 0 &&
+                     (!h->any_bc || h->one_bc);
   for (bool behind = false; done < n_steps; ++done, behind = chain) {
     pf_status st = step_t<S, R>(h, done == n_steps - 1, nullptr, behind);
     if (st != PF_OK) return st;

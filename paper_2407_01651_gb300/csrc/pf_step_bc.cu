@@ -201,6 +201,7 @@ __global__ void __launch_bounds__(YM_THREADS, sizeof(R) == 4 ? 3 : 2)
   __shared__ R ring[NF][4][RW];
   const int t = threadIdx.x;
   const unsigned ps = (unsigned)a.plane_stride;
+  chain_step(a);
 
   for (int tile = a.tile_base + blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
     const DomDesc d = a.doms[a.tile_dom[tile]];
@@ -310,19 +311,20 @@ template <typename S, typename R>
 cudaError_t launch_ymarch_bc(const StepArgs<S, R>& a, bool big, int grid, cudaStream_t st) {
   if constexpr (sizeof(S) == sizeof(R)) {
     // a.bc: 1 boundary sides, 2 among them an inlet or an outlet
+    cudaError_t e = cudaSuccess;
     auto go = [&](auto io) {
       constexpr bool IO = decltype(io)::value;
       if (big) {
-        if (a.thermal) k_step_ymarch_bc<S, R, true, true, IO><<<grid, YM_THREADS, 0, st>>>(a);
-        else k_step_ymarch_bc<S, R, true, false, IO><<<grid, YM_THREADS, 0, st>>>(a);
+        if (a.thermal) e = launch_chained(k_step_ymarch_bc<S, R, true, true, IO>, a, grid, 0, st);
+        else e = launch_chained(k_step_ymarch_bc<S, R, true, false, IO>, a, grid, 0, st);
       } else {
-        if (a.thermal) k_step_ymarch_bc<S, R, false, true, IO><<<grid, YM_THREADS, 0, st>>>(a);
-        else k_step_ymarch_bc<S, R, false, false, IO><<<grid, YM_THREADS, 0, st>>>(a);
+        if (a.thermal) e = launch_chained(k_step_ymarch_bc<S, R, false, true, IO>, a, grid, 0, st);
+        else e = launch_chained(k_step_ymarch_bc<S, R, false, false, IO>, a, grid, 0, st);
       }
     };
     if (a.bc == 2) go(std::true_type{});
     else go(std::false_type{});
-    return cudaGetLastError();
+    return e;
   } else {
     return cudaErrorInvalidValue;   // boundaries need FP32 or FP64 storage (checked on the host)
   }
