@@ -210,9 +210,9 @@ pf_status pf_step(pf_handle *h, int n_steps);
  * domains' sizes, at most 32); variant 2 = the same strips with their input
  * rows staged in shared memory by bulk copies (b ignored; the default for
  * FP16/BF16 storage and, from 786,432 sites on, for FP32, a chosen by size, at
- * most 48; needs every
- * domain's nx to be a multiple of 16 bytes of storage: 4 FP32, 8 FP16/BF16,
- * 2 FP64 sites).  Synchronises the stream and rebuilds the tile table.
+ * most 48; by default a handle of fewer sites marches the strips unstaged, to the
+ * same bits; needs every domain's nx to be a multiple of 16 bytes of storage:
+ * 4 FP32, 8 FP16/BF16, 2 FP64 sites).  Synchronises the stream and rebuilds the tile table.
  * Errors: BAD_ARG. */
 pf_status pf_set_step_config(pf_handle *h, int variant, int a, int b);
 

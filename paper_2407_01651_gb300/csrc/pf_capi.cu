@@ -388,8 +388,8 @@ static void release(pf_handle* h) {
 // they end with the others (thermal, sides: 1024^2 at 18 rows 128, at 6 rows 107;
 // 2048^2 at 36 rows 371, at 12 rows 333).
 static int chunk_by_size(const pf_handle* h, int sms, int ctas_per_sm) {
-  const bool staged = h->variant == STEP_STAGED || h->staged_rows;
-  int top = h->variant == STEP_STAGED ? 48 : (staged ? 36 : 32);
+  const bool staged = h->staged_rows;
+  int top = !staged ? 32 : (h->variant == STEP_STAGED ? 48 : 36);
   if (h->any_bc) {
     double n = 0.0;
     for (const DomDesc& d : h->ddesc) n = std::max(n, (double)d.nx * d.ny);
@@ -419,26 +419,30 @@ static int chunk_by_size(const pf_handle* h, int sms, int ctas_per_sm) {
 }
 
 // The traversal that a step takes.  Where neither the caller nor the autotuner
-// set one, an FP32 y-march stages its rows by bulk copies (the same strips and
-// tiles, the same bits) if the widths allow it and there are sites enough: its
-// prologue fills the stages, so short tiles do not pay.  Measured, us per step
-// y-march / staged: 512^2 18.5 / 22.6, 1024^2 63.6 / 59.5, 2048^2 213 / 183,
-// 4096^2 820 / 677.  FP64 is bound by its arithmetic: 1024^2 1234 / 1261.
+// set one, the FP32 and 16-bit marches stage their rows by bulk copies (the same
+// strips and tiles, the same bits) if the widths allow it and there are sites
+// enough: the prologue fills the stages, so short tiles do not pay.  Measured, us
+// per step y-march / staged: FP32 512^2 18.5 / 22.6, 1024^2 63.6 / 59.5, 2048^2
+// 213 / 183, 4096^2 820 / 677; FP16 128^2 4.7 / 12.0, 256^2 7.7 / 12.6, 512^2 18.9
+// / 24.1, 768^2 34.9 / 37.0, 1024x768 50.7 / 47.4, 2048^2 214 / 197.  FP64 is bound
+// by its arithmetic: 1024^2 1234 / 1261.  Copies dropped by a test are those of
+// the staged march.
 constexpr long long STAGE_SITES = 3ll << 18;
 static StepVariant step_variant(const pf_handle* h) {
-  if (h->variant == STEP_YMARCH && h->staged_rows && !h->own_chunk && h->persistent != 2)
-    return STEP_STAGED;
-  return (StepVariant)h->variant;
+  if (h->own_chunk || h->persistent == 2 || h->variant == STEP_TILE)
+    return (StepVariant)h->variant;
+  if (h->variant == STEP_STAGED && h->drop_copies) return STEP_STAGED;
+  return h->staged_rows ? STEP_STAGED : STEP_YMARCH;
 }
 
 static pf_status choose_chunk(pf_handle* h) {
   if (h->own_chunk || h->variant == STEP_TILE) return PF_OK;
-  h->staged_rows = h->prec == PF_FP32 && h->plane_stride >= STAGE_SITES && staged_ok(h);
+  h->staged_rows = h->prec != PF_FP64 && h->plane_stride >= STAGE_SITES && staged_ok(h);
   int sms = 0;
   PF_CUDA(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
   return dispatch(h, [&](auto s_t, auto r_t) {
     PF_TYPES(s_t, r_t);
-    const int k = step_blocks_per_sm<S, R>(h->staged_rows ? STEP_STAGED : h->variant, h->tx, h->ty,
+    const int k = step_blocks_per_sm<S, R>(h->staged_rows ? STEP_STAGED : STEP_YMARCH, h->tx, h->ty,
                                            h->plane_stride, h->thermal != 0, h->any_bc != 0);
     h->chunk = chunk_by_size(h, std::max(1, sms), std::max(1, k));
     return PF_OK;
@@ -1241,7 +1245,7 @@ static pf_status autotune_t(pf_handle* h, int trial_steps, int out[4]) {
   struct Cand { int variant, a, b, persistent, own = 1; };
   std::vector<Cand> cands;
   const int own0 = h->own_chunk;
-  if (!own0 && h->staged_rows)
+  if (!own0)
     for (int pers : {0, 1}) cands.push_back({h->variant, h->chunk, 0, pers, 0});
   for (int ch : {4, 8, 16, 24, 32, 48, 64, 96})
     for (int pers : {0, 1}) cands.push_back({STEP_YMARCH, ch, 0, pers});
@@ -1321,7 +1325,8 @@ extern "C" pf_status pf_autotune(pf_handle* h, int trial_steps, int out[4]) {
 extern "C" pf_status pf_get_step_config(const pf_handle* h, int out[3]) {
   if (!h || !out) return PF_ERR_BAD_ARG;
   // what pf_set_step_config would take to run the same kernels
-  out[0] = !h->thermal && !h->any_bc ? (int)step_variant(h) : h->variant;
+  // (of a 16-bit march by size the staged form of it, also where it is small)
+  out[0] = !h->thermal && !h->any_bc && h->variant == STEP_YMARCH ? (int)step_variant(h) : h->variant;
   out[1] = h->variant != STEP_TILE ? h->chunk : h->tx;
   out[2] = h->variant == STEP_TILE ? h->ty : 0;
   return PF_OK;
