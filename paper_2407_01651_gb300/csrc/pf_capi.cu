@@ -1827,7 +1827,11 @@ static pf_status adjoint_t(pf_handle* h, int n, const pf_objective* obj, double*
   cudaStream_t A = h->stream;
   // x_0 may be a raw state: its step and its reverse take their own kernels
   const double* raw0 = h->raw[0];
-  auto forward = [&](const StepArgs<S, R>& a, int t, cudaStream_t sx) -> pf_status {
+  // (behind: the step before it is the stream's last operation; 512^2, 100 steps,
+  // K = 25: the call 9707 -> 9504 us.  The recomputed steps and the reverse
+  // kernels, which share the SMs, lose by it: 9877.)
+  auto forward = [&](StepArgs<S, R> a, int t, bool behind, cudaStream_t sx) -> pf_status {
+    a.chained = behind;
     if (t > 0 || !raw0) return launch_all<S, R>(h, a, sx);
     PF_CUDA(h, launch_step_general<S, R>(a, dd, raw0, sx));
     h->launches++;
@@ -1846,7 +1850,8 @@ static pf_status adjoint_t(pf_handle* h, int n, const pf_objective* obj, double*
                                  cudaMemcpyDeviceToDevice, A));
     }
     pf_status st = forward(make_step_args<S, R>(h, h->pop[h->cur], h->aux[h->cur],
-                                                h->pop[h->cur ^ 1], h->aux[h->cur ^ 1], false), t, A);
+                                                h->pop[h->cur ^ 1], h->aux[h->cur ^ 1], false), t,
+                           t % K != 0, A);
     if (st != PF_OK) return st;
     h->cur ^= 1;
     h->steps++;
@@ -1861,7 +1866,7 @@ static pf_status adjoint_t(pf_handle* h, int n, const pf_objective* obj, double*
       const StepArgs<S, R> a = make_step_args<S, R>(
           h, pop_of(bl[j]), aux_of(bl[j]), last ? h->pop[h->cur ^ 1] : pop_of(bl[j + 1]),
           last ? h->aux[h->cur ^ 1] : aux_of(bl[j + 1]), last);
-      pf_status sl = forward(a, t_last + j, A);
+      pf_status sl = forward(a, t_last + j, j > 0, A);
       if (sl != PF_OK) return sl;
     }
     h->cur ^= 1;
@@ -1889,7 +1894,7 @@ static pf_status adjoint_t(pf_handle* h, int n, const pf_objective* obj, double*
     for (int j = 0; j + 1 < K; ++j) {
       const StepArgs<S, R> a = make_step_args<S, R>(h, pop_of(b[j]), aux_of(b[j]),
                                                     pop_of(b[j + 1]), aux_of(b[j + 1]), false);
-      pf_status sl = forward(a, s * K + j, sx);
+      pf_status sl = forward(a, s * K + j, false, sx);
       if (sl != PF_OK) return sl;
     }
     return PF_OK;
