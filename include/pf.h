@@ -218,7 +218,8 @@ pf_status pf_set_step_config(pf_handle *h, int variant, int a, int b);
 
 /* How a step is launched over an ensemble of domains:
  *  per_domain = 0: one launch whose tile list spans every domain (default);
- *               1: one launch per domain, one after the other.
+ *               1: one launch per domain, one after the other (rows per tile chosen
+ *               by size are then those of a domain's own launch).
  *  persistent = 1: the grid is the device's resident CTAs of the step kernel,
  *               each looping over tiles; 0: one CTA per tile (default);
  *               2: as 1, and every step of a pf_step call in one cooperative

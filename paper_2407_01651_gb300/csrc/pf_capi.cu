@@ -398,17 +398,21 @@ static int chunk_by_size(const pf_handle* h, int sms, int ctas_per_sm) {
   const double warm = staged ? 3.0 : 2.0;
   double best = 0.0;
   int pick = top;
+  auto of = [&](long long tiles, int c) {      // a launch of so many tiles
+    if (h->prec == PF_FP64)
+      return (double)((tiles + sms - 1) / sms) * (5.6 * c + 2.0) * (tiles <= sms ? 1.13 : 1.0);
+    const double w = (double)tiles / ((double)sms * ctas_per_sm);
+    return (w > 4.0 ? w + 0.5 : std::ceil(w)) * (c + warm);
+  };
   for (int c = top; c >= 1; --c) {
-    long long tiles = 0;
-    for (const DomDesc& d : h->ddesc)
-      tiles += (long long)((d.nx + YM_W - 1) / YM_W) * ((d.ny + c - 1) / c);
-    double cost;
-    if (h->prec == PF_FP64) {
-      cost = (double)((tiles + sms - 1) / sms) * (5.6 * c + 2.0) * (tiles <= sms ? 1.13 : 1.0);
-    } else {
-      const double w = (double)tiles / ((double)sms * ctas_per_sm);
-      cost = (w > 4.0 ? w + 0.5 : std::ceil(w)) * (c + warm);
+    long long all = 0;
+    double cost = 0.0;
+    for (const DomDesc& d : h->ddesc) {
+      const long long tiles = (long long)((d.nx + YM_W - 1) / YM_W) * ((d.ny + c - 1) / c);
+      all += tiles;
+      if (h->launch_mode) cost += of(tiles, c);   // a launch per domain
     }
+    if (!h->launch_mode) cost = of(all, c);
     // shorter tiles only where they are clearly ahead: they pull more rows twice
     if (c == top || cost < 0.97 * best) {
       best = cost;
@@ -437,7 +441,12 @@ static StepVariant step_variant(const pf_handle* h) {
 
 static pf_status choose_chunk(pf_handle* h) {
   if (h->own_chunk || h->variant == STEP_TILE) return PF_OK;
-  h->staged_rows = h->prec != PF_FP64 && h->plane_stride >= STAGE_SITES && staged_ok(h);
+  long long sites = 0;   // of the largest launch
+  for (const DomDesc& d : h->ddesc) {
+    const long long n = (long long)d.nx * d.ny;
+    sites = h->launch_mode ? std::max(sites, n) : sites + n;
+  }
+  h->staged_rows = h->prec != PF_FP64 && sites >= STAGE_SITES && staged_ok(h);
   int sms = 0;
   PF_CUDA(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device));
   return dispatch(h, [&](auto s_t, auto r_t) {
@@ -1217,12 +1226,20 @@ extern "C" pf_status pf_set_launch(pf_handle* h, int per_domain, int persistent,
     }
   }
   PF_CUDA(h, cudaStreamSynchronize(h->stream));
+  const bool retile = h->launch_mode != per_domain;
   h->launch_mode = per_domain;
   h->persistent = persistent;
   h->graph_steps = graph_steps;
   h->coop_graph_failed = 0;
   for (auto& g : h->gexec)
     if (g) { cudaGraphExecDestroy(g); g = nullptr; }
+  // the tiles by size are those of a launch: 96 domains, 32 each of 256^2, 512x384
+  // and 1024x512, one launch per domain 3311 -> 11236 MLUPS against the whole list's
+  if (retile) {
+    const pf_status st = choose_chunk(h);
+    if (st != PF_OK) return st;
+    return upload_tables(h);
+  }
   return PF_OK;
 }
 
