@@ -36,23 +36,16 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 METRIC = "coupled-step MLUPS at 4096² and % of HBM roofline; adjoint/forward time ratio"
-# Algorithmic HBM bytes per lattice update of the step kernel: 39 planes read
-# + 39 planes written (9 NS, 9 CAC, 5+5+1 dendrite, 5 solute, 5 lagged scalars)
-# and 1 byte of grain id read.
-# The 16-bit forms store the 33 population planes in 2 bytes and keep 7 lagged
-# scalars (with psi) in FP32.
-BYTES_PER_LU = {"fp32": 39 * 4 * 2 + 1, "fp64": 39 * 8 * 2 + 1,
-                "fp16": (33 * 2 + 7 * 4) * 2 + 1, "bf16": (33 * 2 + 7 * 4) * 2 + 1}
+# HBM bytes per lattice update of the step kernel: 29 planes read and written (9
+# NS; of each opposite pair whose sum a density fixes one population: 4 CAC, 5
+# pre- and 3 post-collision dendrite, 2 solute; 6 lagged scalars) and 1 byte of
+# grain id read.  The 16-bit forms store the 23 population planes in 2 bytes and
+# keep 7 lagged scalars (with psi) in FP32.
+BYTES_PER_LU = {"fp32": 29 * 4 * 2 + 1, "fp64": 29 * 8 * 2 + 1,
+                "fp16": (23 * 2 + 7 * 4) * 2 + 1, "bf16": (23 * 2 + 7 * 4) * 2 + 1}
 DTYPE = {"fp32": "f32", "fp64": "f64", "fp16": "f16-storage/f32", "bf16": "bf16-storage/f32"}
-# The strict algorithmic bytes per lattice update of the coupled step: 28
-# populations and 6 temporal scalars read and written, and a 4-byte grain
-# angle read (FP32 276 B); populations in 16 bits with FP32 scalars about 164
-# B.  The library stores the time stretch's pre-collision populations and
-# 1/a_s^2 besides (BYTES_PER_LU): the roofline's achieved rate takes the strict
-# figure and the line also gives the fraction at the stored bytes.
-STRICT_BYTES_PER_LU = {"fp32": 276, "fp16": 164, "bf16": 164, "fp64": 2 * 276 - 4}
-# Thermal mode adds 5 temperature populations and the lagged H: 45 planes.
-BYTES_PER_LU_THERMAL = {"fp32": 45 * 4 * 2 + 1, "fp64": 45 * 8 * 2 + 1}
+# Thermal mode adds rho H, its pair base and 2 temperature populations: 33 planes.
+BYTES_PER_LU_THERMAL = {"fp32": 33 * 4 * 2 + 1, "fp64": 33 * 8 * 2 + 1}
 KERNEL_SOURCES = ("paper_2407_01651_gb300/csrc/pf_step.cu",
                   "paper_2407_01651_gb300/csrc/pf_device.cuh",
                   "paper_2407_01651_gb300/csrc/pf_model.cuh",
@@ -631,9 +624,9 @@ def run_ensemble(args) -> None:
                        "launch": "64 steps per persistent cooperative launch, graph replay",
                        "autotuned_one_launch": cfg_one,
                        "parallelism": f"domains sharded over {world} rank(s)",
-                       "l2": f"{313 * my_sites / 1e9:.1f} GB read+written per step > L2 "
+                       "l2": f"{BYTES_PER_LU['fp32'] * my_sites / 1e9:.1f} GB read+written per step > L2 "
                              "(no flush)"},
-            "roofline": roofline(STRICT_BYTES_PER_LU["fp32"], my_sites, ms / args.steps,
+            "roofline": roofline(BYTES_PER_LU["fp32"], my_sites, ms / args.steps,
                                  "k_step_ymarch_steps (64 steps per cooperative launch, every "
                                  "domain's tiles)", state_bpl=BYTES_PER_LU["fp32"]),
             "modes": res, "ms_per_step_modes": ms_mode,
@@ -691,7 +684,7 @@ def run_precision(args) -> None:
                    "lattice": [lay.nx, lay.ny], "precision": "fp16",
                    "l2": f"{(BYTES_PER_LU['fp16'] - 1) * sites / 1e9:.1f} GB read+written per "
                          "step > L2 (no flush)"},
-        "roofline": roofline(STRICT_BYTES_PER_LU["fp16"], sites, f16["ms_per_step"],
+        "roofline": roofline(BYTES_PER_LU["fp16"], sites, f16["ms_per_step"],
                              "k_step_staged<__half,float> (one launch per step)",
                              recorded_traffic("fp16", 4096) and
                              recorded_traffic("fp16", 4096) * sites / 4096 ** 2,
@@ -764,13 +757,13 @@ def _thermal_like(args, mode: str) -> None:
     h = res[runs[0][0]]
     if mode == "thermal":
         metric = "thermal coupled-step MLUPS at 4096² and % of HBM roofline"
-        kernel = "k_step_ymarch<thermal> (one launch per step)"
+        kernel = "k_step_staged<thermal> (one launch per step)"
         traffic = recorded_traffic(f"thermal_{prec}", args.size)
         extra = {"thermal_cost_vs_isothermal": res["isothermal"]["mlups"] / h["mlups"]}
         cfg = dict(workload_config(lay.nx, prec), thermal=wl.THERMAL_PARAMS)
     else:
         metric = "bounded thermal coupled-step MLUPS at 4096² and % of HBM roofline"
-        kernel = ("k_step_ymarch<thermal> on interior tiles + k_step_ymarch_bc<thermal> on edge "
+        kernel = ("k_step_staged<thermal> on interior tiles + k_step_ymarch_bc<thermal> on edge "
                   "tiles (side stream)")
         traffic = None
         extra = {}
@@ -797,9 +790,9 @@ def run_thermal(args) -> None:
 
 def run_3d(args) -> None:
     """The 3-D dendrite step (psi and C on D3Q7, no gas or flow) on a periodic
-    256^3 melt with 64 seeds: MLUPS and the HBM roofline at 184 B/LU (FP32: 23
+    256^3 melt with 64 seeds: MLUPS and the HBM roofline at 136 B/LU (FP32: 17
     planes read and written, g_pre[7], g_post[7], r, s[7], Q_psi); with the
-    temperature lattice ('3d_thermal') 240 B/LU (30 planes, e[7] added)."""
+    temperature lattice ('3d_thermal') 176 B/LU (22 planes, rho H, base and e[3] added)."""
     import torch
 
     from paper_2407_01651_gb300 import pf
@@ -825,7 +818,7 @@ def run_3d(args) -> None:
     launches = sim.launches - l0
     d = sim.reduce()
     sites = n ** 3
-    planes = 30 if thermal else 23
+    planes = 22 if thermal else 17
     bpl = planes * 2 * (4 if prec == "fp32" else 8)
     extra = {}
     if thermal:
@@ -1028,7 +1021,7 @@ def main() -> None:
     ms_per_step = ms_max / args.steps
     value = world * sites * args.steps / (ms_max / 1e3) / 1e6
     bpl = BYTES_PER_LU[args.precision]
-    roof = roofline(STRICT_BYTES_PER_LU[args.precision], sites, ms / args.steps,
+    roof = roofline(BYTES_PER_LU[args.precision], sites, ms / args.steps,
                     "k_step (one launch per step; average over the timed region)",
                     recorded_traffic(args.precision, args.size), state_bpl=bpl)
 
