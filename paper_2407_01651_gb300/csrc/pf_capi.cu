@@ -376,13 +376,14 @@ static void release(pf_handle* h) {
 // times: long tiles waste little on a large lattice, short ones are what fills
 // the chip on a small one.  Whole waves up to four; beyond that the CTAs run
 // out of step and only half a wave is lost at the end.  Measured (us per step at
-// 32 rows and at the rows chosen): FP32 128^2 43.1 -> 6.2 (1 row), 256^2 45.1 ->
-// 8.2 (1), 512^2 45.1 -> 18.5 (4); staged 1024^2 88.0 -> 55.3 (14), 2048^2 206 ->
-// 183 (27), 4096^2 679 -> 676 (36).
+// 32 rows and at the rows chosen, before steps were chained; now in brackets):
+// FP32 128^2 43.1 -> 6.2 (1 row) [4.4], 256^2 45.1 -> 8.2 (1) [7.0], 512^2 45.1 ->
+// 18.5 (4) [16.4]; staged 1024^2 88.0 -> 55.3 (14), 2048^2 206 -> 183 (27), 4096^2
+// 679 -> 676 (36).
 // FP64 is bound by the FP64 units, so there the SM with the most tiles sets the
 // time, a row costs its update (5.6 pulls' worth with its own pull) plus two
 // warm-up pulls per tile, and one tile alone leaves an SM's units idle for an
-// eighth of the time: 128^2 763 -> 38.9 (1 row), 512^2 804 -> 337 (7).
+// eighth of the time: 128^2 763 -> 38.9 (1 row) [35.3], 512^2 804 -> 337 (7) [323].
 // Tiles at a non-periodic side are several times slower per row and too few to
 // fill the chip: their height is held to a share of the lattice's side, so that
 // they end with the others (thermal, sides: 1024^2 at 18 rows 128, at 6 rows 107;
@@ -426,10 +427,10 @@ static int chunk_by_size(const pf_handle* h, int sms, int ctas_per_sm) {
 // set one, the FP32 and 16-bit marches stage their rows by bulk copies (the same
 // strips and tiles, the same bits) if the widths allow it and there are sites
 // enough: the prologue fills the stages, so short tiles do not pay.  Measured, us
-// per step y-march / staged: FP32 512^2 18.5 / 22.6, 1024^2 63.6 / 59.5, 2048^2
-// 213 / 183, 4096^2 820 / 677; FP16 128^2 4.7 / 12.0, 256^2 7.7 / 12.6, 512^2 18.9
-// / 24.1, 768^2 34.9 / 37.0, 1024x768 50.7 / 47.4, 2048^2 214 / 197.  FP64 is bound
-// by its arithmetic: 1024^2 1234 / 1261.  Copies dropped by a test are those of
+// per step y-march / staged: FP32 (before steps were chained) 512^2 18.5 / 22.6,
+// 1024^2 63.6 / 59.5, 2048^2 213 / 183, 4096^2 820 / 677; FP16 128^2 4.7 / 12.0,
+// 256^2 7.7 / 12.6, 512^2 18.9 / 24.1, 768^2 34.9 / 37.0, 1024x768 50.7 / 47.4,
+// 2048^2 214 / 197.  FP64 is bound by its arithmetic: 1024^2 1234 / 1261.  Copies dropped by a test are those of
 // the staged march.
 constexpr long long STAGE_SITES = 3ll << 18;
 static StepVariant step_variant(const pf_handle* h) {
