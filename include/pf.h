@@ -284,10 +284,13 @@ pf_status pf_run(pf_handle *h, const double *fields6, size_t n, int n_steps, uin
 /* Raw state of domain dom (pf_state_planes(h) planes, FP64) to / from the
  * host: checkpoint and restart.  Synchronise the stream.  pf_set_state marks
  * the domain initialised.  Its populations may be any: where they are not what
- * a step leaves behind (to a few ulp), the planes stay on the device in FP64
- * until the domain's next step, which starts from them.  Errors: BAD_ARG (domain, NULL, a buffer of the
- * wrong size: at least / exactly planes x nx x ny values), OOM (staging),
- * CUDA; pf_get_state also TIMEOUT (a staged step's wait ran out before the
+ * a step leaves behind (to a few ulp), 19 further planes of the domain (25 in
+ * thermal mode) in the storage type keep them on the device until its next
+ * step, which starts from them; the handle then holds no more than if each
+ * state copy had every population (thermal: one value a site more).  Errors:
+ * BAD_ARG (domain, NULL, a buffer of the wrong size: at least / exactly planes
+ * x nx x ny values), OOM (staging, those planes; the domain's state is then
+ * as it was), CUDA; pf_get_state also TIMEOUT (a staged step's wait ran out before the
  * call: the state is invalid), which pf_set_state clears. */
 pf_status pf_get_state(pf_handle *h, int dom, double *host_out, size_t n);
 pf_status pf_set_state(pf_handle *h, int dom, const double *host_in, size_t n);

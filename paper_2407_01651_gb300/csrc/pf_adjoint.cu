@@ -46,7 +46,7 @@ __device__ __forceinline__ local::Coef<R> make_coef(const KParams<R>& kp, const 
 }  // namespace
 
 // ---------------------------------------------------------------------------
-// RAW: x_t is a raw state (its pulls from a.raw; the first state after a
+// RAW: x_t is a raw state (pulls from a.tied too; the first state after a
 // pf_set_state of populations that no collision made).
 template <typename S, typename R, bool BIG, bool RAW>
 __global__ void __launch_bounds__(256, 2) k_adj_local(AdjArgs<S, R> a) {
@@ -59,20 +59,14 @@ __global__ void __launch_bounds__(256, 2) k_adj_local(AdjArgs<S, R> a) {
   const int tid = threadIdx.y * ADJ_TX + threadIdx.x;
   const int tiles_x = (d.nx + ADJ_TX - 1) / ADJ_TX;
   const int ntiles = tiles_x * ((d.ny + ADJ_TY - 1) / ADJ_TY);
-  const RawState<S, R> rs{a.raw, (long long)d.nx * d.ny};
-  const GeneralPull<S, R, false> raw{rs, st, d};
+  const GeneralPull<S, R, false> raw{a.tied, st, d};
   // streamed dendrite populations, phi, psi and the lagged velocity of a site
   auto pull = [&](const Src9& src, int x, int y, R (&g)[5], R& phi, R& psi, R& psio, R& vx, R& vy) {
     V2<R> J;
-    if constexpr (RAW) {
-      raw.hg(x, y, J, g, phi, psi, psio);
-      vx = rs.x(X_VX, raw.local(src.s[0]));
-      vy = rs.x(X_VY, raw.local(src.s[0]));
-    } else {
-      pull_hg<S, R, BIG>(st, src, J, g, phi, psi, psio);
-      vx = ld<R>(st.ain + A_VXO * ps, src.s[0]);
-      vy = ld<R>(st.ain + A_VYO * ps, src.s[0]);
-    }
+    if constexpr (RAW) raw.hg(x, y, J, g, phi, psi, psio);
+    else pull_hg<S, R, BIG>(st, src, J, g, phi, psi, psio);
+    vx = ld<R>(st.ain + A_VXO * ps, src.s[0]);
+    vy = ld<R>(st.ain + A_VYO * ps, src.s[0]);
   };
   R pe = R(0), po = R(0), psg = R(0);
   for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -379,7 +373,7 @@ __global__ void k_adj_omega_init(const R* __restrict__ L, const S* __restrict__ 
 // ---------------------------------------------------------------------------
 template <typename S, typename R>
 cudaError_t launch_adjoint_step(const AdjArgs<S, R>& a, int grid, cudaStream_t st) {
-  if (a.raw)
+  if (a.tied)
     k_adj_local<S, R, true, true><<<grid, dim3(ADJ_TX, ADJ_TY), 0, st>>>(a);
   else if ((unsigned long long)a.step.plane_stride * N_POP >= (1ull << 32))
     k_adj_local<S, R, true, false><<<grid, dim3(ADJ_TX, ADJ_TY), 0, st>>>(a);

@@ -84,18 +84,18 @@ struct pf_handle {
   int* d_tile_dom = nullptr;
   double* partial = nullptr;
   double* d_diag = nullptr;
-  // device error bits written by the step kernels, then the block counter of
-  // the reductions (0 between them)
+  // device error bits written by the step kernels, the block counter of the
+  // reductions (0 between them), the answer of launch_state_general
   unsigned int* d_err = nullptr;
   int* d_tile_ctr = nullptr;      // two tile counters of the one-launch mode
   bool one_bc = false;            // few tiles with sides: one launch (upload_tables)
   int drop_copies = 0;            // testing only (pf_test_drop_staged_copies)
   double* staging = nullptr;    // FP64 device staging (largest domain x 39 planes)
   size_t staging_elems = 0;
-  // raw FP64 planes of a domain whose state pf_set_state gave populations that
-  // no collision made (pf_step_general.cu), until its next step; else nullptr
-  std::vector<double*> raw;
-  std::vector<double*> spent;   // raw planes a step has consumed, freed at the next wait
+  // tied planes of a domain whose state pf_set_state gave populations that no
+  // collision made (pf_raw.cuh), until its next step; else nullptr
+  std::vector<void*> raw;
+  std::vector<void*> spent;   // tied planes a step has consumed, freed at the next wait
   long long steps = 0;
   long long launches = 0;
   std::string err;
@@ -269,18 +269,18 @@ static pf_status check_params(const pf_params* p) {
 template <typename R>
 static R* fields_ptr(pf_handle* h) { return reinterpret_cast<R*>(h->fields); }
 
-// The raw planes of a domain are not its state any more; work that reads them
+// The tied planes of a domain are not its state any more; work that reads them
 // may still be in the stream, so they are freed where the stream was waited for.
 static void drop_raw(pf_handle* h, int dom) {
   if (h->raw[dom]) h->spent.push_back(h->raw[dom]);
   h->raw[dom] = nullptr;
 }
 static void free_spent(pf_handle* h) {
-  for (double* r : h->spent) dev_free(h, r);
+  for (void* r : h->spent) dev_free(h, r);
   h->spent.clear();
 }
 static bool any_raw(const pf_handle* h) {
-  for (const double* r : h->raw)
+  for (const void* r : h->raw)
     if (r) return true;
   return false;
 }
@@ -347,8 +347,8 @@ static void release(pf_handle* h) {
   dev_free(h, h->d_tile_ctr);
   h->d_tile_ctr = nullptr;
   dev_free(h, h->staging);
-  for (double*& r : h->raw) { dev_free(h, r); r = nullptr; }
-  for (double* r : h->spent) dev_free(h, r);
+  for (void*& r : h->raw) { dev_free(h, r); r = nullptr; }
+  for (void* r : h->spent) dev_free(h, r);
   h->spent.clear();
   dev_free(h, h->adj_ws);
   h->adj_ws = nullptr;
@@ -640,13 +640,13 @@ extern "C" pf_status pf_create(const pf_params* p, const pf_domain* doms, int n_
   h->d_doms = (DomDesc*)dev_alloc(h, (size_t)n_doms * sizeof(DomDesc));
   h->partial = (double*)dev_alloc(h, (size_t)REDUCE_BLOCKS * NDIAG * sizeof(double));
   h->d_diag = (double*)dev_alloc(h, (NDIAG + 1) * sizeof(double));
-  h->d_err = (unsigned int*)dev_alloc(h, 2 * sizeof(unsigned int));
+  h->d_err = (unsigned int*)dev_alloc(h, 3 * sizeof(unsigned int));
   (void)max_n;
   if (!h->fields || !h->grain || !h->grain_cs || !h->d_doms || !h->partial || !h->d_diag ||
       !h->d_err)
     return bail(PF_ERR_OOM, "device allocation failed");
   if (cudaMemsetAsync(h->fields, 0, ps * N_FIELDS * h->celem, h->stream) != cudaSuccess ||
-      cudaMemsetAsync(h->d_err, 0, 2 * sizeof(unsigned int), h->stream) != cudaSuccess ||
+      cudaMemsetAsync(h->d_err, 0, 3 * sizeof(unsigned int), h->stream) != cudaSuccess ||
       cudaMemsetAsync(h->grain, 0, ps, h->stream) != cudaSuccess)
     return bail(PF_ERR_CUDA, "memset failed");
   for (int d = 0; d < n_doms; ++d)
@@ -784,14 +784,13 @@ extern "C" pf_status pf_init_fields(pf_handle* h, int dom, const pf_init_spec* s
     if (!std::isfinite(spec->bubbles[i])) return fail(h, PF_ERR_BAD_ARG, "non-finite bubble");
   std::vector<double> angles;
   for (int s = 0; s < spec->n_seeds; ++s) angles.push_back(spec->seeds[3 * s + 2]);
-  drop_raw(h, dom);
-  pf_status st = clear_device_error(h);
-  if (st != PF_OK) return st;
-  st = upload_grain_table(h, dom, angles);
-  if (st != PF_OK) return st;
   const size_t ns = 3 * (size_t)spec->n_seeds, nb = 3 * (size_t)spec->n_bubbles;
   double* buf = (double*)dev_alloc(h, (ns + nb + 1) * sizeof(double));
   if (!buf) return fail(h, PF_ERR_OOM, "init buffer allocation failed");
+  pf_status st = clear_device_error(h);
+  if (st == PF_OK) st = upload_grain_table(h, dom, angles);
+  if (st != PF_OK) { dev_free(h, buf); return st; }
+  drop_raw(h, dom);
   if (ns) PF_CUDA(h, cudaMemcpyAsync(buf, spec->seeds, ns * sizeof(double), cudaMemcpyHostToDevice, h->stream));
   if (nb) PF_CUDA(h, cudaMemcpyAsync(buf + ns, spec->bubbles, nb * sizeof(double), cudaMemcpyHostToDevice, h->stream));
   st = dispatch(h, [&](auto s_t, auto r_t) {
@@ -853,15 +852,16 @@ extern "C" pf_status pf_set_fields(pf_handle* h, int dom, const double* fields6,
       ids[i] = (uint8_t)it->second;
     }
   }
-  drop_raw(h, dom);
-  pf_status st = clear_device_error(h);
+  // page-locked fields are read by the kernel in place; others are staged (the
+  // allocation that may fail before the first change)
+  const double* direct = static_cast<const double*>(host_device_view(fields6));
+  pf_status st = ensure_staging(h, (direct ? 0 : 6 * nn) + (theta ? (nn + 7) / 8 : 0));
+  if (st != PF_OK) return st;
+  st = clear_device_error(h);
   if (st != PF_OK) return st;
   st = upload_grain_table(h, dom, angles);
   if (st != PF_OK) return st;
-  // page-locked fields are read by the kernel in place; others are staged
-  const double* direct = static_cast<const double*>(host_device_view(fields6));
-  st = ensure_staging(h, (direct ? 0 : 6 * nn) + (theta ? (nn + 7) / 8 : 0));
-  if (st != PF_OK) return st;
+  drop_raw(h, dom);
   const double* buf = direct ? direct : h->staging;
   uint8_t* d_ids = nullptr;
   if (!direct)
@@ -1034,7 +1034,7 @@ static pf_status step_t(pf_handle* h, bool write_fields, cudaStream_t stream = n
 }
 
 // The step after a pf_set_state of populations that no collision made: those
-// domains from their raw planes, the others as ever, one launch per domain.
+// domains with their tied planes, the others as ever, one launch per domain.
 template <typename S, typename R>
 static pf_status step_general_t(pf_handle* h, bool write_fields) {
   const StepArgs<S, R> a0 = make_step_args<S, R>(h, h->pop[h->cur], h->aux[h->cur],
@@ -1054,7 +1054,7 @@ static pf_status step_general_t(pf_handle* h, bool write_fields) {
   for (size_t d = 0; d < h->ddesc.size(); ++d) {
     pf_status st;
     if (h->raw[d]) {
-      PF_CUDA(h, launch_step_general<S, R>(a0, h->ddesc[d], h->raw[d], h->stream));
+      PF_CUDA(h, launch_step_general<S, R>(a0, h->ddesc[d], (const S*)h->raw[d], h->stream));
       h->launches++;
     } else if (h->any_bc) {
       if ((st = go(h->plain0[d], h->plain1[d], 0)) != PF_OK) return st;
@@ -1591,14 +1591,10 @@ extern "C" pf_status pf_get_state(pf_handle* h, int dom, double* host_out, size_
   if (st != PF_OK) return st;
   st = dispatch(h, [&](auto s_t, auto r_t) {
     PF_TYPES(s_t, r_t);
-    if (h->raw[dom])
-      PF_CUDA(h, launch_raw_rounded<S, R>(h->raw[dom], (long long)nn, (int)np, h->staging,
-                                          h->stream));
-    else
-      PF_CUDA(h, launch_state_to_f64<S, R>((const S*)h->pop[h->cur], (const R*)h->aux[h->cur],
-                                           h->plane_stride, dd.off, (long long)nn, h->staging,
-                                           h->thermal, h->p.rho_g, h->p.rho_l - h->p.rho_g,
-                                           h->stream));
+    PF_CUDA(h, launch_state_to_f64<S, R>((const S*)h->pop[h->cur], (const R*)h->aux[h->cur],
+                                         h->plane_stride, dd.off, (long long)nn, h->staging,
+                                         h->thermal, h->p.rho_g, h->p.rho_l - h->p.rho_g,
+                                         (const S*)h->raw[dom], h->stream));
     return PF_OK;
   });
   if (st != PF_OK) return st;
@@ -1617,33 +1613,37 @@ extern "C" pf_status pf_set_state(pf_handle* h, int dom, const double* host_in, 
   const size_t np = (size_t)h->n_phys;
   if (n != nn * np)
     return fail(h, PF_ERR_BAD_ARG, "input must hold pf_state_planes(h) planes of nx*ny");
-  drop_raw(h, dom);
-  pf_status st = clear_device_error(h);
-  if (st != PF_OK) return st;
-  st = ensure_staging(h, nn * np);
+  // everything that can run out of memory comes before the first change
+  pf_status st = ensure_staging(h, nn * np);
   if (st != PF_OK) return st;
   PF_CUDA(h, cudaMemcpyAsync(h->staging, host_in, nn * np * sizeof(double),
                              cudaMemcpyHostToDevice, h->stream));
+  PF_CUDA(h, cudaMemsetAsync(h->d_err + 2, 0, sizeof(unsigned int), h->stream));
+  const double drho = h->p.rho_l - h->p.rho_g;
+  PF_CUDA(h, h->celem == 8 ? launch_state_general<double>((long long)nn, h->staging, h->thermal,
+                                                          h->p.rho_g, drho, h->d_err + 2, h->stream)
+                           : launch_state_general<float>((long long)nn, h->staging, h->thermal,
+                                                         h->p.rho_g, drho, h->d_err + 2, h->stream));
+  unsigned int general = 0;
+  PF_CUDA(h, cudaMemcpyAsync(&general, h->d_err + 2, sizeof(general), cudaMemcpyDeviceToHost, h->stream));
+  PF_CUDA(h, cudaStreamSynchronize(h->stream));
+  if (general && !h->raw[dom]) {
+    h->raw[dom] = dev_alloc(h, nn * (h->thermal ? N_TIED_TH : N_TIED) * h->elem);
+    if (!h->raw[dom]) return fail(h, PF_ERR_OOM, "allocation of the state's tied planes failed");
+  } else if (!general) {
+    drop_raw(h, dom);
+  }
+  if ((st = clear_device_error(h)) != PF_OK) return st;
   st = dispatch(h, [&](auto s_t, auto r_t) {
     PF_TYPES(s_t, r_t);
     PF_CUDA(h, launch_state_from_f64<S, R>((S*)h->pop[h->cur], (R*)h->aux[h->cur],
                                            h->plane_stride, dd.off, (long long)nn, h->staging,
-                                           h->thermal, h->p.rho_g, h->p.rho_l - h->p.rho_g,
-                                           h->d_err, h->stream));
+                                           h->thermal, (S*)h->raw[dom], h->stream));
     return PF_OK;
   });
   if (st != PF_OK) return st;
-  h->launches++;
-  unsigned int bits = 0;
-  PF_CUDA(h, cudaMemcpyAsync(&bits, h->d_err, sizeof(bits), cudaMemcpyDeviceToHost, h->stream));
+  h->launches += 2;
   PF_CUDA(h, cudaStreamSynchronize(h->stream));
-  if (bits & ERR_GENERAL_STATE) {
-    // the staged planes are the domain's state until its next step
-    h->raw[dom] = h->staging;
-    h->staging = nullptr;
-    h->staging_elems = 0;
-    if ((st = clear_device_error(h)) != PF_OK) return st;
-  }
   h->inited[dom] = 1;
   return PF_OK;
 }
@@ -1748,9 +1748,10 @@ extern "C" pf_status pf_set_temperature(pf_handle* h, int dom, const double* the
                                             fields_ptr<R>(h), h->plane_stride, dd, h->staging,
                                             make_kparams<R>(h->p), h->stream));
     if (h->raw[dom]) {
-      PF_CUDA(h, launch_raw_temperature<S, R>((const S*)h->pop[h->cur], (const R*)h->aux[h->cur],
-                                              h->plane_stride, dd.off, (long long)nn, h->raw[dom],
-                                              h->p.rho_g, h->p.rho_l - h->p.rho_g, h->stream));
+      PF_CUDA(h, launch_tied_temperature<S, R>((const S*)h->pop[h->cur], (const R*)h->aux[h->cur],
+                                               h->plane_stride, dd.off, (long long)nn,
+                                               (S*)h->raw[dom], h->p.rho_g,
+                                               h->p.rho_l - h->p.rho_g, h->stream));
       h->launches++;
     }
     return PF_OK;
@@ -1770,7 +1771,8 @@ extern "C" pf_status pf_reduce_thermal(pf_handle* h, int dom, double out[3]) {
   pf_status st = dispatch(h, [&](auto s_t, auto r_t) {
     PF_TYPES(s_t, r_t);
     PF_CUDA(h, launch_reduce_thermal<S, R>((const S*)h->pop[h->cur], fields_ptr<R>(h),
-                                           h->plane_stride, dd, h->raw[dom], h->partial, h->d_diag,
+                                           h->plane_stride, dd, (const S*)h->raw[dom], h->partial,
+                                           h->d_diag,
                                            h->d_err + 1, h->d_err, h->stream));
     return PF_OK;
   });
@@ -1844,7 +1846,7 @@ static pf_status adjoint_t(pf_handle* h, int n, const pf_objective* obj, double*
   const bool fresh = h->steps == 0;
   cudaStream_t A = h->stream;
   // x_0 may be a raw state: its step and its reverse take their own kernels
-  const double* raw0 = h->raw[0];
+  const S* raw0 = (const S*)h->raw[0];
   // (behind: the step before it is the stream's last operation; 512^2, 100 steps,
   // K = 25: the call 9707 -> 9504 us.  The recomputed steps and the reverse
   // kernels, which share the SMs, lose by it: 9877.)
@@ -1932,7 +1934,7 @@ static pf_status adjoint_t(pf_handle* h, int n, const pf_objective* obj, double*
       aa.ai = ai;
       aa.partial = partial;
       aa.dfs_dsigma = dfs;
-      aa.raw = t0 + j == 0 ? raw0 : nullptr;
+      aa.tied = t0 + j == 0 ? raw0 : nullptr;
       PF_CUDA(h, launch_adjoint_step<S, R>(aa, grid, A));
       h->launches += ADJ_LAUNCHES_PER_STEP;
       cl ^= 1;

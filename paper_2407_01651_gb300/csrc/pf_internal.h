@@ -86,7 +86,6 @@ struct SetFieldsArgs {
 // Device error bits (pf_handle::d_err).
 constexpr unsigned int ERR_STAGED_TIMEOUT = 1u;   // a staged bulk copy did not complete
 constexpr unsigned int ERR_NONFINITE_INPUT = 2u;  // pf_set_fields met a non-finite value
-constexpr unsigned int ERR_GENERAL_STATE = 4u;    // pf_set_state: not a collision's output
 
 template <typename R>
 struct ReduceArgs {
@@ -148,27 +147,27 @@ cudaError_t launch_set_fields(const SetFieldsArgs<S, R>& a, cudaStream_t st);
 // *flag = 1 if any of the n device values at p is NaN or infinite, else 0.
 cudaError_t launch_flag_nonfinite(const double* p, long long n, unsigned int* flag,
                                   cudaStream_t st);
+// tied: the domain's tied planes (pf_raw.cuh), or nullptr.
 template <typename S, typename R>
 cudaError_t launch_state_to_f64(const S* pin, const R* ain, long long ps, long long off,
                                 long long n, double* out, int thermal, double rho_g, double drho,
-                                cudaStream_t st);
+                                const S* tied, cudaStream_t st);
 template <typename S, typename R>
 cudaError_t launch_state_from_f64(S* pout, R* aout, long long ps, long long off, long long n,
-                                  const double* in, int thermal, double rho_g, double drho,
-                                  unsigned int* err, cudaStream_t st);
-// One step of a domain from raw FP64 planes, whatever their populations.
+                                  const double* in, int thermal, S* tied, cudaStream_t st);
+// Sets *general where raw FP64 planes are not a collision's output.
+template <typename R>
+cudaError_t launch_state_general(long long n, const double* in, int thermal, double rho_g,
+                                 double drho, unsigned int* general, cudaStream_t st);
+// One step of a domain from a raw state, whatever its populations.
 template <typename S, typename R>
-cudaError_t launch_step_general(const StepArgs<S, R>& a, const DomDesc& d, const double* raw,
+cudaError_t launch_step_general(const StepArgs<S, R>& a, const DomDesc& d, const S* tied,
                                 cudaStream_t st);
-// Raw planes: their temperature planes from the stored state; rounded to the
-// storage form.
+// The temperature planes of the tied ones from the stored state.
 template <typename S, typename R>
-cudaError_t launch_raw_temperature(const S* pin, const R* ain, long long ps, long long off,
-                                   long long n, double* raw, double rho_g, double drho,
-                                   cudaStream_t st);
-template <typename S, typename R>
-cudaError_t launch_raw_rounded(const double* raw, long long n, int planes, double* out,
-                               cudaStream_t st);
+cudaError_t launch_tied_temperature(const S* pin, const R* ain, long long ps, long long off,
+                                    long long n, S* tied, double rho_g, double drho,
+                                    cudaStream_t st);
 // Thermal mode: temperature lattice at equilibrium for a theta field (device,
 // n of the domain), and the FP64 totals (sum e, sum theta, sum psi).
 template <typename S, typename R>
@@ -176,7 +175,7 @@ cudaError_t launch_set_temperature(S* out, R* aout, R* fields, long long ps, con
                                    const double* theta, const KParams<R>& kp, cudaStream_t st);
 template <typename S, typename R>
 cudaError_t launch_reduce_thermal(const S* pop, const R* fields, long long ps, const DomDesc& d,
-                                  const double* raw, double* partial, double* out, unsigned int* ctr,
+                                  const S* tied, double* partial, double* out, unsigned int* ctr,
                                   const unsigned int* err, cudaStream_t st);
 template <typename R>
 cudaError_t launch_fields_to_f64(const R* fields, long long ps, long long off, long long n,
@@ -219,7 +218,7 @@ struct AdjArgs {
   R* lam_out;              // lambda_t, 39 planes
   R* ai;                   // input adjoints, N_AI planes
   double* partial;         // per-block parameter adjoints (eps, Omega, sigma), accumulated
-  const double* raw;       // x_t as raw FP64 planes (pf_step_general.cu), or nullptr
+  const S* tied;           // x_t is a raw state: its tied planes (pf_raw.cuh), or nullptr
   double dfs_dsigma;       // d(surface-tension coefficient)/d sigma
 };
 

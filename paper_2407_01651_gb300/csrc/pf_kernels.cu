@@ -210,10 +210,12 @@ __device__ __forceinline__ double sum_pairs5(const double (&v)[5]) {
 }
 __device__ __forceinline__ double sum5(const double (&v)[5]) { return sum_pairs5(v) + v[0]; }
 
+// tied: the populations of the pair-stored lattices are those of the tied planes
+// (a raw state), else those the pairs stand for.
 template <typename S, typename R>
 __global__ void k_state_to_f64(const S* __restrict__ pin, const R* __restrict__ ain, long long ps,
                                long long off, long long n, double* __restrict__ out,
-                               int thermal, double rho_g, double drho) {
+                               int thermal, double rho_g, double drho, const S* __restrict__ tied) {
   constexpr bool offs = Codec<S>::kOffset;
   for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n;
        j += (long long)gridDim.x * blockDim.x) {
@@ -229,6 +231,27 @@ __global__ void k_state_to_f64(const S* __restrict__ pin, const R* __restrict__ 
     const R phio = ain[A_PHIO * ps + s], Co = ain[A_CO * ps + s];
     const R psio = offs ? ain[A_PSIO * ps + s] : R(0);
     for (int i = 0; i < 9; ++i) out[(X_F + i) * n + j] = (double)pop_ns<S, R>(pin + (P_F + i) * ps, s);
+    for (int i = 0; i < 5; ++i)
+      out[(X_GPRE + i) * n + j] = (double)pop_off<S, R>(pin + (P_GPRE + i) * ps, s, w5<R>(i) * psio);
+    out[X_RR * n + j] = (double)ain[A_RR * ps + s];
+    out[X_PHI * n + j] = (double)phio;
+    out[X_C * n + j] = (double)Co;
+    out[X_VX * n + j] = (double)ain[A_VXO * ps + s];
+    out[X_VY * n + j] = (double)ain[A_VYO * ps + s];
+    out[X_Q * n + j] = (double)ain[A_QO * ps + s];
+    if (tied) {
+      auto off_of = [&](int k, R wm) { return (double)dec_off<S, R>(tied[k * n + j], wm); };
+      for (int i = 0; i < 9; ++i) out[(X_H + i) * n + j] = off_of(T_H + i, w9<R>(i) * phio);
+      for (int i = 0; i < 5; ++i) {
+        out[(X_GPOST + i) * n + j] = off_of(T_GPOST + i, w5<R>(i) * psio);
+        out[(X_S + i) * n + j] = off_of(T_S + i, w5<R>(i) * Co);
+      }
+      if (thermal) {
+        for (int i = 0; i < 5; ++i) out[(X_E + i) * n + j] = (double)(R)tied[(T_E + i) * n + j];
+        out[X_HO * n + j] = (double)(R)tied[T_HO * n + j];
+      }
+      continue;
+    }
     const CacBase<R> b(phio);
     out[X_H * n + j] = (double)b.rest(phio);
     for (int i = 1; i < 9; ++i) {
@@ -236,8 +259,6 @@ __global__ void k_state_to_f64(const S* __restrict__ pin, const R* __restrict__ 
       const S v = pop(P_H + pair9(i));
       out[(X_H + i) * n + j] = minus9(i) ? minus(v, base) : plus(v, base);
     }
-    for (int i = 0; i < 5; ++i)
-      out[(X_GPRE + i) * n + j] = (double)pop_off<S, R>(pin + (P_GPRE + i) * ps, s, w5<R>(i) * psio);
     {
       // density m; in the offset forms psi_o + F with F/6 in the first plane
       const double f6 = offs ? (double)dec_off<S, R>(pop(P_GPOST), R(0)) : 0.0;
@@ -261,12 +282,6 @@ __global__ void k_state_to_f64(const S* __restrict__ pin, const R* __restrict__ 
         out[(X_S + i + 2) * n + j] = minus(v, base);
       }
     }
-    out[X_RR * n + j] = (double)ain[A_RR * ps + s];
-    out[X_PHI * n + j] = (double)phio;
-    out[X_C * n + j] = (double)Co;
-    out[X_VX * n + j] = (double)ain[A_VXO * ps + s];
-    out[X_VY * n + j] = (double)ain[A_VYO * ps + s];
-    out[X_Q * n + j] = (double)ain[A_QO * ps + s];
     if (thermal) {
       const R m = Codec<S>::template dec<R>(pop(P_E)), base = Codec<S>::template dec<R>(pop(P_E + 1));
       double e[5];
@@ -281,20 +296,69 @@ __global__ void k_state_to_f64(const S* __restrict__ pin, const R* __restrict__ 
   }
 }
 
-// Sets ERR_GENERAL_STATE where the populations are not a collision's output to
-// rounding (4 ulp of the pair's size in FP32 arithmetic, 16 in FP64): the step
-// that follows then starts from the raw planes (pf_step_general.cu).
-template <typename S, typename R>
-__global__ void k_state_from_f64(S* __restrict__ pout, R* __restrict__ aout, long long ps,
-                                 long long off, long long n, const double* __restrict__ in,
-                                 int thermal, double rho_g, double drho, unsigned int* err) {
+// Sets *flag where the populations are not a collision's output to rounding (4
+// ulp of the pair's size in FP32 arithmetic, 16 in FP64): the state is then kept
+// with all of them (pf_raw.cuh).
+template <typename R>
+__global__ void k_state_general(long long n, const double* __restrict__ in, int thermal,
+                                double rho_g, double drho, unsigned int* flag) {
   constexpr double tol = sizeof(R) == 8 ? 16.0 * 2.220446049250313e-16 : 4.0 * 1.1920928955078125e-7;
-  constexpr bool offs = Codec<S>::kOffset;
   bool general = false;
   // a and b are equal to rounding on the scale of their parts
   auto same = [&](double a, double b, double size) {
     if (!(fabs(a - b) <= tol * size)) general = true;
   };
+  for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n;
+       j += (long long)gridDim.x * blockDim.x) {
+    auto x = [&](int k) { return in[k * n + j]; };
+    const R phio = (R)x(X_PHI), Co = (R)x(X_C);
+    {
+      const CacBase<R> b(phio);
+      double size = fabs(x(X_PHI));
+      for (int i = 0; i < 9; ++i) size = fmax(size, fabs(x(X_H + i)));
+      same(x(X_H), (double)b.rest(phio), size);
+      for (int i : {1, 2, 5, 6})
+        same(x(X_H + i) + x(X_H + i + 2), 2.0 * (double)(i < 5 ? b.axis : b.diag()), size);
+    }
+    {
+      double g[5], size = 0.0;
+      for (int i = 0; i < 5; ++i) {
+        g[i] = x(X_GPOST + i);
+        size = fmax(size, fabs(g[i]));
+      }
+      const double m = sum5(g);
+      same(g[1] + g[3], m / 3.0, 2.0 * size);
+      same(g[2] + g[4], m / 3.0, 2.0 * size);
+    }
+    {
+      const R base = q5_base(Co);
+      double size = fabs(x(X_C));
+      for (int i = 0; i < 5; ++i) size = fmax(size, fabs(x(X_S + i)));
+      same(x(X_S), (double)q5_rest(Co, base), size);
+      for (int i = 1; i < 3; ++i) same(x(X_S + i) + x(X_S + i + 2), 2.0 * (double)base, size);
+    }
+    if (thermal) {
+      double e[5], size = 0.0;
+      for (int i = 0; i < 5; ++i) {
+        e[i] = x(X_E + i);
+        size = fmax(size, fabs(e[i]));
+      }
+      const double md = sum5(e), rhoH = (rho_g + x(X_PHI) * drho) * x(X_HO);
+      const R m = (R)md, b = round_to_multiple((R)(0.5 * (e[1] + e[3])), quantum_quarter_ulp(m));
+      same(e[1] + e[3], 2.0 * (double)b, 2.0 * size);
+      same(e[2] + e[4], 2.0 * (double)b, 2.0 * size);
+      same(md, rhoH, 2.0 * size);
+    }
+  }
+  if (general) atomicOr(flag, 1u);
+}
+
+// tied: also the tied planes of a raw state.
+template <typename S, typename R>
+__global__ void k_state_from_f64(S* __restrict__ pout, R* __restrict__ aout, long long ps,
+                                 long long off, long long n, const double* __restrict__ in,
+                                 int thermal, S* __restrict__ tied) {
+  constexpr bool offs = Codec<S>::kOffset;
   for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n;
        j += (long long)gridDim.x * blockDim.x) {
     const long long s = off + j;
@@ -309,26 +373,14 @@ __global__ void k_state_from_f64(S* __restrict__ pout, R* __restrict__ aout, lon
     for (int i = 0; i < 9; ++i) st_ns<S, R>(pout + (P_F + i) * ps, s, (R)x(X_F + i));
     {
       const CacBase<R> b(phio);
-      double size = fabs(x(X_PHI));
-      for (int i = 0; i < 9; ++i) size = fmax(size, fabs(x(X_H + i)));
-      same(x(X_H), (double)b.rest(phio), size);
-      for (int i : {1, 2, 5, 6}) {
-        const R base = i < 5 ? b.axis : b.diag();
-        same(x(X_H + i) + x(X_H + i + 2), 2.0 * (double)base, size);
-        put(P_H + pair9(i), x(X_H + i), base);
-      }
+      for (int i : {1, 2, 5, 6}) put(P_H + pair9(i), x(X_H + i), i < 5 ? b.axis : b.diag());
     }
     for (int i = 0; i < 5; ++i)
       st_off<S, R>(pout + (P_GPRE + i) * ps, s, (R)x(X_GPRE + i), w5<R>(i) * psio);
     {
-      double g[5], size = 0.0;
-      for (int i = 0; i < 5; ++i) {
-        g[i] = x(X_GPOST + i);
-        size = fmax(size, fabs(g[i]));
-      }
+      double g[5];
+      for (int i = 0; i < 5; ++i) g[i] = x(X_GPOST + i);
       const double m = sum5(g);
-      same(g[1] + g[3], m / 3.0, 2.0 * size);
-      same(g[2] + g[4], m / 3.0, 2.0 * size);
       if constexpr (offs) {
         const R base = q5_base(psio);
         pout[P_GPOST * ps + s] = enc_off<S, R>((R)((m - (double)psio) / 6.0), R(0));
@@ -340,16 +392,7 @@ __global__ void k_state_from_f64(S* __restrict__ pout, R* __restrict__ aout, lon
         put(P_GPOST + 2, g[2], R(0));
       }
     }
-    {
-      const R base = q5_base(Co);
-      double size = fabs(x(X_C));
-      for (int i = 0; i < 5; ++i) size = fmax(size, fabs(x(X_S + i)));
-      same(x(X_S), (double)q5_rest(Co, base), size);
-      for (int i = 1; i < 3; ++i) {
-        same(x(X_S + i) + x(X_S + i + 2), 2.0 * (double)base, size);
-        put(P_S + i - 1, x(X_S + i), base);
-      }
-    }
+    for (int i = 1; i < 3; ++i) put(P_S + i - 1, x(X_S + i), q5_base(Co));
     aout[A_RR * ps + s] = (R)x(X_RR);
     aout[A_PHIO * ps + s] = phio;
     aout[A_CO * ps + s] = Co;
@@ -358,69 +401,45 @@ __global__ void k_state_from_f64(S* __restrict__ pout, R* __restrict__ aout, lon
     aout[A_QO * ps + s] = (R)x(X_Q);
     if constexpr (offs) aout[A_PSIO * ps + s] = psio;
     if (thermal) {
-      double e[5], size = 0.0;
-      for (int i = 0; i < 5; ++i) {
-        e[i] = x(X_E + i);
-        size = fmax(size, fabs(e[i]));
-      }
-      const double md = sum5(e), rhoH = (rho_g + x(X_PHI) * drho) * x(X_HO);
-      const R m = (R)md, b = round_to_multiple((R)(0.5 * (e[1] + e[3])), quantum_quarter_ulp(m));
-      same(e[1] + e[3], 2.0 * (double)b, 2.0 * size);
-      same(e[2] + e[4], 2.0 * (double)b, 2.0 * size);
-      same(md, rhoH, 2.0 * size);
+      double e[5];
+      for (int i = 0; i < 5; ++i) e[i] = x(X_E + i);
+      const R m = (R)sum5(e);
       st<S, R>(pout + (P_E + 0) * ps, s, m);
-      st<S, R>(pout + (P_E + 1) * ps, s, b);
+      st<S, R>(pout + (P_E + 1) * ps, s,
+               round_to_multiple((R)(0.5 * (e[1] + e[3])), quantum_quarter_ulp(m)));
       st<S, R>(pout + (P_E + 2) * ps, s, (R)e[1]);
       st<S, R>(pout + (P_E + 3) * ps, s, (R)e[2]);
     }
+    if (!tied) continue;
+    for (int i = 0; i < 9; ++i) tied[(T_H + i) * n + j] = enc_off<S, R>((R)x(X_H + i), w9<R>(i) * phio);
+    for (int i = 0; i < 5; ++i) {
+      tied[(T_GPOST + i) * n + j] = enc_off<S, R>((R)x(X_GPOST + i), w5<R>(i) * psio);
+      tied[(T_S + i) * n + j] = enc_off<S, R>((R)x(X_S + i), w5<R>(i) * Co);
+    }
+    if (thermal) {
+      for (int i = 0; i < 5; ++i) st<S, R>(tied + (T_E + i) * n, j, (R)x(X_E + i));
+      st<S, R>(tied + T_HO * n, j, (R)x(X_HO));
+    }
   }
-  if (general) atomicOr(err, ERR_GENERAL_STATE);
 }
 
-// The temperature planes of a raw state from the stored ones (after
-// pf_set_temperature rewrote those).
+// The temperature planes of the tied ones from the stored state (after
+// pf_set_temperature rewrote that).
 template <typename S, typename R>
-__global__ void k_raw_temperature(const S* __restrict__ pin, const R* __restrict__ ain,
-                                  long long ps, long long off, long long n,
-                                  double* __restrict__ raw, double rho_g, double drho) {
+__global__ void k_tied_temperature(const S* __restrict__ pin, const R* __restrict__ ain,
+                                   long long ps, long long off, long long n,
+                                   S* __restrict__ tied, double rho_g, double drho) {
   for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n;
        j += (long long)gridDim.x * blockDim.x) {
     const long long s = off + j;
     const R m = ld<R>(pin + P_E * ps, s), b = ld<R>(pin + (P_E + 1) * ps, s);
     const R e1 = ld<R>(pin + (P_E + 2) * ps, s), e2 = ld<R>(pin + (P_E + 3) * ps, s);
-    raw[X_E * n + j] = (double)q5_rest(m, b);
-    raw[(X_E + 1) * n + j] = (double)e1;
-    raw[(X_E + 2) * n + j] = (double)e2;
-    raw[(X_E + 3) * n + j] = (double)fma(R(2), b, -e1);
-    raw[(X_E + 4) * n + j] = (double)fma(R(2), b, -e2);
-    raw[X_HO * n + j] = (double)m / (rho_g + raw[X_PHI * n + j] * drho);
-    raw[X_Q * n + j] = (double)ain[A_QO * ps + s];
-  }
-}
-
-// A raw state rounded to the storage form (as pf_get_state returns it).
-template <typename S, typename R>
-__global__ void k_raw_rounded(const double* __restrict__ raw, long long n, int planes,
-                              double* __restrict__ out) {
-  for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n;
-       j += (long long)gridDim.x * blockDim.x) {
-    auto x = [&](int k) { return (R)raw[k * n + j]; };
-    R psio = R(0);
-    for (int i = 0; i < 5; ++i) psio += x(X_GPRE + i);
-    for (int k = 0; k < planes; ++k) {
-      R v = x(k);
-      if (k < X_H) {
-        if constexpr (Codec<S>::kOffset)
-          v = Codec<S>::template dec<R>(Codec<S>::template enc<R>(v * R(kNSScale))) * R(kNSInvScale);
-      } else if (k < X_PHI && k != X_RR) {
-        const R wm = k < X_GPRE ? w9<R>(k - X_H) * x(X_PHI)
-                                : (k < X_GPOST ? w5<R>(k - X_GPRE) * psio
-                                               : (k < X_RR ? w5<R>(k - X_GPOST) * psio
-                                                           : w5<R>(k - X_S) * x(X_C)));
-        v = dec_off<S, R>(enc_off<S, R>(v, wm), wm);
-      }
-      out[k * n + j] = (double)v;
-    }
+    st<S, R>(tied + T_E * n, j, q5_rest(m, b));
+    st<S, R>(tied + (T_E + 1) * n, j, e1);
+    st<S, R>(tied + (T_E + 2) * n, j, e2);
+    st<S, R>(tied + (T_E + 3) * n, j, fma(R(2), b, -e1));
+    st<S, R>(tied + (T_E + 4) * n, j, fma(R(2), b, -e2));
+    st<S, R>(tied + T_HO * n, j, (R)((double)m / (rho_g + (double)ain[A_PHIO * ps + s] * drho)));
   }
 }
 
@@ -498,21 +517,21 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce(ReduceArgs<R> a, double*
 }
 
 // Thermal totals (FP64): sum over sites of the five temperature populations
-// (the total of rho H: their density plane, or the raw state's populations),
+// (the total of rho H: their density plane, or the tied populations),
 // sum theta, sum psi; then the device error bits.
 template <typename S, typename R>
 __global__ void __launch_bounds__(RED_THREADS) k_reduce_thermal(
     const S* __restrict__ pop, const R* __restrict__ fields, long long ps, DomDesc d,
-    const double* __restrict__ raw, double* __restrict__ partial, double* __restrict__ out, unsigned int* __restrict__ ctr,
+    const S* __restrict__ tied, double* __restrict__ partial, double* __restrict__ out, unsigned int* __restrict__ ctr,
     const unsigned int* __restrict__ err) {
   double acc[3] = {0.0, 0.0, 0.0};
   const long long n = (long long)d.nx * d.ny;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
     const long long site = d.off + i;
-    if (raw) {
+    if (tied) {
       double se = 0.0;
-      for (int q = 0; q < 5; ++q) se += (double)(R)raw[(X_E + q) * n + i];
+      for (int q = 0; q < 5; ++q) se += (double)ld<R>(tied + (T_E + q) * n, i);
       acc[0] += se;
     } else {
       acc[0] += (double)ld<R>(pop + P_E * ps, site);
@@ -608,32 +627,30 @@ cudaError_t launch_set_fields(const SetFieldsArgs<S, R>& a, cudaStream_t st) {
 template <typename S, typename R>
 cudaError_t launch_state_to_f64(const S* pin, const R* ain, long long ps, long long off,
                                 long long n, double* out, int thermal, double rho_g, double drho,
-                                cudaStream_t st) {
-  k_state_to_f64<S, R><<<1024, 256, 0, st>>>(pin, ain, ps, off, n, out, thermal, rho_g, drho);
+                                const S* tied, cudaStream_t st) {
+  k_state_to_f64<S, R><<<1024, 256, 0, st>>>(pin, ain, ps, off, n, out, thermal, rho_g, drho, tied);
   return cudaGetLastError();
 }
 
 template <typename S, typename R>
 cudaError_t launch_state_from_f64(S* pout, R* aout, long long ps, long long off, long long n,
-                                  const double* in, int thermal, double rho_g, double drho,
-                                  unsigned int* err, cudaStream_t st) {
-  k_state_from_f64<S, R><<<1024, 256, 0, st>>>(pout, aout, ps, off, n, in, thermal, rho_g, drho,
-                                               err);
+                                  const double* in, int thermal, S* tied, cudaStream_t st) {
+  k_state_from_f64<S, R><<<1024, 256, 0, st>>>(pout, aout, ps, off, n, in, thermal, tied);
+  return cudaGetLastError();
+}
+
+template <typename R>
+cudaError_t launch_state_general(long long n, const double* in, int thermal, double rho_g,
+                                 double drho, unsigned int* general, cudaStream_t st) {
+  k_state_general<R><<<1024, 256, 0, st>>>(n, in, thermal, rho_g, drho, general);
   return cudaGetLastError();
 }
 
 template <typename S, typename R>
-cudaError_t launch_raw_temperature(const S* pin, const R* ain, long long ps, long long off,
-                                   long long n, double* raw, double rho_g, double drho,
-                                   cudaStream_t st) {
-  k_raw_temperature<S, R><<<1024, 256, 0, st>>>(pin, ain, ps, off, n, raw, rho_g, drho);
-  return cudaGetLastError();
-}
-
-template <typename S, typename R>
-cudaError_t launch_raw_rounded(const double* raw, long long n, int planes, double* out,
-                               cudaStream_t st) {
-  k_raw_rounded<S, R><<<1024, 256, 0, st>>>(raw, n, planes, out);
+cudaError_t launch_tied_temperature(const S* pin, const R* ain, long long ps, long long off,
+                                    long long n, S* tied, double rho_g, double drho,
+                                    cudaStream_t st) {
+  k_tied_temperature<S, R><<<1024, 256, 0, st>>>(pin, ain, ps, off, n, tied, rho_g, drho);
   return cudaGetLastError();
 }
 
@@ -654,10 +671,10 @@ static int reduce_grid(long long n) {
 
 template <typename S, typename R>
 cudaError_t launch_reduce_thermal(const S* pop, const R* fields, long long ps, const DomDesc& d,
-                                  const double* raw, double* partial, double* out, unsigned int* ctr,
+                                  const S* tied, double* partial, double* out, unsigned int* ctr,
                                   const unsigned int* err, cudaStream_t st) {
   k_reduce_thermal<S, R><<<reduce_grid((long long)d.nx * d.ny), RED_THREADS, 0, st>>>(
-      pop, fields, ps, d, raw, partial, out, ctr, err);
+      pop, fields, ps, d, tied, partial, out, ctr, err);
   return cudaGetLastError();
 }
 
@@ -698,20 +715,17 @@ cudaError_t launch_reduce(const ReduceArgs<R>& a, double* partial, double* out, 
   template cudaError_t launch_set_fields<S, R>(const SetFieldsArgs<S, R>&, cudaStream_t);    \
   template cudaError_t launch_state_to_f64<S, R>(const S*, const R*, long long, long long,   \
                                                  long long, double*, int, double, double,    \
-                                                 cudaStream_t);                              \
+                                                 const S*, cudaStream_t);                    \
   template cudaError_t launch_state_from_f64<S, R>(S*, R*, long long, long long, long long,  \
-                                                   const double*, int, double, double,       \
-                                                   unsigned int*, cudaStream_t);             \
-  template cudaError_t launch_raw_temperature<S, R>(const S*, const R*, long long, long long, \
-                                                    long long, double*, double, double,      \
-                                                    cudaStream_t);                           \
-  template cudaError_t launch_raw_rounded<S, R>(const double*, long long, int, double*,      \
-                                                cudaStream_t);                               \
+                                                   const double*, int, S*, cudaStream_t);    \
+  template cudaError_t launch_tied_temperature<S, R>(const S*, const R*, long long, long long, \
+                                                     long long, S*, double, double,          \
+                                                     cudaStream_t);                          \
   template cudaError_t launch_set_temperature<S, R>(S*, R*, R*, long long, const DomDesc&,   \
                                                     const double*, const KParams<R>&,        \
                                                     cudaStream_t);                           \
   template cudaError_t launch_reduce_thermal<S, R>(const S*, const R*, long long,            \
-                                                   const DomDesc&, const double*, double*,   \
+                                                   const DomDesc&, const S*, double*,        \
                                                    double*, unsigned int*,                   \
                                                    const unsigned int*,                      \
                                                    cudaStream_t);
@@ -731,6 +745,10 @@ template cudaError_t launch_fields_to_f64_range<double>(const double*, long long
 template cudaError_t launch_fields_to_f64_range<float>(const float*, long long, long long,
                                                        long long, long long, long long, uint32_t,
                                                        double*, cudaStream_t);
+template cudaError_t launch_state_general<double>(long long, const double*, int, double, double,
+                                                  unsigned int*, cudaStream_t);
+template cudaError_t launch_state_general<float>(long long, const double*, int, double, double,
+                                                 unsigned int*, cudaStream_t);
 template cudaError_t launch_rho_bar<double>(const double*, long long, double*, unsigned int*,
                                             DomDesc*, int, double, double, cudaStream_t);
 template cudaError_t launch_rho_bar<float>(const double*, long long, double*, unsigned int*,

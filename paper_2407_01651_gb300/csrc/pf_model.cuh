@@ -61,6 +61,12 @@ constexpr int N_PHYS = 39;
 // Thermal mode: + e[5], H_o.
 constexpr int N_PHYS_TH = 45;
 
+// What the stored form leaves out of a state whose populations no collision
+// made (pf_raw.cuh): every population of the pair-stored lattices and the lagged
+// H, in planes of the domain's sites, in the storage type.
+constexpr int T_H = 0, T_GPOST = 9, T_S = 14, T_E = 19, T_HO = 24;
+constexpr int N_TIED = 19, N_TIED_TH = 25;
+
 enum Field : int { FLD_PHI, FLD_PSI, FLD_C, FLD_U, FLD_P, FLD_VX, FLD_VY, FLD_MU, FLD_THETA, N_FIELDS };
 
 // Boundary type of a domain side, placed half-way between the last site and

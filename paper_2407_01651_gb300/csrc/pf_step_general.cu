@@ -4,9 +4,9 @@
 // The step kernels keep one population of each opposite pair where a collision
 // fixes the other (pf_model.cuh).  A state that came out of a step or of an
 // initialisation has that form; one written by pf_set_state need not.  Such a
-// state stays in its raw FP64 planes, this kernel takes the first step from
-// them (every population rounded to the storage form on the way, with the
-// pulls, sides and per-site arithmetic of the other kernels), and what it
+// state keeps every population of those lattices in planes beside the stored
+// ones (pf_raw.cuh), this kernel takes the first step from them with the
+// pulls, sides and per-site arithmetic of the other kernels, and what it
 // writes is a collision's output again.  It runs once after such a call, so it
 // is written for any lattice rather than for speed: 32 x 8 tiles with a halo
 // of the stencil fields in shared memory.
@@ -18,11 +18,10 @@ constexpr int GX = 32, GY = 8;
 
 template <typename S, typename R, bool TH>
 __global__ void __launch_bounds__(GX * GY) k_step_general(StepArgs<S, R> a, DomDesc d,
-                                                          const double* raw) {
+                                                          const S* tied) {
   constexpr int NF = TH ? 5 : 4;
   __shared__ R ring[NF][GY + 2][GX + 2];
-  const RawState<S, R> s{raw, (long long)d.nx * d.ny};
-  const GeneralPull<S, R, TH> pull{s, a, d};
+  const GeneralPull<S, R, TH> pull{tied, a, d};
   const int tiles_x = (d.nx + GX - 1) / GX;
   const int x0 = (int)(blockIdx.x % tiles_x) * GX, y0 = (int)(blockIdx.x / tiles_x) * GY;
   const int tid = threadIdx.y * GX + threadIdx.x;
@@ -43,9 +42,8 @@ __global__ void __launch_bounds__(GX * GY) k_step_general(StepArgs<S, R> a, DomD
     R v[NF], g[5], po;
     V2<R> J;
     pull.hg(ex, ey, J, g, v[0], v[1], po);
-    const unsigned j = pull.local(site_at(d, ex, ey));
-    v[2] = s.x(X_VX, j);
-    v[3] = s.x(X_VY, j);
+    v[2] = pull.aux(A_VXO, site_at(d, ex, ey));
+    v[3] = pull.aux(A_VYO, site_at(d, ex, ey));
     if constexpr (TH) {
       R sv[5];
       pull.solute(ex, ey, sv);
@@ -78,22 +76,22 @@ __global__ void __launch_bounds__(GX * GY) k_step_general(StepArgs<S, R> a, DomD
 }
 
 template <typename S, typename R>
-cudaError_t launch_step_general(const StepArgs<S, R>& a, const DomDesc& d, const double* raw,
+cudaError_t launch_step_general(const StepArgs<S, R>& a, const DomDesc& d, const S* tied,
                                 cudaStream_t st) {
   const unsigned tiles = (unsigned)((d.nx + GX - 1) / GX) * (unsigned)((d.ny + GY - 1) / GY);
   if constexpr (sizeof(S) == sizeof(R)) {
     if (a.thermal) {
-      k_step_general<S, R, true><<<tiles, dim3(GX, GY), 0, st>>>(a, d, raw);
+      k_step_general<S, R, true><<<tiles, dim3(GX, GY), 0, st>>>(a, d, tied);
       return cudaGetLastError();
     }
   }
-  k_step_general<S, R, false><<<tiles, dim3(GX, GY), 0, st>>>(a, d, raw);
+  k_step_general<S, R, false><<<tiles, dim3(GX, GY), 0, st>>>(a, d, tied);
   return cudaGetLastError();
 }
 
 #define PF_GENERAL_INST(S, R)                                                             \
   template cudaError_t launch_step_general<S, R>(const StepArgs<S, R>&, const DomDesc&,   \
-                                                 const double*, cudaStream_t);
+                                                 const S*, cudaStream_t);
 PF_GENERAL_INST(double, double)
 PF_GENERAL_INST(float, float)
 PF_GENERAL_INST(__half, float)
