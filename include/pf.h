@@ -200,7 +200,10 @@ pf_status pf_set_fields(pf_handle *h, int dom, const double *fields6, const doub
 
 /* Advance every domain by n_steps coupled steps (Section 3 unified LBE and
  * Appendix B).  n_steps >= 0.  Enqueued on the stream; returns without
- * waiting.  Errors: STATE (no init), CUDA. */
+ * waiting.  The call may be captured into a CUDA graph of the caller's (which
+ * has to end before the handle does): a replay starts from the state that the
+ * buffer then holds, also one that pf_set_state has put there before or after
+ * the capture.  Errors: STATE (no init), CUDA. */
 pf_status pf_step(pf_handle *h, int n_steps);
 
 /* Traversal of the step kernel (same arithmetic, results identical to

@@ -85,17 +85,26 @@ struct pf_handle {
   double* partial = nullptr;
   double* d_diag = nullptr;
   // device error bits written by the step kernels, the block counter of the
-  // reductions (0 between them), the answer of launch_state_general
+  // reductions (0 between them), the answer of launch_state_general, the block
+  // counter of launch_step_tied
   unsigned int* d_err = nullptr;
   int* d_tile_ctr = nullptr;      // two tile counters of the one-launch mode
   bool one_bc = false;            // few tiles with sides: one launch (upload_tables)
   int drop_copies = 0;            // testing only (pf_test_drop_staged_copies)
   double* staging = nullptr;    // FP64 device staging (largest domain x 39 planes)
   size_t staging_elems = 0;
-  // tied planes of a domain whose state pf_set_state gave populations that no
-  // collision made (pf_raw.cuh), until its next step; else nullptr
-  std::vector<void*> raw;
-  std::vector<void*> spent;   // tied planes a step has consumed, freed at the next wait
+  // Tied planes of the domains whose state in buffer 0 / 1 pf_set_state gave
+  // populations that no collision made (pf_raw.cuh), until the buffer is
+  // overwritten; else nullptr.  The device holds the same (d_tied, the table of
+  // pf_step_general.cu): a step that a caller captured into a graph finds the
+  // raw domains there when it runs, and takes out what it overwrites, so once a
+  // step was captured the table says which entries here still stand (settle_raw).
+  std::vector<void*> raw[2];
+  int n_raw = 0;                        // entries of raw
+  unsigned long long* d_tied = nullptr;
+  bool captured = false;                // some step is in a caller's graph
+  std::vector<void*> spent;   // tied planes that are no domain's state any more, freed
+                              // at the next wait
   long long steps = 0;
   long long launches = 0;
   std::string err;
@@ -269,18 +278,53 @@ static pf_status check_params(const pf_params* p) {
 template <typename R>
 static R* fields_ptr(pf_handle* h) { return reinterpret_cast<R*>(h->fields); }
 
-// The tied planes of a domain are not its state any more; work that reads them
-// may still be in the stream, so they are freed where the stream was waited for.
-static void drop_raw(pf_handle* h, int dom) {
-  if (h->raw[dom]) h->spent.push_back(h->raw[dom]);
-  h->raw[dom] = nullptr;
+// Row of state buffer b in the table of tied planes.
+static unsigned long long* tied_row(const pf_handle* h, int b) {
+  return h->d_tied + (size_t)b * (h->ddesc.size() + 1);
+}
+// The domain's state in buffer b is not raw (any more).  Work that reads its tied
+// planes may still be in the stream, so they are freed where that was waited for.
+static pf_status drop_raw(pf_handle* h, int b, int dom) {
+  if (!h->raw[b][dom]) return PF_OK;
+  h->spent.push_back(h->raw[b][dom]);
+  h->raw[b][dom] = nullptr;
+  h->n_raw--;
+  PF_CUDA(h, cudaMemsetAsync(tied_row(h, b) + 1 + dom, 0, sizeof(unsigned long long), h->stream));
+  return PF_OK;
+}
+// Buffer b was overwritten.
+static pf_status drop_raw_row(pf_handle* h, int b) {
+  for (int d = 0; h->n_raw && d < (int)h->raw[b].size(); ++d) {
+    const pf_status st = drop_raw(h, b, d);
+    if (st != PF_OK) return st;
+  }
+  return PF_OK;
+}
+// Takes out the entries that a graph's steps have overwritten (waits, and only
+// where a state is raw and some step was captured).
+static pf_status settle_raw(pf_handle* h) {
+  if (!h->captured || !h->n_raw) return PF_OK;
+  const size_t nd = h->ddesc.size();
+  std::vector<unsigned long long> t(2 * (nd + 1));
+  PF_CUDA(h, cudaMemcpyAsync(t.data(), h->d_tied, t.size() * sizeof(t[0]), cudaMemcpyDeviceToHost,
+                             h->stream));
+  PF_CUDA(h, cudaStreamSynchronize(h->stream));
+  for (int b = 0; b < 2; ++b)
+    for (size_t d = 0; d < nd; ++d)
+      if (h->raw[b][d] && !t[b * (nd + 1) + 1 + d]) {
+        h->spent.push_back(h->raw[b][d]);
+        h->raw[b][d] = nullptr;
+        h->n_raw--;
+      }
+  return PF_OK;
 }
 static void free_spent(pf_handle* h) {
   for (void* r : h->spent) dev_free(h, r);
   h->spent.clear();
 }
+// Some domain's current state is raw.
 static bool any_raw(const pf_handle* h) {
-  for (const void* r : h->raw)
+  for (const void* r : h->raw[h->cur])
     if (r) return true;
   return false;
 }
@@ -347,7 +391,10 @@ static void release(pf_handle* h) {
   dev_free(h, h->d_tile_ctr);
   h->d_tile_ctr = nullptr;
   dev_free(h, h->staging);
-  for (void*& r : h->raw) { dev_free(h, r); r = nullptr; }
+  for (auto& row : h->raw)
+    for (void*& r : row) { dev_free(h, r); r = nullptr; }
+  dev_free(h, h->d_tied);
+  h->d_tied = nullptr;
   for (void* r : h->spent) dev_free(h, r);
   h->spent.clear();
   dev_free(h, h->adj_ws);
@@ -597,7 +644,7 @@ extern "C" pf_status pf_create(const pf_params* p, const pf_domain* doms, int n_
   h->n_phys = p->thermal ? N_PHYS_TH : N_PHYS;
   h->doms.assign(doms, doms + n_doms);
   h->inited.assign(n_doms, 0);
-  h->raw.assign(n_doms, nullptr);
+  for (auto& row : h->raw) row.assign(n_doms, nullptr);
   long long off = 0;
   size_t max_n = 0;
   for (int d = 0; d < n_doms; ++d) {
@@ -640,13 +687,16 @@ extern "C" pf_status pf_create(const pf_params* p, const pf_domain* doms, int n_
   h->d_doms = (DomDesc*)dev_alloc(h, (size_t)n_doms * sizeof(DomDesc));
   h->partial = (double*)dev_alloc(h, (size_t)REDUCE_BLOCKS * NDIAG * sizeof(double));
   h->d_diag = (double*)dev_alloc(h, (NDIAG + 1) * sizeof(double));
-  h->d_err = (unsigned int*)dev_alloc(h, 3 * sizeof(unsigned int));
+  h->d_err = (unsigned int*)dev_alloc(h, 4 * sizeof(unsigned int));
+  const size_t tied_b = 2 * ((size_t)n_doms + 1) * sizeof(unsigned long long);
+  h->d_tied = (unsigned long long*)dev_alloc(h, tied_b);
   (void)max_n;
   if (!h->fields || !h->grain || !h->grain_cs || !h->d_doms || !h->partial || !h->d_diag ||
-      !h->d_err)
+      !h->d_err || !h->d_tied)
     return bail(PF_ERR_OOM, "device allocation failed");
   if (cudaMemsetAsync(h->fields, 0, ps * N_FIELDS * h->celem, h->stream) != cudaSuccess ||
-      cudaMemsetAsync(h->d_err, 0, 3 * sizeof(unsigned int), h->stream) != cudaSuccess ||
+      cudaMemsetAsync(h->d_err, 0, 4 * sizeof(unsigned int), h->stream) != cudaSuccess ||
+      cudaMemsetAsync(h->d_tied, 0, tied_b, h->stream) != cudaSuccess ||
       cudaMemsetAsync(h->grain, 0, ps, h->stream) != cudaSuccess)
     return bail(PF_ERR_CUDA, "memset failed");
   for (int d = 0; d < n_doms; ++d)
@@ -789,8 +839,8 @@ extern "C" pf_status pf_init_fields(pf_handle* h, int dom, const pf_init_spec* s
   if (!buf) return fail(h, PF_ERR_OOM, "init buffer allocation failed");
   pf_status st = clear_device_error(h);
   if (st == PF_OK) st = upload_grain_table(h, dom, angles);
+  if (st == PF_OK) st = drop_raw(h, h->cur, dom);
   if (st != PF_OK) { dev_free(h, buf); return st; }
-  drop_raw(h, dom);
   if (ns) PF_CUDA(h, cudaMemcpyAsync(buf, spec->seeds, ns * sizeof(double), cudaMemcpyHostToDevice, h->stream));
   if (nb) PF_CUDA(h, cudaMemcpyAsync(buf + ns, spec->bubbles, nb * sizeof(double), cudaMemcpyHostToDevice, h->stream));
   st = dispatch(h, [&](auto s_t, auto r_t) {
@@ -861,7 +911,7 @@ extern "C" pf_status pf_set_fields(pf_handle* h, int dom, const double* fields6,
   if (st != PF_OK) return st;
   st = upload_grain_table(h, dom, angles);
   if (st != PF_OK) return st;
-  drop_raw(h, dom);
+  if ((st = drop_raw(h, h->cur, dom)) != PF_OK) return st;
   const double* buf = direct ? direct : h->staging;
   uint8_t* d_ids = nullptr;
   if (!direct)
@@ -1033,38 +1083,22 @@ static pf_status step_t(pf_handle* h, bool write_fields, cudaStream_t stream = n
   return PF_OK;
 }
 
-// The step after a pf_set_state of populations that no collision made: those
-// domains with their tied planes, the others as ever, one launch per domain.
+// The first step of a call where a domain may be raw: every domain as ever, then
+// the raw ones once more from their tied planes (so a raw domain does not change
+// how the others step).  In a caller's capture the second launch is always there,
+// since the graph may run on a raw state later: us a replay of a graph of one call
+// without and with it, FP32: 2 steps of 128^2 12.3 and 12.3, of 512^2 34.8 and 36.5;
+// 30 steps 129.1 and 129.1, 477.2 and 478.3.
 template <typename S, typename R>
-static pf_status step_general_t(pf_handle* h, bool write_fields) {
-  const StepArgs<S, R> a0 = make_step_args<S, R>(h, h->pop[h->cur], h->aux[h->cur],
-                                                 h->pop[h->cur ^ 1], h->aux[h->cur ^ 1],
-                                                 write_fields);
-  auto go = [&](int t0, int t1, int bc) -> pf_status {
-    if (t1 <= t0) return PF_OK;
-    StepArgs<S, R> a = a0;
-    a.tile_base = t0;
-    a.ntiles = t1;
-    a.bc = bc;
-    PF_CUDA(h, launch_step<S, R>(a, bc ? STEP_YMARCH : step_variant(h), h->tx, h->ty, t1 - t0,
-                                 h->stream));
-    h->launches++;
-    return PF_OK;
-  };
-  for (size_t d = 0; d < h->ddesc.size(); ++d) {
-    pf_status st;
-    if (h->raw[d]) {
-      PF_CUDA(h, launch_step_general<S, R>(a0, h->ddesc[d], (const S*)h->raw[d], h->stream));
-      h->launches++;
-    } else if (h->any_bc) {
-      if ((st = go(h->plain0[d], h->plain1[d], 0)) != PF_OK) return st;
-      if ((st = go(h->edge0[d], h->edge1[d], h->any_io ? 2 : 1)) != PF_OK) return st;
-    } else {
-      const int t1 = d + 1 < h->ddesc.size() ? h->ddesc[d + 1].tile0 : h->ntiles;
-      if ((st = go(h->ddesc[d].tile0, t1, 0)) != PF_OK) return st;
-    }
-  }
-  for (size_t d = 0; d < h->raw.size(); ++d) drop_raw(h, (int)d);
+static pf_status step_tied_t(pf_handle* h, int n_steps) {
+  const StepArgs<S, R> a = make_step_args<S, R>(h, h->pop[h->cur], h->aux[h->cur],
+                                                h->pop[h->cur ^ 1], h->aux[h->cur ^ 1],
+                                                n_steps == 1);
+  pf_status st = launch_all<S, R>(h, a, h->stream);
+  if (st != PF_OK) return st;
+  PF_CUDA(h, launch_step_tied<S, R>(a, h->d_doms, (int)h->ddesc.size(), h->d_tied, h->cur,
+                                    n_steps > 1, h->d_err + 3, std::max(1, h->sms), h->stream));
+  h->launches++;
   h->cur ^= 1;
   h->steps++;
   return PF_OK;
@@ -1107,14 +1141,9 @@ static pf_status ensure_graph(pf_handle* h) {
   return PF_OK;
 }
 
+// The steps of a call behind its first `done`; captured: into a caller's graph.
 template <typename S, typename R>
-static pf_status step_n(pf_handle* h, int n_steps) {
-  int done = 0;
-  if (n_steps > 0 && any_raw(h)) {
-    pf_status st = step_general_t<S, R>(h, n_steps == 1);
-    if (st != PF_OK) return st;
-    done = 1;
-  }
+static pf_status step_rest(pf_handle* h, int n_steps, int done, bool captured) {
   if (steps_in_one_launch(h)) {
     // graph_steps > 0: whole graph_steps-step launches replayed from graphs,
     // then the rest (with the field output) in one more launch
@@ -1144,15 +1173,35 @@ static pf_status step_n(pf_handle* h, int n_steps) {
   }
   // steps behind the first, one launch each: chained (see chain_step), except in
   // a caller's capture, whose graph keeps plain edges
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (n_steps - done > 1) PF_CUDA(h, cudaStreamIsCapturing(h->stream, &cs));
-  const bool chain = cs == cudaStreamCaptureStatusNone && h->launch_mode == 0 &&
-                     (!h->any_bc || h->one_bc);
+  const bool chain = !captured && h->launch_mode == 0 && (!h->any_bc || h->one_bc);
   for (bool behind = false; done < n_steps; ++done, behind = chain) {
     pf_status st = step_t<S, R>(h, done == n_steps - 1, nullptr, behind);
     if (st != PF_OK) return st;
   }
   return PF_OK;
+}
+
+template <typename S, typename R>
+static pf_status step_n(pf_handle* h, int n_steps) {
+  if (n_steps == 0) return PF_OK;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  PF_CUDA(h, cudaStreamIsCapturing(h->stream, &cs));
+  pf_status st;
+  if (cs != cudaStreamCaptureStatusNone) {
+    h->captured = true;
+    if ((st = step_tied_t<S, R>(h, n_steps)) != PF_OK) return st;
+    return step_rest<S, R>(h, n_steps, 1, true);
+  }
+  if ((st = settle_raw(h)) != PF_OK) return st;
+  int done = 0;
+  if (h->n_raw && any_raw(h)) {
+    if ((st = step_tied_t<S, R>(h, n_steps)) != PF_OK) return st;
+    done = 1;
+  }
+  if ((st = step_rest<S, R>(h, n_steps, done, false)) != PF_OK) return st;
+  // the buffers the steps wrote: the one that is current now, two steps on both
+  if ((st = drop_raw_row(h, h->cur)) != PF_OK) return st;
+  return n_steps > 1 ? drop_raw_row(h, h->cur ^ 1) : PF_OK;
 }
 
 // The staged variant needs every domain's nx to be a multiple of its copy
@@ -1310,6 +1359,8 @@ static pf_status autotune_t(pf_handle* h, int trial_steps, int out[4]) {
   h->steps = steps0;
   h->launches = launches0;
   h->own_chunk = own0;
+  // the trials overwrote the other buffer, this one is as it was
+  if (const pf_status sr = drop_raw_row(h, cur0 ^ 1); sr != PF_OK) return sr;
   if (st != PF_OK) return st;
   h->variant = bc.variant;
   if (bc.variant != STEP_TILE) h->chunk = bc.a; else { h->tx = bc.a; h->ty = bc.b; }
@@ -1449,7 +1500,8 @@ static pf_status run_banded(pf_handle* h, const double* in6, int n_steps, uint32
   if (!h->run_phi) PF_CUDA(h, cudaEventCreateWithFlags(&h->run_phi, cudaEventDisableTiming));
   if (!h->run_ctl) PF_CUDA(h, cudaEventCreateWithFlags(&h->run_ctl, cudaEventDisableTiming));
   cudaStream_t S0 = h->stream;
-  drop_raw(h, 0);
+  for (int b = 0; b < 2; ++b)   // the equilibria overwrite one, the first step the other
+    if ((st = drop_raw_row(h, b)) != PF_OK) return st;
   st = clear_device_error(h);
   if (st != PF_OK) return st;
   st = upload_grain_table(h, 0, {});
@@ -1587,14 +1639,16 @@ extern "C" pf_status pf_get_state(pf_handle* h, int dom, double* host_out, size_
   const size_t nn = (size_t)dd.nx * dd.ny;
   const size_t np = (size_t)h->n_phys;
   if (n < nn * np) return fail(h, PF_ERR_BAD_ARG, "output buffer too small");
-  pf_status st = ensure_staging(h, nn * np);
+  pf_status st = settle_raw(h);
+  if (st != PF_OK) return st;
+  st = ensure_staging(h, nn * np);
   if (st != PF_OK) return st;
   st = dispatch(h, [&](auto s_t, auto r_t) {
     PF_TYPES(s_t, r_t);
     PF_CUDA(h, launch_state_to_f64<S, R>((const S*)h->pop[h->cur], (const R*)h->aux[h->cur],
                                          h->plane_stride, dd.off, (long long)nn, h->staging,
                                          h->thermal, h->p.rho_g, h->p.rho_l - h->p.rho_g,
-                                         (const S*)h->raw[dom], h->stream));
+                                         (const S*)h->raw[h->cur][dom], h->stream));
     return PF_OK;
   });
   if (st != PF_OK) return st;
@@ -1614,7 +1668,9 @@ extern "C" pf_status pf_set_state(pf_handle* h, int dom, const double* host_in, 
   if (n != nn * np)
     return fail(h, PF_ERR_BAD_ARG, "input must hold pf_state_planes(h) planes of nx*ny");
   // everything that can run out of memory comes before the first change
-  pf_status st = ensure_staging(h, nn * np);
+  pf_status st = settle_raw(h);
+  if (st != PF_OK) return st;
+  st = ensure_staging(h, nn * np);
   if (st != PF_OK) return st;
   PF_CUDA(h, cudaMemcpyAsync(h->staging, host_in, nn * np * sizeof(double),
                              cudaMemcpyHostToDevice, h->stream));
@@ -1627,18 +1683,24 @@ extern "C" pf_status pf_set_state(pf_handle* h, int dom, const double* host_in, 
   unsigned int general = 0;
   PF_CUDA(h, cudaMemcpyAsync(&general, h->d_err + 2, sizeof(general), cudaMemcpyDeviceToHost, h->stream));
   PF_CUDA(h, cudaStreamSynchronize(h->stream));
-  if (general && !h->raw[dom]) {
-    h->raw[dom] = dev_alloc(h, nn * (h->thermal ? N_TIED_TH : N_TIED) * h->elem);
-    if (!h->raw[dom]) return fail(h, PF_ERR_OOM, "allocation of the state's tied planes failed");
-  } else if (!general) {
-    drop_raw(h, dom);
+  void*& tied = h->raw[h->cur][dom];
+  if (general && !tied) {
+    tied = dev_alloc(h, nn * (h->thermal ? N_TIED_TH : N_TIED) * h->elem);
+    if (!tied) return fail(h, PF_ERR_OOM, "allocation of the state's tied planes failed");
+    h->n_raw++;
+    const unsigned long long entry = reinterpret_cast<unsigned long long>(tied), some = 1;
+    unsigned long long* row = tied_row(h, h->cur);
+    PF_CUDA(h, cudaMemcpyAsync(row + 1 + dom, &entry, sizeof(entry), cudaMemcpyHostToDevice, h->stream));
+    PF_CUDA(h, cudaMemcpyAsync(row, &some, sizeof(some), cudaMemcpyHostToDevice, h->stream));
+  } else if (!general && (st = drop_raw(h, h->cur, dom)) != PF_OK) {
+    return st;
   }
   if ((st = clear_device_error(h)) != PF_OK) return st;
   st = dispatch(h, [&](auto s_t, auto r_t) {
     PF_TYPES(s_t, r_t);
     PF_CUDA(h, launch_state_from_f64<S, R>((S*)h->pop[h->cur], (R*)h->aux[h->cur],
                                            h->plane_stride, dd.off, (long long)nn, h->staging,
-                                           h->thermal, (S*)h->raw[dom], h->stream));
+                                           h->thermal, (S*)tied, h->stream));
     return PF_OK;
   });
   if (st != PF_OK) return st;
@@ -1728,7 +1790,9 @@ extern "C" pf_status pf_set_temperature(pf_handle* h, int dom, const double* the
   const DomDesc& dd = h->ddesc[dom];
   const size_t nn = (size_t)dd.nx * dd.ny;
   if (n != nn) return fail(h, PF_ERR_BAD_ARG, "n must equal nx*ny of the domain");
-  pf_status st = ensure_staging(h, nn + 1);
+  pf_status st = settle_raw(h);
+  if (st != PF_OK) return st;
+  st = ensure_staging(h, nn + 1);
   if (st != PF_OK) return st;
   PF_CUDA(h, cudaMemcpyAsync(h->staging, theta, nn * sizeof(double), cudaMemcpyHostToDevice,
                              h->stream));
@@ -1747,10 +1811,10 @@ extern "C" pf_status pf_set_temperature(pf_handle* h, int dom, const double* the
     PF_CUDA(h, launch_set_temperature<S, R>((S*)h->pop[h->cur], (R*)h->aux[h->cur],
                                             fields_ptr<R>(h), h->plane_stride, dd, h->staging,
                                             make_kparams<R>(h->p), h->stream));
-    if (h->raw[dom]) {
+    if (void* tied = h->raw[h->cur][dom]) {
       PF_CUDA(h, launch_tied_temperature<S, R>((const S*)h->pop[h->cur], (const R*)h->aux[h->cur],
                                                h->plane_stride, dd.off, (long long)nn,
-                                               (S*)h->raw[dom], h->p.rho_g,
+                                               (S*)tied, h->p.rho_g,
                                                h->p.rho_l - h->p.rho_g, h->stream));
       h->launches++;
     }
@@ -1768,11 +1832,13 @@ extern "C" pf_status pf_reduce_thermal(pf_handle* h, int dom, double out[3]) {
   if (dom < 0 || dom >= (int)h->doms.size() || !out)
     return fail(h, PF_ERR_BAD_ARG, "bad domain or output");
   const DomDesc& dd = h->ddesc[dom];
-  pf_status st = dispatch(h, [&](auto s_t, auto r_t) {
+  pf_status st = settle_raw(h);
+  if (st != PF_OK) return st;
+  st = dispatch(h, [&](auto s_t, auto r_t) {
     PF_TYPES(s_t, r_t);
     PF_CUDA(h, launch_reduce_thermal<S, R>((const S*)h->pop[h->cur], fields_ptr<R>(h),
-                                           h->plane_stride, dd, (const S*)h->raw[dom], h->partial,
-                                           h->d_diag,
+                                           h->plane_stride, dd, (const S*)h->raw[h->cur][dom],
+                                           h->partial, h->d_diag,
                                            h->d_err + 1, h->d_err, h->stream));
     return PF_OK;
   });
@@ -1846,7 +1912,8 @@ static pf_status adjoint_t(pf_handle* h, int n, const pf_objective* obj, double*
   const bool fresh = h->steps == 0;
   cudaStream_t A = h->stream;
   // x_0 may be a raw state: its step and its reverse take their own kernels
-  const S* raw0 = (const S*)h->raw[0];
+  if (pf_status sr = settle_raw(h); sr != PF_OK) return sr;
+  const S* raw0 = (const S*)h->raw[h->cur][0];
   // (behind: the step before it is the stream's last operation; 512^2, 100 steps,
   // K = 25: the call 9707 -> 9504 us.  The recomputed steps and the reverse
   // kernels, which share the SMs, lose by it: 9877.)
@@ -1999,8 +2066,9 @@ static pf_status adjoint_t(pf_handle* h, int n, const pf_objective* obj, double*
   PF_CUDA(h, cudaMemcpyAsync(hp.data(), partial, hp.size() * sizeof(double),
                              cudaMemcpyDeviceToHost, A));
   PF_CUDA(h, cudaStreamSynchronize(A));
-  drop_raw(h, 0);
-  free_spent(h);
+  // the sweep of several segments overwrote both buffers, that of one the current
+  if (pf_status sr = drop_raw_row(h, h->cur); sr != PF_OK) return sr;
+  if (pf_status sr = nseg > 1 ? drop_raw_row(h, h->cur ^ 1) : PF_OK; sr != PF_OK) return sr;
   double g[3] = {0.0, 0.0, 0.0};
   for (int b = 0; b < grid; ++b)
     for (int q = 0; q < 3; ++q) g[q] += hp[(size_t)b * 3 + q];

@@ -163,6 +163,12 @@ cudaError_t launch_state_general(long long n, const double* in, int thermal, dou
 template <typename S, typename R>
 cudaError_t launch_step_general(const StepArgs<S, R>& a, const DomDesc& d, const S* tied,
                                 cudaStream_t st);
+// The raw domains again, from the device table of tied planes, behind a step that
+// read state buffer `row` (pf_step_general.cu).  ctr: a device counter at 0.
+template <typename S, typename R>
+cudaError_t launch_step_tied(const StepArgs<S, R>& a, const DomDesc* doms, int n_doms,
+                             unsigned long long* table, int row, int both, unsigned int* ctr,
+                             int grid, cudaStream_t st);
 // The temperature planes of the tied ones from the stored state.
 template <typename S, typename R>
 cudaError_t launch_tied_temperature(const S* pin, const R* ain, long long ps, long long off,
