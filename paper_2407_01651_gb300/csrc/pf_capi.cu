@@ -319,6 +319,8 @@ static pf_status settle_raw(pf_handle* h) {
   return PF_OK;
 }
 static void free_spent(pf_handle* h) {
+  if (h->spent.empty()) return;
+  if (h->adj_stream) cudaStreamSynchronize(h->adj_stream);   // an adjoint that failed midway
   for (void* r : h->spent) dev_free(h, r);
   h->spent.clear();
 }
@@ -1913,7 +1915,14 @@ static pf_status adjoint_t(pf_handle* h, int n, const pf_objective* obj, double*
   cudaStream_t A = h->stream;
   // x_0 may be a raw state: its step and its reverse take their own kernels
   if (pf_status sr = settle_raw(h); sr != PF_OK) return sr;
-  const S* raw0 = (const S*)h->raw[h->cur][0];
+  const int b0 = h->cur;
+  const S* raw0 = (const S*)h->raw[b0][0];
+  // its tied planes outlive the state: the reverse sweep still reads them
+  struct Keep {
+    pf_handle* h;
+    void* p = nullptr;
+    ~Keep() { if (p) h->spent.push_back(p); }
+  } keep{h};
   // (behind: the step before it is the stream's last operation; 512^2, 100 steps,
   // K = 25: the call 9707 -> 9504 us.  The recomputed steps and the reverse
   // kernels, which share the SMs, lose by it: 9877.)
@@ -1958,6 +1967,14 @@ static pf_status adjoint_t(pf_handle* h, int n, const pf_objective* obj, double*
     }
     h->cur ^= 1;
     h->steps += L;
+  }
+  // the state is x_T from here on, whatever fails; a sweep of several segments has
+  // overwritten x_0's buffer too
+  if (pf_status sr = drop_raw_row(h, b0 ^ 1); sr != PF_OK) return sr;
+  if (raw0 && nseg > 1) {
+    if (pf_status sr = drop_raw(h, b0, 0); sr != PF_OK) return sr;
+    keep.p = h->spent.back();
+    h->spent.pop_back();
   }
   // objective J(x_T) and its adjoint lambda_T
   pf_diag dg{};
@@ -2066,9 +2083,6 @@ static pf_status adjoint_t(pf_handle* h, int n, const pf_objective* obj, double*
   PF_CUDA(h, cudaMemcpyAsync(hp.data(), partial, hp.size() * sizeof(double),
                              cudaMemcpyDeviceToHost, A));
   PF_CUDA(h, cudaStreamSynchronize(A));
-  // the sweep of several segments overwrote both buffers, that of one the current
-  if (pf_status sr = drop_raw_row(h, h->cur); sr != PF_OK) return sr;
-  if (pf_status sr = nseg > 1 ? drop_raw_row(h, h->cur ^ 1) : PF_OK; sr != PF_OK) return sr;
   double g[3] = {0.0, 0.0, 0.0};
   for (int b = 0; b < grid; ++b)
     for (int q = 0; q < 3; ++q) g[q] += hp[(size_t)b * 3 + q];
