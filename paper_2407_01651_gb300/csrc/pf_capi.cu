@@ -744,6 +744,7 @@ static pf_status check_device_error(pf_handle* h) {
   unsigned int bits = 0;
   PF_CUDA(h, cudaMemcpyAsync(&bits, h->d_err, sizeof(bits), cudaMemcpyDeviceToHost, h->stream));
   PF_CUDA(h, cudaStreamSynchronize(h->stream));
+  free_spent(h);
   return report_device_error(h, bits);
 }
 
@@ -1708,6 +1709,7 @@ extern "C" pf_status pf_set_state(pf_handle* h, int dom, const double* host_in, 
   if (st != PF_OK) return st;
   h->launches += 2;
   PF_CUDA(h, cudaStreamSynchronize(h->stream));
+  free_spent(h);
   h->inited[dom] = 1;
   return PF_OK;
 }
@@ -1734,6 +1736,7 @@ extern "C" pf_status pf_reduce(pf_handle* h, int dom, const pf_probe* probe, pf_
   double buf[NDIAG + 1];   // the diagnostics and the error bits in one copy
   PF_CUDA(h, cudaMemcpyAsync(buf, h->d_diag, sizeof(buf), cudaMemcpyDeviceToHost, h->stream));
   PF_CUDA(h, cudaStreamSynchronize(h->stream));
+  free_spent(h);
   static_assert(sizeof(pf_diag) == NDIAG * sizeof(double), "pf_diag layout");
   std::memcpy(out, buf, sizeof(pf_diag));
   return report_device_error(h, (unsigned int)buf[NDIAG]);
@@ -1849,6 +1852,7 @@ extern "C" pf_status pf_reduce_thermal(pf_handle* h, int dom, double out[3]) {
   double buf[4];
   PF_CUDA(h, cudaMemcpyAsync(buf, h->d_diag, sizeof(buf), cudaMemcpyDeviceToHost, h->stream));
   PF_CUDA(h, cudaStreamSynchronize(h->stream));
+  free_spent(h);
   std::memcpy(out, buf, 3 * sizeof(double));
   return report_device_error(h, (unsigned int)buf[3]);
 }

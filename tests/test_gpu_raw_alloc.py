@@ -111,3 +111,16 @@ def test_an_allocation_that_fails_leaves_the_state(allocator, what):
     ref.step(1)
     for d in (0, 1):
         assert np.array_equal(sim.get_state(d), ref.get_state(d))
+
+
+@pytest.mark.parametrize("wait", ["sync", "reduce", "reduce_thermal", "set_state"])
+def test_every_wait_releases_used_planes(allocator, wait):
+    """Planes that a step has used go at the next call that waits for the stream."""
+    sim = ensemble([(64, 48)], "fp32", 1)
+    ordinary, st = sim.get_state(0), general(sim, 0, 1)
+    before = allocator.bytes()
+    sim.set_state(0, st)
+    sim.step(2)
+    assert allocator.bytes() - before == 25 * 4 * 64 * 48
+    sim.set_state(0, ordinary) if wait == "set_state" else getattr(sim, wait)()
+    assert allocator.bytes() == before
