@@ -203,7 +203,9 @@ pf_status pf_set_fields(pf_handle *h, int dom, const double *fields6, const doub
  * waiting.  The call may be captured into a CUDA graph of the caller's (which
  * has to end before the handle does): a replay starts from the state that the
  * buffer then holds, also one that pf_set_state has put there before or after
- * the capture.  Errors: STATE (no init), CUDA. */
+ * the capture.  pf_set_step_config, pf_autotune and pf_set_boundaries replace
+ * tables that such a graph reads: capture it anew behind them.
+ * Errors: STATE (no init), CUDA. */
 pf_status pf_step(pf_handle *h, int n_steps);
 
 /* Traversal of the step kernel (same arithmetic, results identical to
@@ -222,7 +224,8 @@ pf_status pf_set_step_config(pf_handle *h, int variant, int a, int b);
 /* How a step is launched over an ensemble of domains:
  *  per_domain = 0: one launch whose tile list spans every domain (default);
  *               1: one launch per domain, one after the other (rows per tile chosen
- *               by size are then those of a domain's own launch).
+ *               by size are then those of a domain's own launch, unless a pf_step
+ *               was captured by the caller before: its graph holds the tiles).
  *  persistent = 1: the grid is the device's resident CTAs of the step kernel,
  *               each looping over tiles; 0: one CTA per tile (default);
  *               2: as 1, and every step of a pf_step call in one cooperative

@@ -1287,8 +1287,9 @@ extern "C" pf_status pf_set_launch(pf_handle* h, int per_domain, int persistent,
   for (auto& g : h->gexec)
     if (g) { cudaGraphExecDestroy(g); g = nullptr; }
   // the tiles by size are those of a launch: 96 domains, 32 each of 256^2, 512x384
-  // and 1024x512, one launch per domain 3311 -> 11236 MLUPS against the whole list's
-  if (retile) {
+  // and 1024x512, one launch per domain 3311 -> 11236 MLUPS against the whole list's.
+  // A caller's graph holds the tiles of its capture, so they stay from then on.
+  if (retile && !h->captured) {
     const pf_status st = choose_chunk(h);
     if (st != PF_OK) return st;
     return upload_tables(h);
