@@ -103,6 +103,7 @@ struct pf_handle {
   int n_raw = 0;                        // entries of raw
   unsigned long long* d_tied = nullptr;
   bool captured = false;                // some step is in a caller's graph
+  size_t runs_n = 0, tiles_n = 0;       // entries that d_runs and d_tile_dom hold
   std::vector<void*> spent;   // tied planes that are no domain's state any more, freed
                               // at the next wait
   long long steps = 0;
@@ -508,6 +509,19 @@ static pf_status choose_chunk(pf_handle* h) {
   });
 }
 
+// Device memory of a tile table for n entries of `size` bytes: the one there is if
+// it holds as many, so that initialising a domain, whose rho_bar the run
+// descriptors carry, leaves the tables where a caller's graph reads them.
+static pf_status resize_table(pf_handle* h, void** table, size_t* held, size_t n, size_t size) {
+  if (*table && *held == n) return PF_OK;
+  dev_free(h, *table);
+  *held = 0;
+  *table = dev_alloc(h, n * size);
+  if (!*table) return fail(h, PF_ERR_OOM, "tile table allocation failed");
+  *held = n;
+  return PF_OK;
+}
+
 static pf_status upload_tables(pf_handle* h) {
   // tiles of every domain, in domain order
   std::vector<int> tile_dom;
@@ -558,15 +572,19 @@ static pf_status upload_tables(pf_handle* h) {
       if (pass == 0) h->n_plain = (int)order.size();
     }
     tile_dom.swap(order);
-    dev_free(h, h->d_runs);
-    h->d_runs = (DomDesc*)dev_alloc(h, runs.size() * sizeof(DomDesc));
-    if (!h->d_runs) return fail(h, PF_ERR_OOM, "tile table allocation failed");
+    void* t = h->d_runs;
+    const pf_status st = resize_table(h, &t, &h->runs_n, runs.size(), sizeof(DomDesc));
+    h->d_runs = (DomDesc*)t;
+    if (st != PF_OK) return st;
     PF_CUDA(h, cudaMemcpyAsync(h->d_runs, runs.data(), runs.size() * sizeof(DomDesc),
                                cudaMemcpyHostToDevice, h->stream));
   }
-  dev_free(h, h->d_tile_dom);
-  h->d_tile_dom = (int*)dev_alloc(h, tile_dom.size() * sizeof(int));
-  if (!h->d_tile_dom) return fail(h, PF_ERR_OOM, "tile table allocation failed");
+  {
+    void* t = h->d_tile_dom;
+    const pf_status st = resize_table(h, &t, &h->tiles_n, tile_dom.size(), sizeof(int));
+    h->d_tile_dom = (int*)t;
+    if (st != PF_OK) return st;
+  }
   PF_CUDA(h, cudaMemcpyAsync(h->d_tile_dom, tile_dom.data(), tile_dom.size() * sizeof(int),
                              cudaMemcpyHostToDevice, h->stream));
   PF_CUDA(h, cudaMemcpyAsync(h->d_doms, h->ddesc.data(), h->ddesc.size() * sizeof(DomDesc),

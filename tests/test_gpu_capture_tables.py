@@ -4,6 +4,7 @@ import pytest
 
 from paper_2407_01651_gb300 import pf
 from paper_2407_01651_gb300 import workload as wl
+from tests.test_gpu_boundaries import F, P, S, W
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -60,3 +61,28 @@ def test_launch_mode_keeps_the_tiles_of_a_captured_step():
         del g
         for s in (sim, ref, fresh, again):
             s.close()
+
+
+@pytest.mark.parametrize("bc", [None, (S, S, W, F), (P, P, W, W)])
+def test_initialising_again_keeps_what_a_graph_reads(bc):
+    """A domain initialised again behind the capture (another mean density): the
+    graph steps the new state with the new buoyancy reference."""
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        sim, ref = handle(bc), handle(bc)
+        sim.sync()
+        g = capture(sim, stream, 2)
+        for s in (sim, ref):
+            s.init_fields(1, [(30.0, 18.0, 0.1)], 6.0, [(70.0, 18.0, 9.0)])
+        g.replay()
+        ref.step(2)
+        assert same(sim, ref)
+        f = ref.fields(0)
+        for s in (sim, ref):
+            s.set_fields(0, f["phi"][::-1], f["psi"], f["C"])
+        g.replay()
+        ref.step(2)
+        assert same(sim, ref)
+        del g
+        sim.close()
+        ref.close()
