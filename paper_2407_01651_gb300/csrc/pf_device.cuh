@@ -50,7 +50,9 @@ constexpr float kNSInvScale = 1.0f / 4096.0f;
 
 // Load from a state plane: a plain coherent load (a chained step starts while the
 // step that writes the plane still runs, so the read-only path is not for it) that
-// the compiler may move past the stores, which go to the other state.
+// the compiler may move past the stores, which go to the other state.  To the
+// compiler it is a function of its address, so a kernel that reads an address
+// again after it was rewritten passes the pointers through fresh_state in between.
 __device__ __forceinline__ float ldp(const float* p) {
   float v;
   asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));

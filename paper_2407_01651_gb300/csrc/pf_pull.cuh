@@ -8,6 +8,13 @@
 
 namespace pf {
 
+// The state pointers of a step as values the compiler has not seen: loads of the
+// step (ldp) can neither be merged with those before this point nor move above it.
+template <typename S, typename R>
+__device__ __forceinline__ void fresh_state(StepArgs<S, R>& a) {
+  asm volatile("" : "+l"(a.in), "+l"(a.ain)::"memory");
+}
+
 // A step launched behind another (StepArgs::chained): its CTAs are placed while
 // the last ones of that step run and wait here until it is complete and its
 // writes are visible; then the next step's CTAs may be placed.  The launch of a

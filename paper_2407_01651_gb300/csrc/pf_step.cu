@@ -221,6 +221,7 @@ __global__ void __launch_bounds__(YM_THREADS, sizeof(R) == 4 ? (TH ? 3 : 4) : 2)
       b.aout = const_cast<R*>(a.ain);
     }
     b.fields = step + 1 == nsteps ? fields : nullptr;
+    fresh_state(b);   // both states' addresses were read two steps ago
     ymarch_tiles<S, R, BIG, TH, true>(b, ring, ctr + (step & 1));
     if (step + 1 < nsteps) grid.sync();
   }
