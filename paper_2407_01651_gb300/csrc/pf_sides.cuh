@@ -82,12 +82,6 @@ __device__ __forceinline__ PullSrc scalar_src(const DomDesc& d, int x, int y, in
   return p;
 }
 
-// A pull source of (x, y) lies beyond a non-periodic side.
-__device__ __forceinline__ bool near_side(const DomDesc& d, int x, int y) {
-  return (x == 0 && d.bc[0]) || (x == d.nx - 1 && d.bc[1]) || (y == 0 && d.bc[2]) ||
-         (y == d.ny - 1 && d.bc[3]);
-}
-
 // Ring fields: 0 phi, 1 psi, 2 vx_o, 3 vy_o, 4 U.  Ghost value across one side
 // of type t on axis (0: x, 1: y) from the mirror site's value v.
 template <typename R, bool IO>

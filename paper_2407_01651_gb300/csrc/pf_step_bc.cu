@@ -229,9 +229,21 @@ __global__ void __launch_bounds__(YM_THREADS, sizeof(R) == 4 ? 3 : 2)
       else col = x0 + w >= nx ? x0 + w - nx : x0 + w;
     }
 
+    // Whether the warp's columns in row y are pulled as next to a side: one path
+    // per warp, the same for the same tile whatever the scheduling (every lane takes
+    // part in the vote, once a tile; those without a column say no); away from the
+    // side both paths pull the same values.
+    const bool side_col = (col == 0 && d.bc[0]) || (col == nx - 1 && d.bc[1]);
+    const bool near_col = __any_sync(0xffffffffu, active && side_col) != 0;
+    const bool near_in = __any_sync(0xffffffffu, interior && side_col) != 0;
+    auto side_row = [&](int y) { return (y == 0 && d.bc[2]) || (y == ny - 1 && d.bc[3]); };
+    // row of the lattice that row yr of the ring comes from
+    auto inside_row = [&](int yr) {
+      return yr < 0 ? (d.bc[2] ? 0 : yr + ny) : (yr >= ny ? (d.bc[3] ? ny - 1 : yr - ny) : yr);
+    };
     // ring values of row yr (ya-1 .. yb, possibly a ghost row) and the
     // streamed h, g of the site (col, row) they were computed at
-    auto fill = [&](int yr, V2<R>& J, R (&g)[5], R& po) {
+    auto fill = [&](int yr, bool near, V2<R>& J, R (&g)[5], R& po) {
       int ey = yr, ty = -1;
       if (yr < 0) {
         if (d.bc[2]) { ey = 0; ty = d.bc[2]; } else ey = yr + ny;
@@ -239,8 +251,6 @@ __global__ void __launch_bounds__(YM_THREADS, sizeof(R) == 4 ? 3 : 2)
         if (d.bc[3]) { ey = ny - 1; ty = d.bc[3]; } else ey = yr - ny;
       }
       R v[NF];
-      // one path per warp: lanes away from the side pull the same values there
-      const bool near = __any_sync(__activemask(), near_side(d, col, ey));
       if (near) pull_hg_b<S, R, BIG, IO>(a, d, col, ey, J, g, v[0], v[1], po);
       else pull_hg<S, R, BIG>(a, sources(d, col, ey), J, g, v[0], v[1], po);
       const unsigned s0 = site_at(d, col, ey);
@@ -262,10 +272,11 @@ __global__ void __launch_bounds__(YM_THREADS, sizeof(R) == 4 ? 3 : 2)
     V2<R> JC = vec2(R(0), R(0));
     R gC[5], poC = R(0);
     for (int k = 0; k < 2; ++k) {
+      const bool near = near_col || side_row(inside_row(ya - 1 + k));
       if (active) {
         V2<R> J;
         R g[5], po;
-        fill(ya - 1 + k, J, g, po);
+        fill(ya - 1 + k, near, J, g, po);
         if (k == 1) {
           JC = J;
 #pragma unroll
@@ -279,7 +290,7 @@ __global__ void __launch_bounds__(YM_THREADS, sizeof(R) == 4 ? 3 : 2)
       SiteIn<R> in;
       Src9 srcj;
       if (interior) {
-        if (__any_sync(__activemask(), near_side(d, col, j))) {
+        if (near_in || side_row(j)) {
           load_site_b<S, R, BIG, TH, IO>(a, d, col, j, in);
           srcj.s[0] = site_at(d, col, j);
         } else {
@@ -289,7 +300,7 @@ __global__ void __launch_bounds__(YM_THREADS, sizeof(R) == 4 ? 3 : 2)
       }
       V2<R> JL = vec2(R(0), R(0));
       R gL[5], poL = R(0);
-      if (active) fill(j + 1, JL, gL, poL);
+      if (active) fill(j + 1, near_col || side_row(inside_row(j + 1)), JL, gL, poL);
       if (interior) load_grain(a, sd, in);
       __syncthreads();
       if (interior) {
