@@ -217,8 +217,11 @@ pf_status pf_step(pf_handle *h, int n_steps);
  * FP16/BF16 storage and, from 786,432 sites on, for FP32, a chosen by size, at
  * most 48; by default a handle of fewer sites marches the strips unstaged, to the
  * same bits; needs every domain's nx to be a multiple of 16 bytes of storage:
- * 4 FP32, 8 FP16/BF16, 2 FP64 sites).  Synchronises the stream and rebuilds the tile table.
- * Errors: BAD_ARG. */
+ * 4 FP32, 8 FP16/BF16, 2 FP64 sites).  Thermal handles and those with sides take
+ * variant 1 only, though chosen by size they stage their rows too.  What
+ * pf_get_step_config gives is taken back on every handle and keeps the kernels
+ * that run (pinned: later calls do not choose by size again).  Synchronises the
+ * stream and rebuilds the tile table.  Errors: BAD_ARG. */
 pf_status pf_set_step_config(pf_handle *h, int variant, int a, int b);
 
 /* How a step is launched over an ensemble of domains:
@@ -247,8 +250,9 @@ pf_status pf_set_launch(pf_handle *h, int per_domain, int persistent, int graph_
  * persistent.  Errors: BAD_ARG, STATE, OOM, CUDA. */
 pf_status pf_autotune(pf_handle *h, int trial_steps, int out[4]);
 
-/* Current traversal: out[0] variant, out[1] a, out[2] b.  Errors: BAD_ARG
- * (NULL). */
+/* Current traversal: out[0] variant, out[1] a, out[2] b; of the march chosen by
+ * size 2 where it stages its rows, and for FP16/BF16 storage at every size.
+ * Errors: BAD_ARG (NULL). */
 pf_status pf_get_step_config(const pf_handle *h, int out[3]);
 
 /* Copy the fields of the last step of domain dom to host_out (FP64,

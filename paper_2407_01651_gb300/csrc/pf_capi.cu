@@ -60,7 +60,10 @@ struct pf_handle {
   int variant = STEP_YMARCH;  // step kernel traversal
   int tx = 32, ty = 8;      // tile of the 2-D variant
   int chunk = 32;           // rows per tile of the y-march variants
-  int own_chunk = 0;        // 1: set by the caller or the autotuner, else chosen by size
+  // traversal and rows per tile: chosen by size; set by the caller or the
+  // autotuner; or the choice by size, kept by a caller who set what was reported
+  enum { BY_SIZE = 0, SET = 1, KEPT = 2 };
+  int own_chunk = BY_SIZE;
   bool staged_rows = false; // the y-march chosen by size stages its rows (step_variant)
   int ntiles = 0;
   int grid = 0;
@@ -484,14 +487,20 @@ static int chunk_by_size(const pf_handle* h, int sms, int ctas_per_sm) {
 // the staged march.
 constexpr long long STAGE_SITES = 3ll << 18;
 static StepVariant step_variant(const pf_handle* h) {
-  if (h->own_chunk || h->persistent == 2 || h->variant == STEP_TILE)
+  if (h->own_chunk == pf_handle::SET || h->persistent == 2 || h->variant == STEP_TILE)
     return (StepVariant)h->variant;
   if (h->variant == STEP_STAGED && h->drop_copies) return STEP_STAGED;
   return h->staged_rows ? STEP_STAGED : STEP_YMARCH;
 }
 
+// The variant that pf_get_step_config gives: the one a step takes, but of a 16-bit
+// march chosen by size the staged form also where it is small.
+static int reported_variant(const pf_handle* h) {
+  return h->variant == STEP_YMARCH ? (int)step_variant(h) : h->variant;
+}
+
 static pf_status choose_chunk(pf_handle* h) {
-  if (h->own_chunk || h->variant == STEP_TILE) return PF_OK;
+  if (h->own_chunk != pf_handle::BY_SIZE || h->variant == STEP_TILE) return PF_OK;
   long long sites = 0;   // of the largest launch
   for (const DomDesc& d : h->ddesc) {
     const long long n = (long long)d.nx * d.ny;
@@ -1247,6 +1256,13 @@ static bool staged_ok(const pf_handle* h) {
 
 extern "C" pf_status pf_set_step_config(pf_handle* h, int variant, int a, int b) {
   if (!h) return PF_ERR_BAD_ARG;
+  // what pf_get_step_config gave keeps the kernels that it was given for
+  if (h->own_chunk != pf_handle::SET && h->variant != STEP_TILE &&
+      variant == reported_variant(h) && a == h->chunk) {
+    h->own_chunk = pf_handle::KEPT;
+    PF_CUDA(h, cudaStreamSynchronize(h->stream));
+    return PF_OK;
+  }
   if (h->thermal && variant != STEP_YMARCH)
     return fail(h, PF_ERR_BAD_ARG, "thermal mode runs the y-march traversal (variant 1) only");
   if (h->any_bc && variant != STEP_YMARCH)
@@ -1267,7 +1283,7 @@ extern "C" pf_status pf_set_step_config(pf_handle* h, int variant, int a, int b)
   } else {
     return fail(h, PF_ERR_BAD_ARG, "unknown step variant");
   }
-  h->own_chunk = 1;
+  h->own_chunk = pf_handle::SET;
   PF_CUDA(h, cudaStreamSynchronize(h->stream));
   h->variant = variant;
   // captured graphs hold the old tile table's size and chunk: drop them
@@ -1331,11 +1347,11 @@ static pf_status autotune_t(pf_handle* h, int trial_steps, int out[4]) {
   PF_CUDA(h, cudaMemcpyAsync(snap_p, h->pop[cur0], pop_b, cudaMemcpyDeviceToDevice, h->stream));
   PF_CUDA(h, cudaMemcpyAsync(snap_a, h->aux[cur0], aux_b, cudaMemcpyDeviceToDevice, h->stream));
   // own: as pf_set_step_config would take it; else the tiles chosen by size
-  struct Cand { int variant, a, b, persistent, own = 1; };
+  struct Cand { int variant, a, b, persistent, own = pf_handle::SET; };
   std::vector<Cand> cands;
   const int own0 = h->own_chunk;
-  if (!own0)
-    for (int pers : {0, 1}) cands.push_back({h->variant, h->chunk, 0, pers, 0});
+  if (own0 != pf_handle::SET)
+    for (int pers : {0, 1}) cands.push_back({h->variant, h->chunk, 0, pers, own0});
   for (int ch : {4, 8, 16, 24, 32, 48, 64, 96})
     for (int pers : {0, 1}) cands.push_back({STEP_YMARCH, ch, 0, pers});
   if (!h->thermal && !h->any_bc) {
@@ -1415,9 +1431,7 @@ extern "C" pf_status pf_autotune(pf_handle* h, int trial_steps, int out[4]) {
 
 extern "C" pf_status pf_get_step_config(const pf_handle* h, int out[3]) {
   if (!h || !out) return PF_ERR_BAD_ARG;
-  // what pf_set_step_config would take to run the same kernels
-  // (of a 16-bit march by size the staged form of it, also where it is small)
-  out[0] = !h->thermal && !h->any_bc && h->variant == STEP_YMARCH ? (int)step_variant(h) : h->variant;
+  out[0] = reported_variant(h);   // pf_set_step_config takes it back
   out[1] = h->variant != STEP_TILE ? h->chunk : h->tx;
   out[2] = h->variant == STEP_TILE ? h->ty : 0;
   return PF_OK;
@@ -1637,7 +1651,7 @@ extern "C" pf_status pf_run(pf_handle* h, const double* fields6, size_t n, int n
   int B = std::min(PF_RUN_BANDS, ((dd.ny + th - 1) / th) / 4);
   // tiles chosen by size are short on a small lattice, whose bands would step
   // faster than the host can launch them one by one: 2^18 sites a band (13 us)
-  if (!h->own_chunk) B = (int)std::min<size_t>(B, nn >> 18);
+  if (h->own_chunk != pf_handle::SET) B = (int)std::min<size_t>(B, nn >> 18);
   if (n_steps == 0 || h->thermal || h->any_bc || B < 3) {
     // one after the other
     pf_status st = pf_set_fields(h, 0, fields6, nullptr, n);
@@ -1790,7 +1804,7 @@ extern "C" pf_status pf_set_boundaries(pf_handle* h, int dom, const int bc[4]) {
     }
   if (h->any_bc && h->variant != STEP_YMARCH) {
     h->variant = STEP_YMARCH;
-    h->own_chunk = 0;
+    h->own_chunk = pf_handle::BY_SIZE;
   }
   pf_status cs = choose_chunk(h);
   if (cs != PF_OK) return cs;
