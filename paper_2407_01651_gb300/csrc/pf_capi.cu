@@ -623,11 +623,13 @@ static pf_status upload_tables(pf_handle* h) {
   return PF_OK;
 }
 
-// Grain table of a domain: the given angles, then the lattice's own frame.
-static pf_status upload_grain_table(pf_handle* h, int dom, const std::vector<double>& angles) {
+// Grain table of a domain, or of `doms` domains from it on alike: the given
+// angles, then the lattice's own frame.
+static pf_status upload_grain_table(pf_handle* h, int dom, const std::vector<double>& angles,
+                                    int doms = 1) {
   return dispatch(h, [&](auto s_t, auto r_t) {
     PF_TYPES(s_t, r_t);
-    std::vector<GrainCS<R>> cs(MAX_GRAINS, GrainCS<R>{R(1), R(0)});
+    std::vector<GrainCS<R>> cs((size_t)doms * MAX_GRAINS, GrainCS<R>{R(1), R(0)});
     for (size_t i = 0; i < angles.size(); ++i)
       cs[i] = GrainCS<R>{(R)std::cos(angles[i]), (R)std::sin(angles[i])};
     PF_CUDA(h, cudaMemcpyAsync(reinterpret_cast<GrainCS<R>*>(h->grain_cs) + (size_t)dom * MAX_GRAINS,
@@ -728,9 +730,8 @@ extern "C" pf_status pf_create(const pf_params* p, const pf_domain* doms, int n_
       cudaMemsetAsync(h->d_tied, 0, tied_b, h->stream) != cudaSuccess ||
       cudaMemsetAsync(h->grain, 0, ps, h->stream) != cudaSuccess)
     return bail(PF_ERR_CUDA, "memset failed");
-  for (int d = 0; d < n_doms; ++d)
-    if (upload_grain_table(h, d, {}) != PF_OK)
-      return bail(PF_ERR_CUDA, "grain table upload failed");
+  if (upload_grain_table(h, 0, {}, n_doms) != PF_OK)
+    return bail(PF_ERR_CUDA, "grain table upload failed");
   // default traversal: the staged y-march for the 16-bit storage forms
   // (measured faster at 4096^2), the plain y-march otherwise
   if ((prec == PF_FP16_OFFSET || prec == PF_BF16_OFFSET) && staged_ok(h))
