@@ -430,7 +430,7 @@ static void release(pf_handle* h) {
 // the chip on a small one.  Whole waves up to four; beyond that the CTAs run
 // out of step and only half a wave is lost at the end.  Measured (us per step at
 // 32 rows and at the rows chosen, before steps were chained; now in brackets):
-// FP32 128^2 43.1 -> 6.2 (1 row) [4.4], 256^2 45.1 -> 8.2 (1) [7.0], 512^2 45.1 ->
+// FP32 128^2 43.1 -> 6.2 (1 row) [4.4], 256^2 45.1 -> 8.2 (1) [7.0], 512^2 51.1 ->
 // 18.5 (4) [16.4]; staged 1024^2 88.0 -> 55.3 (14), 2048^2 206 -> 183 (27), 4096^2
 // 679 -> 676 (36).
 // FP64 is bound by the FP64 units, so there the SM with the most tiles sets the

@@ -106,7 +106,10 @@ __device__ __forceinline__ R lap18(const R (*Pm)[HX], const R (*P0)[HX], const R
 // CTAs: `top` where that gives waves enough, else the length whose tiles, each
 // with 2 warm-up planes and the columns' last ones shorter, end first. `alone`:
 // what a plane takes longer where a tile has an SM to itself; a shorter length
-// has to be `gain` ahead. Chosen once per handle.
+// has to be `gain` ahead. Chosen once per handle. Between the small lattices and
+// 256^3, where `top` was tuned (us per step by this rule, and the best of six
+// lengths): FP32 two-phase 160^3 477.7, 192^3 815.4, 224^3 1272, all the best; melt
+// 160^3 140.7 (24 planes 137.6), 192^3 236.1 (20: 228.7), 224^3 365.1 (24: 353.0).
 inline int planes_by_size(int nx, int ny, int nz, int ty, int slots, int top, double alone,
                           double gain) {
   const long long xy = (long long)((nx + TX - 1) / TX) * ((ny + ty - 1) / ty);
