@@ -1223,8 +1223,9 @@ static pf_status step_n(pf_handle* h, int n_steps) {
     if ((st = step_tied_t<S, R>(h, n_steps)) != PF_OK) return st;
     return step_rest<S, R>(h, n_steps, 1, true);
   }
-  if ((st = settle_raw(h)) != PF_OK) return st;
   int done = 0;
+  // (an entry that a graph has overwritten is out of the table already: the kernel
+  // then leaves the domain as the step made it)
   if (h->n_raw && any_raw(h)) {
     if ((st = step_tied_t<S, R>(h, n_steps)) != PF_OK) return st;
     done = 1;

@@ -133,3 +133,28 @@ def test_thermal_calls_between_replays():
         del g
         sim.close()
         ref.close()
+
+
+def test_steps_behind_a_replay_do_not_wait():
+    """pf_step on a state that a replay has used enqueues and returns, also while
+    the host has not looked whether it is raw still."""
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        sim, ref = handle("fp32", 0, None, (0, 0, 0)), handle("fp32", 0, None, (0, 0, 0))
+        raw = general(ref.get_state(1), 0, 11)
+        sim.sync()
+        g = capture(sim, stream, 30)
+        for s in (sim, ref):
+            s.set_state(1, raw)
+        torch.cuda.synchronize()
+        for _ in range(20):
+            g.replay()
+        done = torch.cuda.Event()
+        done.record()
+        sim.step(1)              # about 5 ms of replays are in front of it
+        assert not done.query()
+        ref.step(601)
+        assert all(np.array_equal(x, y) for x, y in zip(states(sim), states(ref)))
+        del g
+        sim.close()
+        ref.close()
